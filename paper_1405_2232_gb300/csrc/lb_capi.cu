@@ -517,15 +517,18 @@ lb_status create(const lb_params* p, void* stream, lb_ctx** out) {
     if (strip && !c->fd && !c->kp.walls &&
         (p->precision == LB_PREC_FP16_DEV || p->precision == LB_PREC_BF16_DEV)) {
         // the 16-bit strip kernel stores each collided row of a strip with
-        // one tensor copy: dims (nx columns, ny rows, planes), box (strip
-        // width, 1 row, every plane); columns past nx are clipped by the copy
+        // one tensor copy: dims (the columns in whole 16-byte units, ny rows,
+        // planes), box (strip width, 1 row, every plane); the copy clips the
+        // columns past the map (a lattice narrower than one unit never
+        // stores through its map)
         PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
         if (!enc) {
             release(c);
             return fail(LB_ERR_CUDA, "the driver provides no cuTensorMapEncodeTiled");
         }
         const int npl = pop_planes(p->precision);
-        const cuuint64_t dims[3] = {(cuuint64_t)p->nx, (cuuint64_t)p->ny, (cuuint64_t)npl};
+        const cuuint64_t dims[3] = {(cuuint64_t)(p->nx < 8 ? 8 : dev_map_columns(p->nx)), (cuuint64_t)p->ny,
+                                    (cuuint64_t)npl};
         const cuuint64_t strides[2] = {(cuuint64_t)(pitch * (long long)es), (cuuint64_t)(plane * (long long)es)};
         const cuuint32_t box[3] = {(cuuint32_t)c->p.tile_x, 1, (cuuint32_t)npl};
         const cuuint32_t estr[3] = {1, 1, 1};

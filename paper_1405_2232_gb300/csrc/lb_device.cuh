@@ -309,6 +309,10 @@ constexpr int STRIP_GHOST = 2;
 constexpr int FD_HALO = 4;
 constexpr int FD_GHOST = 3;
 
+// Columns of a row that the 16-bit strip kernel stores through its tensor map:
+// the whole 16-byte units of the row.
+__host__ __device__ constexpr int dev_map_columns(int nx) { return nx & ~7; }
+
 // Periodic ghost columns of the strip layout: the value stored at column x of
 // a row is also stored at column x + nx when x < kp.ghost and at x - nx when
 // x >= nx - kp.ghost, so that a row segment with its column halo is one

@@ -14,9 +14,11 @@
 //     into buffer m mod 3, laid out [plane][column]) and leave the CTA as
 //     one tensor copy each (cp.async.bulk.tensor.3d shared -> global through
 //     the map of the destination buffer: x the column, y the row, z the
-//     plane; the copy clips the columns past nx), so no thread forms twenty
-//     64-bit store addresses per site; the periodic ghost copies of the edge
-//     columns are stored by their threads directly.  Lane 0 of the halo warp
+//     plane), so no thread forms twenty 64-bit store addresses per site; the
+//     periodic ghost copies of the edge columns are stored by their threads
+//     directly, and so are the last nx mod 8 columns: a tensor copy writes
+//     whole 16-byte units, so a map that ended inside a unit would overwrite
+//     the ghost columns beside it (dev_map_columns);  lane 0 of the halo warp
 //     issues the copies (twenty per-plane bulk copies, whose operands are
 //     uniform registers, made the issuing warp step through its lanes one by
 //     one, which loaded its SM sub-partition more than the others): after
@@ -109,7 +111,7 @@ template <class S, int SEGW, int BX, bool EQ24>
 __device__ __forceinline__ void dev_collide_site(const KParams& kp, const typename S::elem* st, int c, float Hf,
                                                  float Hg, float Fx, float Fy, typename S::elem* d,
                                                  typename S::elem* o, uint32_t plane, bool ghost_lo,
-                                                 bool ghost_hi) {
+                                                 bool ghost_hi, bool tail) {
     constexpr int NPL = S::NPLANES;
     float h[9], q[9];
 #pragma unroll
@@ -123,6 +125,10 @@ __device__ __forceinline__ void dev_collide_site(const KParams& kp, const typena
 #pragma unroll
     for (int p = 0; p < NPL; ++p) o[p * BX] = v[p];
     fence_proxy_async_smem();
+    if (tail) {
+#pragma unroll
+        for (int p = 0; p < NPL; ++p) d[(size_t)p * plane] = v[p];
+    }
     put_ghost_copies<S>(d, plane, kp.nx, v, ghost_lo, ghost_hi);
 }
 
@@ -192,8 +198,10 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     const int r_psi = halo ? (lane == 0 ? 0 : W + 1) : t + 1;
     const bool has_psi = halo ? lane < 2 : t < W;
     const int c_psi = r_psi - 1 + HALO;   // smem column of the psi site
-    const bool issuer = halo && lane == 0;  // copies the collided rows out
+    // copies the collided rows out (a strip with no whole 16-byte unit has none)
+    const bool issuer = halo && lane == 0 && x0 < dev_map_columns(nx);
     const int xg = x0 + t;
+    const bool tail = xg >= dev_map_columns(nx);
     const bool ghost_lo = xg < STRIP_GHOST, ghost_hi = xg >= nx - STRIP_GHOST;
     const int c = t + HALO;               // smem column of the collided site
     int flags = 0;
@@ -268,7 +276,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     dev_collide_site<S, SEGW, BX, EQ24>(kp, stage + sm * (NPL * SEGW), c, Hf_p, Hg_p, FxA, FyA,
                                                         dst + ((size_t)y * pitch + (size_t)xg),
                                                         outb + (size_t)bA * NPL * BX + t, plane,
-                                                        ghost_lo, ghost_hi);
+                                                        ghost_lo, ghost_hi, tail);
                 }
                 __syncwarp();
                 if (lane == 0) mbar_arrive(written);
@@ -277,7 +285,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     dev_collide_site<S, SEGW, BX, EQ24>(kp, stage + s0 * (NPL * SEGW), c, Hf_0, Hg_0, FxB, FyB,
                                                         dst + ((size_t)y * pitch + (size_t)xg),
                                                         outb + (size_t)b0 * NPL * BX + t, plane,
-                                                        ghost_lo, ghost_hi);
+                                                        ghost_lo, ghost_hi, tail);
                 }
             } else {
                 __syncwarp();

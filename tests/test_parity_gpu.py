@@ -495,3 +495,22 @@ def test_16bit_slab_error_report(lb, prec):
     print(f"{prec} slab 64^2 200 steps: e_rho={e[0]:.3e} e_u={e[1]:.3e} e_T={e[2]:.3e}")
     bound = 0.05 if prec == "fp16" else 0.5
     assert np.all(np.isfinite(m[0])) and e[0] < bound and e[2] < bound
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec,u", [("fp16", 2.0 ** -11), ("bf16", 2.0 ** -8)])
+@pytest.mark.parametrize("nx,ny", [(1021, 37), (490, 41), (257, 24), (263, 16), (5, 32)])
+def test_16bit_strip_ragged_columns_over_several_steps(lb, prec, u, nx, ny):
+    """Widths that are not whole 16-byte units on the 16-bit strip kernel, 20
+    steps: the ghost columns beside the last column keep the periodic copies.
+    Each step rounds the eight moving deviations (|h| < 0.03 here) with unit
+    roundoff u, so rho differs from FP32 by at most 20 * 8 * 0.03 u."""
+    rho, T = I.spinodal_fields(nx, ny)
+    out = {}
+    for p in ("fp32", prec):
+        with lb.Lattice(rho, T, nx=nx, ny=ny, precision=p, beta=1.3, tile_x=256, tile_y=0, psi_uses_local_T=0,
+                        T_psi=0.75 * I.CS_TC) as L:
+            L.step(20)
+            L.synchronize()
+            out[p] = L.moments()[0]
+    assert np.abs(out[prec] - out["fp32"]).max() <= 20 * 8 * 0.03 * u
