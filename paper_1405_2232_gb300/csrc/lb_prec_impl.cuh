@@ -62,16 +62,20 @@ constexpr int strip_stages() {
 }
 
 // 16-bit deviation storage: k_step_strip_dev; FP32 / FP64: k_step_strip.
-template <int BX, int ST, bool EQ24, int BM>
+// (TAIL: the width is not in whole 16-byte units)
+template <int BX, int ST, bool EQ24, int BM, bool TAIL>
 auto strip_kernel() {
     if constexpr (Store<LBGB_PREC>::SPLIT)
-        return k_step_strip_dev<LBGB_PREC, BX, ST, EQ24, BM>;
+        return k_step_strip_dev<LBGB_PREC, BX, ST, EQ24, BM, TAIL>;
     else
         return k_step_strip<LBGB_PREC, BX, ST, EQ24, BM>;
 }
 
-template <int BX, bool EQ24, int BM>
+template <int BX, bool EQ24, int BM, bool TAIL = false>
 cudaError_t strip_launch(const StepLaunch& L) {
+    if constexpr (Store<LBGB_PREC>::SPLIT && !TAIL) {
+        if (dev_map_columns(L.kp.nx) != L.kp.nx) return strip_launch<BX, EQ24, BM, true>(L);
+    }
     using E = typename Store<LBGB_PREC>::elem;
     constexpr int ST = strip_stages<BX>();
     static_assert(ST >= 3, "strip kernel needs at least three stages");
@@ -79,7 +83,7 @@ cudaError_t strip_launch(const StepLaunch& L) {
     constexpr size_t smem =
         DEV ? strip_dev_smem_bytes<LBGB_PREC, BX, ST>() : strip_smem_bytes<LBGB_PREC, BX, ST>();
     static_assert(smem <= 110 * 1024, "two CTAs per SM");
-    auto kern = strip_kernel<BX, ST, EQ24, BM>();
+    auto kern = strip_kernel<BX, ST, EQ24, BM, TAIL>();
     static unsigned long long configured = 0;  // per instantiation, one bit per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -107,7 +107,7 @@ __device__ __forceinline__ void dev_psi_site(const KParams& kp, const typename S
 // Eq. (1) + F_i and Eq. (7) / (24) for one site: its stored form into row
 // buffer column o (fenced for the tensor copy), the ghost copies of an edge
 // column straight to its planes at d.
-template <class S, int SEGW, int BX, bool EQ24>
+template <class S, int SEGW, int BX, bool EQ24, bool TAIL>
 __device__ __forceinline__ void dev_collide_site(const KParams& kp, const typename S::elem* st, int c, float Hf,
                                                  float Hg, float Fx, float Fy, typename S::elem* d,
                                                  typename S::elem* o, uint32_t plane, bool ghost_lo,
@@ -125,14 +125,19 @@ __device__ __forceinline__ void dev_collide_site(const KParams& kp, const typena
 #pragma unroll
     for (int p = 0; p < NPL; ++p) o[p * BX] = v[p];
     fence_proxy_async_smem();
-    if (tail) {
+    if constexpr (TAIL) {
+        if (tail) {
 #pragma unroll
-        for (int p = 0; p < NPL; ++p) d[(size_t)p * plane] = v[p];
+            for (int p = 0; p < NPL; ++p) d[(size_t)p * plane] = v[p];
+        }
     }
     put_ghost_copies<S>(d, plane, kp.nx, v, ghost_lo, ghost_hi);
 }
 
-template <int PREC, int BX, int STAGES, bool EQ24, int BMODE>
+// TAIL: nx is not a multiple of 8, so the last columns are stored by their
+// threads (a variant of its own: the store's code alone cost the aligned widths
+// 3 - 7%).
+template <int PREC, int BX, int STAGES, bool EQ24, int BMODE, bool TAIL>
 __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     k_step_strip_dev(const typename Store<PREC>::elem* __restrict__ src,
                      typename Store<PREC>::elem* __restrict__ dst, const KParams kp, int nchunks,
@@ -199,9 +204,9 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     const bool has_psi = halo ? lane < 2 : t < W;
     const int c_psi = r_psi - 1 + HALO;   // smem column of the psi site
     // copies the collided rows out (a strip with no whole 16-byte unit has none)
-    const bool issuer = halo && lane == 0 && x0 < dev_map_columns(nx);
+    const bool issuer = halo && lane == 0 && (!TAIL || x0 < dev_map_columns(nx));
     const int xg = x0 + t;
-    const bool tail = xg >= dev_map_columns(nx);
+    const bool tail = TAIL && xg >= dev_map_columns(nx);
     const bool ghost_lo = xg < STRIP_GHOST, ghost_hi = xg >= nx - STRIP_GHOST;
     const int c = t + HALO;               // smem column of the collided site
     int flags = 0;
@@ -273,7 +278,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     ring_psi2 + qm1 * RW + r, ring_psi2 + q * RW + r, ring_psi2 + (q + 1) * RW + r, FxB, FyB);
                 if (c0) {
                     const int y = y_start - 1 + m0;
-                    dev_collide_site<S, SEGW, BX, EQ24>(kp, stage + sm * (NPL * SEGW), c, Hf_p, Hg_p, FxA, FyA,
+                    dev_collide_site<S, SEGW, BX, EQ24, TAIL>(kp, stage + sm * (NPL * SEGW), c, Hf_p, Hg_p, FxA, FyA,
                                                         dst + ((size_t)y * pitch + (size_t)xg),
                                                         outb + (size_t)bA * NPL * BX + t, plane,
                                                         ghost_lo, ghost_hi, tail);
@@ -282,7 +287,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                 if (lane == 0) mbar_arrive(written);
                 if (c1) {
                     const int y = y_start - 1 + m1;
-                    dev_collide_site<S, SEGW, BX, EQ24>(kp, stage + s0 * (NPL * SEGW), c, Hf_0, Hg_0, FxB, FyB,
+                    dev_collide_site<S, SEGW, BX, EQ24, TAIL>(kp, stage + s0 * (NPL * SEGW), c, Hf_0, Hg_0, FxB, FyB,
                                                         dst + ((size_t)y * pitch + (size_t)xg),
                                                         outb + (size_t)b0 * NPL * BX + t, plane,
                                                         ghost_lo, ghost_hi, tail);
