@@ -265,13 +265,13 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                 {
                     const int r = r_psi;
                     const int c = r - 1 + HALO;
-                    real f[9], g[9], rho, T, psi, psi2;
+                    real f[9], g[9], rho, e, T, psi, psi2;
 #pragma unroll
                     for (int i = 0; i < 9; ++i) {
                         f[i] = S::load(st + i * SEGW + c - ex(i), (real)kp.base_f[i]);
                         g[i] = S::load(st + (9 + i) * SEGW + c - ex(i), (real)kp.base_g[i]);
                     }
-                    site_psi<real, BMODE>(kp, f, g, rho, T, psi, psi2, flags);
+                    site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
                     if (BMODE != BETA_ZERO) rp[r] = psi;
                     if (BMODE != BETA_ONE) rq[r] = psi2;
                 }

@@ -43,14 +43,14 @@ __global__ void __launch_bounds__(CAV_BX* CAV_BY)
     for (int s = tid; s < WX * WY; s += NT) {
         const int ly = s / WX, lx = s - ly * WX;
         const int gx = clampc(x0 + lx - 1, nx), gy = clampc(y0 + ly - 1, ny);
-        real f[9], g[9], rho, T, psi, psi2;
+        real f[9], g[9], rho, e, T, psi, psi2;
         const long long off = (long long)gy * kp.pitch + gx;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             f[i] = S::load(src + (long long)i * kp.plane + off, (real)kp.base_f[i]);
             g[i] = S::load(src + (long long)(9 + i) * kp.plane + off, (real)kp.base_g[i]);
         }
-        site_psi<real, BMODE>(kp, f, g, rho, T, psi, psi2, flags);
+        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
         if (BMODE != BETA_ZERO) s_psi[s] = psi;
         if (BMODE != BETA_ONE) s_psi2[s] = psi2;
     }
@@ -126,14 +126,14 @@ __global__ void __launch_bounds__(CAV_BX* CAV_BY)
     for (int s = tid; s < WX * WY; s += NT) {
         const int ly = s / WX, lx = s - ly * WX;
         const int gx = clampc(x0 + lx - 1, nx), gy = clampc(y0 + ly - 1, ny);
-        real f[9], g[9], rho, T, psi, psi2;
+        real f[9], g[9], rho, e, T, psi, psi2;
         const long long off = (long long)gy * kp.pitch + gx;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
             f[i] = S::load(src + (long long)i * kp.plane + off, (real)kp.base_f[i]);
             g[i] = S::load(src + (long long)(9 + i) * kp.plane + off, (real)kp.base_g[i]);
         }
-        site_psi<real, BMODE>(kp, f, g, rho, T, psi, psi2, flags);
+        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
         if (BMODE != BETA_ZERO) s_psi[s] = psi;
         if (BMODE != BETA_ONE) s_psi2[s] = psi2;
     }

@@ -17,6 +17,8 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include "lb.h"
 
 namespace lbgb {
@@ -196,10 +198,16 @@ struct KParams {
     int halo_rows;               // 0: periodic in y; H > 0: rows [0, H) and [ny - H, ny) are ghost
                                  // rows of a y-decomposed lattice, the step updates [H, ny - H)
     // 16-bit modes, collision in deviation variables (collide_dev):
+    // FP64 step: products and scalings of the parameters above that are formed
+    // once on the host (kp_fill_derived); each is the double the printed
+    // formula forms per site
+    double b4;                   // b / 4 (exact)
+    double gw[3], cwc[3];        // guo_pre w and corr_pre w c_v (rest, axis, diagonal)
+    int g_pow2;                  // |G| is a power of two: 2 x / G = x (2 / G), both exact scalings
     float sum_bf, sum_bg;        // sum_i base_f[i], sum_i base_g[i]
     float dsum_f, dsum_g;        // sum_i base_f[i] - rho0, sum_i base_g[i] - rho0 c_v T0
     float cw_f[3], cw_g[3];      // w rho0 - base_f, w rho0 c_v T0 - base_g (rest, axis, diagonal)
-    // the doubles above rounded to float once on the host (kp_fill_float):
+    // the doubles above rounded to float once on the host (kp_fill_derived):
     // the 16-bit kernels read these (KPR, collide_dev), since converting a
     // double at each use runs on the FP64 pipe, which is narrow on this GPU
     struct {
@@ -217,8 +225,16 @@ struct KParams {
     } d;
 };
 
-// Set KParams::f from the double fields (call after they are final).
-inline void kp_fill_float(KParams& k) {
+// Set the fields derived from the double parameters (call after they are final).
+inline void kp_fill_derived(KParams& k) {
+    k.b4 = k.b * 0.25;
+    for (int c = 0; c < 3; ++c) {
+        const double w = wd(c == 0 ? 0 : (c == 1 ? 1 : 5));
+        k.gw[c] = k.guo_pre * w;
+        k.cwc[c] = k.corr_pre * w * k.cv;
+    }
+    int ex2 = 0;
+    k.g_pow2 = std::frexp(std::fabs(k.G), &ex2) == 0.5 && ex2 > -1000 && ex2 < 1000;
     k.f.omega_f = (float)k.omega_f;
     k.f.omega_g = (float)k.omega_g;
     k.f.guo_pre = (float)k.guo_pre;
@@ -278,19 +294,57 @@ constexpr long long WAIT_CYCLES_DEFAULT = 2000000000LL;
 
 enum BetaMode { BETA_ZERO = 0, BETA_ONE = 1, BETA_MIXED = 2 };
 
+// Division of the FP64 mode by its two constants, c_s^2 = fl(1/3) and
+// c_s^4 = fl(c_s^2 c_s^2), in two operations with the correctly rounded
+// result.  c_s^2 = (1 - 2^-54)/3, so x / c_s^2 = 3x (1 + 2^-54 + 2^-108 ...): the
+// fused multiply-add rounds 3x + fl(3x 2^-54) once, and what is dropped (below
+// 2^-106 of the quotient) cannot reach a rounding boundary: the quotients closest
+// to one (for each small r, the x with 2x 2^k = (2q + 1) c + r on the integer
+// mantissas) were enumerated and all round alike.  The same holds for
+// 1 / c_s^4 = 9 (1 + 2^-54 ...).  Exact for any x of magnitude above 2^-900 (below,
+// the product may lose bits of a term that is added to a population, where it
+// is absorbed).  The GPU's FP64 units take one warp instruction per 16 cycles
+// of an SM and bound every FP64 kernel; a general division is about nine of
+// them.  With these, each printed product shared between opposite directions
+// and the site's rho, sum g and T carried from its psi to its collision, the
+// strip step of a 384 x 320 lattice went from 232 to 130 us, the 150 x 150 cavity
+// from 53 to 31 us.
+template <int HALVES = 0>  // HALVES = 1: of x / 2
+__device__ __forceinline__ double div_cs2(double x) {
+    constexpr double m = HALVES ? 1.5 : 3.0;
+    return fma(m, x, x * (m * 0x1p-54));
+}
+template <int HALVES = 0>
+__device__ __forceinline__ double div_cs4(double x) {
+    constexpr double m = HALVES ? 4.5 : 9.0;
+    return fma(m, x, x * (m * 0x1p-54));
+}
+
+// isfinite(x) and x < 0 of a double on the integer units (the comparison
+// instruction would take an FP64 slot)
+__device__ __forceinline__ bool finite_bits(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool negative_bits(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x), mag = hi & 0x7fffffffu;
+    return (hi >> 31) && (mag | lo) != 0u && (mag < 0x7ff00000u || (mag == 0x7ff00000u && lo == 0u));
+}
+__device__ __forceinline__ bool finite_bits(float x) { return isfinite(x); }
+__device__ __forceinline__ bool negative_bits(float x) { return x < 0.0f; }
+
 template <typename real>
 __device__ __forceinline__ real p_eos(const KParams& kp, real rho, real T) {
     const real R = KPR(kp, R), a = KPR(kp, a), b = KPR(kp, b);
     if (kp.eos == LB_EOS_IDEAL) return rho * R * T;
     if (kp.eos == LB_EOS_VDW) return rho * R * T / ((real)1 - b * rho) - a * rho * rho;
     // Carnahan-Starling, eta = b rho / 4
-    const real eta = b * rho / (real)4;
     if constexpr (sizeof(real) == 8) {
         // FP64 parity mode: the printed polynomial, evaluated term by term
+        // (the division by 4 is exact, so it is taken on b)
+        const real eta = kp.b4 * rho;
         const real num = (real)1 + eta + eta * eta - eta * eta * eta;
         const real den = ((real)1 - eta) * ((real)1 - eta) * ((real)1 - eta);
         return rho * R * T * num / den - a * rho * rho;
     } else {
+        const real eta = b * rho / (real)4;
         const real num = (real)1 + eta * ((real)1 + eta * ((real)1 - eta));
         const real d = (real)1 - eta;
         return rho * R * T * num / (d * d * d) - a * rho * rho;
@@ -505,29 +559,43 @@ __device__ __forceinline__ void pull18_dev(const typename S::elem* __restrict__ 
     }
 }
 
-// rho, T and the pseudopotential (psi^2, and psi when beta != 0) of one site.
+// The pseudopotential (psi^2, and psi when beta != 0) of a site of density r
+// and temperature T.
+template <typename real, int BMODE>
+__device__ __forceinline__ void site_psi_T(const KParams& kp, real r, real T, real& psi, real& psi2,
+                                           int& flags) {
+    const real Te = kp.psi_local_T ? T : KPR(kp, T_psi);
+    if constexpr (sizeof(real) == 8) {
+        const real d = p_eos<real>(kp, r, Te) - r * (real)(1.0 / 3.0);
+        if (kp.g_pow2)
+            psi2 = d * kp.two_over_G;
+        else
+            psi2 = (real)2 * d / kp.G;
+    } else {
+        psi2 = (p_eos<real>(kp, r, Te) - r * (real)(1.0 / 3.0)) * KPR(kp, two_over_G);
+    }
+    psi = (real)0;
+    if (BMODE != BETA_ZERO) {
+        if (negative_bits(psi2)) flags |= 1 << LB_ERR_PSI_DOMAIN;
+        psi = sqrt(psi2);
+    }
+    if (!finite_bits(r) || !finite_bits(T)) flags |= 1 << LB_ERR_NONFINITE;
+}
+
+// rho, the energy density e = sum g, T and the pseudopotential of one site.
 template <typename real, int BMODE>
 __device__ __forceinline__ void site_psi(const KParams& kp, const real f[9], const real g[9],
-                                         real& rho, real& T, real& psi, real& psi2, int& flags) {
-    real r = f[0], e = g[0];
+                                         real& rho, real& e, real& T, real& psi, real& psi2, int& flags) {
+    real r = f[0], es = g[0];
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
         r += f[i];
-        e += g[i];
+        es += g[i];
     }
     rho = r;
-    T = e / (r * KPR(kp, cv));
-    const real Te = kp.psi_local_T ? T : KPR(kp, T_psi);
-    if constexpr (sizeof(real) == 8)
-        psi2 = (real)2 * (p_eos<real>(kp, r, Te) - r * (real)(1.0 / 3.0)) / KPR(kp, G);
-    else
-        psi2 = (p_eos<real>(kp, r, Te) - r * (real)(1.0 / 3.0)) * KPR(kp, two_over_G);
-    psi = (real)0;
-    if (BMODE != BETA_ZERO) {
-        if (psi2 < (real)0) flags |= 1 << LB_ERR_PSI_DOMAIN;
-        psi = sqrt(psi2);
-    }
-    if (!isfinite(r) || !isfinite(T)) flags |= 1 << LB_ERR_NONFINITE;
+    e = es;
+    T = es / (r * KPR(kp, cv));
+    site_psi_T<real, BMODE>(kp, r, T, psi, psi2, flags);
 }
 
 // Eq. (4) force (Eq. (2) when beta = 1) from a shared-memory window with
@@ -539,6 +607,7 @@ __device__ __forceinline__ void force_from_window(const KParams& kp, const real*
                                                   real& Fx, real& Fy) {
     const real w1 = (real)(1.0 / 3.0), w2 = (real)(1.0 / 12.0);
     real fx = 0, fy = 0;
+    constexpr bool first = sizeof(real) == 8;  // FP64: no 0 + x (the compiler keeps it for x = -0)
     if (BMODE != BETA_ZERO) {
         const real* p = s_psi;
         const real E = p[c + 1], Wv = p[c - 1], N = p[c + W], S = p[c - W];
@@ -547,8 +616,8 @@ __device__ __forceinline__ void force_from_window(const KParams& kp, const real*
         const real s1x = w1 * (E - Wv) + w2 * (d1 + d2);
         const real s1y = w1 * (N - S) + w2 * (d1 + d3);
         const real pc = (BMODE == BETA_ONE) ? p[c] : KPR(kp, beta) * p[c];
-        fx += pc * s1x;
-        fy += pc * s1y;
+        fx = first ? pc * s1x : fx + pc * s1x;
+        fy = first ? pc * s1y : fy + pc * s1y;
     }
     if (BMODE != BETA_ONE) {
         const real* p = s_psi2;
@@ -558,8 +627,8 @@ __device__ __forceinline__ void force_from_window(const KParams& kp, const real*
         const real s2x = w1 * (E - Wv) + w2 * (d1 + d2);
         const real s2y = w1 * (N - S) + w2 * (d1 + d3);
         const real h = (BMODE == BETA_ZERO) ? (real)0.5 : KPR(kp, half_1mbeta);
-        fx += h * s2x;
-        fy += h * s2y;
+        fx = first && BMODE == BETA_ZERO ? h * s2x : fx + h * s2x;
+        fy = first && BMODE == BETA_ZERO ? h * s2y : fy + h * s2y;
     }
     Fx = -KPR(kp, G) * fx;
     Fy = -KPR(kp, G) * fy;
@@ -579,54 +648,69 @@ __device__ __forceinline__ void force_from_window(const KParams& kp, const real*
 // kp.d, (1 - omega) f_i + P +- Q (see below); measured faster in the fused
 // finite-difference kernel (+2.6%), slower in the strip and batched steps
 // (-8% and -0.5%), which keep the direct form.
-template <typename real, bool EQ24, bool FMA = false>
-__device__ __forceinline__ void collide(const KParams& kp, real f[9], real g[9], real rho,
-                                        real Fx, real Fy, real& ux_out, real& uy_out,
-                                        real& T_out) {
+// GIVEN: e = sum g and T are the caller's (formed with the site's psi), else
+// they are formed here.
+template <typename real, bool EQ24, bool FMA, bool GIVEN>
+__device__ __forceinline__ void collide_et(const KParams& kp, real f[9], real g[9], real rho, real e, real& T,
+                                           real Fx, real Fy, real& ux_out, real& uy_out) {
     if constexpr (sizeof(real) == 8) {
-        const double cs2 = 1.0 / 3.0;
+        if constexpr (!GIVEN) {
+            e = g[0];
+#pragma unroll
+            for (int i = 1; i < 9; ++i) e += g[i];
+            T = e / (rho * kp.cv);
+        }
         // sum_i e_i f_i in index order
         const double mx = ((((f[1] - f[3]) + f[5]) - f[6]) - f[7]) + f[8];
         const double my = ((((f[2] - f[4]) + f[5]) + f[6]) - f[7]) - f[8];
-        double e = g[0];
-#pragma unroll
-        for (int i = 1; i < 9; ++i) e += g[i];
         const double ux = (mx + 0.5 * Fx) / rho;
         const double uy = (my + 0.5 * Fy) / rho;
-        const double T = e / (rho * kp.cv);
-        const double usq = ux * ux + uy * uy;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            const double w = wd(i);
-            // e_i.u, e_i.F with the zero components dropped (exact)
-            const double eu = ex(i) == 0 ? (ey(i) == 0 ? 0.0 : (ey(i) > 0 ? uy : -uy))
-                                         : (ey(i) == 0 ? (ex(i) > 0 ? ux : -ux)
-                                                       : (ex(i) > 0 ? ux : -ux) + (ey(i) > 0 ? uy : -uy));
-            const double eF = ex(i) == 0 ? (ey(i) == 0 ? 0.0 : (ey(i) > 0 ? Fy : -Fy))
-                                         : (ey(i) == 0 ? (ex(i) > 0 ? Fx : -Fx)
-                                                       : (ex(i) > 0 ? Fx : -Fx) + (ey(i) > 0 ? Fy : -Fy));
-            const double emuF = ((double)ex(i) - ux) * Fx + ((double)ey(i) - uy) * Fy;
-            const double feq = rho * w * (1.0 + eu / cs2 + 0.5 * eu * eu / (cs2 * cs2) - 0.5 * usq / cs2);
-            const double Fi = kp.guo_pre * w * (emuF / cs2 + eu * eF / (cs2 * cs2));
+        const double cu = div_cs2<1>(ux * ux + uy * uy);  // 0.5 u^2 / cs^2
+        const double cvT = kp.cv * T;
+        // (e_i - u).F = (e_ix - ux) Fx + (e_iy - uy) Fy from its products, by e_ix, e_iy in {0, 1, -1}
+        const double ax[3] = {-(ux * Fx), (1.0 - ux) * Fx, (-1.0 - ux) * Fx};
+        const double ay[3] = {-(uy * Fy), (1.0 - uy) * Fy, (-1.0 - uy) * Fy};
+        auto emuF = [&](int i) {
+            return ax[ex(i) == 0 ? 0 : (ex(i) > 0 ? 1 : 2)] + ay[ey(i) == 0 ? 0 : (ey(i) > 0 ? 1 : 2)];
+        };
+        // one population: f_i - omega (f_i - f^eq_i) + F_i, g_i - omega (g_i - c_v T f^eq_i) + C_i
+        // with feq = f^eq_i and q = (e.u)(e.F)/cs^4
+        auto update = [&](int i, double feq, double Fi, double Ci) {
             f[i] = f[i] - kp.omega_f * (f[i] - feq) + Fi;
-            const double geq = kp.cv * T * feq;
-            double gs = g[i] - kp.omega_g * (g[i] - geq);
-            if (EQ24) gs += kp.corr_pre * w * kp.cv * T * eF / cs2;
-            g[i] = gs;
+            const double gs = g[i] - kp.omega_g * (g[i] - cvT * feq);
+            g[i] = EQ24 && i ? gs + Ci : gs;
+        };
+        update(0, rho * wd(0) * (1.0 - cu), kp.gw[0] * div_cs2(emuF(0)), 0.0);
+        // Pairs of opposite directions (1,3), (2,4), (5,7), (6,8): e.u, e.F and
+        // C_i only change sign between the two, their squares and products
+        // not at all, so each is formed once (the same doubles as printed).
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+            const int i = p < 2 ? 1 + p : 3 + p, k = i + 2, c = p < 2 ? 1 : 2;
+            const double eu = p == 0 ? ux : (p == 1 ? uy : (p == 2 ? ux + uy : uy - ux));
+            const double eF = p == 0 ? Fx : (p == 1 ? Fy : (p == 2 ? Fx + Fy : Fy - Fx));
+            const double rw = rho * wd(i);
+            const double a = div_cs2(eu);             // e.u / cs^2
+            const double b = div_cs4<1>(eu * eu);     // 0.5 (e.u)^2 / cs^4
+            const double q = div_cs4(eu * eF);
+            const double C = EQ24 ? div_cs2(kp.cwc[c] * T * eF) : 0.0;
+            update(i, rw * (1.0 + a + b - cu), kp.gw[c] * (div_cs2(emuF(i)) + q), C);
+            update(k, rw * (1.0 - a + b - cu), kp.gw[c] * (div_cs2(emuF(k)) + q), -C);
         }
         ux_out = ux;
         uy_out = uy;
-        T_out = T;
     } else {
         const real mx = (f[1] - f[3]) + ((f[5] - f[7]) + (f[8] - f[6]));
         const real my = (f[2] - f[4]) + ((f[5] - f[7]) + (f[6] - f[8]));
-        real e = g[0];
+        if constexpr (!GIVEN) {
+            e = g[0];
 #pragma unroll
-        for (int i = 1; i < 9; ++i) e += g[i];
+            for (int i = 1; i < 9; ++i) e += g[i];
+        }
         const real inv_rho = (real)1 / rho;
         const real ux = (mx + (real)0.5 * Fx) * inv_rho;
         const real uy = (my + (real)0.5 * Fy) * inv_rho;
-        const real T = e / (rho * KPR(kp, cv));
+        if constexpr (!GIVEN) T = e / (rho * KPR(kp, cv));
         const real cvT = KPR(kp, cv) * T;
         if constexpr (FMA) {
             const real m15u2 = (real)-1.5 * fmaf(ux, ux, uy * uy);
@@ -724,8 +808,13 @@ __device__ __forceinline__ void collide(const KParams& kp, real f[9], real g[9],
         g[0] = e - sg;
         ux_out = ux;
         uy_out = uy;
-        T_out = T;
     }
+}
+
+template <typename real, bool EQ24, bool FMA = false>
+__device__ __forceinline__ void collide(const KParams& kp, real f[9], real g[9], real rho, real Fx, real Fy,
+                                        real& ux_out, real& uy_out, real& T_out) {
+    collide_et<real, EQ24, FMA, false>(kp, f, g, rho, (real)0, T_out, Fx, Fy, ux_out, uy_out);
 }
 
 // 16-bit modes: the collision of Eq. (1) with F_i and of Eq. (7) / (24) in the
@@ -853,10 +942,10 @@ __global__ void __launch_bounds__(BX* BY)
     for (int s = tid; s < WX * WY; s += NT) {
         const int ly = s / WX, lx = s - ly * WX;
         const int gx = wrapc(x0 + lx - 1, kp.nx), gy = wrapc(y0 + ly - 1, kp.ny);
-        real f[9], g[9], rho, T, psi, psi2;
+        real f[9], g[9], rho, e, T, psi, psi2;
         int fl = 0;
         pull18<S>(src, kp, gx, gy, f, g);
-        site_psi<real, BMODE>(kp, f, g, rho, T, psi, psi2, fl);
+        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, fl);
         // ring rows beyond the updated range (ghost rows' own ring) do not report
         if (y0 + ly - 1 <= kp.ny - H) flags |= fl;
         if (BMODE != BETA_ZERO) s_psi[s] = psi;
@@ -914,9 +1003,9 @@ __global__ void __launch_bounds__(BX* BY)
     for (int s = tid; s < WX * WY; s += NT) {
         const int ly = s / WX, lx = s - ly * WX;
         const int gx = ringc(kp, x0 + lx - 1, kp.nx), gy = ringc(kp, y0 + ly - 1, kp.ny);
-        real f[9], g[9], rho, T, psi, psi2;
+        real f[9], g[9], rho, e, T, psi, psi2;
         pull18<S>(src, kp, gx, gy, f, g);
-        site_psi<real, BMODE>(kp, f, g, rho, T, psi, psi2, flags);
+        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
         if (BMODE != BETA_ZERO) s_psi[s] = psi;
         if (BMODE != BETA_ONE) s_psi2[s] = psi2;
     }

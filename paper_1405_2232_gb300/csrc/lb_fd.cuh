@@ -53,23 +53,6 @@ __device__ __forceinline__ void pull9(const typename S::elem* __restrict__ src, 
     }
 }
 
-// psi^2 (and psi) of a site with rho from f and T given
-template <typename real, int BMODE>
-__device__ __forceinline__ void site_psi_T(const KParams& kp, real r, real T, real& psi, real& psi2,
-                                           int& flags) {
-    const real Te = kp.psi_local_T ? T : KPR(kp, T_psi);
-    if constexpr (sizeof(real) == 8)
-        psi2 = (real)2 * (p_eos<real>(kp, r, Te) - r * (real)(1.0 / 3.0)) / KPR(kp, G);
-    else
-        psi2 = (p_eos<real>(kp, r, Te) - r * (real)(1.0 / 3.0)) * KPR(kp, two_over_G);
-    psi = (real)0;
-    if (BMODE != BETA_ZERO) {
-        if (psi2 < (real)0) flags |= 1 << LB_ERR_PSI_DOMAIN;
-        psi = sqrt(psi2);
-    }
-    if (!isfinite(r) || !isfinite(T)) flags |= 1 << LB_ERR_NONFINITE;
-}
-
 // Density step (STEP) or moments (!STEP) of the FD treatment.
 //   STEP:  f (src, pre-collision at n) -> dst (post-collision, stored at the
 //          source site; cavity: pushed, bounced back at the walls);

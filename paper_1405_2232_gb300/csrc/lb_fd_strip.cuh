@@ -49,46 +49,73 @@ constexpr int fd_fused_stages() {
     return s > 12 ? 12 : (int)s;
 }
 
-// K(X) of Eq. (26) at one site from three row pointers (south, centre, north,
-// each at the site's column) of X and of rho.  FP64: the stencil and order of
-// operations of the printed form (divisions by c_s^2 included); FP32: the
-// same sums with the divisions by c_s^2 = 1/3 taken as products by 3 and the
-// division by rho as the fast division.
-template <typename real>
-__device__ __forceinline__ real fd_K_rows(const real* Xs, const real* Xc, const real* Xn, const real* Rs,
-                                          const real* Rc, const real* Rn, real ux, real uy, real chi) {
-    real gTx = 0, gTy = 0, grx = 0, gry = 0, lap = 0;
-    const real X0 = Xc[0];
+// FP64: the printed sums over the eight neighbours X[i], R[i] in their order,
+// without the products by e_i = 0 (which add zero), each w X[i] formed once for
+// both gradient components, and the divisions by c_s^2 as div_cs2.
+__device__ __forceinline__ double fd_K_fp64(const double X[9], const double R[9], double ux, double uy, double chi) {
+    double gTx = 0, gTy = 0, grx = 0, gry = 0, lap = 0;
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
-        const real w = (real)wd(i);
-        const real* xr = ey(i) == 1 ? Xn : (ey(i) == -1 ? Xs : Xc);
-        const real* rr = ey(i) == 1 ? Rn : (ey(i) == -1 ? Rs : Rc);
-        const real Xv = xr[ex(i)], rn = rr[ex(i)];
-        gTx += w * (real)ex(i) * Xv;
-        gTy += w * (real)ey(i) * Xv;
-        grx += w * (real)ex(i) * rn;
-        gry += w * (real)ey(i) * rn;
-        lap += w * (Xv - X0);
+        const double w = wd(i), wX = w * X[i], wR = w * R[i];
+        if (ex(i)) {
+            gTx = ex(i) > 0 ? gTx + wX : gTx - wX;
+            grx = ex(i) > 0 ? grx + wR : grx - wR;
+        }
+        if (ey(i)) {
+            gTy = ey(i) > 0 ? gTy + wX : gTy - wX;
+            gry = ey(i) > 0 ? gry + wR : gry - wR;
+        }
+        lap += w * (X[i] - X[0]);
     }
+    gTx = div_cs2(gTx);
+    gTy = div_cs2(gTy);
+    grx = div_cs2(grx);
+    gry = div_cs2(gry);
+    lap *= 2.0 / (1.0 / 3.0);
+    return -(ux * gTx + uy * gTy) + chi * (lap + (grx * gTx + gry * gTy) / R[0]);
+}
+
+// K(X) of Eq. (26) from X and rho of a site and its eight neighbours.  FP64: the
+// order of operations of the printed form (fd_K_fp64); FP32: the same sums with
+// the divisions by c_s^2 = 1/3 taken as products by 3 and the division by rho
+// as the fast division.
+template <typename real>
+__device__ __forceinline__ real fd_K(const real X[9], const real R[9], real ux, real uy, real chi) {
     if constexpr (sizeof(real) == 8) {
-        const real cs2 = (real)(1.0 / 3.0);
-        gTx /= cs2;
-        gTy /= cs2;
-        grx /= cs2;
-        gry /= cs2;
-        lap *= (real)2 / cs2;
+        return fd_K_fp64(X, R, ux, uy, chi);
     } else {
+        real gTx = 0, gTy = 0, grx = 0, gry = 0, lap = 0;
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const real w = (real)wd(i);
+            gTx += w * (real)ex(i) * X[i];
+            gTy += w * (real)ey(i) * X[i];
+            grx += w * (real)ex(i) * R[i];
+            gry += w * (real)ey(i) * R[i];
+            lap += w * (X[i] - X[0]);
+        }
         gTx *= (real)3;
         gTy *= (real)3;
         grx *= (real)3;
         gry *= (real)3;
         lap *= (real)6;
+        // the fast division (a few ulp; +3% on the issue-bound fused step)
+        return -(ux * gTx + uy * gTy) + chi * (lap + __fdividef(grx * gTx + gry * gTy, R[0]));
     }
-    if constexpr (sizeof(real) == 8)
-        return -(ux * gTx + uy * gTy) + chi * (lap + (grx * gTx + gry * gTy) / Rc[0]);
-    else  // FP32: the fast division (a few ulp; +3% on the issue-bound fused step)
-        return -(ux * gTx + uy * gTy) + chi * (lap + __fdividef(grx * gTx + gry * gTy, Rc[0]));
+}
+
+// K(X) of Eq. (26) at one site from three row pointers (south, centre, north,
+// each at the site's column) of X and of rho.
+template <typename real>
+__device__ __forceinline__ real fd_K_rows(const real* Xs, const real* Xc, const real* Xn, const real* Rs,
+                                          const real* Rc, const real* Rn, real ux, real uy, real chi) {
+    real X[9], R[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        X[i] = (ey(i) == 1 ? Xn : (ey(i) == -1 ? Xs : Xc))[ex(i)];
+        R[i] = (ey(i) == 1 ? Rn : (ey(i) == -1 ? Rs : Rc))[ex(i)];
+    }
+    return fd_K<real>(X, R, ux, uy, chi);
 }
 
 // FP32: the same K with the terms that depend only on the site's density and
@@ -395,36 +422,13 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
 template <typename real>
 __device__ __forceinline__ real fd_K_tile(const real* X, int xs, int xc, const real* R, int rs, int rc, real ux,
                                           real uy, real chi) {
-    real gTx = 0, gTy = 0, grx = 0, gry = 0, lap = 0;
-    const real Xc = X[xc];
+    real Xv[9], Rv[9];
 #pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const real w = (real)wd(i);
-        const real Xn = X[xc + ey(i) * xs + ex(i)], rn = R[rc + ey(i) * rs + ex(i)];
-        gTx += w * (real)ex(i) * Xn;
-        gTy += w * (real)ey(i) * Xn;
-        grx += w * (real)ex(i) * rn;
-        gry += w * (real)ey(i) * rn;
-        lap += w * (Xn - Xc);
+    for (int i = 0; i < 9; ++i) {
+        Xv[i] = X[xc + ey(i) * xs + ex(i)];
+        Rv[i] = R[rc + ey(i) * rs + ex(i)];
     }
-    if constexpr (sizeof(real) == 8) {
-        const real cs2 = (real)(1.0 / 3.0);
-        gTx /= cs2;
-        gTy /= cs2;
-        grx /= cs2;
-        gry /= cs2;
-        lap *= (real)2 / cs2;
-    } else {
-        gTx *= (real)3;
-        gTy *= (real)3;
-        grx *= (real)3;
-        gry *= (real)3;
-        lap *= (real)6;
-    }
-    if constexpr (sizeof(real) == 8)
-        return -(ux * gTx + uy * gTy) + chi * (lap + (grx * gTx + gry * gTy) / R[rc]);
-    else
-        return -(ux * gTx + uy * gTy) + chi * (lap + __fdividef(grx * gTx + gry * gTy, R[rc]));
+    return fd_K<real>(Xv, Rv, ux, uy, chi);
 }
 
 // Ghost value of a temperature-like field X at (rx, ry) outside the lattice

@@ -119,6 +119,7 @@ __device__ __forceinline__ void force_from_rows(const KParams& kp, const real* p
                                                 const real* qn, real& Fx, real& Fy) {
     const real w1 = (real)(1.0 / 3.0), w2 = (real)(1.0 / 12.0);
     real fx = 0, fy = 0;
+    constexpr bool first = sizeof(real) == 8;  // FP64: no 0 + x (the compiler keeps it for x = -0)
     if (BMODE != BETA_ZERO) {
         const real E = pc[1], Wv = pc[-1], N = pn[0], S = ps[0];
         const real NE = pn[1], NW = pn[-1], SE = ps[1], SW = ps[-1];
@@ -126,8 +127,8 @@ __device__ __forceinline__ void force_from_rows(const KParams& kp, const real* p
         const real s1x = w1 * (E - Wv) + w2 * (d1 + d2);
         const real s1y = w1 * (N - S) + w2 * (d1 + d3);
         const real c = (BMODE == BETA_ONE) ? pc[0] : KPR(kp, beta) * pc[0];
-        fx += c * s1x;
-        fy += c * s1y;
+        fx = first ? c * s1x : fx + c * s1x;
+        fy = first ? c * s1y : fy + c * s1y;
     }
     if (BMODE != BETA_ONE) {
         const real E = qc[1], Wv = qc[-1], N = qn[0], S = qs[0];
@@ -136,8 +137,8 @@ __device__ __forceinline__ void force_from_rows(const KParams& kp, const real* p
         const real s2x = w1 * (E - Wv) + w2 * (d1 + d2);
         const real s2y = w1 * (N - S) + w2 * (d1 + d3);
         const real h = (BMODE == BETA_ZERO) ? (real)0.5 : KPR(kp, half_1mbeta);
-        fx += h * s2x;
-        fy += h * s2y;
+        fx = first && BMODE == BETA_ZERO ? h * s2x : fx + h * s2x;
+        fy = first && BMODE == BETA_ZERO ? h * s2y : fy + h * s2y;
     }
     Fx = -KPR(kp, G) * fx;
     Fy = -KPR(kp, G) * fy;
@@ -309,9 +310,16 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     const bool has_psi = halo ? (t & 31) < 2 : t < W;
     int flags = 0;
     bool aborted = false;
+    // FP64: rho, sum g and T of this thread's site in the newest row and in the
+    // row behind it, which collides next (the FP64 units bound that kernel, so the
+    // sums and the division are not formed again)
+    real rho1 = 0, e1 = 0, T1 = 0, rho0 = 0, e0 = 0, T0 = 0;
     for (int j = 0; j < njobs; ++j) {
         const int s = j % STAGES;
         if (!mbar_wait_bounded(&full[s], (uint32_t)((j / STAGES) & 1), kp.wait_cycles)) s_abort[j & 1] = 1;
+        rho0 = rho1;
+        e0 = e1;
+        T0 = T1;
         // 1. rho, T, psi of pre-collision row j at ring column r_psi
         if (has_psi) {
             const elem* st = stage + (size_t)s * NPL * SEGW;
@@ -320,7 +328,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
             {
                 const int r = r_psi;
                 const int c = r - 1 + HALO;  // smem column of the site
-                real rho, T, psi, psi2;
+                real rho, e, T, psi, psi2;
                 if constexpr (S::SPLIT) {
                     // rho and the energy density from the sums of the stored deviations
                     float Hf = 0.0f, Hg = 0.0f;
@@ -339,10 +347,15 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                         f[i] = load_pop<S>(st + i * SEGW + c - ex(i), SEGW, i, (real)kp.base_f[i]);
                         g[i] = load_pop<S>(st + (9 + i) * SEGW + c - ex(i), SEGW, 9 + i, (real)kp.base_g[i]);
                     }
-                    site_psi<real, BMODE>(kp, f, g, rho, T, psi, psi2, flags);
+                    site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
                 }
                 if (BMODE != BETA_ZERO) rp[r] = psi;
                 if (BMODE != BETA_ONE) rq[r] = psi2;
+                if constexpr (sizeof(real) == 8) {
+                    rho1 = rho;
+                    e1 = e;
+                    T1 = T;
+                }
             }
         }
         consumer_sync<BX + 32>();
@@ -386,11 +399,15 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     f[i] = load_pop_acc<S>(st + i * SEGW + c - ex(i), SEGW, i, (real)kp.base_f[i], Hf);
                     g[i] = load_pop_acc<S>(st + (9 + i) * SEGW + c - ex(i), SEGW, 9 + i, (real)kp.base_g[i], Hg);
                 }
-                real rho = f[0];
-#pragma unroll
-                for (int i = 1; i < 9; ++i) rho += f[i];
                 real ux, uy, T;
-                collide<real, EQ24>(kp, f, g, rho, Fx, Fy, ux, uy, T);
+                if constexpr (sizeof(real) == 8) {
+                    collide_et<real, EQ24, false, true>(kp, f, g, rho0, e0, T0, Fx, Fy, ux, uy);
+                } else {
+                    real rho = f[0];
+#pragma unroll
+                    for (int i = 1; i < 9; ++i) rho += f[i];
+                    collide<real, EQ24>(kp, f, g, rho, Fx, Fy, ux, uy, T);
+                }
                 store_site<S>(dst + off, plane, kp, f, g, Hf, Hg, xg < STRIP_GHOST, xg >= nx - STRIP_GHOST);
             }
         }

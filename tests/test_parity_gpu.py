@@ -514,3 +514,20 @@ def test_16bit_strip_ragged_columns_over_several_steps(lb, prec, u, nx, ny):
             L.synchronize()
             out[p] = L.moments()[0]
     assert np.abs(out[prec] - out["fp32"]).max() <= 20 * 8 * 0.03 * u
+
+
+@pytest.mark.parametrize("tile", [(128, 0), (32, 8)])
+@pytest.mark.parametrize("G,beta", [(-0.9, 1.3), (-2.0, 1.0), (-0.75, 1.0)])
+def test_fp64_interaction_strengths_bit_identical(lb, G, beta, tile):
+    """2 x / G as a scaling (|G| a power of two) and as a division."""
+    nx, ny = 45, 37
+    rho, T = I.slab_fields(nx, ny, width=20, noise=1e-3)
+    T_psi = 0.85 * I.CS_TC
+    P = oracle_params(O.THERMAL_EQ24, 0, T_psi, nx=nx, ny=ny, G=G, beta=beta)
+    f0, g0 = O.init_equilibrium(P, rho, T)
+    f_ref, g_ref, _ = O.step(P, f0, g0, n=40, check=False)
+    with gpu_lattice(lb, rho, T, O.THERMAL_EQ24, "fp64", 0, T_psi, G=G, beta=beta, tile_x=tile[0],
+                     tile_y=tile[1]) as L:
+        L.step(40)
+        f, g = L.populations()
+    assert np.array_equal(f, f_ref) and np.array_equal(g, g_ref)
