@@ -44,7 +44,10 @@ def nvcc() -> str:
 EXTRA_FLAGS = {"lb_prec_fp64.cu": ["--fmad=false"], "lb_batch_fp64.cu": ["--fmad=false"],
                "lb_init_balanced.cu": ["--fmad=false"],
                "lb_prec_fp16.cu": ["-prec-div=false", "-prec-sqrt=false", "-DLB_KP_FLOAT"],
-               "lb_prec_bf16.cu": ["-prec-div=false", "-prec-sqrt=false", "-DLB_KP_FLOAT"]}
+               "lb_prec_bf16.cu": ["-prec-div=false", "-prec-sqrt=false", "-DLB_KP_FLOAT"],
+               "lb_tile_fp64.cu": ["--fmad=false"], "lb_tile_fp32.cu": ["-DLB_KP_FLOAT"],
+               "lb_tile_fp16.cu": ["-prec-div=false", "-prec-sqrt=false", "-DLB_KP_FLOAT"],
+               "lb_tile_bf16.cu": ["-prec-div=false", "-prec-sqrt=false", "-DLB_KP_FLOAT"]}
 
 
 def _sources():

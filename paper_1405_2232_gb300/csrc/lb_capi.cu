@@ -172,6 +172,8 @@ struct lb_ctx {
     int64_t ref_time = 0;
     int64_t t = 0;
     int nchunks = 1;            // strip kernel: row chunks per strip
+    int tile_by = 0;            // see StepLaunch
+    int sms = 152;
     bool have_out_map = false;  // 16-bit strip contexts: out_map[b] describes buf[b]
     CUtensorMap out_map[2];
     long long pitch = 0, plane = 0;  // population layout (elements)
@@ -261,12 +263,11 @@ cudaError_t dispatch_step(const lb_ctx* c, const void* src, void* dst) {
     L.bx = c->p.tile_x;
     L.by = c->p.tile_y;
     L.nchunks = c->nchunks;
+    // (a caller-set wait limit is about the strip kernel's waits: it runs then)
+    L.tile_by = c->kp.walls || c->kp.wait_cycles == WAIT_CYCLES_DEFAULT ? c->tile_by : 0;
+    L.sms = c->sms;
     L.stream = c->stream;
     if (c->have_out_map) L.dst_map = &c->out_map[dst == c->buf[0] ? 0 : 1];
-    if (c->p.walls == LB_WALLS_CHANNEL)
-        return c->p.precision == LB_PREC_FP64 ? launch_step_channel_fp64(L) : launch_step_channel_fp32(L);
-    if (c->kp.walls)
-        return c->p.precision == LB_PREC_FP64 ? launch_step_cavity_fp64(L) : launch_step_cavity_fp32(L);
     switch (c->p.precision) {
         case LB_PREC_FP64: return launch_step_fp64(L);
         case LB_PREC_FP32: return launch_step_fp32(L);
@@ -356,6 +357,41 @@ cudaError_t dispatch_fd_moments(lb_ctx* c, double* rho, double* ux, double* uy, 
 cudaError_t dispatch_fd_set_T(lb_ctx* c, const double* d_T0) {
     return c->p.precision == LB_PREC_FP64 ? launch_fd_set_T_fp64(c->Tf[c->tcur], d_T0, c->kp, c->stream)
                                           : launch_fd_set_T_fp32(c->Tf[c->tcur], d_T0, c->kp, c->stream);
+}
+
+// Rows of the tile kernel's 32-column tiles for a lattice whose caller asked for no
+// shape; 0: the strip kernel (never in a cavity or channel).
+//
+// FP64: the FP64 units bound both kernels, so the tiles are balanced over the SMs: the
+// height that minimises (tiles per SM) x (285 operations of a row's collision + 65
+// of each warp's psi, ring included).  The strip kernel wastes less on halos and takes
+// over at 2^20 sites (1024^2: 749 us against 751 us; 512^2: 234 against 192).
+// FP32, 16-bit: up to four tiles per SM the same balance, at most ten rows, with the
+// collision and psi of a row weighing alike; beyond, the height whose blocks fill the
+// SMs best with the kernel's registers (seven rows: four blocks of ten warps in FP32;
+// six rows: four of nine in the 16-bit modes).  The strip kernel reads less and takes
+// over where the state outgrows the L2 cache: at 2^21 sites in FP32 (1448^2: 61.6 us
+// against 59.4, 2048^2: 109 against 114), at 1.5 x 2^20 in the 16-bit modes (1024^2:
+// 28.7 against 26.7, 1448^2: 51 against 52).
+int default_tile_rows(int prec, int nx, int rows, int sms, bool walls) {
+    const bool fp64 = prec == LB_PREC_FP64, fp32 = prec == LB_PREC_FP32;
+    const long long sites = (long long)nx * rows;
+    if (!walls && sites > (fp64 ? (1LL << 20) - 1 : (fp32 ? 1LL << 21 : 3LL << 19))) return 0;
+    const long long cols = (nx + 31) / 32;
+    const int fill = fp32 ? 7 : 6;
+    if (!fp64 && cols * ((rows + fill - 1) / fill) > 4LL * sms) return fill;
+    const double own = fp64 ? 285.0 : 0.55, psi = fp64 ? 65.0 : 0.45;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int by = 1; by <= (fp64 ? 14 : 10); ++by) {
+        const long long tiles = cols * ((rows + by - 1) / by);
+        const double cost = (double)((tiles + sms - 1) / sms) * (own * by + psi * (tile_threads(32, by) / 32));
+        if (by == 1 || cost < best_cost) {
+            best = by;
+            best_cost = cost;
+        }
+    }
+    return best;
 }
 
 void release(lb_ctx* c) {
@@ -501,12 +537,15 @@ lb_status create(const lb_params* p, void* stream, lb_ctx** out) {
     c->kp.ghost = strip ? (c->fd ? FD_GHOST : STRIP_GHOST) : 0;
     c->pitch = pitch;
     c->plane = plane;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess && sms > 0)
+        c->sms = sms;
+    sms = c->sms;
+    if (c->kp.walls || (strip && !p->tile_x && !p->tile_y && !c->fd))
+        c->tile_by = default_tile_rows(p->precision, p->nx, p->ny - 2 * p->halo_rows, sms, c->kp.walls != 0);
     if (strip) {
         // one wave of two resident CTAs per SM: strips x chunks <= 2 x SMs
         // (chunks of at least 8 rows)
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || sms <= 0)
-            sms = 152;
         const int strips = (p->nx + c->p.tile_x - 1) / c->p.tile_x;
         const int rows = p->ny - 2 * p->halo_rows;
         const int max_ch = rows / 8 > 0 ? rows / 8 : 1;

@@ -484,8 +484,7 @@ __device__ __forceinline__ int ringc(const KParams& kp, int v, int n) {
 
 // Pull the 18 pre-collision populations of site (x, y).
 template <class S>
-__device__ __forceinline__ void pull18(const typename S::elem* __restrict__ src,
-                                       const KParams& kp, int x, int y,
+__device__ __forceinline__ void pull18(const typename S::elem* src, const KParams& kp, int x, int y,
                                        typename S::real f[9], typename S::real g[9]) {
     if (kp.walls) {  // cavity: populations stored pre-collision at their own site
         const long long off = (long long)y * kp.pitch + x;
@@ -510,52 +509,6 @@ __device__ __forceinline__ void pull18(const typename S::elem* __restrict__ src,
         f[i] = load_pop<S>(src + (long long)i * kp.plane + off, kp.plane, i, (typename S::real)kp.base_f[i]);
         g[i] = load_pop<S>(src + (long long)(9 + i) * kp.plane + off, kp.plane, 9 + i,
                            (typename S::real)kp.base_g[i]);
-    }
-}
-
-// pull18 of a periodic site that also returns the sums of the stored
-// deviations (16-bit modes; zero otherwise), which store_site closes on.
-template <class S>
-__device__ __forceinline__ void pull18h(const typename S::elem* __restrict__ src, const KParams& kp, int x,
-                                        int y, typename S::real f[9], typename S::real g[9],
-                                        typename S::real& Hf, typename S::real& Hg) {
-    Hf = Hg = (typename S::real)0;
-    const int xm = x == 0 ? kp.nx - 1 : x - 1;
-    const int xp = x == kp.nx - 1 ? 0 : x + 1;
-    const long long r0 = (long long)y * kp.pitch;
-    const long long rm = (long long)(y == 0 ? kp.ny - 1 : y - 1) * kp.pitch;
-    const long long rp = (long long)(y == kp.ny - 1 ? 0 : y + 1) * kp.pitch;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const int sx = ex(i) == 1 ? xm : (ex(i) == -1 ? xp : x);
-        const long long sr = ey(i) == 1 ? rm : (ey(i) == -1 ? rp : r0);
-        const long long off = sr + sx;
-        f[i] = load_pop_acc<S>(src + (long long)i * kp.plane + off, kp.plane, i, (typename S::real)kp.base_f[i], Hf);
-        g[i] = load_pop_acc<S>(src + (long long)(9 + i) * kp.plane + off, kp.plane, 9 + i,
-                               (typename S::real)kp.base_g[i], Hg);
-    }
-}
-
-// The stored deviations of the 18 pre-collision populations of a periodic
-// site (16-bit modes) and their sums Hf, Hg.
-template <class S>
-__device__ __forceinline__ void pull18_dev(const typename S::elem* __restrict__ src, const KParams& kp, int x,
-                                           int y, float h[9], float q[9], float& Hf, float& Hg) {
-    Hf = Hg = 0.0f;
-    const int xm = x == 0 ? kp.nx - 1 : x - 1;
-    const int xp = x == kp.nx - 1 ? 0 : x + 1;
-    const long long r0 = (long long)y * kp.pitch;
-    const long long rm = (long long)(y == 0 ? kp.ny - 1 : y - 1) * kp.pitch;
-    const long long rp = (long long)(y == kp.ny - 1 ? 0 : y + 1) * kp.pitch;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        const int sx = ex(i) == 1 ? xm : (ex(i) == -1 ? xp : x);
-        const long long sr = ey(i) == 1 ? rm : (ey(i) == -1 ? rp : r0);
-        const long long off = sr + sx;
-        h[i] = dev_of<S>(src + (long long)i * kp.plane + off, i, rest_lo_offset(i) * kp.plane);
-        q[i] = dev_of<S>(src + (long long)(9 + i) * kp.plane + off, 9 + i, rest_lo_offset(9 + i) * kp.plane);
-        Hf += h[i];
-        Hg += q[i];
     }
 }
 
@@ -917,66 +870,6 @@ __device__ __forceinline__ void store_site_dev(typename S::elem* d, IT stride, c
     typename S::elem v[S::NPLANES];
     encode_site_dev<S>(h, q, Hf, Hg, v);
     put_planes<S>(d, stride, kp.nx, v, ghost_lo, ghost_hi);
-}
-
-// ---------------------------------------------------------------- step
-// One fused time step.  CTA tile BX x BY; phase 1 computes psi for the tile
-// plus a one-site ring from pulled populations (ring pulls hit L2), phase 2
-// pulls each tile site again (L1), applies the stencil and both collisions,
-// and stores 18 values at the site (the next step pulls them).
-template <int PREC, int BX, int BY, bool EQ24, int BMODE>
-__global__ void __launch_bounds__(BX* BY)
-    k_step(const typename Store<PREC>::elem* __restrict__ src,
-           typename Store<PREC>::elem* __restrict__ dst, const KParams kp) {
-    using S = Store<PREC>;
-    using real = typename S::real;
-    constexpr int WX = BX + 2, WY = BY + 2, NT = BX * BY;
-    __shared__ real s_psi[BMODE != BETA_ZERO ? WX * WY : 1];
-    __shared__ real s_psi2[BMODE != BETA_ONE ? WX * WY : 1];
-
-    const int tid = threadIdx.x + threadIdx.y * BX;
-    // rows updated: [H, ny - H) (H = kp.halo_rows; 0 on a periodic lattice)
-    const int H = kp.halo_rows;
-    const int x0 = blockIdx.x * BX, y0 = H + blockIdx.y * BY;
-    int flags = 0;
-    for (int s = tid; s < WX * WY; s += NT) {
-        const int ly = s / WX, lx = s - ly * WX;
-        const int gx = wrapc(x0 + lx - 1, kp.nx), gy = wrapc(y0 + ly - 1, kp.ny);
-        real f[9], g[9], rho, e, T, psi, psi2;
-        int fl = 0;
-        pull18<S>(src, kp, gx, gy, f, g);
-        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, fl);
-        // ring rows beyond the updated range (ghost rows' own ring) do not report
-        if (y0 + ly - 1 <= kp.ny - H) flags |= fl;
-        if (BMODE != BETA_ZERO) s_psi[s] = psi;
-        if (BMODE != BETA_ONE) s_psi2[s] = psi2;
-    }
-    __syncthreads();
-
-    const int gx = x0 + threadIdx.x, gy = y0 + threadIdx.y;
-    if (gx < kp.nx && gy < kp.ny - H) {
-        real Fx, Fy, ux, uy, T;
-        force_from_window<real, BMODE>(kp, s_psi, s_psi2, (threadIdx.y + 1) * WX + threadIdx.x + 1,
-                                       WX, Fx, Fy);
-        const long long off = (long long)gy * kp.pitch + gx;
-        if constexpr (S::SPLIT) {
-            float h[9], q[9], Hf, Hg;
-            pull18_dev<S>(src, kp, gx, gy, h, q, Hf, Hg);
-            collide_dev<EQ24>(kp, h, q, Hf, Hg, Fx, Fy);
-            store_site_dev<S>(dst + off, kp.plane, kp, h, q, Hf, Hg, false, false);
-        } else {
-            real f[9], g[9], Hf, Hg;
-            pull18h<S>(src, kp, gx, gy, f, g, Hf, Hg);
-            real rho = f[0];
-#pragma unroll
-            for (int i = 1; i < 9; ++i) rho += f[i];
-            collide<real, EQ24>(kp, f, g, rho, Fx, Fy, ux, uy, T);
-            store_site<S>(dst + off, kp.plane, kp, f, g, Hf, Hg, false, false);
-        }
-    } else {
-        flags = 0;
-    }
-    if (flags) atomicOr(kp.err, flags);
 }
 
 // ---------------------------------------------------------------- moments

@@ -22,8 +22,8 @@
 // order of its printed form (compiled without contraction).
 #pragma once
 
-#include "lb_cavity.cuh"
 #include "lb_device.cuh"
+#include "lb_step_tile.cuh"
 
 namespace lbgb {
 

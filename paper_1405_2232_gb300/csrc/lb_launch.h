@@ -18,6 +18,9 @@ struct StepLaunch {
     int bmode;      // BetaMode
     int bx, by;     // CTA tile; by == 0: strip kernel of width bx
     int nchunks;    // strip kernel: row chunks per strip
+    int tile_by;    // > 0: rows of the 32-column tiles that run where no tile is
+                    // asked for (by == 0, cavity, channel) instead of the strip kernel
+    int sms;        // SMs of the device
     cudaStream_t stream;
     // 16-bit strip kernel: tensor map of dst (x: dev_map_columns(nx) columns,
     // y: ny rows, z: the planes; box bx x 1 x NPLANES) that its collided rows
@@ -109,6 +112,7 @@ inline PopLayout pop_layout(int prec, int nx, int ny, bool strip) {
 
 #define LBGB_DECLARE_PREC(NAME)                                                       \
     cudaError_t launch_step_##NAME(const StepLaunch& L);                               \
+    cudaError_t launch_tile_##NAME(const StepLaunch& L);                               \
     cudaError_t launch_moments_##NAME(const MomentsLaunch& L);                         \
     cudaError_t launch_init_##NAME(void* dst, const KParams& kp, const double* rho0,   \
                                    const double* T0, cudaStream_t st);                 \
@@ -116,8 +120,6 @@ inline PopLayout pop_layout(int prec, int nx, int ny, bool strip) {
                                      cudaStream_t st);                                 \
     cudaError_t launch_scatter_##NAME(void* dst, const KParams& kp, const double* in,  \
                                       cudaStream_t st);                                \
-    cudaError_t launch_step_cavity_##NAME(const StepLaunch& L);                        \
-    cudaError_t launch_step_channel_##NAME(const StepLaunch& L);                       \
     cudaError_t launch_fd_step_##NAME(const FdLaunch& L);                              \
     cudaError_t launch_fd_moments_##NAME(const FdLaunch& L);                           \
     cudaError_t launch_fd_set_T_##NAME(void* T, const double* T0, const KParams& kp, cudaStream_t st);

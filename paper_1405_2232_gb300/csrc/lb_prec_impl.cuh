@@ -3,7 +3,6 @@
 // value) and LBGB_NAME (the suffix of the launch functions).
 #pragma once
 
-#include "lb_cavity.cuh"
 #include "lb_fd.cuh"
 #include "lb_fd_strip.cuh"
 #include "lb_launch.h"
@@ -16,29 +15,6 @@ namespace lbgb {
 #define LBGB_CAT(a, b) LBGB_CAT2(a, b)
 
 namespace {
-
-template <int BX, int BY>
-cudaError_t step_tile(const StepLaunch& L) {
-    using E = typename Store<LBGB_PREC>::elem;
-    const dim3 block(BX, BY);
-    const dim3 grid((L.kp.nx + BX - 1) / BX, (L.kp.ny - 2 * L.kp.halo_rows + BY - 1) / BY);
-    const E* src = static_cast<const E*>(L.src);
-    E* dst = static_cast<E*>(L.dst);
-    if (L.eq24) {
-        switch (L.bmode) {
-            case BETA_ZERO: k_step<LBGB_PREC, BX, BY, true, BETA_ZERO><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            case BETA_ONE: k_step<LBGB_PREC, BX, BY, true, BETA_ONE><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            default: k_step<LBGB_PREC, BX, BY, true, BETA_MIXED><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-        }
-    } else {
-        switch (L.bmode) {
-            case BETA_ZERO: k_step<LBGB_PREC, BX, BY, false, BETA_ZERO><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            case BETA_ONE: k_step<LBGB_PREC, BX, BY, false, BETA_ONE><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            default: k_step<LBGB_PREC, BX, BY, false, BETA_MIXED><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-        }
-    }
-    return cudaGetLastError();
-}
 
 // Everything in this anonymous namespace depends on LBGB_PREC without carrying
 // it as a template argument, so it must have internal linkage: each precision
@@ -124,17 +100,12 @@ cudaError_t step_strip(const StepLaunch& L) {
 }  // namespace
 
 cudaError_t LBGB_CAT(launch_step_, LBGB_NAME)(const StepLaunch& L) {
-    if (L.by == 0) {
-        if (L.bx == 128) return step_strip<128>(L);
-        // (LB_PREC_* are enum constants, invisible to the preprocessor)
-        if constexpr (LBGB_PREC != LB_PREC_FP64) {
-            if (L.bx == 256) return step_strip<256>(L);
-        }
-        return cudaErrorInvalidValue;
+    if (L.by != 0 || L.tile_by) return LBGB_CAT(launch_tile_, LBGB_NAME)(L);
+    if (L.bx == 128) return step_strip<128>(L);
+    // (LB_PREC_* are enum constants, invisible to the preprocessor)
+    if constexpr (LBGB_PREC != LB_PREC_FP64) {
+        if (L.bx == 256) return step_strip<256>(L);
     }
-    if (L.bx == 32 && L.by == 8) return step_tile<32, 8>(L);
-    if (L.bx == 32 && L.by == 16) return step_tile<32, 16>(L);
-    if (L.bx == 64 && L.by == 4) return step_tile<64, 4>(L);
     return cudaErrorInvalidValue;
 }
 
@@ -187,63 +158,6 @@ cudaError_t LBGB_CAT(launch_scatter_, LBGB_NAME)(void* dst, const KParams& kp, c
     using E = typename Store<LBGB_PREC>::elem;
     k_scatter<LBGB_PREC><<<elementwise_blocks(kp), 256, 0, st>>>(static_cast<E*>(dst), kp, in);
     return cudaGetLastError();
-}
-
-// ------------------------------------------------ cavity (Sec. III B)
-cudaError_t LBGB_CAT(launch_step_cavity_, LBGB_NAME)(const StepLaunch& L) {
-    if constexpr (LBGB_PREC != LB_PREC_FP64 && LBGB_PREC != LB_PREC_FP32) {
-        return cudaErrorNotSupported;
-    } else {
-        using E = typename Store<LBGB_PREC>::elem;
-        const dim3 block(CAV_BX, CAV_BY);
-        const dim3 grid((L.kp.nx + CAV_BX - 1) / CAV_BX, (L.kp.ny + CAV_BY - 1) / CAV_BY);
-        const E* src = static_cast<const E*>(L.src);
-        E* dst = static_cast<E*>(L.dst);
-        if (L.eq24) {
-            switch (L.bmode) {
-                case BETA_ZERO: k_step_cavity<LBGB_PREC, true, BETA_ZERO><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                case BETA_ONE: k_step_cavity<LBGB_PREC, true, BETA_ONE><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                default: k_step_cavity<LBGB_PREC, true, BETA_MIXED><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            }
-        } else {
-            switch (L.bmode) {
-                case BETA_ZERO: k_step_cavity<LBGB_PREC, false, BETA_ZERO><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                case BETA_ONE: k_step_cavity<LBGB_PREC, false, BETA_ONE><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                default: k_step_cavity<LBGB_PREC, false, BETA_MIXED><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            }
-        }
-        return cudaGetLastError();
-    }
-}
-
-// ------------------------------------------------ channel (Sec. III A)
-cudaError_t LBGB_CAT(launch_step_channel_, LBGB_NAME)(const StepLaunch& L) {
-    if constexpr (LBGB_PREC != LB_PREC_FP64 && LBGB_PREC != LB_PREC_FP32) {
-        return cudaErrorNotSupported;
-    } else {
-        using E = typename Store<LBGB_PREC>::elem;
-        const dim3 block(CAV_BX, CAV_BY);
-        const dim3 grid((L.kp.nx + CAV_BX - 1) / CAV_BX, (L.kp.ny + CAV_BY - 1) / CAV_BY);
-        const E* src = static_cast<const E*>(L.src);
-        E* dst = static_cast<E*>(L.dst);
-        if (L.eq24) {
-            switch (L.bmode) {
-                case BETA_ZERO: k_step_channel<LBGB_PREC, true, BETA_ZERO><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                case BETA_ONE: k_step_channel<LBGB_PREC, true, BETA_ONE><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                default: k_step_channel<LBGB_PREC, true, BETA_MIXED><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            }
-        } else {
-            switch (L.bmode) {
-                case BETA_ZERO: k_step_channel<LBGB_PREC, false, BETA_ZERO><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                case BETA_ONE: k_step_channel<LBGB_PREC, false, BETA_ONE><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-                default: k_step_channel<LBGB_PREC, false, BETA_MIXED><<<grid, block, 0, L.stream>>>(src, dst, L.kp); break;
-            }
-        }
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_channel_outlet<LBGB_PREC><<<(L.kp.ny + 127) / 128, 128, 0, L.stream>>>(dst, L.kp);
-        return cudaGetLastError();
-    }
 }
 
 // ------------------------------------------------ finite-difference T (Eqs. 26-27)

@@ -1,0 +1,95 @@
+// lb_tile_impl.cuh -- instantiates the tile kernels (lb_step_tile.cuh) of one
+// storage precision.  Included by lb_tile_<name>.cu after defining LBGB_PREC
+// (an LB_PREC_* value) and LBGB_NAME (the suffix of the launch function).  A unit
+// of its own: a thread of these kernels has one site, so the parameters are read
+// as float copies (LB_KP_FLOAT) where the strip kernels convert the doubles once
+// per chunk of rows.
+#pragma once
+
+#include <atomic>
+
+#include "lb_launch.h"
+#include "lb_step_tile.cuh"
+
+namespace lbgb {
+
+#define LBGB_CAT2(a, b) a##b
+#define LBGB_CAT(a, b) LBGB_CAT2(a, b)
+
+namespace {  // (see lb_prec_impl.cuh: depends on LBGB_PREC, internal linkage)
+
+template <int BX, int WALLS>
+auto tile_kernel(const StepLaunch& L) -> void (*)(const typename Store<LBGB_PREC>::elem*,
+                                                   typename Store<LBGB_PREC>::elem*, const KParams, int) {
+    if (L.eq24) {
+        if (L.bmode == BETA_ZERO) return k_step_tile<LBGB_PREC, BX, WALLS, true, BETA_ZERO>;
+        if (L.bmode == BETA_ONE) return k_step_tile<LBGB_PREC, BX, WALLS, true, BETA_ONE>;
+        return k_step_tile<LBGB_PREC, BX, WALLS, true, BETA_MIXED>;
+    }
+    if (L.bmode == BETA_ZERO) return k_step_tile<LBGB_PREC, BX, WALLS, false, BETA_ZERO>;
+    if (L.bmode == BETA_ONE) return k_step_tile<LBGB_PREC, BX, WALLS, false, BETA_ONE>;
+    return k_step_tile<LBGB_PREC, BX, WALLS, false, BETA_MIXED>;
+}
+
+// Dynamic shared memory of a launch of `tiles` blocks: what the psi window needs,
+// or more where at most eight blocks run per SM, so that no SM takes more than
+// ceil(tiles / SMs) of them.  The blocks of a step are dispatched while the step
+// before it still runs, and an SM that happens to be free then would take several,
+// which keeps the next steps unbalanced as well (FP64 150 x 150 cavity, 150 tiles of
+// five rows: 32.4 us per step without, 19.0 us with).
+size_t tile_smem(const StepLaunch& L, long long tiles, size_t need) {
+    const long long k = (tiles + L.sms - 1) / L.sms;
+    if (k > 8) return need;
+    const size_t pad = TILE_SM_SMEM / (size_t)(k + 1);  // k + 1 blocks (and 1 KB each) do not fit
+    return pad > need ? pad : need;
+}
+
+template <int BX, int WALLS>
+cudaError_t step_tile(const StepLaunch& L, int by) {
+    using E = typename Store<LBGB_PREC>::elem;
+    auto kern = tile_kernel<BX, WALLS>(L);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((L.kp.nx + BX - 1) / BX, (L.kp.ny - 2 * L.kp.halo_rows + by - 1) / by);
+    cfg.blockDim = dim3(tile_threads(BX, by));
+    cfg.dynamicSmemBytes = tile_smem(L, (long long)cfg.gridDim.x * cfg.gridDim.y,
+                                     L.bmode == BETA_MIXED ? tile_smem_bytes<LBGB_PREC, BETA_MIXED>(BX, by)
+                                                           : tile_smem_bytes<LBGB_PREC, BETA_ONE>(BX, by));
+    cfg.stream = L.stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cfg.dynamicSmemBytes > 48 * 1024) {
+        // opt in once per kernel (by its slot among the variants) and device
+        static std::atomic<unsigned long long> configured[6];
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        auto& done = configured[(L.eq24 ? 3 : 0) + L.bmode];
+        if (dev >= 64 || !(done.load() >> dev & 1ULL)) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TILE_SM_SMEM / 2));
+            if (e != cudaSuccess) return e;
+            if (dev < 64) done.fetch_or(1ULL << dev);
+        }
+    }
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, by);
+}
+
+}  // namespace
+
+cudaError_t LBGB_CAT(launch_tile_, LBGB_NAME)(const StepLaunch& L) {
+    if (L.kp.walls) {
+        if constexpr (LBGB_PREC == LB_PREC_FP64 || LBGB_PREC == LB_PREC_FP32) {
+            if (L.kp.walls == LB_WALLS_CAVITY) return step_tile<32, LB_WALLS_CAVITY>(L, L.tile_by);
+            return step_tile<32, LB_WALLS_CHANNEL>(L, L.tile_by);
+        }
+        return cudaErrorNotSupported;
+    }
+    if (L.by == 0) return step_tile<32, 0>(L, L.tile_by);
+    if (L.bx == 32 && (L.by == 8 || L.by == 16)) return step_tile<32, 0>(L, L.by);
+    if (L.bx == 64 && L.by == 4) return step_tile<64, 0>(L, L.by);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace lbgb
