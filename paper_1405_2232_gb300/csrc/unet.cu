@@ -890,8 +890,22 @@ lb_status un_warm_fields(int32_t N, int32_t H, int32_t W, const float* d_pred, d
     a.rho = d_rho;
     a.T = d_T;
     a.P = (long long)H * W;
-    unk::k_warm<<<N, 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
-    UCU(cudaGetLastError(), "un_warm_fields");
+    // blocks per case: as many as leave each thread at least WARM_KEEP sites
+    int blocks = 1;
+    while (blocks < unk::WARM_MAX_CLUSTER && a.P > (long long)blocks * unk::WARM_THREADS * unk::WARM_KEEP) blocks *= 2;
+    if (blocks > 8)
+        UCU(cudaFuncSetAttribute(unk::k_warm, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "un_warm_fields");
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)blocks;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)N * (unsigned)blocks);
+    cfg.blockDim = dim3(unk::WARM_THREADS);
+    cfg.stream = static_cast<cudaStream_t>(stream);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    UCU(cudaLaunchKernelEx(&cfg, unk::k_warm, a), "un_warm_fields");
     return LB_OK;
 }
 

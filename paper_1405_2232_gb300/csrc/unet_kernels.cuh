@@ -18,6 +18,7 @@
 // contiguous block for the tensor copies of the tcgen05 convolution.
 #pragma once
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -954,73 +955,124 @@ __device__ __forceinline__ double warm_T_hat(const WarmArgs& a, long long i) {
     return a.T0[i] * (1.0 + a.t_dev_scale * (double)a.pred[2 * i + 1]);
 }
 
-// fixed-order block reduction of NV values (sum, or min/max where asked)
+constexpr int WARM_THREADS = 512;    // threads of a block
+constexpr int WARM_KEEP = 8;         // sites a thread keeps in registers
+constexpr int WARM_MAX_CLUSTER = 16;
+
+// Reduction of NV values over the cluster (sum, or min/max where asked), the same
+// on every thread: lanes, warps and blocks each in a fixed order.  The 16 warps'
+// values and the blocks' are each joined by half a warp per value (every thread
+// joining them cost more FP64 operations than the passes themselves).
 template <int NV>
-__device__ void block_reduce(double (&v)[NV], double (*red)[256], const int (&op)[NV]) {
+__device__ __forceinline__ void cluster_reduce(double (&v)[NV], const int (&op)[NV],
+                                               double (*s_warp)[5], double* s_block, double* s_all) {
+    namespace cg = cooperative_groups;
+    static_assert(WARM_THREADS == 512 && WARM_MAX_CLUSTER == 16 && NV <= 5, "half a warp per value");
+    cg::cluster_group cl = cg::this_cluster();
+    const int t = threadIdx.x, k16 = t >> 4, l16 = t & 15;
+    auto join = [](int o, double a, double b) { return o == 0 ? a + b : (o < 0 ? fmin(a, b) : fmax(a, b)); };
+    int my_op = 0;
 #pragma unroll
-    for (int k = 0; k < NV; ++k) red[k][threadIdx.x] = v[k];
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
+    for (int k = 0; k < NV; ++k)
+        if (k == k16) my_op = op[k];
+    const double none = my_op == 0 ? 0.0 : (my_op < 0 ? INFINITY : -INFINITY);
+    auto join16 = [&](double x) {
 #pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                const double a = red[k][threadIdx.x], b = red[k][threadIdx.x + w];
-                red[k][threadIdx.x] = op[k] == 0 ? a + b : (op[k] < 0 ? fmin(a, b) : fmax(a, b));
-            }
-        __syncthreads();
+        for (int o = 8; o > 0; o >>= 1) {
+            const double y = __shfl_xor_sync(0xffffffffu, x, o);
+            x = my_op == 0 ? x + y : (my_op < 0 ? fmin(x, y) : fmax(x, y));
+        }
+        return x;
+    };
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v[k] = join(op[k], v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+        if ((t & 31) == 0) s_warp[t >> 5][k] = v[k];
     }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = red[k][0];
     __syncthreads();
+    if (t < 96) {  // (whole warps shuffle; five values are two and a half)
+        const double x = join16(k16 < NV ? s_warp[l16][k16] : none);
+        if (k16 < NV && l16 == 0) s_block[k16] = x;
+    }
+    cl.sync();
+    if (t < 96) {
+        const double x =
+            join16(k16 < NV && l16 < (int)cl.num_blocks() ? *cl.map_shared_rank(s_block + k16, l16) : none);
+        if (k16 < NV && l16 == 0) s_all[k16] = x;
+    }
+    cl.sync();  // (and no block overwrites its values before all have read them)
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = s_all[k];
 }
 
-// One block per case.  Mass is moved inside the interfaces with the weight
-// w = (rho_hat - lo)(hi - rho_hat) (zero in both bulk phases), then a final
-// scaling makes it exact; T is scaled to the initial energy.
-__global__ void __launch_bounds__(256) k_warm(WarmArgs a) {
-    __shared__ double red[5][256];
-    const long long base = (long long)blockIdx.x * a.P;
+// One cluster of 1 - 16 blocks per case.  Mass is moved inside the interfaces with
+// the weight w = (rho_hat - lo)(hi - rho_hat) (zero in both bulk phases), then a
+// final scaling makes it exact; T is scaled to the initial energy.  Three
+// reductions over the case, each needing the one before, bound by the FP64 units
+// (about 30 operations per site): with one block per case 8 cases of 256^2 kept 8
+// SMs busy for 727 us; a cluster spreads a case over up to 16 SMs, which
+// exchange their sums through distributed shared memory in the same launch, and a
+// thread keeps rho_hat and T_hat of its first WARM_KEEP sites (all, up to 65,536
+// sites per case) between the passes: 86 us.
+__global__ void __launch_bounds__(WARM_THREADS) k_warm(WarmArgs a) {
+    namespace cg = cooperative_groups;
+    __shared__ double s_warp[WARM_THREADS / 32][5];
+    __shared__ double s_block[5], s_all[5];
+    cg::cluster_group cl = cg::this_cluster();
+    const long long base = (long long)(blockIdx.x / cl.num_blocks()) * a.P;
+    const long long first = (long long)cl.block_rank() * WARM_THREADS + threadIdx.x;
+    const long long step = (long long)cl.num_blocks() * WARM_THREADS;
+    double rk[WARM_KEEP], tk[WARM_KEEP];
+    // f(i, rho_hat, T_hat) over this thread's sites
+    auto kept = [&](auto f) {
+#pragma unroll
+        for (int k = 0; k < WARM_KEEP; ++k)
+            if (first + k * step < a.P) f(base + first + k * step, rk[k], tk[k]);
+        for (long long i = first + WARM_KEEP * step; i < a.P; i += step)
+            f(base + i, warm_rho_hat(a, base + i), warm_T_hat(a, base + i));
+    };
+#pragma unroll
+    for (int k = 0; k < WARM_KEEP; ++k)
+        if (first + k * step < a.P) {
+            rk[k] = warm_rho_hat(a, base + first + k * step);
+            tk[k] = warm_T_hat(a, base + first + k * step);
+        }
     // pass 1: S0 = sum rho0, S1 = sum rho_hat, E0 = sum rho0 T0, lo, hi
     double v1[5] = {0.0, 0.0, 0.0, INFINITY, -INFINITY};
-    for (long long i = threadIdx.x; i < a.P; i += 256) {
-        const double r = warm_rho_hat(a, base + i);
-        v1[0] += a.rho0[base + i];
+    kept([&](long long i, double r, double) {
+        v1[0] += a.rho0[i];
         v1[1] += r;
-        v1[2] += a.rho0[base + i] * a.T0[base + i];
+        v1[2] += a.rho0[i] * a.T0[i];
         v1[3] = fmin(v1[3], r);
         v1[4] = fmax(v1[4], r);
-    }
+    });
     const int op1[5] = {0, 0, 0, -1, 1};
-    block_reduce<5>(v1, red, op1);
+    cluster_reduce<5>(v1, op1, s_warp, s_block, s_all);
     const double S0 = v1[0], S1 = v1[1], E0 = v1[2], lo = v1[3], hi = v1[4];
     // pass 2: SW = sum w
     double v2[1] = {0.0};
-    for (long long i = threadIdx.x; i < a.P; i += 256) {
-        const double r = warm_rho_hat(a, base + i);
-        v2[0] += (r - lo) * (hi - r);
-    }
+    kept([&](long long, double r, double) { v2[0] += (r - lo) * (hi - r); });
     const int op2[1] = {0};
-    block_reduce<1>(v2, red, op2);
+    cluster_reduce<1>(v2, op2, s_warp, s_block, s_all);
     double lam = v2[0] > 0.0 ? (S0 - S1) / v2[0] : 0.0;
     const double cap = hi > lo ? 1.0 / (hi - lo) : 1.0;
     lam = fmin(fmax(lam, -cap), cap);
     // pass 3: S2 = sum rho1, Q = sum rho1 T_hat
     double v3[2] = {0.0, 0.0};
-    for (long long i = threadIdx.x; i < a.P; i += 256) {
-        const double r = warm_rho_hat(a, base + i);
+    kept([&](long long, double r, double t) {
         const double r1 = r + lam * (r - lo) * (hi - r);
         v3[0] += r1;
-        v3[1] += r1 * warm_T_hat(a, base + i);
-    }
+        v3[1] += r1 * t;
+    });
     const int op3[2] = {0, 0};
-    block_reduce<2>(v3, red, op3);
+    cluster_reduce<2>(v3, op3, s_warp, s_block, s_all);
     const double fr = S0 / v3[0];
     const double ft = E0 / (fr * v3[1]);
-    for (long long i = threadIdx.x; i < a.P; i += 256) {
-        const double r = warm_rho_hat(a, base + i);
-        a.rho[base + i] = (r + lam * (r - lo) * (hi - r)) * fr;
-        a.T[base + i] = warm_T_hat(a, base + i) * ft;
-    }
+    kept([&](long long i, double r, double t) {
+        a.rho[i] = (r + lam * (r - lo) * (hi - r)) * fr;
+        a.T[i] = t * ft;
+    });
 }
 
 }  // namespace unk

@@ -254,6 +254,26 @@ def test_warm_handoff(torch, N):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("n,h,w", [(2, 64, 64), (3, 65, 64), (2, 200, 123), (2, 256, 256), (1, 264, 320)])
+def test_warm_handoff_clusters(torch, N, n, h, w):
+    """Cases spread over 1 - 16 blocks of a cluster, with sites past the ones a
+    thread keeps; sums of up to 84,480 terms in another order than numpy's."""
+    r = np.random.default_rng(29)
+    pred = r.standard_normal((n, h, w, 2)).astype(np.float32)
+    rho0 = 0.05 + 0.3 * r.random((n, h, w))
+    T0 = 0.08 + 0.01 * r.random((n, h, w))
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    d_rho, d_T = d(rho0), d(T0)
+    N.warm_fields(n, h, w, d(pred), I.UNET_NORM, d_rho, d_T, d_rho, d_T)  # in place
+    torch.cuda.synchronize()
+    nm = I.UNET_NORM
+    rh, th = U.denormalise(pred.astype(np.float64), nm["rho_dev_scale"], nm["t_dev_scale"], rho0, T0)
+    rr, tr = U.warm_project(rh, th, rho0, T0)
+    assert np.allclose(d_rho.cpu().numpy(), rr, rtol=1e-12, atol=0)
+    assert np.allclose(d_T.cpu().numpy(), tr, rtol=1e-12, atol=0)
+
+
+@pytest.mark.gpu
 def test_warmstart_training_learns_without_per_step_sync(torch, N):
     """warmstart.train issues its steps without synchronising and builds every
     augmented batch with torch ops; with the network on the same stream as the
