@@ -103,6 +103,7 @@ struct lb_batch {
     int have_ref = 0;
     int64_t t = 0;
     int64_t ref_time = 0;
+    int64_t checked_t = -1;       // time of the check that wrote the reference fields (-1: none is current)
     cudaGraphExec_t graph = nullptr;
     int graph_k = 0;
     int graph_cur = -1;
@@ -151,7 +152,7 @@ cudaError_t launch_batch_check(lb_batch* b) {
             b->d_ref_rho, b->d_ref_T, b->have_ref, b->d_part);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_batch_fold<<<(b->n + 127) / 128, 128, 0, b->stream>>>(b->d_part, b->d_tile_begin, b->n, b->d_out6);
+    k_batch_fold<<<b->n, 32, 0, b->stream>>>(b->d_part, b->d_tile_begin, b->d_out6);
     return cudaGetLastError();
 }
 
@@ -183,7 +184,7 @@ lb_status rebuild_lists(lb_batch* b) {
                 items.push_back(it);
             }
         }
-        for (int first = 0; first < nx * ny; first += 256) tiles.push_back(BatchTile{d, first});
+        for (int first = 0; first < nx * ny; first += CHECK_SITES) tiles.push_back(BatchTile{d, first});
     }
     begin[b->n] = (int)tiles.size();
     if ((int)items.size() > b->max_items || (int)tiles.size() > b->max_tiles)
@@ -361,7 +362,7 @@ lb_status lb_batch_init(const lb_params* params, int32_t n, const double* const*
         off += 18 * plane;
         fld += (long long)p.nx * p.ny;
         max_items += ((p.nx + b->bx - 1) / b->bx) * ((p.ny + MIN_CHUNK_ROWS - 1) / MIN_CHUNK_ROWS);
-        max_tiles += (p.nx * p.ny + 255) / 256;
+        max_tiles += (p.nx * p.ny + CHECK_SITES - 1) / CHECK_SITES;
     }
     b->n_sites = fld;
     b->buf_bytes = (size_t)off * es;
@@ -464,6 +465,7 @@ lb_status lb_batch_check(lb_batch* b, double* residual, double* mass, double* en
     }
     b->have_ref = 1;
     b->ref_time = b->t;
+    b->checked_t = b->t;
     return LB_OK;
 }
 
@@ -515,6 +517,7 @@ lb_status lb_batch_run(lb_batch* b, double tol, int64_t K, int64_t max_steps, in
         if (st) return st;
         const int64_t Kr = b->t - b->ref_time;
         b->ref_time = b->t;
+        b->checked_t = b->t;
         bool changed = false;
         for (int d = 0; d < b->n; ++d) {
             if (b->frozen[d] >= 0) continue;
@@ -548,11 +551,13 @@ lb_status lb_batch_fields(lb_batch* b, int32_t d, double* rho, double* T) {
     if (!b || d < 0 || d >= b->n) return err(LB_ERR_ARG, "lb_batch_fields: invalid domain");
     BCU(cudaSetDevice(b->device), "cudaSetDevice");
     // a check refreshes the reference fields, which are rho and T of every
-    // active domain; frozen domains keep the fields of their last check
-    if (b->frozen[d] < 0) {
+    // active domain, unless one has at this time; frozen domains keep the
+    // fields of their last check
+    if (b->frozen[d] < 0 && b->checked_t != b->t) {
         BCU(launch_batch_check(b), "batch fields");
         b->have_ref = 1;
         b->ref_time = b->t;
+        b->checked_t = b->t;
     }
     const size_t nb = sizeof(double) * (size_t)b->params[d].nx * b->params[d].ny;
     if (rho) BCU(cudaMemcpyAsync(rho, b->d_ref_rho + b->doms[d].fld_off, nb, cudaMemcpyDeviceToHost, b->stream), "fields download");
@@ -573,6 +578,7 @@ lb_status lb_batch_restart(lb_batch* b, int32_t d, const double* rho0, const dou
     // the fields are staged in the domain's residual reference (its next
     // residual compares with them), then the state is built in the buffer the
     // active domains currently hold
+    b->checked_t = -1;  // (the staged fields are not the state's rounded rho and T)
     BCU(cudaMemcpyAsync(r, rho0, nb, cudaMemcpyDefault, b->stream), "restart fields");
     BCU(cudaMemcpyAsync(tt, T0, nb, cudaMemcpyDefault, b->stream), "restart fields");
     void* dst = b->prec == LB_PREC_FP32 ? static_cast<void*>(static_cast<float*>(b->buf[b->cur]) + D.off)

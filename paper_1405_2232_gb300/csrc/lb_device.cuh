@@ -330,6 +330,23 @@ __device__ __forceinline__ bool negative_bits(double x) {
 __device__ __forceinline__ bool finite_bits(float x) { return isfinite(x); }
 __device__ __forceinline__ bool negative_bits(float x) { return x < 0.0f; }
 
+// (double)x on the integer units where x is normal or zero
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x), mag = b & 0x7fffffffu;
+    if (mag - 0x00800000u < 0x7f000000u)  // normal
+        return __hiloint2double((int)((b & 0x80000000u) | ((mag >> 3) + (896u << 20))), (int)(b << 29));
+    if (mag == 0u) return __hiloint2double((int)b, 0);
+    return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
+// s += x, the rounding error of the addition added to err
+__device__ __forceinline__ void add_exact(float& s, float x, float& err) {
+    const float t = s + x, d = t - s;
+    err += (s - (t - d)) + (x - d);
+    s = t;
+}
+
 template <typename real>
 __device__ __forceinline__ real p_eos(const KParams& kp, real rho, real T) {
     const real R = KPR(kp, R), a = KPR(kp, a), b = KPR(kp, b);

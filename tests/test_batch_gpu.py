@@ -250,3 +250,50 @@ def test_batch_many_items_per_cta_match_lone_runs(lb, precision):
                 e_rho = np.abs(rho - m[0]).max() / np.abs(m[0]).max()
                 e_T = np.abs(T - m[3]).max() / np.abs(m[3]).max()
                 assert e_rho < 1e-6 and e_T < 1e-6, (d, specs[d][:2], e_rho, e_T)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_check_sums_are_the_exact_sums(lb, prec):
+    """Mass and energy of the check at the edges of its 2,048-site tiles: the FP64
+    sums of the stored populations of a lone context (sums of at most 50,000
+    terms: 1e-14), and the residual's norms from the fields."""
+    sizes = [(3, 3), (64, 32), (45, 45), (64, 33), (31, 67), (90, 61)]
+    params, rhos, Ts = [], [], []
+    for k, (nx, ny) in enumerate(sizes):
+        rho, T = I.slab_fields(nx, ny, width=max(2, nx // 2), noise=1e-3, seed=k + 1)
+        params.append(lb.lb_params_default(nx=nx, ny=ny, precision=prec, psi_uses_local_T=0, T_psi=0.85 * I.CS_TC))
+        rhos.append(rho)
+        Ts.append(T)
+    with lb.Batch(params, rhos, Ts) as B:
+        _, mass, energy, status = B.check()
+        before = [B.fields(d) for d in range(len(sizes))]
+        B.step(7)
+        resid, _, _, _ = B.check()
+        after = [B.fields(d) for d in range(len(sizes))]
+    assert not status.any()
+    for d, p in enumerate(params):
+        with lb.Lattice(rhos[d], Ts[d], nx=p.nx, ny=p.ny, precision=prec) as L:
+            f, g = L.populations()
+        assert abs(mass[d] - f.sum()) <= 1e-14 * f.sum() and abs(energy[d] - g.sum()) <= 1e-14 * g.sum()
+        r = max(np.linalg.norm(a - b) / (7 * np.linalg.norm(a)) for a, b in zip(after[d], before[d]))
+        assert abs(resid[d] - r) <= 1e-12 * r
+
+
+@pytest.mark.gpu
+def test_fields_after_restart_are_the_state(lb):
+    """fields() reuses the check of the same time, but not across a restart, whose
+    staged FP64 fields are not yet the FP32 state's."""
+    rho, T = I.slab_fields(40, 36, noise=1e-3)
+    p = [lb.lb_params_default(nx=40, ny=36, precision="fp32") for _ in range(2)]
+    with lb.Batch(p, [rho, rho], [T, T]) as B:
+        fresh = B.fields(0)
+        B.step(3)
+        moved = B.fields(0)
+        again = B.fields(0)
+        B.restart(0, rho, T)
+        back = B.fields(0)
+        other = B.fields(1)
+    assert np.array_equal(moved[0], again[0]) and np.array_equal(other[0], moved[0])
+    assert np.array_equal(back[0], fresh[0]) and np.array_equal(back[1], fresh[1])
+    assert not np.array_equal(back[0], rho) and not np.array_equal(back[0], moved[0])
