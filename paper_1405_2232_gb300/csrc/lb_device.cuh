@@ -889,96 +889,6 @@ __device__ __forceinline__ void store_site_dev(typename S::elem* d, IT stride, c
     put_planes<S>(d, stride, kp.nx, v, ghost_lo, ghost_hi);
 }
 
-// ---------------------------------------------------------------- moments
-// Same front end as the step; phase 2 writes rho, u (with F/2), T (any
-// pointer may be null) and, if `part` is set, reduces FP64 totals per CTA:
-//   part[blk*8 + k], k = mass, energy, rho ux, rho uy, |d rho|^2, rho^2, |dT|^2, T^2
-// against the reference fields ref_rho/ref_T (may be null).
-template <int PREC, int BX, int BY, int BMODE>
-__global__ void __launch_bounds__(BX* BY)
-    k_moments(const typename Store<PREC>::elem* __restrict__ src, const KParams kp,
-              double* __restrict__ o_rho, double* __restrict__ o_ux, double* __restrict__ o_uy,
-              double* __restrict__ o_T, const double* __restrict__ ref_rho,
-              const double* __restrict__ ref_T, double* __restrict__ part) {
-    using S = Store<PREC>;
-    using real = typename S::real;
-    constexpr int WX = BX + 2, WY = BY + 2, NT = BX * BY;
-    __shared__ real s_psi[BMODE != BETA_ZERO ? WX * WY : 1];
-    __shared__ real s_psi2[BMODE != BETA_ONE ? WX * WY : 1];
-    __shared__ double s_red[NT / 32][8];
-
-    const int tid = threadIdx.x + threadIdx.y * BX;
-    const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
-    int flags = 0;
-    for (int s = tid; s < WX * WY; s += NT) {
-        const int ly = s / WX, lx = s - ly * WX;
-        const int gx = ringc(kp, x0 + lx - 1, kp.nx), gy = ringc(kp, y0 + ly - 1, kp.ny);
-        real f[9], g[9], rho, e, T, psi, psi2;
-        pull18<S>(src, kp, gx, gy, f, g);
-        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
-        if (BMODE != BETA_ZERO) s_psi[s] = psi;
-        if (BMODE != BETA_ONE) s_psi2[s] = psi2;
-    }
-    __syncthreads();
-
-    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    const int gx = x0 + threadIdx.x, gy = y0 + threadIdx.y;
-    if (gx < kp.nx && gy < kp.ny) {
-        real f[9], g[9];
-        pull18<S>(src, kp, gx, gy, f, g);
-        real rho = f[0];
-        double m = (double)f[0], e = (double)g[0];
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            rho += f[i];
-            m += (double)f[i];
-            e += (double)g[i];
-        }
-        real Fx, Fy, ux, uy, T;
-        force_from_window<real, BMODE>(kp, s_psi, s_psi2, (threadIdx.y + 1) * WX + threadIdx.x + 1,
-                                       WX, Fx, Fy);
-        if (kp.walls) Fy += -rho * KPR(kp, g_grav);  // cavity buoyancy
-        collide<real, false>(kp, f, g, rho, Fx, Fy, ux, uy, T);
-        const long long idx = (long long)gy * kp.nx + gx;
-        if (o_rho) o_rho[idx] = (double)rho;
-        if (o_ux) o_ux[idx] = (double)ux;
-        if (o_uy) o_uy[idx] = (double)uy;
-        if (o_T) o_T[idx] = (double)T;
-        if (part) {
-            const double dr = (double)rho, dT = (double)T;
-            v[0] = m;
-            v[1] = e;
-            v[2] = dr * (double)ux;
-            v[3] = dr * (double)uy;
-            if (ref_rho) {
-                const double a = dr - ref_rho[idx], b = dT - ref_T[idx];
-                v[4] = a * a;
-                v[6] = b * b;
-            }
-            v[5] = dr * dr;
-            v[7] = dT * dT;
-        }
-    } else {
-        flags = 0;
-    }
-    if (flags) atomicOr(kp.err, flags);
-    if (!part) return;
-    // deterministic block reduction: warp tree, then warps in order
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        double x = v[k];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-        if ((tid & 31) == 0) s_red[tid >> 5][k] = x;
-    }
-    __syncthreads();
-    if (tid < 8) {
-        double x = 0.0;
-        for (int w = 0; w < NT / 32; ++w) x += s_red[w][tid];
-        part[(long long)(blockIdx.y * gridDim.x + blockIdx.x) * 8 + tid] = x;
-    }
-}
-
 // ---------------------------------------------------------------- init / gather
 // Initial state f = f^eq(rho0, 0) = w_i rho0, g = c_v T0 w_i rho0, written at
 // the source position so the first pull sees it at its own site.

@@ -109,28 +109,6 @@ cudaError_t LBGB_CAT(launch_step_, LBGB_NAME)(const StepLaunch& L) {
     return cudaErrorInvalidValue;
 }
 
-cudaError_t LBGB_CAT(launch_moments_, LBGB_NAME)(const MomentsLaunch& L) {
-    using E = typename Store<LBGB_PREC>::elem;
-    const dim3 block(MOM_BX, MOM_BY);
-    const dim3 grid((L.kp.nx + MOM_BX - 1) / MOM_BX, (L.kp.ny + MOM_BY - 1) / MOM_BY);
-    const E* src = static_cast<const E*>(L.src);
-    switch (L.bmode) {
-        case BETA_ZERO:
-            k_moments<LBGB_PREC, MOM_BX, MOM_BY, BETA_ZERO><<<grid, block, 0, L.stream>>>(
-                src, L.kp, L.rho, L.ux, L.uy, L.T, L.ref_rho, L.ref_T, L.part);
-            break;
-        case BETA_ONE:
-            k_moments<LBGB_PREC, MOM_BX, MOM_BY, BETA_ONE><<<grid, block, 0, L.stream>>>(
-                src, L.kp, L.rho, L.ux, L.uy, L.T, L.ref_rho, L.ref_T, L.part);
-            break;
-        default:
-            k_moments<LBGB_PREC, MOM_BX, MOM_BY, BETA_MIXED><<<grid, block, 0, L.stream>>>(
-                src, L.kp, L.rho, L.ux, L.uy, L.T, L.ref_rho, L.ref_T, L.part);
-            break;
-    }
-    return cudaGetLastError();
-}
-
 namespace {
 int elementwise_blocks(const KParams& kp) {
     const long long n = (long long)kp.nx * kp.ny;

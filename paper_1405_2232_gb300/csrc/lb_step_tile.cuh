@@ -161,6 +161,26 @@ struct PullAt {
     }
 };
 
+// Site (lx, ly) of thread tid relative to the tile's first: the tile row by row, then
+// the ring (the rows below and above with their corners, then the sides in turn).
+template <int BX>
+__device__ __forceinline__ void tile_site(int tid, int by, int& lx, int& ly) {
+    constexpr int WX = BX + 2;
+    if (tid < BX * by) {
+        lx = tid % BX;
+        ly = tid / BX;
+        return;
+    }
+    const int r = tid - BX * by;
+    if (r < 2 * WX) {
+        lx = (r < WX ? r : r - WX) - 1;
+        ly = r < WX ? -1 : by;
+    } else {
+        lx = (r & 1) ? BX : -1;
+        ly = (r - 2 * WX) >> 1;  // (past the ring: ly >= by)
+    }
+}
+
 // One step of the tile at (x0, y0): see the head of the file.  Every thread of
 // the block calls it (one barrier inside).
 template <int PREC, int BX, int WALLS, bool EQ24, int BMODE>
@@ -174,23 +194,10 @@ __device__ __forceinline__ void tile_step(const typename Store<PREC>::elem* src,
     const int tid = threadIdx.x, nx = kp.nx, ny = kp.ny;
     const bool own = tid < BX * by;
     int lx, ly;
-    if (own) {
-        lx = tid % BX;
-        ly = tid / BX;
-    } else {
-        const int r = tid - BX * by;
-        if (r < 2 * WX) {
-            lx = (r < WX ? r : r - WX) - 1;
-            ly = r < WX ? -1 : by;
-        } else {
-            lx = (r & 1) ? BX : -1;
-            ly = (r - 2 * WX) >> 1;  // past the ring: ly >= by, out of range below
-        }
-    }
+    tile_site<BX>(tid, by, lx, ly);
     // rows updated: [H, ny - H) (H = kp.halo_rows; 0 on a periodic lattice)
     const int W = min(BX, nx - x0), Hh = min(by, ny - kp.halo_rows - y0);
-    const bool in_ring = own || tid - BX * by < 2 * WX + 2 * by;
-    const bool need = in_ring && lx <= W && ly <= Hh;  // the tile and one site around it
+    const bool need = tid - BX * by < tile_ring(BX, by) && lx <= W && ly <= Hh;  // the tile and one site around it
     real f[9], g[9], rho = 0, e = 0, T = 0;  // (16-bit modes: the stored deviations)
     float Hf = 0.0f, Hg = 0.0f;
     // (the tile starts inside the lattice: one site past it at most is needed)
@@ -260,6 +267,137 @@ __global__ void __launch_bounds__(tile_threads(BX, tile_max_by(BX)))
     tile_step<PREC, BX, WALLS, EQ24, BMODE>(src, dst, kp, blockIdx.x * BX, kp.halo_rows + blockIdx.y * by, by, s_psi,
                                             s_psi2, flags);
     if (flags) atomicOr(kp.err, flags);
+}
+
+// ---------------------------------------------------------------- moments
+// Sum of v[0..7] over the warp: halving steps exchange half of the values each
+// (nine additions instead of eight times five).  Lane 4 k returns the sum of v[k].
+__device__ __forceinline__ double warp_sum8(double v[8], int lane) {
+#pragma unroll
+    for (int h = 4; h > 0; h >>= 1) {
+        const bool up = lane & (4 * h);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k < h) {
+                const double send = up ? v[k] : v[k + h], keep = up ? v[k + h] : v[k];
+                v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+            }
+    }
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+    v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+    return v[0];
+}
+
+// Macroscopic fields of the state as the step forms them: rho, u (with F/2), T (any
+// pointer may be null), on the tile and psi ring of tile_step, and with PART the
+// FP64 totals of each block:
+//   part[blk*8 + k], k = mass, energy, rho ux, rho uy, |d rho|^2, rho^2, |dT|^2, T^2
+// against the reference fields ref_rho/ref_T (may be null).  Each site pulled once,
+// the parameters read as floats and the results widened on the integer units:
+// 4096^2 FP32 fields 340 us, 1,543 us with the two pulls, the FP64 conversions and the
+// whole collision of the kernel before (bytes: 72 read, 32 written per site).
+template <int PREC, int BMODE, bool PART>
+__global__ void __launch_bounds__(tile_threads(32, 8))
+    k_moments(const typename Store<PREC>::elem* __restrict__ src, const KParams kp,
+              double* __restrict__ o_rho, double* __restrict__ o_ux, double* __restrict__ o_uy,
+              double* __restrict__ o_T, const double* __restrict__ ref_rho,
+              const double* __restrict__ ref_T, double* __restrict__ part) {
+    using S = Store<PREC>;
+    using real = typename S::real;
+    constexpr int BX = 32, BY = 8, WX = BX + 2, WY = BY + 2;
+    __shared__ real s_psi[BMODE != BETA_ZERO ? WX * WY : 1];
+    __shared__ real s_psi2[BMODE != BETA_ONE ? WX * WY : 1];
+    __shared__ double s_red[BY][8];
+    const int tid = threadIdx.x, nx = kp.nx, ny = kp.ny;
+    const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
+    const bool own = tid < BX * BY;
+    int lx, ly;
+    tile_site<BX>(tid, BY, lx, ly);
+    const int W = min(BX, nx - x0), Hh = min(BY, ny - y0);
+    const bool active = own && lx < W && ly < Hh;
+    int gx = x0 + lx, gy = y0 + ly, flags = 0;
+    real rho = 0, e = 0, T = 0, mx = 0, my = 0;
+    double m = 0, en = 0;
+    if (tid - BX * BY < tile_ring(BX, BY) && lx <= W && ly <= Hh) {
+        gx = kp.walls ? clampc(gx, nx) : (gx < 0 ? gx + nx : (gx >= nx ? gx - nx : gx));
+        gy = kp.walls ? clampc(gy, ny) : (gy < 0 ? gy + ny : (gy >= ny ? gy - ny : gy));
+        real f[9], g[9], psi, psi2;
+        pull18<S>(src, kp, gx, gy, f, g);
+        site_psi<real, BMODE>(kp, f, g, rho, e, T, psi, psi2, flags);
+        if (BMODE != BETA_ZERO) s_psi[(ly + 1) * WX + lx + 1] = psi;
+        if (BMODE != BETA_ONE) s_psi2[(ly + 1) * WX + lx + 1] = psi2;
+        if constexpr (sizeof(real) == 8) {
+            mx = ((((f[1] - f[3]) + f[5]) - f[6]) - f[7]) + f[8];
+            my = ((((f[2] - f[4]) + f[5]) + f[6]) - f[7]) - f[8];
+        } else {
+            mx = (f[1] - f[3]) + ((f[5] - f[7]) + (f[8] - f[6]));
+            my = (f[2] - f[4]) + ((f[5] - f[7]) + (f[6] - f[8]));
+        }
+        if constexpr (PART) {
+            if constexpr (sizeof(real) == 8) {
+                m = rho;
+                en = e;
+            } else {
+                // rho and e with their rounding errors: the exact sums
+                float r = f[0], q = g[0], r_err = 0.0f, q_err = 0.0f;
+#pragma unroll
+                for (int i = 1; i < 9; ++i) {
+                    add_exact(r, f[i], r_err);
+                    add_exact(q, g[i], q_err);
+                }
+                m = widen(r) + widen(r_err);
+                en = widen(q) + widen(q_err);
+            }
+        }
+    }
+    if (flags) atomicOr(kp.err, flags);
+    __syncthreads();
+    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (active) {
+        real Fx, Fy, ux, uy;
+        force_from_window<real, BMODE>(kp, s_psi, s_psi2, (ly + 1) * WX + lx + 1, WX, Fx, Fy);
+        if (kp.walls) Fy += -rho * KPR(kp, g_grav);  // cavity buoyancy
+        if constexpr (sizeof(real) == 8) {
+            ux = (mx + 0.5 * Fx) / rho;
+            uy = (my + 0.5 * Fy) / rho;
+        } else {
+            const real inv_rho = (real)1 / rho;
+            ux = (mx + (real)0.5 * Fx) * inv_rho;
+            uy = (my + (real)0.5 * Fy) * inv_rho;
+        }
+        const long long idx = (long long)gy * nx + gx;
+        const double dr = widen(rho), dux = widen(ux), duy = widen(uy), dT = widen(T);
+        if (o_rho) o_rho[idx] = dr;
+        if (o_ux) o_ux[idx] = dux;
+        if (o_uy) o_uy[idx] = duy;
+        if (o_T) o_T[idx] = dT;
+        if constexpr (PART) {
+            v[0] = m;
+            v[1] = en;
+            v[2] = dr * dux;
+            v[3] = dr * duy;
+            if (ref_rho) {
+                const double a = dr - ref_rho[idx], b = dT - ref_T[idx];
+                v[4] = a * a;
+                v[6] = b * b;
+            }
+            v[5] = dr * dr;
+            v[7] = dT * dT;
+        }
+    }
+    if constexpr (PART) {
+        // deterministic block reduction: lanes, then warps in order
+        if (own) {
+            const double x = warp_sum8(v, tid & 31);
+            if ((tid & 3) == 0) s_red[tid >> 5][(tid & 31) >> 2] = x;
+        }
+        __syncthreads();
+        if (tid < 8) {
+            double x = 0.0;
+            for (int w = 0; w < BY; ++w) x += s_red[w][tid];
+            part[(long long)(blockIdx.y * gridDim.x + blockIdx.x) * 8 + tid] = x;
+        }
+    }
 }
 
 }  // namespace lbgb

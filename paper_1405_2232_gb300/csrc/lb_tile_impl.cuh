@@ -92,4 +92,25 @@ cudaError_t LBGB_CAT(launch_tile_, LBGB_NAME)(const StepLaunch& L) {
     return cudaErrorInvalidValue;
 }
 
+namespace {
+template <int BM, bool PART>
+void moments(const MomentsLaunch& L, dim3 grid) {
+    using E = typename Store<LBGB_PREC>::elem;
+    k_moments<LBGB_PREC, BM, PART><<<grid, tile_threads(MOM_BX, MOM_BY), 0, L.stream>>>(
+        static_cast<const E*>(L.src), L.kp, L.rho, L.ux, L.uy, L.T, L.ref_rho, L.ref_T, L.part);
+}
+}  // namespace
+
+cudaError_t LBGB_CAT(launch_moments_, LBGB_NAME)(const MomentsLaunch& L) {
+    static_assert(MOM_BX == 32 && MOM_BY == 8, "the tile of k_moments");
+    const dim3 grid((L.kp.nx + MOM_BX - 1) / MOM_BX, (L.kp.ny + MOM_BY - 1) / MOM_BY);
+    if (L.bmode == BETA_ZERO)
+        L.part ? moments<BETA_ZERO, true>(L, grid) : moments<BETA_ZERO, false>(L, grid);
+    else if (L.bmode == BETA_ONE)
+        L.part ? moments<BETA_ONE, true>(L, grid) : moments<BETA_ONE, false>(L, grid);
+    else
+        L.part ? moments<BETA_MIXED, true>(L, grid) : moments<BETA_MIXED, false>(L, grid);
+    return cudaGetLastError();
+}
+
 }  // namespace lbgb
