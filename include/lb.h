@@ -380,13 +380,17 @@ int64_t lb_batch_time(const lb_batch* b);
 /* Release the batch.  NULL is accepted. */
 lb_status lb_batch_free(lb_batch* b);
 
-/* Work-list granularity: every domain strip is cut into row chunks of about
- * `rows` rows (>= 16; default 64); smaller chunks balance uneven domains over
- * the persistent CTAs, larger ones re-read fewer halo rows.
- * lb_batch_set_chunk_rows rebuilds the lists (synchronises); LB_ERR_ARG for
- * rows < 16.  lb_batch_chunk_rows returns the current height (-1 for NULL).
+/* Work-list granularity of the strip kernel: every domain strip is cut into row
+ * chunks of about `rows` rows (>= 16; default 64); smaller chunks balance uneven
+ * domains over the persistent CTAs, larger ones re-read fewer halo rows.  Without a
+ * height set or tuned, the library runs small batches on the tile kernel and takes
+ * the height in 16 .. 64 that balances the active domains on the others.
+ * lb_batch_set_chunk_rows runs the strip kernel at that height (rebuilds the lists,
+ * synchronises); LB_ERR_ARG for rows < 16.  lb_batch_chunk_rows returns the height
+ * set or tuned (64 before; -1 for NULL).
  * lb_batch_autotune times `steps` batched steps (after 2 warm-up steps) for
- * each of the LB_BATCH_TUNE_N heights 16, 32, 64, 128, keeps the fastest and
+ * each of the LB_BATCH_TUNE_N heights 16, 32, 64, 128, keeps the fastest (or the
+ * tile kernel, where the library would run it and it is faster still) and
  * writes it to *chunk_rows (may be NULL); ms_per_step[k] (may be NULL) gets
  * each height's time per step.  The batch state, its time and its error
  * words are restored afterwards, bit for bit (one temporary device copy of

@@ -87,7 +87,13 @@ struct lb_batch {
     int* d_err = nullptr;
     // work lists
     BatchItem* d_items = nullptr;
-    int* d_counts = nullptr;      // [0] items, [1] tiles
+    int* d_counts = nullptr;      // [0] items, [1] check tiles, [2] step tiles
+    // tile step (tile_by > 0): its tiles instead of the strip kernel's items
+    int tile_by = 0;
+    bool strip_asked = false;     // the caller set a chunk height: the strip kernel
+    int n_step_tiles = 0;
+    int cap_step_tiles = 0;
+    BatchStepTile* d_step_tiles = nullptr;
     int* d_next = nullptr;        // takes from the work counter in the current step (the step resets it)
     int max_items = 0;
     BatchTile* d_tiles = nullptr;
@@ -107,6 +113,8 @@ struct lb_batch {
     cudaGraphExec_t graph = nullptr;
     int graph_k = 0;
     int graph_cur = -1;
+    int graph_by = 0;
+    int graph_grid = 0;           // tile step: blocks of the captured launches
 };
 
 namespace {
@@ -114,6 +122,13 @@ namespace {
 // Launch one batched step src -> dst; with src == nullptr only set the
 // kernel's shared-memory attribute (done once, outside any stream capture).
 cudaError_t launch_batch_step(lb_batch* b, const void* src, void* dst) {
+    if (b->tile_by || !src) {
+        const BatchTileLaunch L = {src, dst, b->d_doms, b->d_step_tiles, b->d_counts + 2, b->n_step_tiles, b->tile_by,
+                                   b->eq24, b->bmode, b->sms, b->stream};
+        if (src && !b->n_step_tiles) return cudaSuccess;
+        const cudaError_t e = b->prec == LB_PREC_FP32 ? launch_batch_tile_fp32(L) : launch_batch_tile_fp64(L);
+        if (src || e != cudaSuccess) return e;
+    }
     const int grid = 2 * b->sms;
     if (b->prec == LB_PREC_FP32) {
         using E = float;
@@ -156,8 +171,94 @@ cudaError_t launch_batch_check(lb_batch* b) {
     return cudaGetLastError();
 }
 
+// Height of the tiles the active domains step in (0: the strip kernel): up to 1.5 x
+// 2^20 sites in FP32 (12 domains of 174,000 sites 84 -> 7.6 us per step, a lone 64^2 68
+// -> 2.8 us; 2.1 million sites in 128 domains 84 us on strips against 90), 2^20 in FP64.
+int batch_tile_rows(const lb_batch* b) {
+    if (b->strip_asked) return 0;
+    long long sites = 0;
+    for (int d = 0; d < b->n; ++d)
+        if (b->frozen[d] < 0) sites += (long long)b->params[d].nx * b->params[d].ny;
+    if (sites > (b->prec == LB_PREC_FP32 ? 3LL << 19 : (1LL << 20) - 1)) return 0;
+    return balanced_tile_rows(b->prec, b->sms, 1, [&](int by) {
+        long long t = 0;
+        for (int d = 0; d < b->n; ++d)
+            if (b->frozen[d] < 0) t += (long long)((b->params[d].nx + 31) / 32) * ((b->params[d].ny + by - 1) / by);
+        return t;
+    });
+}
+
+// Cost of a work item of the strip kernel: its jobs (rows plus the two halo rows; a
+// half item's two halves march together, so the left half's rows) times the
+// columns they keep busy plus a per-row constant (a narrow strip still pays the
+// row's barrier and latencies).
+long long item_cost(const lb_batch* b, int nx, int strip, int y0, int y1, int half) {
+    const long long w = std::min(b->bx, nx - strip * b->bx);
+    if (half) return (long long)(batch_split(y0, y1) - y0 + 2) * (2 * w + 64);
+    return (long long)(y1 - y0 + 2) * (w + 64);
+}
+
+// Height of the strip kernel's row chunks: the caller's, or with none asked the one
+// in 16 .. chunk_rows whose items finish first by their cost, where the tallest gives
+// the persistent CTAs fewer than four items each (n items of mean m and longest c on G
+// CTAs: the lesser of ceil(n/G) c and sum/G + m/2).  28 domains of 3.3 million sites:
+// 64 rows 123 us per step, 16 rows 110; 128 domains of 128^2: 84 and 90.
+int chunk_rows_used(const lb_batch* b) {
+    if (b->strip_asked) return b->chunk_rows;
+    const double G = 2.0 * b->sms;
+    int best = b->chunk_rows;
+    double best_cost = 0.0;
+    for (int rows = b->chunk_rows; rows >= MIN_CHUNK_ROWS; rows -= MIN_CHUNK_ROWS / 2) {
+        double sum = 0.0, longest = 0.0, n = 0.0;
+        for (int d = 0; d < b->n; ++d) {
+            if (b->frozen[d] >= 0) continue;
+            const int nx = b->params[d].nx, ny = b->params[d].ny;
+            const int strips = (nx + b->bx - 1) / b->bx, chunks = (ny + rows - 1) / rows;
+            for (int s = 0; s < strips; ++s) {
+                const int half = 2 * std::min(b->bx, nx - s * b->bx) <= b->bx ? 1 : 0;
+                const double c = (double)item_cost(b, nx, s, 0, (ny + chunks - 1) / chunks, half);
+                n += chunks;
+                sum += c * chunks;
+                longest = std::max(longest, c);
+            }
+        }
+        if (rows == b->chunk_rows && n >= 4.0 * G) return rows;
+        const double cost = std::max(sum / G, std::min(std::ceil(n / G) * longest, sum / G + 0.5 * sum / std::max(n, 1.0)));
+        if (rows == b->chunk_rows || cost < 0.98 * best_cost) {
+            best = rows;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
 // Rebuild the step work list and the check tile list from the active set.
 lb_status rebuild_lists(lb_batch* b) {
+    std::vector<BatchStepTile> step_tiles;
+    b->tile_by = batch_tile_rows(b);
+    for (int d = 0; d < b->n && b->tile_by; ++d) {
+        if (b->frozen[d] >= 0) continue;
+        for (int y = 0; y < b->params[d].ny; y += b->tile_by)
+            for (int x = 0; x < b->params[d].nx; x += 32) step_tiles.push_back(BatchStepTile{d, x, y, 0});
+    }
+    b->n_step_tiles = (int)step_tiles.size();
+    if (b->n_step_tiles > b->cap_step_tiles) {
+        if (b->graph) {  // it holds the list's address
+            cudaGraphExecDestroy(b->graph);
+            b->graph = nullptr;
+        }
+        cudaFree(b->d_step_tiles);
+        b->d_step_tiles = nullptr;
+        b->cap_step_tiles = 0;
+        BCU(cudaMalloc(&b->d_step_tiles, sizeof(BatchStepTile) * step_tiles.size()), "step tile list");
+        b->cap_step_tiles = b->n_step_tiles;
+    }
+    if (b->graph && (b->graph_by != b->tile_by || b->n_step_tiles > b->graph_grid ||
+                     (b->tile_by && 4 * b->n_step_tiles < b->graph_grid))) {
+        cudaGraphExecDestroy(b->graph);  // another kernel, or a grid too small or mostly idle
+        b->graph = nullptr;
+    }
+    const int rows = chunk_rows_used(b);
     std::vector<BatchItem> items;
     std::vector<BatchTile> tiles;
     std::vector<int> begin(b->n + 1, 0);
@@ -166,7 +267,7 @@ lb_status rebuild_lists(lb_batch* b) {
         if (b->frozen[d] >= 0) continue;
         const int nx = b->params[d].nx, ny = b->params[d].ny;
         const int strips = (nx + b->bx - 1) / b->bx;
-        const int chunks = (ny + b->chunk_rows - 1) / b->chunk_rows;
+        const int chunks = (ny + rows - 1) / rows;
         for (int s = 0; s < strips; ++s) {
             // a strip at most half the kernel's width runs as half items: the
             // chunk's rows split between the two halves of the CTA, so the item
@@ -190,19 +291,16 @@ lb_status rebuild_lists(lb_batch* b) {
     if ((int)items.size() > b->max_items || (int)tiles.size() > b->max_tiles)
         return err(LB_ERR_ARG, "batch work list larger than allocated");
     // Longest item first: the persistent CTAs take items in this order from a
-    // global counter, so the short items fill in at the end.  Cost of an item:
-    // its jobs (rows plus the two halo rows; a half item's two halves march
-    // together, so the left half's rows) times the columns they keep busy
-    // plus a per-row constant (a narrow strip still pays the row's barrier
-    // and latencies).
+    // global counter, so the short items fill in at the end.
     auto cost = [&](const BatchItem& a) {
-        const long long w = std::min(b->bx, b->params[a.domain].nx - a.strip * b->bx);
-        if (a.half) return (long long)(batch_split(a.y0, a.y1) - a.y0 + 2) * (2 * w + 64);
-        return (long long)(a.y1 - a.y0 + 2) * (w + 64);
+        return item_cost(b, b->params[a.domain].nx, a.strip, a.y0, a.y1, a.half);
     };
     std::stable_sort(items.begin(), items.end(),
                      [&](const BatchItem& a, const BatchItem& c) { return cost(a) > cost(c); });
-    int counts[2] = {(int)items.size(), (int)tiles.size()};
+    int counts[3] = {(int)items.size(), (int)tiles.size(), b->n_step_tiles};
+    if (b->n_step_tiles)
+        BCU(cudaMemcpyAsync(b->d_step_tiles, step_tiles.data(), sizeof(BatchStepTile) * step_tiles.size(),
+                            cudaMemcpyHostToDevice, b->stream), "step tile list upload");
     if (!items.empty())
         BCU(cudaMemcpyAsync(b->d_items, items.data(), sizeof(BatchItem) * items.size(),
                             cudaMemcpyHostToDevice, b->stream), "work list upload");
@@ -233,6 +331,7 @@ void release(lb_batch* b) {
     cudaFree(b->d_counts);
     cudaFree(b->d_next);
     cudaFree(b->d_tiles);
+    cudaFree(b->d_step_tiles);
     cudaFree(b->d_tile_begin);
     cudaFree(b->d_part);
     cudaFree(b->d_out6);
@@ -373,7 +472,7 @@ lb_status lb_batch_init(const lb_params* params, int32_t n, const double* const*
     if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(int) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_doms, sizeof(BatchDomain) * n);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(BatchItem) * (max_items > 0 ? max_items : 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_counts, sizeof(int) * 2);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_counts, sizeof(int) * 3);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_next, sizeof(int) * 2);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_next, 0, sizeof(int) * 2, b->stream);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, sizeof(BatchTile) * (max_tiles > 0 ? max_tiles : 1));
@@ -507,6 +606,8 @@ lb_status lb_batch_run(lb_batch* b, double tol, int64_t K, int64_t max_steps, in
             cudaGraphDestroy(g);
             if (e != cudaSuccess) return cuerr(e, "instantiating the batch graph");
             b->graph_k = (int)K;
+            b->graph_by = b->tile_by;
+            b->graph_grid = b->n_step_tiles;
             b->graph_cur = b->cur;
         }
         BCU(cudaGraphLaunch(b->graph, b->stream), "graph launch");
@@ -610,6 +711,7 @@ lb_status lb_batch_set_chunk_rows(lb_batch* b, int32_t rows) {
         return err(LB_ERR_ARG, "lb_batch_set_chunk_rows: rows must be >= %d", MIN_CHUNK_ROWS);
     BCU(cudaSetDevice(b->device), "cudaSetDevice");
     b->chunk_rows = rows;
+    b->strip_asked = true;
     return rebuild_lists(b);
 }
 
@@ -634,11 +736,18 @@ lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
     lb_status st = LB_OK;
     double best = INFINITY;
     int best_rows = rows0;
-    for (int k = 0; k < LB_BATCH_TUNE_N && e == cudaSuccess && st == LB_OK; ++k) {
-        if (ms_per_step) ms_per_step[k] = NAN;
-        b->chunk_rows = kChunkCand[k];
+    // the strip kernel at every height, then the tile step where the library would
+    // run it (the tuned batch keeps the faster kernel)
+    const bool asked0 = b->strip_asked;
+    bool strip_best = true;
+    for (int k = 0; k <= LB_BATCH_TUNE_N && e == cudaSuccess && st == LB_OK; ++k) {
+        const bool strip = k < LB_BATCH_TUNE_N;
+        if (strip && ms_per_step) ms_per_step[k] = NAN;
+        if (strip) b->chunk_rows = kChunkCand[k];
+        b->strip_asked = strip;
         st = rebuild_lists(b);
         if (st != LB_OK) break;
+        if (!strip && !b->tile_by) break;
         for (int w = 0; w < 2 && e == cudaSuccess; ++w) {
             e = launch_batch_step(b, b->buf[b->cur], b->buf[b->cur ^ 1]);
             b->cur ^= 1;
@@ -654,14 +763,16 @@ lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, ev[0], ev[1]);
         if (e != cudaSuccess) break;
         const double per = (double)ms / steps;
-        if (ms_per_step) ms_per_step[k] = per;
+        if (strip && ms_per_step) ms_per_step[k] = per;
         if (per < best) {
             best = per;
-            best_rows = kChunkCand[k];
+            strip_best = strip;
+            if (strip) best_rows = kChunkCand[k];
         }
     }
     // restore the snapshot, whatever happened
     b->cur = cur0;
+    b->strip_asked = e == cudaSuccess && st == LB_OK ? strip_best : asked0;
     cudaError_t e2 = cudaMemcpyAsync(b->buf[cur0], snap, b->buf_bytes, cudaMemcpyDeviceToDevice, b->stream);
     if (e2 == cudaSuccess)
         e2 = cudaMemcpyAsync(b->d_err, errw.data(), sizeof(int) * b->n, cudaMemcpyHostToDevice, b->stream);

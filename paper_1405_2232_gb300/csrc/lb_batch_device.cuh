@@ -34,6 +34,7 @@
 // a halo warp computes the halo psi columns.
 #pragma once
 
+#include "lb_launch.h"
 #include "lb_step_strip.cuh"
 
 namespace lbgb {
@@ -41,13 +42,6 @@ namespace lbgb {
 // Item indices the producer may run ahead of the consumers (it is at most
 // STAGES jobs ahead, and every item has at least three jobs).
 constexpr int BATCH_QN = 16;
-
-// One domain of a batch.
-struct BatchDomain {
-    KParams kp;          // physics, sizes, pitch/plane (elements) and error word
-    long long off;       // element offset of the domain's 18 planes in each buffer
-    long long fld_off;   // site offset of the domain in the dense field arrays
-};
 
 // One work item of the persistent step kernel.
 struct BatchItem {

@@ -14,6 +14,7 @@
 #include <new>
 
 #include "lb.h"
+#include "lb_fd.cuh"
 #include "lb_launch.h"
 #include "tensor_map.h"
 
@@ -378,21 +379,9 @@ int default_tile_rows(int prec, int nx, int rows, int sms, bool walls) {
     const long long sites = (long long)nx * rows;
     if (!walls && sites > (fp64 ? (1LL << 20) - 1 : (fp32 ? 1LL << 21 : 3LL << 19))) return 0;
     const long long cols = (nx + 31) / 32;
-    const int fill = fp32 ? 7 : 6, low = (rows + 65534) / 65535;  // (at most 65,535 blocks down a grid)
-    if (!walls && low > fill) return 0;
-    if (!fp64 && fill >= low && cols * ((rows + fill - 1) / fill) > 4LL * sms) return fill;
-    const double own = fp64 ? 285.0 : 0.55, psi = fp64 ? 65.0 : 0.45;
-    int best = low;
-    double best_cost = 0.0;
-    for (int by = low; by <= (fp64 ? 14 : 10); ++by) {
-        const long long tiles = cols * ((rows + by - 1) / by);
-        const double cost = (double)((tiles + sms - 1) / sms) * (own * by + psi * (tile_threads(32, by) / 32));
-        if (by == low || cost < best_cost) {
-            best = by;
-            best_cost = cost;
-        }
-    }
-    return best;
+    const int low = (rows + 65534) / 65535;  // (at most 65,535 blocks down a grid)
+    if (!walls && low > (fp64 ? 1 : TILE_FILL_DEV)) return 0;
+    return balanced_tile_rows(prec, sms, low, [&](int by) { return cols * ((rows + by - 1) / by); });
 }
 
 void release(lb_ctx* c) {

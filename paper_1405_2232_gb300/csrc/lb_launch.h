@@ -6,9 +6,16 @@
 #include <cuda_runtime.h>
 
 #include "lb_device.cuh"
-#include "lb_fd.cuh"
 
 namespace lbgb {
+
+// Most rows of a tile, and the threads of a block for a tile of bx x by
+// (tile and ring, each in whole warps).
+__host__ __device__ constexpr int tile_max_by(int bx) { return bx == 32 ? 16 : 4; }
+__host__ __device__ constexpr int tile_ring(int bx, int by) { return 2 * (bx + 2) + 2 * by; }
+__host__ __device__ constexpr int tile_threads(int bx, int by) {
+    return bx * by + (tile_ring(bx, by) + 31) / 32 * 32;
+}
 
 struct StepLaunch {
     const void* src;
@@ -27,6 +34,57 @@ struct StepLaunch {
     // are stored through; nullptr elsewhere
     const CUtensorMap* dst_map = nullptr;
 };
+
+// One domain of a batch.
+struct BatchDomain {
+    KParams kp;          // physics, sizes, pitch/plane (elements) and error word
+    long long off;       // element offset of the domain's 18 planes in each buffer
+    long long fld_off;   // site offset of the domain in the dense field arrays
+};
+
+// One tile of the batched tile step: its domain and first site.
+struct BatchStepTile {
+    int domain, x0, y0, pad;
+};
+
+// One step of the active domains of a batch on the tile kernel: `grid` blocks, of
+// which the first *n_tiles (device) have a tile of 32 columns and `by` rows.  With
+// src == nullptr only the kernel's attributes are set (outside stream capture).
+struct BatchTileLaunch {
+    const void* src;
+    void* dst;
+    const BatchDomain* doms;
+    const BatchStepTile* tiles;
+    const int* n_tiles;
+    int grid, by;
+    int eq24, bmode;
+    int sms;
+    cudaStream_t stream;
+};
+cudaError_t launch_batch_tile_fp32(const BatchTileLaunch& L);
+cudaError_t launch_batch_tile_fp64(const BatchTileLaunch& L);
+
+// Rows of the 32-column tiles that run a set of lattices best (0: the strip
+// kernels): tiles(by) counts the tiles of `by` rows, `low` is the least height
+// allowed.  See default_tile_rows in lb_capi.cu.
+constexpr int TILE_FILL_FP32 = 7, TILE_FILL_DEV = 6;
+template <class Count>
+int balanced_tile_rows(int prec, int sms, int low, Count tiles) {
+    const bool fp64 = prec == LB_PREC_FP64;
+    const int fill = prec == LB_PREC_FP32 ? TILE_FILL_FP32 : TILE_FILL_DEV;
+    if (!fp64 && fill >= low && tiles(fill) > 4LL * sms) return fill;
+    const double own = fp64 ? 285.0 : 0.55, psi = fp64 ? 65.0 : 0.45;
+    int best = low;
+    double best_cost = 0.0;
+    for (int by = low; by <= (fp64 ? 14 : 10); ++by) {
+        const double cost = (double)((tiles(by) + sms - 1) / sms) * (own * by + psi * (tile_threads(32, by) / 32));
+        if (by == low || cost < best_cost) {
+            best = by;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
 
 struct MomentsLaunch {
     const void* src;

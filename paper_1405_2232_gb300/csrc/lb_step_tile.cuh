@@ -44,6 +44,7 @@
 #pragma once
 
 #include "lb_device.cuh"
+#include "lb_launch.h"
 
 namespace lbgb {
 
@@ -51,13 +52,6 @@ __host__ __device__ constexpr int opp(int i) {
     return i == 0 ? 0 : (i <= 4 ? ((i + 1) % 4) + 1 : ((i - 5 + 2) % 4) + 5);
 }
 
-// Most rows of a tile, and the threads of a block for a tile of bx x by
-// (tile and ring, each in whole warps).
-__host__ __device__ constexpr int tile_max_by(int bx) { return bx == 32 ? 16 : 4; }
-__host__ __device__ constexpr int tile_ring(int bx, int by) { return 2 * (bx + 2) + 2 * by; }
-__host__ __device__ constexpr int tile_threads(int bx, int by) {
-    return bx * by + (tile_ring(bx, by) + 31) / 32 * 32;
-}
 template <int PREC, int BMODE>
 __host__ __device__ constexpr size_t tile_smem_bytes(int bx, int by) {
     return (size_t)(BMODE == BETA_MIXED ? 2 : 1) * (bx + 2) * (by + 2) * sizeof(typename Store<PREC>::real);
@@ -267,6 +261,35 @@ __global__ void __launch_bounds__(tile_threads(BX, tile_max_by(BX)))
     tile_step<PREC, BX, WALLS, EQ24, BMODE>(src, dst, kp, blockIdx.x * BX, kp.halo_rows + blockIdx.y * by, by, s_psi,
                                             s_psi2, flags);
     if (flags) atomicOr(kp.err, flags);
+}
+
+// One step of the active domains of a batch: block b takes tile b of the list (domain
+// and first site), with its domain's parameters read from the device table.  The
+// list and the table are written before the steps, not by them, so a block has
+// read its tile when the step before it ends.  (Each block has its tile whatever the
+// others do, so small domains need no balancing; the persistent strip kernel of
+// lb_batch_device.cuh re-reads less and takes over for large batches.)
+template <int PREC, bool EQ24, int BMODE>
+__global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
+    k_batch_tile(const typename Store<PREC>::elem* __restrict__ src, typename Store<PREC>::elem* __restrict__ dst,
+                 const BatchDomain* __restrict__ doms, const BatchStepTile* __restrict__ tiles,
+                 const int* __restrict__ n_tiles, int by) {
+    using real = typename Store<PREC>::real;
+    extern __shared__ __align__(16) unsigned char tile_smem[];
+    real* s_psi = reinterpret_cast<real*>(tile_smem);
+    real* s_psi2 = BMODE == BETA_MIXED ? s_psi + 34 * (by + 2) : s_psi;
+    grid_dependency_launch();
+    if ((int)blockIdx.x >= *n_tiles) {  // the grid covers the longest list
+        grid_dependency_wait();         // (no block ends before the step ahead of it)
+        return;
+    }
+    const BatchStepTile t = tiles[blockIdx.x];
+    const BatchDomain& D = doms[t.domain];
+    const long long off = D.off;
+    int flags = 0;
+    grid_dependency_wait();
+    tile_step<PREC, 32, 0, EQ24, BMODE>(src + off, dst + off, D.kp, t.x0, t.y0, by, s_psi, s_psi2, flags);
+    if (flags) atomicOr(D.kp.err, flags);
 }
 
 // ---------------------------------------------------------------- moments

@@ -1,6 +1,7 @@
 // lb_tile_impl.cuh -- instantiates the tile kernels (lb_step_tile.cuh) of one
 // storage precision.  Included by lb_tile_<name>.cu after defining LBGB_PREC
-// (an LB_PREC_* value) and LBGB_NAME (the suffix of the launch function).  A unit
+// (an LB_PREC_* value) and LBGB_NAME (the suffix of the launch functions); with
+// LBGB_BATCH also the batched tile step.  A unit
 // of its own: a thread of these kernels has one site, so the parameters are read
 // as float copies (LB_KP_FLOAT) where the strip kernels convert the doubles once
 // per chunk of rows.
@@ -37,11 +38,23 @@ auto tile_kernel(const StepLaunch& L) -> void (*)(const typename Store<LBGB_PREC
 // before it still runs, and an SM that happens to be free then would take several,
 // which keeps the next steps unbalanced as well (FP64 150 x 150 cavity, 150 tiles of
 // five rows: 32.4 us per step without, 19.0 us with).
-size_t tile_smem(const StepLaunch& L, long long tiles, size_t need) {
-    const long long k = (tiles + L.sms - 1) / L.sms;
+size_t tile_smem(int sms, long long tiles, size_t need) {
+    const long long k = (tiles + sms - 1) / sms;
     if (k > 8) return need;
     const size_t pad = TILE_SM_SMEM / (size_t)(k + 1);  // k + 1 blocks (and 1 KB each) do not fit
     return pad > need ? pad : need;
+}
+
+// Lets a kernel have the padded size; once per kernel (`done`) and device.
+template <class K>
+cudaError_t opt_in_smem(std::atomic<unsigned long long>& done, K kern) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 64 && (done.load() >> dev & 1ULL)) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TILE_SM_SMEM / 2));
+    if (e == cudaSuccess && dev < 64) done.fetch_or(1ULL << dev);
+    return e;
 }
 
 template <int BX, int WALLS>
@@ -54,24 +67,16 @@ cudaError_t step_tile(const StepLaunch& L, int by) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((L.kp.nx + BX - 1) / BX, (L.kp.ny - 2 * L.kp.halo_rows + by - 1) / by);
     cfg.blockDim = dim3(tile_threads(BX, by));
-    cfg.dynamicSmemBytes = tile_smem(L, (long long)cfg.gridDim.x * cfg.gridDim.y,
+    cfg.dynamicSmemBytes = tile_smem(L.sms, (long long)cfg.gridDim.x * cfg.gridDim.y,
                                      L.bmode == BETA_MIXED ? tile_smem_bytes<LBGB_PREC, BETA_MIXED>(BX, by)
                                                            : tile_smem_bytes<LBGB_PREC, BETA_ONE>(BX, by));
     cfg.stream = L.stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     if (cfg.dynamicSmemBytes > 48 * 1024) {
-        // opt in once per kernel (by its slot among the variants) and device
         static std::atomic<unsigned long long> configured[6];
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        cudaError_t e = opt_in_smem(configured[(L.eq24 ? 3 : 0) + L.bmode], kern);
         if (e != cudaSuccess) return e;
-        auto& done = configured[(L.eq24 ? 3 : 0) + L.bmode];
-        if (dev >= 64 || !(done.load() >> dev & 1ULL)) {
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(TILE_SM_SMEM / 2));
-            if (e != cudaSuccess) return e;
-            if (dev < 64) done.fetch_or(1ULL << dev);
-        }
     }
     return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, by);
 }
@@ -91,6 +96,46 @@ cudaError_t LBGB_CAT(launch_tile_, LBGB_NAME)(const StepLaunch& L) {
     if (L.bx == 64 && L.by == 4) return step_tile<64, 0>(L, L.by);
     return cudaErrorInvalidValue;
 }
+
+#ifdef LBGB_BATCH
+namespace {
+auto batch_tile_kernel(int eq24, int bmode)
+    -> void (*)(const typename Store<LBGB_PREC>::elem*, typename Store<LBGB_PREC>::elem*, const BatchDomain*,
+                const BatchStepTile*, const int*, int) {
+    if (eq24) {
+        if (bmode == BETA_ZERO) return k_batch_tile<LBGB_PREC, true, BETA_ZERO>;
+        if (bmode == BETA_ONE) return k_batch_tile<LBGB_PREC, true, BETA_ONE>;
+        return k_batch_tile<LBGB_PREC, true, BETA_MIXED>;
+    }
+    if (bmode == BETA_ZERO) return k_batch_tile<LBGB_PREC, false, BETA_ZERO>;
+    if (bmode == BETA_ONE) return k_batch_tile<LBGB_PREC, false, BETA_ONE>;
+    return k_batch_tile<LBGB_PREC, false, BETA_MIXED>;
+}
+}  // namespace
+
+cudaError_t LBGB_CAT(launch_batch_tile_, LBGB_NAME)(const BatchTileLaunch& L) {
+    using E = typename Store<LBGB_PREC>::elem;
+    auto kern = batch_tile_kernel(L.eq24, L.bmode);
+    if (!L.src) {
+        static std::atomic<unsigned long long> configured[6];
+        return opt_in_smem(configured[(L.eq24 ? 3 : 0) + L.bmode], kern);
+    }
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(L.grid);
+    cfg.blockDim = dim3(tile_threads(32, L.by));
+    cfg.dynamicSmemBytes = tile_smem(L.sms, L.grid, L.bmode == BETA_MIXED
+                                                        ? tile_smem_bytes<LBGB_PREC, BETA_MIXED>(32, L.by)
+                                                        : tile_smem_bytes<LBGB_PREC, BETA_ONE>(32, L.by));
+    cfg.stream = L.stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.doms, L.tiles,
+                              L.n_tiles, L.by);
+}
+#endif
 
 namespace {
 template <int BM, bool PART>

@@ -297,3 +297,33 @@ def test_fields_after_restart_are_the_state(lb):
     assert np.array_equal(moved[0], again[0]) and np.array_equal(other[0], moved[0])
     assert np.array_equal(back[0], fresh[0]) and np.array_equal(back[1], fresh[1])
     assert not np.array_equal(back[0], rho) and not np.array_equal(back[0], moved[0])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec,eps", [("fp64", 0.0), ("fp32", 2.0 ** -24)])
+def test_tile_and_strip_steps_agree(lb, prec, eps):
+    """The tile kernel that small batches run by default against the strip kernel (a
+    chunk height set): sizes at the edges of tiles, and a run that takes domains off
+    the list on the way.  FP32: one rounding (eps, of values below 0.4) per
+    population and step."""
+    sizes = [(3, 3), (32, 14), (33, 15), (64, 5), (31, 130), (97, 64), (5, 7)]
+    params, rhos, Ts = [], [], []
+    for k, (nx, ny) in enumerate(sizes):
+        rho, T = I.slab_fields(nx, ny, width=max(2, nx // 2), noise=1e-3, seed=k + 1)
+        params.append(lb.lb_params_default(nx=nx, ny=ny, precision=prec, beta=1.3, G=-1.0 + 0.05 * k,
+                                           psi_uses_local_T=0, T_psi=0.85 * I.CS_TC))
+        rhos.append(rho)
+        Ts.append(T)
+    with lb.Batch(params, rhos, Ts) as A, lb.Batch(params, rhos, Ts) as B:
+        B.chunk_rows = 16
+        A.step(25)
+        B.step(25)
+        for d in range(len(sizes)):
+            for a, b in zip(A.fields(d), B.fields(d)):
+                assert np.abs(a - b).max() <= 25 * 9 * eps * 0.4
+        ra, rb = A.run(2e-6, K=20, max_steps=600), B.run(2e-6, K=20, max_steps=600)
+        if prec == "fp64":
+            assert np.array_equal(ra[0], rb[0]) and np.array_equal(ra[2], rb[2])
+            assert len(set(ra[0].tolist())) > 1  # some left the list before others
+            for d in range(len(sizes)):
+                assert np.array_equal(A.fields(d)[0], B.fields(d)[0]), d
