@@ -177,6 +177,7 @@ struct lb_ctx {
     int sms = 152;
     bool have_out_map = false;  // 16-bit strip contexts: out_map[b] describes buf[b]
     CUtensorMap out_map[2];
+    DevLoadMaps in_maps[2];     // and the loads from buf[b]
     long long pitch = 0, plane = 0;  // population layout (elements)
     // finite-difference temperature treatment (Eqs. 26-27)
     bool fd = false;
@@ -268,7 +269,10 @@ cudaError_t dispatch_step(const lb_ctx* c, const void* src, void* dst) {
     L.tile_by = c->kp.walls || c->kp.wait_cycles == WAIT_CYCLES_DEFAULT ? c->tile_by : 0;
     L.sms = c->sms;
     L.stream = c->stream;
-    if (c->have_out_map) L.dst_map = &c->out_map[dst == c->buf[0] ? 0 : 1];
+    if (c->have_out_map) {
+        L.dst_map = &c->out_map[dst == c->buf[0] ? 0 : 1];
+        L.src_maps = &c->in_maps[src == c->buf[0] ? 0 : 1];
+    }
     switch (c->p.precision) {
         case LB_PREC_FP64: return launch_step_fp64(L);
         case LB_PREC_FP32: return launch_step_fp32(L);
@@ -556,18 +560,36 @@ lb_status create(const lb_params* p, void* stream, lb_ctx** out) {
             return fail(LB_ERR_CUDA, "the driver provides no cuTensorMapEncodeTiled");
         }
         const int npl = pop_planes(p->precision);
+        auto encode = [&](CUtensorMap* m, CUtensorMapDataType type, int rank, void* base, const cuuint64_t* dims,
+                          const cuuint64_t* strides, const cuuint32_t* box) {
+            const cuuint32_t one[4] = {1, 1, 1, 1};
+            return enc(m, type, rank, base, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                       CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+        };
+        const cuuint64_t row = (cuuint64_t)(pitch * (long long)es), pl = (cuuint64_t)(plane * (long long)es);
         const cuuint64_t dims[3] = {(cuuint64_t)(p->nx < 8 ? 8 : dev_map_columns(p->nx)), (cuuint64_t)p->ny,
                                     (cuuint64_t)npl};
-        const cuuint64_t strides[2] = {(cuuint64_t)(pitch * (long long)es), (cuuint64_t)(plane * (long long)es)};
+        const cuuint64_t strides[2] = {row, pl};
         const cuuint32_t box[3] = {(cuuint32_t)c->p.tile_x, 1, (cuuint32_t)npl};
-        const cuuint32_t estr[3] = {1, 1, 1};
-        for (int b = 0; b < 2; ++b) {
-            if (enc(&c->out_map[b], CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, c->buf[b], dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
-                release(c);
-                return fail(LB_ERR_CUDA, "encoding the tensor map of population buffer %d", b);
-            }
+        // loads: the strip with its 8-column halo on each side
+        const cuuint32_t words = (cuuint32_t)(c->p.tile_x + 2 * strip_halo(p->precision)) / 2;
+        const cuuint64_t ldims[4] = {row / 4, (cuuint64_t)p->ny, 9, 2}, lstrides[3] = {row, pl, 9 * pl};
+        const cuuint32_t box4[4] = {words, 1, 2, 2}, box2[4] = {words, 1, 1, 2};
+        const cuuint64_t wdims[3] = {row / 4, (cuuint64_t)p->ny, 2};
+        const cuuint32_t boxw[3] = {words, 1, 2};
+        static_assert(DEV_ROW_ORIGIN * 2 == 128, "pop_layout's origin of the 16-bit modes");
+        bool ok = true;
+        for (int b = 0; b < 2 && ok; ++b) {
+            ok = encode(&c->out_map[b], CU_TENSOR_MAP_DATA_TYPE_UINT16, 3, c->buf[b], dims, strides, box) &&
+                 encode(&c->in_maps[b].four, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, c->alloc[b], ldims, lstrides, box4) &&
+                 encode(&c->in_maps[b].two, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, c->alloc[b], ldims, lstrides, box2) &&
+                 encode(&c->in_maps[b].low, CU_TENSOR_MAP_DATA_TYPE_UINT32, 3,
+                        static_cast<char*>(c->alloc[b]) + 18 * pl, wdims, strides, boxw);
+        }
+        if (!ok) {
+            release(c);
+            return fail(LB_ERR_CUDA, "encoding the tensor maps of the population buffers");
         }
         c->have_out_map = true;
     }

@@ -13,6 +13,7 @@
 // the pre-collision value f_i(x, t) is read ("pulled") from x - e_i.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -379,6 +380,15 @@ constexpr int STRIP_GHOST = 2;
 // contexts.
 constexpr int FD_HALO = 4;
 constexpr int FD_GHOST = 3;
+
+// Tensor maps of a population buffer that the 16-bit strip kernel loads through, in
+// 32-bit words (two columns) from the start of the padded rows, which begin
+// DEV_ROW_ORIGIN columns left of column 0: x, y, population i, f or g (four: two
+// populations of both, two: one of both), and x, y, half for the two low-half planes.
+struct DevLoadMaps {
+    CUtensorMap four, two, low;
+};
+constexpr int DEV_ROW_ORIGIN = 64;
 
 // Columns of a row that the 16-bit strip kernel stores through its tensor map:
 // the whole 16-byte units of the row.

@@ -33,6 +33,7 @@ struct StepLaunch {
     // y: ny rows, z: the planes; box bx x 1 x NPLANES) that its collided rows
     // are stored through; nullptr elsewhere
     const CUtensorMap* dst_map = nullptr;
+    const DevLoadMaps* src_maps = nullptr;  // and those its rows are loaded through
 };
 
 // One domain of a batch.

@@ -28,8 +28,13 @@ template <int BX>
 constexpr int strip_stages() {
     using C = StripCfg<LBGB_PREC>;
     constexpr int NPL = Store<LBGB_PREC>::NPLANES;
-    constexpr size_t stage = (size_t)NPL * (BX + 2 * C::HALO) * C::ES;
     constexpr bool DEV = Store<LBGB_PREC>::SPLIT;
+    constexpr size_t stage = [] {
+        if constexpr (DEV)
+            return (size_t)dev_stage<BX + 2 * C::HALO>() * C::ES;
+        else
+            return (size_t)NPL * (BX + 2 * C::HALO) * C::ES;
+    }();
     constexpr size_t ring = (size_t)(DEV ? 2 * DEV_PSI_ROWS : 8) * (BX + 2) * sizeof(typename C::real);
     constexpr size_t out = DEV ? (size_t)DEV_OUT_BUFS * NPL * BX * C::ES : 0;
     constexpr size_t budget = 110 * 1024 - 32 - (DEV ? (2 * 12 + 2) * 8 : 0);
@@ -56,8 +61,12 @@ cudaError_t strip_launch(const StepLaunch& L) {
     constexpr int ST = strip_stages<BX>();
     static_assert(ST >= 3, "strip kernel needs at least three stages");
     constexpr bool DEV = Store<LBGB_PREC>::SPLIT;
-    constexpr size_t smem =
-        DEV ? strip_dev_smem_bytes<LBGB_PREC, BX, ST>() : strip_smem_bytes<LBGB_PREC, BX, ST>();
+    constexpr size_t smem = [] {
+        if constexpr (DEV)
+            return strip_dev_smem_bytes<LBGB_PREC, BX, ST>();
+        else
+            return strip_smem_bytes<LBGB_PREC, BX, ST>();
+    }();
     static_assert(smem <= 110 * 1024, "two CTAs per SM");
     auto kern = strip_kernel<BX, ST, EQ24, BM, TAIL>();
     static unsigned long long configured = 0;  // per instantiation, one bit per device
@@ -71,9 +80,9 @@ cudaError_t strip_launch(const StepLaunch& L) {
     }
     const dim3 grid((L.kp.nx + BX - 1) / BX, L.nchunks);
     if constexpr (DEV) {
-        if (!L.dst_map) return cudaErrorInvalidValue;  // the kernel stores through it
-        kern<<<grid, strip_threads<BX>(), smem, L.stream>>>(static_cast<const E*>(L.src), static_cast<E*>(L.dst),
-                                                             L.kp, L.nchunks, *L.dst_map);
+        if (!L.dst_map || !L.src_maps) return cudaErrorInvalidValue;  // the kernel loads and stores through them
+        kern<<<grid, strip_threads<BX>(), smem, L.stream>>>(static_cast<E*>(L.dst), L.kp, L.nchunks, *L.dst_map,
+                                                             *L.src_maps);
     } else {
         kern<<<grid, strip_threads<BX>(), smem, L.stream>>>(static_cast<const E*>(L.src), static_cast<E*>(L.dst),
                                                              L.kp, L.nchunks);

@@ -2,7 +2,7 @@
 // storage modes (FP16 / BF16 deviations, FP32 rest populations in two halves).
 //
 // The pipeline of k_step_strip (producer warp streaming plane-row segments
-// into a stage ring, column threads computing psi into a ring of psi rows
+// into a stage ring, here with seven tensor copies per row, column threads computing psi into a ring of psi rows
 // and colliding the rows whose psi neighbourhood is complete, halo warp for
 // the two halo psi columns), changed where these modes, which are bound by
 // instruction issue rather than by HBM bandwidth, spent instructions:
@@ -48,6 +48,95 @@
 
 namespace lbgb {
 
+// A stage holds the 20 plane rows of a job in the order its seven tensor copies write
+// them: populations 0, 1 then 5, 6 then 7, 8 of f and of g (four rows each, f_i, f_i+1,
+// g_i, g_i+1), then 2, 3, 4 of f and g and the two low-half rows (two rows each).  A copy
+// starts on 128 bytes, so the two-row groups are padded.  Elements:
+template <int SEGW>
+__host__ __device__ constexpr int dev_pair() {  // a two-row group
+    return (2 * SEGW + 63) / 64 * 64;
+}
+template <int SEGW>
+__host__ __device__ constexpr int dev_stage() {
+    static_assert(4 * SEGW % 64 == 0, "four-row groups start on 128 bytes");
+    return 12 * SEGW + 4 * dev_pair<SEGW>();
+}
+template <int SEGW>
+__host__ __device__ constexpr int dev_row(int p) {  // first element of plane p's row
+    if (p >= 18) return 12 * SEGW + 3 * dev_pair<SEGW>() + (p - 18) * SEGW;
+    const int i = p % 9, g = p / 9;
+    if (i >= 2 && i <= 4) return 12 * SEGW + (i - 2) * dev_pair<SEGW>() + g * SEGW;
+    const int group = i < 2 ? 0 : (i < 7 ? 1 : 2), k = i < 2 ? i : (i < 7 ? i - 5 : i - 7);
+    return (4 * group + 2 * g + k) * SEGW;
+}
+template <int SEGW>
+__host__ __device__ constexpr int dev_lo(int p) {  // from the high half of a rest population to its low half
+    return p == 0 ? dev_row<SEGW>(18) - dev_row<SEGW>(0) : dev_row<SEGW>(19) - dev_row<SEGW>(9);
+}
+
+__device__ __forceinline__ void tensor_load_4d(void* dst, const CUtensorMap* map, int x, int y, int z, int w,
+                                               uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+        "[%6];" ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w),
+        "r"(smem_u32(bar))
+        : "memory");
+}
+__device__ __forceinline__ void tensor_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            smem_u32(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+        : "memory");
+}
+
+// The producer warp (strip_produce's protocol): lane 0 issues a job's seven copies.
+// The rows of a job come from three source rows (y - e_y), so no single copy can
+// take them, but f_i and g_i lie nine planes apart and 0, 1 / 5, 6 / 7, 8 share their
+// e_y: four rows at a time.  (Twenty bulk copies of one row each kept an SM's copy
+// engine at about 34 cycles apiece: streaming the same rows alone ran at 4.6 TB/s,
+// copies of four rows at 7.2 TB/s.  4096^2 BF16 step 303 us, 325 us before.)
+template <class S, int STAGES, int SEGW>
+__device__ __forceinline__ void strip_produce_dev(const DevLoadMaps& maps, typename S::elem* stage, uint64_t* full,
+                                                  uint64_t* empty, const KParams& kp, int lane, int njobs, int y_start,
+                                                  int x0) {
+    constexpr int HALO = 16 / (int)sizeof(typename S::elem);
+    const int ny = kp.ny;
+    // maps count in 32-bit words from the start of the padded rows
+    const int xw = (DEV_ROW_ORIGIN + x0 - HALO) / 2;
+    int issued = 0;
+    for (int j = 0; j < njobs; ++j) {
+        const int s = j % STAGES;
+        if (j >= STAGES) {
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&empty[s], (uint32_t)(((j / STAGES) - 1) & 1),
+                                                           kp.wait_cycles))) {
+                if (lane == 0) atomicOr(kp.err, 1 << LB_ERR_TIMEOUT);
+                break;
+            }
+        }
+        int y = y_start - 1 + j;
+        y = y < 0 ? y + ny : (y >= ny ? y - ny : y);
+        const int yb = y == 0 ? ny - 1 : y - 1, ya = y == ny - 1 ? 0 : y + 1;  // sources of e_y = 1 and -1
+        if (lane == 0) {
+            typename S::elem* st = stage + (size_t)s * dev_stage<SEGW>();
+            uint64_t* bar = &full[s];
+            mbar_arrive_expect_tx(bar, (uint32_t)(S::NPLANES * SEGW * sizeof(typename S::elem)));
+            tensor_load_4d(st + dev_row<SEGW>(0), &maps.four, xw, y, 0, 0, bar);
+            tensor_load_4d(st + dev_row<SEGW>(5), &maps.four, xw, yb, 5, 0, bar);
+            tensor_load_4d(st + dev_row<SEGW>(7), &maps.four, xw, ya, 7, 0, bar);
+            tensor_load_4d(st + dev_row<SEGW>(2), &maps.two, xw, yb, 2, 0, bar);
+            tensor_load_4d(st + dev_row<SEGW>(3), &maps.two, xw, y, 3, 0, bar);
+            tensor_load_4d(st + dev_row<SEGW>(4), &maps.two, xw, ya, 4, 0, bar);
+            tensor_load_3d(st + dev_row<SEGW>(18), &maps.low, xw, y, 0, bar);
+        }
+        __syncwarp();
+        issued = j + 1;
+    }
+    if (lane == 0)
+        for (int j = (issued > STAGES ? issued - STAGES : 0); j < issued; ++j)
+            (void)mbar_wait_bounded(&full[j % STAGES], (uint32_t)((j / STAGES) & 1));
+}
+
 constexpr int DEV_OUT_BUFS = 3;  // row buffers: job m collides into buffer m mod 3
 
 // 3D tensor copy shared -> global of the box at (x, y, z) (bulk async group
@@ -79,7 +168,7 @@ template <int PREC, int BX, int STAGES>
 constexpr size_t strip_dev_smem_bytes() {
     using C = StripCfg<PREC>;
     constexpr int NPL = Store<PREC>::NPLANES;
-    return (size_t)STAGES * NPL * (BX + 2 * C::HALO) * C::ES + (size_t)DEV_OUT_BUFS * NPL * BX * C::ES +
+    return (size_t)STAGES * dev_stage<BX + 2 * C::HALO>() * C::ES + (size_t)DEV_OUT_BUFS * NPL * BX * C::ES +
            (size_t)2 * DEV_PSI_ROWS * (BX + 2) * sizeof(float) + (size_t)(2 * STAGES + 1) * 8 + 16;
 }
 
@@ -91,8 +180,8 @@ __device__ __forceinline__ void dev_psi_site(const KParams& kp, const typename S
     float hf = 0.0f, hg = 0.0f;
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        hf = acc_dev<S>(st + i * SEGW + c - ex(i), i, rest_lo_offset(i) * SEGW, hf);
-        hg = acc_dev<S>(st + (9 + i) * SEGW + c - ex(i), 9 + i, rest_lo_offset(9 + i) * SEGW, hg);
+        hf = acc_dev<S>(st + dev_row<SEGW>(i) + c - ex(i), i, dev_lo<SEGW>(i), hf);
+        hg = acc_dev<S>(st + dev_row<SEGW>(9 + i) + c - ex(i), 9 + i, dev_lo<SEGW>(9 + i), hg);
     }
     const float rho = kp.sum_bf + hf;
     const float T = (kp.sum_bg + hg) / (rho * kp.f.cv);
@@ -116,8 +205,8 @@ __device__ __forceinline__ void dev_collide_site(const KParams& kp, const typena
     float h[9], q[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
-        h[i] = dev_of<S>(st + i * SEGW + c - ex(i), i, rest_lo_offset(i) * SEGW);
-        q[i] = dev_of<S>(st + (9 + i) * SEGW + c - ex(i), 9 + i, rest_lo_offset(9 + i) * SEGW);
+        h[i] = dev_of<S>(st + dev_row<SEGW>(i) + c - ex(i), i, dev_lo<SEGW>(i));
+        q[i] = dev_of<S>(st + dev_row<SEGW>(9 + i) + c - ex(i), 9 + i, dev_lo<SEGW>(9 + i));
     }
     collide_dev<EQ24>(kp, h, q, Hf, Hg, Fx, Fy);
     typename S::elem v[NPL];
@@ -139,9 +228,8 @@ __device__ __forceinline__ void dev_collide_site(const KParams& kp, const typena
 // 3 - 7%).
 template <int PREC, int BX, int STAGES, bool EQ24, int BMODE, bool TAIL>
 __global__ void __launch_bounds__(strip_threads<BX>(), 2)
-    k_step_strip_dev(const typename Store<PREC>::elem* __restrict__ src,
-                     typename Store<PREC>::elem* __restrict__ dst, const KParams kp, int nchunks,
-                     const __grid_constant__ CUtensorMap dst_map) {
+    k_step_strip_dev(typename Store<PREC>::elem* __restrict__ dst, const KParams kp, int nchunks,
+                     const __grid_constant__ CUtensorMap dst_map, const __grid_constant__ DevLoadMaps src_maps) {
     using S = Store<PREC>;
     static_assert(S::SPLIT, "16-bit deviation storage only");
     using C = StripCfg<PREC>;
@@ -154,8 +242,8 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     constexpr int ES = C::ES;
 
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    elem* stage = reinterpret_cast<elem*>(smem_raw);                 // [STAGES][NPL][SEGW]
-    elem* outb = stage + (size_t)STAGES * NPL * SEGW;                 // [DEV_OUT_BUFS][NPL][BX]
+    elem* stage = reinterpret_cast<elem*>(smem_raw);                 // [STAGES][dev_stage]
+    elem* outb = stage + (size_t)STAGES * dev_stage<SEGW>();          // [DEV_OUT_BUFS][NPL][BX]
     float* ring_psi = reinterpret_cast<float*>(outb + (size_t)DEV_OUT_BUFS * NPL * BX);  // [6][RW]
     float* ring_psi2 = ring_psi + DEV_PSI_ROWS * RW;                                     // [6][RW]
     uint64_t* full = reinterpret_cast<uint64_t*>(
@@ -189,7 +277,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     __syncthreads();
 
     if (t >= BX + 32) {
-        strip_produce<S, STAGES, SEGW>(src, stage, full, empty, kp, t - BX - 32, njobs, y_start, x0, W);
+        strip_produce_dev<S, STAGES, SEGW>(src_maps, stage, full, empty, kp, t - BX - 32, njobs, y_start, x0);
         return;
     }
 
@@ -229,10 +317,10 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
         if (!ok) s_abort[k & 1] = 1;
         float Hf_0 = 0.0f, Hg_0 = 0.0f, Hf_1 = 0.0f, Hg_1 = 0.0f;
         if (has_psi && ok) {
-            dev_psi_site<S, SEGW, BMODE>(kp, stage + s0 * (NPL * SEGW), c_psi, Hf_0, Hg_0,
+            dev_psi_site<S, SEGW, BMODE>(kp, stage + s0 * dev_stage<SEGW>(), c_psi, Hf_0, Hg_0,
                                          ring_psi + q * RW + r_psi, ring_psi2 + q * RW + r_psi, flags);
             if (has1)
-                dev_psi_site<S, SEGW, BMODE>(kp, stage + s1 * (NPL * SEGW), c_psi, Hf_1, Hg_1,
+                dev_psi_site<S, SEGW, BMODE>(kp, stage + s1 * dev_stage<SEGW>(), c_psi, Hf_1, Hg_1,
                                              ring_psi + (q + 1) * RW + r_psi, ring_psi2 + (q + 1) * RW + r_psi,
                                              flags);
         }
@@ -278,7 +366,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     ring_psi2 + qm1 * RW + r, ring_psi2 + q * RW + r, ring_psi2 + (q + 1) * RW + r, FxB, FyB);
                 if (c0) {
                     const int y = y_start - 1 + m0;
-                    dev_collide_site<S, SEGW, BX, EQ24, TAIL>(kp, stage + sm * (NPL * SEGW), c, Hf_p, Hg_p, FxA, FyA,
+                    dev_collide_site<S, SEGW, BX, EQ24, TAIL>(kp, stage + sm * dev_stage<SEGW>(), c, Hf_p, Hg_p, FxA, FyA,
                                                         dst + ((size_t)y * pitch + (size_t)xg),
                                                         outb + (size_t)bA * NPL * BX + t, plane,
                                                         ghost_lo, ghost_hi, tail);
@@ -287,7 +375,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                 if (lane == 0) mbar_arrive(written);
                 if (c1) {
                     const int y = y_start - 1 + m1;
-                    dev_collide_site<S, SEGW, BX, EQ24, TAIL>(kp, stage + s0 * (NPL * SEGW), c, Hf_0, Hg_0, FxB, FyB,
+                    dev_collide_site<S, SEGW, BX, EQ24, TAIL>(kp, stage + s0 * dev_stage<SEGW>(), c, Hf_0, Hg_0, FxB, FyB,
                                                         dst + ((size_t)y * pitch + (size_t)xg),
                                                         outb + (size_t)b0 * NPL * BX + t, plane,
                                                         ghost_lo, ghost_hi, tail);
