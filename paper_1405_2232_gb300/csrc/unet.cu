@@ -135,9 +135,11 @@ struct un_net {
     bf16* gup[UN_LEVELS] = {};   // index 1..3
     bf16* gs[UN_LEVELS - 1] = {};
     // reductions
-    float* wpart = nullptr;
-    long long wpart_cap = 0;
-    float* bpart = nullptr;   // [1024][256]
+    float* wpart = nullptr;   // weight-gradient partials, each layer's own
+    long long wpart_off[UN_LAYERS] = {}, wpart_cap[UN_LAYERS] = {};
+    float* bpart = nullptr;   // bias-gradient partials likewise: splits x cout
+    long long bpart_off[UN_LAYERS] = {};
+    unk::SumJobs sums;        // the sums of the pass being issued
     float* hpart = nullptr;   // [hblocks][2C + 2]
     double* lpart = nullptr;  // [hblocks]
     double* d_loss = nullptr;
@@ -174,12 +176,6 @@ cudaError_t alloc(un_net* n, T** p, long long count) {
 int grid_for(long long work, int per_block = 256) {
     long long b = (work + per_block - 1) / per_block;
     return (int)(b < 1 ? 1 : (b > 1 << 20 ? 1 << 20 : b));
-}
-
-// blocks of k_sum_splits for n outputs (32 per block, grid-stride beyond)
-int sum_grid(long long n) {
-    const long long b = (n + 31) / 32;
-    return (int)(b < 1 ? 1 : (b > 65536 ? 65536 : b));
 }
 
 // splits of the weight-gradient kernel for a layer at M pixels
@@ -289,6 +285,15 @@ cudaError_t conv(un_net* n, const bf16* x, int xC, int xoff, int Cin, const bf16
     return cudaGetLastError();
 }
 
+// the sums over layer k's splits, for the launch at the end of the pass
+cudaError_t queue_sums(un_net* n, int k, int splits) {
+    const Layer& L = n->L[k];
+    const bool ok =
+        n->sums.add(n->wpart + n->wpart_off[k], splits, (long long)L.cout * 9 * L.cin, false, n->grad + L.woff) &&
+        n->sums.add(n->bpart + n->bpart_off[k], splits, L.cout, true, n->grad + L.boff);
+    return ok ? cudaGetLastError() : cudaErrorInvalidValue;
+}
+
 // weight and bias gradient of layer k: g (gradient at its output) and x (its input)
 cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16* x, int xC, int xoff, int N, int l) {
     const Layer& L = n->L[k];
@@ -310,9 +315,8 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
         long long S = n->sms / units;
         if (S < 1) S = 1;
         if (S > items) S = items;
-        const long long cap = n->wpart_cap / nw;
+        const long long cap = n->wpart_cap[k] / nw;
         if (S > cap) S = cap;
-        if (S > 1024LL * 256 / L.cout) S = 1024LL * 256 / L.cout;
         if (S >= 1) {
             const long long per = (items + S - 1) / S;
             const int splits = (int)((items + per - 1) / per);
@@ -330,8 +334,8 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
             a.W = W;
             a.splits = splits;
             a.items_per_split = (int)per;
-            a.part = n->wpart;
-            a.bpart = n->bpart;
+            a.part = n->wpart + n->wpart_off[k];
+            a.bpart = n->bpart + n->bpart_off[k];
             a.err = n->d_err;
             const int na = xm ? 32 : NBW;
             const int stages = unk::tw_stages(na, xm, segw);
@@ -345,9 +349,7 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
                 unk::k_wgrad_tc<64, false><<<grid, unk::TW_THREADS, smem, n->stream>>>(a, gmap, xmap, stages);
             else
                 unk::k_wgrad_tc<32, false><<<grid, unk::TW_THREADS, smem, n->stream>>>(a, gmap, xmap, stages);
-            unk::k_sum_splits<<<sum_grid(nw), dim3(32, 8), 0, n->stream>>>(n->wpart, splits, nw, n->grad + L.woff);
-            unk::k_sum_splits_wide<<<L.cout, 256, 0, n->stream>>>(n->bpart, splits, L.cout, n->grad + L.boff);
-            return cudaGetLastError();
+            return queue_sums(n, k, splits);
         }
     }
     if (W % unk::HT_W == 0 && H % unk::HT_H == 0) {
@@ -372,12 +374,10 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
         const long long tps = (n_tiles + sp - 1) / sp;
         const int splits = (int)((n_tiles + tps - 1) / tps);
         a.tiles_per_split = (int)tps;
-        a.part = n->wpart;
-        a.bpart = n->bpart;
+        a.part = n->wpart + n->wpart_off[k];
+        a.bpart = n->bpart + n->bpart_off[k];
         unk::k_wgrad_halo<<<dim3(blocks, splits), 256, unk::wgrad_halo_smem_bytes(), n->stream>>>(a);
-        unk::k_sum_splits<<<sum_grid(nw), dim3(32, 8), 0, n->stream>>>(n->wpart, splits, nw, n->grad + L.woff);
-        unk::k_sum_splits_wide<<<L.cout, 256, 0, n->stream>>>(n->bpart, splits, L.cout, n->grad + L.boff);
-        return cudaGetLastError();
+        return queue_sums(n, k, splits);
     }
     int MT, NT, tiles, splits, cps;
     wgrad_shape(n, L, M, &MT, &NT, &tiles, &splits, &cps);
@@ -394,17 +394,15 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
     a.H = Hl(n, l);
     a.W = Wl(n, l);
     a.chunks_per_split = cps;
-    a.part = n->wpart;
-    a.bpart = n->bpart;
+    a.part = n->wpart + n->wpart_off[k];
+    a.bpart = n->bpart + n->bpart_off[k];
     const dim3 grid(tiles, splits);
     if (MT == 32 && NT == 32) unk::k_wgrad<32, 32><<<grid, 256, 0, n->stream>>>(a);
     else if (MT == 32) unk::k_wgrad<32, 64><<<grid, 256, 0, n->stream>>>(a);
     else if (NT == 32) unk::k_wgrad<64, 32><<<grid, 256, 0, n->stream>>>(a);
     else unk::k_wgrad<64, 64><<<grid, 256, 0, n->stream>>>(a);
-    unk::k_sum_splits<<<sum_grid(nw), dim3(32, 8), 0, n->stream>>>(n->wpart, splits, nw, n->grad + L.woff);
-    // bias: partials of the centre-tap CTAs, summed over the splits in order
-    unk::k_sum_splits_wide<<<L.cout, 256, 0, n->stream>>>(n->bpart, splits, L.cout, n->grad + L.boff);
-    return cudaGetLastError();
+    // (bias: partials of the centre-tap CTAs, summed over the splits in order)
+    return queue_sums(n, k, splits);
 }
 
 const bf16* Wb(const un_net* n, int k) { return n->wb + n->L[k].qoff; }
@@ -521,7 +519,8 @@ cudaError_t backward(un_net* n, int N, const float* d_target) {
             break;
         default: return cudaErrorInvalidValue;
     }
-    unk::k_sum_splits_wide<<<2 * C + 2, 256, 0, n->stream>>>(n->hpart, hb, 2LL * C + 2, n->grad + H.woff);
+    n->sums.count = 0;
+    n->sums.add(n->hpart, hb, 2LL * C + 2, true, n->grad + H.woff);
     unk::k_sum_doubles<<<1, 256, 0, n->stream>>>(n->lpart, hb, n->d_loss);
     // decoder, finest level first
     for (int l = 0; l < LV - 1; ++l) {
@@ -552,6 +551,7 @@ cudaError_t backward(un_net* n, int N, const float* d_target) {
                 n->gs[l - 1]);
         }
     }
+    unk::k_sum_splits<<<n->sums.first[n->sums.count], 256, 0, n->stream>>>(n->sums);
     return cudaGetLastError();
 }
 
@@ -689,9 +689,9 @@ lb_status un_create(const un_config* cfg, void* stream, un_net** out) {
     if (e == cudaSuccess) e = alloc(n, &n->d0, Pl(n, 0, N) * Cl(n, 0));
     if (e == cudaSuccess) e = alloc(n, &n->gd0, Pl(n, 0, N) * Cl(n, 0));
     if (e == cudaSuccess) e = alloc(n, &n->y, Pl(n, 0, N) * UN_OUT);
-    // weight-gradient partials: the largest split count any layer can use
+    // weight- and bias-gradient partials: the largest split count each layer can use
     // (the split count grows with the pixel count, so max_batch bounds it)
-    long long cap = 0;
+    long long cap = 0, bcap = 0;
     for (int k = 0; k < UN_LAYERS; ++k) {
         if (n->L[k].k != 3) continue;
         int MT, NT, tiles, splits, cps;
@@ -712,12 +712,17 @@ lb_status un_create(const un_config* cfg, void* stream, un_net** out) {
             const long long s_tc = n->sms / units > 1 ? n->sms / units : 1;
             if (s_tc > smax) smax = s_tc;
         }
-        const long long need = smax * n->L[k].cout * 9 * n->L[k].cin;
-        if (need > cap) cap = need;
+        // (a split has at least one row segment of 16 pixels)
+        const long long pixels = Pl(n, lev, N);
+        if (smax > pixels / 16 + 1) smax = pixels / 16 + 1;
+        n->wpart_off[k] = cap;
+        n->wpart_cap[k] = smax * n->L[k].cout * 9 * n->L[k].cin;
+        n->bpart_off[k] = bcap;
+        cap += n->wpart_cap[k];
+        bcap += smax * n->L[k].cout;
     }
-    n->wpart_cap = cap;
     if (e == cudaSuccess) e = alloc(n, &n->wpart, cap);
-    if (e == cudaSuccess) e = alloc(n, &n->bpart, 1024LL * 256);
+    if (e == cudaSuccess) e = alloc(n, &n->bpart, bcap);
     n->hblocks = 2 * n->sms;
     if (e == cudaSuccess) e = alloc(n, &n->hpart, (long long)n->hblocks * (2 * cfg->base + 2));
     if (e == cudaSuccess) e = alloc(n, &n->lpart, n->hblocks);

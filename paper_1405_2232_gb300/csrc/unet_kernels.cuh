@@ -621,45 +621,76 @@ __global__ void __launch_bounds__(256) k_wgrad_halo(WgradHaloArgs a) {
         }
 }
 
-// out[i] = sum_s part[s * n + i] in a fixed order: blocks of 32 x 8 threads,
-// threadIdx.x the output within a chunk of 32, threadIdx.y a lane of splits
-// (s = y, y + 8, ...); the 8 lane sums are then added in order of y
-__global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ part, int splits, long long n,
-                                                     float* __restrict__ out) {
-    __shared__ float red[8][33];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    for (long long i0 = blockIdx.x * 32LL; i0 < n; i0 += (long long)gridDim.x * 32) {
-        const long long i = i0 + tx;
-        float s = 0.0f;
-        if (i < n)
-            for (int k = ty; k < splits; k += 8) s += part[(long long)k * n + i];
-        red[ty][tx] = s;
-        __syncthreads();
-        if (ty == 0 && i < n) {
-            float t = 0.0f;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) t += red[k][tx];
-            out[i] = t;
-        }
-        __syncthreads();
+// Sums over splits of every layer's weight- and bias-gradient partials, one launch per
+// backward pass: out[i] = sum_s part[s * n + i] in a fixed order.  Each job has its own
+// partials, so the sums wait until all are written (one pair of launches per layer, 28
+// in all, took 206 us and their gaps at 256^2 x 16, most of it latency: 55 us now).
+//  narrow (weights: many outputs, a multiple of four): 128 outputs per block, four per
+//   t & 31 (with one each the launch had 62,530 blocks of two loads: 137 us), t >> 5 a
+//   lane of splits (s = lane, lane + 8, ...); the 8 lane sums are added in order;
+//  wide (biases, head: few outputs, many partials): one output per block, a strided
+//   sum per thread and a fixed-order tree.
+constexpr int SUM_MAX_JOBS = 32;
+struct SumJobs {
+    int count;
+    int first[SUM_MAX_JOBS + 1];  // first block of each job
+    const float* part[SUM_MAX_JOBS];
+    float* out[SUM_MAX_JOBS];
+    int n[SUM_MAX_JOBS], splits[SUM_MAX_JOBS];
+    bool wide[SUM_MAX_JOBS];
+    bool add(const float* p, int splits_, long long n_, bool wide_, float* o) {
+        if (count == SUM_MAX_JOBS) return false;
+        if (count == 0) first[0] = 0;
+        part[count] = p;
+        out[count] = o;
+        n[count] = (int)n_;
+        splits[count] = splits_;
+        wide[count] = wide_;
+        first[count + 1] = first[count] + (int)(wide_ ? n_ : (n_ + 127) / 128);
+        ++count;
+        return true;
     }
-}
+};
 
-// out[i] = sum_s part[s * n + i] for few outputs and many partials: one block
-// per output, a strided per-thread sum and a fixed-order tree (deterministic)
-__global__ void __launch_bounds__(256) k_sum_splits_wide(const float* __restrict__ part, int splits, long long n,
-                                                          float* __restrict__ out) {
-    __shared__ float red[256];
-    const long long i = blockIdx.x;
-    float s = 0.0f;
-    for (int k = threadIdx.x; k < splits; k += 256) s += part[(long long)k * n + i];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
+__global__ void __launch_bounds__(256) k_sum_splits(const __grid_constant__ SumJobs a) {
+    __shared__ float4 red4[8][32];
+    float* red = &red4[0][0].x;
+    const int t = threadIdx.x, b = blockIdx.x;
+    int k = 0;
+    while (b >= a.first[k + 1]) ++k;
+    const int q = b - a.first[k], n = a.n[k], splits = a.splits[k];
+    const float* part = a.part[k];
+    if (a.wide[k]) {
+        float s = 0.0f;
+        for (int c = t; c < splits; c += 256) s += part[(long long)c * n + q];
+        red[t] = s;
         __syncthreads();
+        for (int w = 128; w > 0; w >>= 1) {
+            if (t < w) red[t] += red[t + w];
+            __syncthreads();
+        }
+        if (t == 0) a.out[k][q] = red[0];
+        return;
     }
-    if (threadIdx.x == 0) out[i] = red[0];
+    const int tx = t & 31, ty = t >> 5, i = q * 128 + 4 * tx;
+    float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (i < n)
+#pragma unroll 4
+        for (int c = ty; c < splits; c += 8) {
+            const float4 v = *reinterpret_cast<const float4*>(part + (long long)c * n + i);
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    red4[ty][tx] = s;
+    __syncthreads();
+    if (t < 128 && q * 128 + t < n) {
+        float v = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v += red[c * 128 + t];
+        a.out[k][q * 128 + t] = v;
+    }
 }
 
 // ------------------------------------------------------ element-wise parts
