@@ -25,6 +25,18 @@
 
 namespace unk {
 
+// Programmatic dependent launch (both return at once without it).  grid_wait: what the
+// kernel before this one wrote is complete; before any access to global memory.
+// grid_launch: the next kernel's blocks may become resident; in a kernel that
+// allocates TMEM only once it holds it, since a waiting block of the next kernel
+// could otherwise hold the columns that this one needs to finish.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_begin() {
+    grid_launch();
+    grid_wait();
+}
+
 typedef __nv_bfloat16 bf16;
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
@@ -119,6 +131,7 @@ constexpr int CV_STAGES = 3;
 
 template <int NT>
 __global__ void __launch_bounds__(256) k_conv3(ConvArgs a) {
+    grid_begin();
     __shared__ __align__(128) bf16 sA[CV_STAGES][CV_MT * CV_LD];
     __shared__ __align__(128) bf16 sB[CV_STAGES][NT * CV_LD];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -264,6 +277,7 @@ constexpr int HT_B = 9 * HT_NT * CV_LD;       // halves per weight stage
 __host__ __device__ constexpr size_t halo_smem_bytes() { return (size_t)2 * (HT_A + HT_B) * 2; }
 
 __global__ void __launch_bounds__(256) k_conv3_halo(ConvArgs a) {
+    grid_begin();
     extern __shared__ __align__(128) bf16 ht_smem[];
     bf16* sA = ht_smem;                 // [2][HT_A]
     bf16* sB = ht_smem + 2 * HT_A;      // [2][HT_B]
@@ -404,6 +418,7 @@ struct WgradArgs {
 
 template <int MT, int NT>
 __global__ void __launch_bounds__(256) k_wgrad(WgradArgs a) {
+    grid_begin();
     constexpr int LG = MT + 8, LX = NT + 8;
     __shared__ __align__(128) bf16 sG[2][32 * LG];
     __shared__ __align__(128) bf16 sX[2][32 * LX];
@@ -524,6 +539,7 @@ constexpr int WH_X = HT_HH * HT_HW * CV_LD;     // halves per halo stage
 __host__ __device__ constexpr size_t wgrad_halo_smem_bytes() { return (size_t)2 * (WH_G + WH_X) * 2; }
 
 __global__ void __launch_bounds__(256) k_wgrad_halo(WgradHaloArgs a) {
+    grid_begin();
     extern __shared__ __align__(128) bf16 wh_smem[];
     bf16* sG = wh_smem;              // [2][WH_G]: [pixel][co]
     bf16* sX = wh_smem + 2 * WH_G;   // [2][WH_X]: [halo pixel][ci]
@@ -653,6 +669,7 @@ struct SumJobs {
 };
 
 __global__ void __launch_bounds__(256) k_sum_splits(const __grid_constant__ SumJobs a) {
+    grid_begin();
     __shared__ float4 red4[8][32];
     float* red = &red4[0][0].x;
     const int t = threadIdx.x, b = blockIdx.x;
@@ -697,6 +714,7 @@ __global__ void __launch_bounds__(256) k_sum_splits(const __grid_constant__ SumJ
 // network input: 3 float32 planes [P][3] (pixel-major) -> BF16, 32 channels
 // (zero padded); one thread per (row, channel group, x), x fastest
 __global__ void k_input(const float* __restrict__ in, long long rows, int W, bf16* __restrict__ x0) {
+    grid_begin();
     const long long total = rows * 4 * W;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(i % W);
@@ -715,6 +733,7 @@ __global__ void k_input(const float* __restrict__ in, long long rows, int W, bf1
 // N x H/2 x W/2 pixels and C channels; one thread per output (row, group, x)
 __global__ void k_pool(const bf16* __restrict__ s, int sC, int soff, int C, int N, int H, int W,
                        bf16* __restrict__ out) {
+    grid_begin();
     const int C8 = C / 8, H2 = H / 2, W2 = W / 2;
     const long long total = (long long)N * H2 * C8 * W2;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -742,6 +761,7 @@ __global__ void k_pool(const bf16* __restrict__ s, int sC, int soff, int C, int 
 // (y, x) = (sum of the 2x2 fine block of g) * (mask at fine (2y, 2x) > 0)
 __global__ void k_up_bwd(const bf16* __restrict__ g, int gC, int goff, const bf16* __restrict__ mask, int mC,
                          int moff, int C, int N, int H, int W, bf16* __restrict__ out) {
+    grid_begin();
     const int C8 = C / 8, H2 = H / 2, W2 = W / 2;
     const long long total = (long long)N * H2 * C8 * W2;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -772,6 +792,7 @@ __global__ void k_up_bwd(const bf16* __restrict__ g, int gC, int goff, const bf1
 __global__ void k_skip_bwd(const bf16* __restrict__ gp, const bf16* __restrict__ gcat, int gC, int goff,
                            const bf16* __restrict__ s, int sC, int soff, int C, int N, int H, int W,
                            bf16* __restrict__ out) {
+    grid_begin();
     const int C8 = C / 8;
     const long long total = (long long)N * H * C8 * W;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -794,6 +815,7 @@ __global__ void k_skip_bwd(const bf16* __restrict__ gp, const bf16* __restrict__
 template <int C>
 __global__ void k_head_fwd(const bf16* __restrict__ h, const float* __restrict__ Wh, const float* __restrict__ bh,
                            long long P, int W, float* __restrict__ y) {
+    grid_begin();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
         float y0 = bh[0], y1 = bh[1];
         const long long row = p / W;
@@ -822,6 +844,7 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, co
                                                    long long P, int W, int rows_per_block, float inv_count2,
                                                    bf16* __restrict__ gh, float* __restrict__ pw,
                                                    double* __restrict__ pl) {
+    grid_begin();
     constexpr int NV = 2 * C + 2;
     __shared__ float sw[8][NV];
     __shared__ double sl[8];
@@ -894,6 +917,7 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, co
 
 // *out = sum of n doubles: strided per-thread sums, fixed-order tree (one block of 256)
 __global__ void __launch_bounds__(256) k_sum_doubles(const double* __restrict__ part, int n, double* __restrict__ out) {
+    grid_begin();
     __shared__ double red[256];
     double s = 0.0;
     for (int k = threadIdx.x; k < n; k += 256) s += part[k];
@@ -938,6 +962,7 @@ struct AdamRefreshArgs {
 // wt[ci][8 - tap][co] (shift_{8 - tap} = -shift_tap), and the stage images
 // of both for the streamed tensor-core convolution.
 __global__ void k_adam_refresh(AdamRefreshArgs a) {
+    grid_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.n; i += (long long)gridDim.x * blockDim.x) {
         float pi = a.p[i];
         if (a.adam) {

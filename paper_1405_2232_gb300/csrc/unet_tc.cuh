@@ -267,6 +267,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         *s_abort = 0;
     }
+    grid_wait();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(s_tmem)),
                      "r"(tc_tmem_cols<N>())
@@ -289,6 +290,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *s_tmem;
+    grid_launch();  // (after the TMEM allocation, which the next kernel's must not come before)
 
     if (warp == 0) {
         // ------------------------------------------------ producer warp
