@@ -41,12 +41,11 @@ constexpr size_t fd_fused_smem_bytes() {
     return (size_t)STAGES * 10 * (BX + 2 * FD_HALO) * C::ES + fd_fused_ring_bytes<PREC, BX>() +
            (size_t)2 * STAGES * 8 + 16;
 }
+// Four stages, as the ring rows: the loop is unrolled by four, so that every stage and
+// ring row is a constant offset.
 template <int PREC, int BX>
 constexpr int fd_fused_stages() {
-    using C = StripCfg<PREC>;
-    constexpr size_t stage = (size_t)10 * (BX + 2 * FD_HALO) * C::ES;
-    constexpr size_t s = (110 * 1024 - 32 - fd_fused_ring_bytes<PREC, BX>()) / stage;
-    return s > 12 ? 12 : (int)s;
+    return 4;
 }
 
 // FP64: the printed sums over the eight neighbours X[i], R[i] in their order,
@@ -270,11 +269,21 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     const bool own_col = !halo && t < W;
     int flags = 0;
     bool aborted = false;
-    for (int j = 0; j < njobs + 2; ++j) {
+    // row r (constant relative to the group of four) of an eight-row ring: `cur` is the
+    // half of rows 4 g .. 4 g + 3 of group g, `prv` the other
+    static_assert(STAGES == 4, "stages and four-row rings share the unrolled index");
+    uint32_t ph = 0;  // parity of "full": the group's
+    real *rho_cur = r_rho, *rho_prv = r_rho + 4 * RA, *T_cur = r_T, *T_prv = r_T + 4 * RA;
+    for (int jb = 0; jb < njobs + 2 && !aborted; jb += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int j = jb + u;
+        if (j >= njobs + 2) break;
+        auto row8 = [&](real* cur, real* prv, int r) { return ((r >= 0 || r < -4) ? cur : prv) + (r & 3) * RA; };
         // A(j)
         if (j < njobs) {
-            const int s = j % STAGES;
-            if (!mbar_wait_bounded(&full[s], (uint32_t)((j / STAGES) & 1), kp.wait_cycles)) s_abort[j & 1] = 1;
+            const int s = u;
+            if (!mbar_wait_bounded(&full[s], ph, kp.wait_cycles)) s_abort[u & 1] = 1;
             if (colA != -99) {
                 const elem* st = stage + (size_t)s * NP * SEGW;
                 const int c = colA + HALO;
@@ -287,16 +296,16 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                 const real T = (real)st[9 * SEGW + c];
                 site_psi_T<real, BMODE>(kp, rho, T, psi, psi2, flags);
                 const int ia = colA + 2;
-                if (BMODE != BETA_ZERO) r_psi[(j & 3) * RA + ia] = psi;
-                if (BMODE != BETA_ONE) r_psi2[(j & 3) * RA + ia] = psi2;
-                r_rho[(j & 7) * RA + ia] = rho;
-                r_T[(j & 7) * RA + ia] = T;
+                if (BMODE != BETA_ZERO) r_psi[u * RA + ia] = psi;
+                if (BMODE != BETA_ONE) r_psi2[u * RA + ia] = psi2;
+                row8(rho_cur, rho_prv, u)[ia] = rho;
+                row8(T_cur, T_prv, u)[ia] = T;
             }
         }
         consumer_sync<BX + 32>();
         // (a thread that times out at job j + 1 writes the other slot than the
         // one read here, so every consumer leaves at the same job)
-        if (s_abort[j & 1]) {
+        if (s_abort[u & 1]) {
             aborted = true;
             break;
         }
@@ -304,7 +313,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
         {
             const int k = j - 1;
             if (k >= 1 && k <= njobs - 2 && colB != -99) {
-                const elem* st = stage + (size_t)(k % STAGES) * NP * SEGW;
+                const elem* st = stage + (size_t)((u + 3) & 3) * NP * SEGW;
                 const int c = colB + HALO;
                 real f[9], g[9];
 #pragma unroll
@@ -312,15 +321,13 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     f[i] = S::load(st + i * SEGW + c - ex(i), (real)kp.base_f[i]);
                     g[i] = (real)0;
                 }
-                real rho = f[0];
-#pragma unroll
-                for (int i = 1; i < 9; ++i) rho += f[i];
                 const int ia = colB + 2;
+                const real rho = row8(rho_cur, rho_prv, u - 1)[ia];
                 real Fx, Fy, ux, uy, Tg;
                 force_from_rows<real, BMODE>(
-                    kp, r_psi + ((k - 1) & 3) * RA + ia, r_psi + (k & 3) * RA + ia, r_psi + ((k + 1) & 3) * RA + ia,
-                    r_psi2 + ((k - 1) & 3) * RA + ia, r_psi2 + (k & 3) * RA + ia,
-                    r_psi2 + ((k + 1) & 3) * RA + ia, Fx, Fy);
+                    kp, r_psi + ((u + 2) & 3) * RA + ia, r_psi + ((u + 3) & 3) * RA + ia, r_psi + ((u + 0) & 3) * RA + ia,
+                    r_psi2 + ((u + 2) & 3) * RA + ia, r_psi2 + ((u + 3) & 3) * RA + ia,
+                    r_psi2 + ((u + 0) & 3) * RA + ia, Fx, Fy);
                 // the f half of the collision; g (zero here) is not used
                 // (FP32: the fused multiply-add form, faster in this kernel)
                 collide<real, false, true>(kp, f, g, rho, Fx, Fy, ux, uy, Tg);
@@ -328,13 +335,13 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                     // FP32: the rings keep a = chi grad(rho) / rho - u, which
                     // both stages' K share (fd_K_rows_a)
                     real ax, ay;
-                    fd_a_rows(r_rho + ((k - 1) & 7) * RA + ia, r_rho + (k & 7) * RA + ia,
-                              r_rho + ((k + 1) & 7) * RA + ia, ux, uy, chi, ax, ay);
-                    r_ux[(k & 3) * RB + colB + 1] = ax;
-                    r_uy[(k & 3) * RB + colB + 1] = ay;
+                    fd_a_rows(row8(rho_cur, rho_prv, u - 2) + ia, row8(rho_cur, rho_prv, u - 1) + ia,
+                              row8(rho_cur, rho_prv, u) + ia, ux, uy, chi, ax, ay);
+                    r_ux[((u + 3) & 3) * RB + colB + 1] = ax;
+                    r_uy[((u + 3) & 3) * RB + colB + 1] = ay;
                 } else {
-                    r_ux[(k & 3) * RB + colB + 1] = ux;
-                    r_uy[(k & 3) * RB + colB + 1] = uy;
+                    r_ux[((u + 3) & 3) * RB + colB + 1] = ux;
+                    r_uy[((u + 3) & 3) * RB + colB + 1] = uy;
                 }
                 if (own_col && k >= 2 && k <= njobs - 3) {
                     int y = y_start - 2 + k;
@@ -361,18 +368,18 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
             const int k = j - 2;
             if (k >= 1 && k <= njobs - 2 && colB != -99) {
                 const int ia = colB + 2, ib = colB + 1;
-                const real* Ts_ = r_T + ((k - 1) & 7) * RA + ia;
-                const real* Tc_ = r_T + (k & 7) * RA + ia;
-                const real* Tn_ = r_T + ((k + 1) & 7) * RA + ia;
+                const real* Ts_ = row8(T_cur, T_prv, u - 3) + ia;
+                const real* Tc_ = row8(T_cur, T_prv, u - 2) + ia;
+                const real* Tn_ = row8(T_cur, T_prv, u - 1) + ia;
                 real K;
                 if constexpr (sizeof(real) == 4)
-                    K = fd_K_rows_a(Ts_, Tc_, Tn_, r_ux[(k & 3) * RB + ib], r_uy[(k & 3) * RB + ib], chi);
+                    K = fd_K_rows_a(Ts_, Tc_, Tn_, r_ux[((u + 2) & 3) * RB + ib], r_uy[((u + 2) & 3) * RB + ib], chi);
                 else
-                    K = fd_K_rows<real>(Ts_, Tc_, Tn_, r_rho + ((k - 1) & 7) * RA + ia, r_rho + (k & 7) * RA + ia,
-                                        r_rho + ((k + 1) & 7) * RA + ia, r_ux[(k & 3) * RB + ib],
-                                        r_uy[(k & 3) * RB + ib], chi);
-                r_h1[(k & 3) * RB + ib] = K;
-                r_Ts[(k & 3) * RB + ib] = Tc_[0] + a * K;
+                    K = fd_K_rows<real>(Ts_, Tc_, Tn_, row8(rho_cur, rho_prv, u - 3) + ia, row8(rho_cur, rho_prv, u - 2) + ia,
+                                        row8(rho_cur, rho_prv, u - 1) + ia, r_ux[((u + 2) & 3) * RB + ib],
+                                        r_uy[((u + 2) & 3) * RB + ib], chi);
+                r_h1[((u + 2) & 3) * RB + ib] = K;
+                r_Ts[((u + 2) & 3) * RB + ib] = Tc_[0] + a * K;
             }
         }
         // D(k), k = j - 4: stage 2 on own rows and columns
@@ -382,15 +389,15 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                 const int ia = t + 2, ib = t + 1;
                 real K;
                 if constexpr (sizeof(real) == 4)
-                    K = fd_K_rows_a(r_Ts + ((k - 1) & 3) * RB + ib, r_Ts + (k & 3) * RB + ib,
-                                    r_Ts + ((k + 1) & 3) * RB + ib, r_ux[(k & 3) * RB + ib], r_uy[(k & 3) * RB + ib],
+                    K = fd_K_rows_a(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + ((u + 0) & 3) * RB + ib,
+                                    r_Ts + ((u + 1) & 3) * RB + ib, r_ux[((u + 0) & 3) * RB + ib], r_uy[((u + 0) & 3) * RB + ib],
                                     chi);
                 else
-                    K = fd_K_rows<real>(r_Ts + ((k - 1) & 3) * RB + ib, r_Ts + (k & 3) * RB + ib,
-                                        r_Ts + ((k + 1) & 3) * RB + ib, r_rho + ((k - 1) & 7) * RA + ia,
-                                        r_rho + (k & 7) * RA + ia, r_rho + ((k + 1) & 7) * RA + ia,
-                                        r_ux[(k & 3) * RB + ib], r_uy[(k & 3) * RB + ib], chi);
-                const real v = r_T[(k & 7) * RA + ia] + (real)0.5 * (r_h1[(k & 3) * RB + ib] + K);
+                    K = fd_K_rows<real>(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + ((u + 0) & 3) * RB + ib,
+                                        r_Ts + ((u + 1) & 3) * RB + ib, row8(rho_cur, rho_prv, u - 5) + ia,
+                                        row8(rho_cur, rho_prv, u - 4) + ia, row8(rho_cur, rho_prv, u - 3) + ia,
+                                        r_ux[((u + 0) & 3) * RB + ib], r_uy[((u + 0) & 3) * RB + ib], chi);
+                const real v = row8(T_cur, T_prv, u - 4)[ia] + (real)0.5 * (r_h1[((u + 0) & 3) * RB + ib] + K);
                 int y = y_start - 2 + k;
                 y = y >= ny ? y - ny : y;
                 const int xg = x0 + t;
@@ -404,8 +411,16 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
         // the stage of job j-1 has had its last reader (A at j-1, B at j)
         if (j >= 1 && j <= njobs - 1 && !halo) {
             __syncwarp();
-            if ((t & 31) == 0) mbar_arrive(&empty[(j - 1) % STAGES]);
+            if ((t & 31) == 0) mbar_arrive(&empty[(u + 3) & 3]);
         }
+      }
+        ph ^= 1u;
+        real* x = rho_cur;
+        rho_cur = rho_prv;
+        rho_prv = x;
+        x = T_cur;
+        T_cur = T_prv;
+        T_prv = x;
     }
     if (aborted) {
         if (t == 0) atomicOr(kp.err, 1 << LB_ERR_TIMEOUT);
