@@ -1,6 +1,5 @@
 // lb_fd_strip.cuh -- the finite-difference temperature treatment (Eqs. 26-27)
-// in one pass over HBM on strip contexts (k_fd_fused), and the fused RK2
-// stages used after the tile front on other lattices (k_fd_rk2).
+// in one pass over HBM on strip contexts (k_fd_fused).
 //
 // k_fd_fused is k_step_strip (lb_step_strip.cuh) with the g populations
 // replaced by the temperature field and the RK2 update of Eq. (27) folded in:
@@ -10,14 +9,9 @@
 // row rings for psi, rho, T^n, u^n, h1 and the intermediate T.  Per site it
 // reads f and T^n and writes f and T^{n+1} once (80 B in FP32).
 //
-// k_fd_rk2 evaluates T^{n+1} = T^n + (h1 + K(T^n + a h1))/2, h1 = K(T^n), in
-// one launch: a tile stages T^n and rho^n with a two-site ring, u^n with a
-// one-site ring, computes h1 and the intermediate T on the tile plus one ring
-// in shared memory, then the second stage on the tile (each thread two rows).
-//
 // K uses the isotropic central stencils of the D2Q9 lattice; in FP64 every
 // formula is evaluated in its printed order (compiled without contraction),
-// so the fused kernel and the tile front + k_fd_rk2 give the same bits.
+// so the fused kernel and the tile kernels (lb_fd_tile.cuh) give the same bits.
 #pragma once
 
 #include "lb_fd.cuh"
@@ -48,111 +42,15 @@ constexpr int fd_fused_stages() {
     return 4;
 }
 
-// FP64: the printed sums over the eight neighbours X[i], R[i] in their order,
-// without the products by e_i = 0 (which add zero), each w X[i] formed once for
-// both gradient components, and the divisions by c_s^2 as div_cs2.
-__device__ __forceinline__ double fd_K_fp64(const double X[9], const double R[9], double ux, double uy, double chi) {
-    double gTx = 0, gTy = 0, grx = 0, gry = 0, lap = 0;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const double w = wd(i), wX = w * X[i], wR = w * R[i];
-        if (ex(i)) {
-            gTx = ex(i) > 0 ? gTx + wX : gTx - wX;
-            grx = ex(i) > 0 ? grx + wR : grx - wR;
-        }
-        if (ey(i)) {
-            gTy = ey(i) > 0 ? gTy + wX : gTy - wX;
-            gry = ey(i) > 0 ? gry + wR : gry - wR;
-        }
-        lap += w * (X[i] - X[0]);
-    }
-    gTx = div_cs2(gTx);
-    gTy = div_cs2(gTy);
-    grx = div_cs2(grx);
-    gry = div_cs2(gry);
-    lap *= 2.0 / (1.0 / 3.0);
-    return -(ux * gTx + uy * gTy) + chi * (lap + (grx * gTx + gry * gTy) / R[0]);
-}
-
-// K(X) of Eq. (26) from X and rho of a site and its eight neighbours.  FP64: the
-// order of operations of the printed form (fd_K_fp64); FP32: the same sums with
-// the divisions by c_s^2 = 1/3 taken as products by 3 and the division by rho
-// as the fast division.
-template <typename real>
-__device__ __forceinline__ real fd_K(const real X[9], const real R[9], real ux, real uy, real chi) {
-    if constexpr (sizeof(real) == 8) {
-        return fd_K_fp64(X, R, ux, uy, chi);
-    } else {
-        real gTx = 0, gTy = 0, grx = 0, gry = 0, lap = 0;
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            const real w = (real)wd(i);
-            gTx += w * (real)ex(i) * X[i];
-            gTy += w * (real)ey(i) * X[i];
-            grx += w * (real)ex(i) * R[i];
-            gry += w * (real)ey(i) * R[i];
-            lap += w * (X[i] - X[0]);
-        }
-        gTx *= (real)3;
-        gTy *= (real)3;
-        grx *= (real)3;
-        gry *= (real)3;
-        lap *= (real)6;
-        // the fast division (a few ulp; +3% on the issue-bound fused step)
-        return -(ux * gTx + uy * gTy) + chi * (lap + __fdividef(grx * gTx + gry * gTy, R[0]));
-    }
-}
-
-// K(X) of Eq. (26) at one site from three row pointers (south, centre, north,
-// each at the site's column) of X and of rho.
-template <typename real>
-__device__ __forceinline__ real fd_K_rows(const real* Xs, const real* Xc, const real* Xn, const real* Rs,
-                                          const real* Rc, const real* Rn, real ux, real uy, real chi) {
-    real X[9], R[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        X[i] = (ey(i) == 1 ? Xn : (ey(i) == -1 ? Xs : Xc))[ex(i)];
-        R[i] = (ey(i) == 1 ? Rn : (ey(i) == -1 ? Rs : Rc))[ex(i)];
-    }
-    return fd_K<real>(X, R, ux, uy, chi);
-}
-
-// FP32: the same K with the terms that depend only on the site's density and
-// velocity folded into a = chi grad(rho) / rho - u, which both RK2 stages
-// share (formed once per site in the fused kernel's velocity phase):
-// K = a . grad(X) + chi lap(X), the stencil of X alone.
-__device__ __forceinline__ float fd_K_rows_a(const float* Xs, const float* Xc, const float* Xn, float ax,
-                                             float ay, float chi) {
-    float gTx = 0.0f, gTy = 0.0f, lap = 0.0f;
-    const float X0 = Xc[0];
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const float w = (float)wd(i);
-        const float* xr = ey(i) == 1 ? Xn : (ey(i) == -1 ? Xs : Xc);
-        const float Xv = xr[ex(i)];
-        gTx += w * (float)ex(i) * Xv;
-        gTy += w * (float)ey(i) * Xv;
-        lap += w * (Xv - X0);
-    }
-    return fmaf(ax, 3.0f * gTx, fmaf(ay, 3.0f * gTy, chi * (6.0f * lap)));
-}
-
-// a = chi grad(rho) / rho - u at a site (FP32; see fd_K_rows_a), from the
-// density rows (south, centre, north, each at the site's column)
-__device__ __forceinline__ void fd_a_rows(const float* Rs, const float* Rc, const float* Rn, float ux, float uy,
-                                          float chi, float& ax, float& ay) {
-    float grx = 0.0f, gry = 0.0f;
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        const float w = (float)wd(i);
-        const float* rr = ey(i) == 1 ? Rn : (ey(i) == -1 ? Rs : Rc);
-        const float rn = rr[ex(i)];
-        grx += w * (float)ex(i) * rn;
-        gry += w * (float)ey(i) * rn;
-    }
-    const float cr = __fdividef(chi, Rc[0]);
-    ax = fmaf(cr, 3.0f * grx, -ux);
-    ay = fmaf(cr, 3.0f * gry, -uy);
+// K(X) of Eq. (26) in FP64 from three row pointers (south, centre, north, each at the
+// site's column) of X and of rho.
+__device__ __forceinline__ double fd_K_rows(const double* Xs, const double* Xc, const double* Xn, const double* Rs,
+                                            const double* Rc, const double* Rn, double ux, double uy, double chi) {
+    double X[9], R[9], grx, gry;
+    fd_window(Xs, Xc, Xn, X);
+    fd_window(Rs, Rc, Rn, R);
+    fd_grad_fp64(R, grx, gry);
+    return fd_K_fp64(X, grx, gry, R[0], ux, uy, chi);
 }
 
 // One whole FD step (Eqs. 1, 26, 27) on a strip context, one pass over HBM:
@@ -375,7 +273,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                 if constexpr (sizeof(real) == 4)
                     K = fd_K_rows_a(Ts_, Tc_, Tn_, r_ux[((u + 2) & 3) * RB + ib], r_uy[((u + 2) & 3) * RB + ib], chi);
                 else
-                    K = fd_K_rows<real>(Ts_, Tc_, Tn_, row8(rho_cur, rho_prv, u - 3) + ia, row8(rho_cur, rho_prv, u - 2) + ia,
+                    K = fd_K_rows(Ts_, Tc_, Tn_, row8(rho_cur, rho_prv, u - 3) + ia, row8(rho_cur, rho_prv, u - 2) + ia,
                                         row8(rho_cur, rho_prv, u - 1) + ia, r_ux[((u + 2) & 3) * RB + ib],
                                         r_uy[((u + 2) & 3) * RB + ib], chi);
                 r_h1[((u + 2) & 3) * RB + ib] = K;
@@ -393,7 +291,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
                                     r_Ts + ((u + 1) & 3) * RB + ib, r_ux[((u + 0) & 3) * RB + ib], r_uy[((u + 0) & 3) * RB + ib],
                                     chi);
                 else
-                    K = fd_K_rows<real>(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + ((u + 0) & 3) * RB + ib,
+                    K = fd_K_rows(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + ((u + 0) & 3) * RB + ib,
                                         r_Ts + ((u + 1) & 3) * RB + ib, row8(rho_cur, rho_prv, u - 5) + ia,
                                         row8(rho_cur, rho_prv, u - 4) + ia, row8(rho_cur, rho_prv, u - 3) + ia,
                                         r_ux[((u + 0) & 3) * RB + ib], r_uy[((u + 0) & 3) * RB + ib], chi);
@@ -425,127 +323,6 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     if (aborted) {
         if (t == 0) atomicOr(kp.err, 1 << LB_ERR_TIMEOUT);
         return;
-    }
-    if (flags) atomicOr(kp.err, flags);
-}
-
-// K(X) of Eq. (26) from shared-memory tiles: X and R (rho) with row strides
-// xs and rs, centre indices xc and rc.  FP64: the stencil and order of
-// operations of the printed form (divisions by c_s^2 included); FP32:
-// the same sums with the divisions by c_s^2 = 1/3 taken as products by 3 and
-// the division by rho as the fast division.
-template <typename real>
-__device__ __forceinline__ real fd_K_tile(const real* X, int xs, int xc, const real* R, int rs, int rc, real ux,
-                                          real uy, real chi) {
-    real Xv[9], Rv[9];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        Xv[i] = X[xc + ey(i) * xs + ex(i)];
-        Rv[i] = R[rc + ey(i) * rs + ex(i)];
-    }
-    return fd_K<real>(Xv, Rv, ux, uy, chi);
-}
-
-// Ghost value of a temperature-like field X at (rx, ry) outside the lattice
-// of a cavity (walls 1) or channel (walls 2) context, from the value Xm at the
-// mirror node (the clamped position): reflected about the boundary value,
-// 2 T_b - Xm, across an isothermal boundary (cavity side walls; channel
-// plates at T_w and inlet at T_in); Xm across an adiabatic one (cavity bottom
-// and top, channel lower plate in Case B, channel outlet).  A position outside
-// in both directions takes the side-wall rule in the cavity and the plate
-// rule in the channel.
-template <typename real>
-__device__ __forceinline__ real fd_ghost(const KParams& kp, int rx, int ry, real Xm) {
-    const int nx = kp.nx, ny = kp.ny;
-    if (kp.walls == 1) {
-        if (rx < 0) return (real)2.0 * KPR(kp, T_hot) - Xm;
-        if (rx >= nx) return (real)2.0 * KPR(kp, T_cold) - Xm;
-        return Xm;
-    }
-    if (ry < 0 || ry >= ny) {
-        if (ry < 0 && kp.adiabatic_bottom) return Xm;
-        return (real)2.0 * KPR(kp, T_w) - Xm;
-    }
-    if (rx < 0) return (real)2.0 * KPR(kp, T_in) - Xm;
-    return Xm;
-}
-
-// tile of k_fd_rk2: FDR_BX x FDR_BY threads, FDR_ROWS rows of sites per thread
-constexpr int FDR_BX = 32, FDR_BY = 8, FDR_ROWS = 2;
-
-// Both RK2 stages of Eq. (27): T (T^n) and T_next in the context's T layout
-// (row pitch kp.pitch; ghost columns written when kp.ghost), rho, ux, uy dense.
-template <typename real>
-__global__ void __launch_bounds__(FDR_BX* FDR_BY)
-    k_fd_rk2(const real* __restrict__ T, const real* __restrict__ rho, const real* __restrict__ ux,
-             const real* __restrict__ uy, real* __restrict__ T_next, const KParams kp, real chi, real a) {
-    constexpr int BX = FDR_BX, BY = FDR_BY * FDR_ROWS, NT = FDR_BX * FDR_BY;
-    constexpr int W2 = BX + 4, H2 = BY + 4;  // tile + two-site ring (T, rho)
-    constexpr int W1 = BX + 2, H1 = BY + 2;  // tile + one-site ring (u, h1, Ts)
-    __shared__ real sT[H2 * W2], sR[H2 * W2];
-    __shared__ real sUx[H1 * W1], sUy[H1 * W1], sH1[H1 * W1], sTs[H1 * W1];
-    const int nx = kp.nx, ny = kp.ny;
-    const long long pitch = kp.pitch;
-    const int tid = threadIdx.x + threadIdx.y * FDR_BX;
-    const int x0 = blockIdx.x * BX, y0 = blockIdx.y * BY;
-    // cavity and channel (kp.walls): a neighbour outside reads the ghost of
-    // fd_ghost (reflected about an isothermal boundary, mirrored across an
-    // adiabatic one); rho and u the mirror node's
-    const bool walls = kp.walls != 0;
-    for (int s = tid; s < H2 * W2; s += NT) {
-        const int ly = s / W2, lx = s - ly * W2;
-        const int rx = x0 + lx - 2, ry = y0 + ly - 2;
-        const int gx = ringc(kp, rx, nx), gy = ringc(kp, ry, ny);
-        const real Tv = T[(long long)gy * pitch + gx];
-        sT[s] = walls && (rx < 0 || rx >= nx || ry < 0 || ry >= ny) ? fd_ghost<real>(kp, rx, ry, Tv) : Tv;
-        sR[s] = rho[(long long)gy * nx + gx];
-    }
-    for (int s = tid; s < H1 * W1; s += NT) {
-        const int ly = s / W1, lx = s - ly * W1;
-        const int gx = ringc(kp, x0 + lx - 1, nx), gy = ringc(kp, y0 + ly - 1, ny);
-        sUx[s] = ux[(long long)gy * nx + gx];
-        sUy[s] = uy[(long long)gy * nx + gx];
-    }
-    __syncthreads();
-    // stage 1 on the tile and its ring: h1 = K(T^n), Ts = T^n + a h1
-    for (int s = tid; s < H1 * W1; s += NT) {
-        const int ly = s / W1, lx = s - ly * W1;
-        const int rx = x0 + lx - 1, ry = y0 + ly - 1;
-        if (walls && (rx < 0 || rx >= nx || ry < 0 || ry >= ny)) continue;  // ghost: filled below
-        const int c2 = (ly + 1) * W2 + lx + 1;
-        const real K = fd_K_tile<real>(sT, W2, c2, sR, W2, c2, sUx[s], sUy[s], chi);
-        sH1[s] = K;
-        sTs[s] = sT[c2] + a * K;
-    }
-    __syncthreads();
-    if (walls) {
-        // intermediate temperature at the ghost sites of the ring, by the same rule
-        for (int s = tid; s < H1 * W1; s += NT) {
-            const int ly = s / W1, lx = s - ly * W1;
-            const int rx = x0 + lx - 1, ry = y0 + ly - 1;
-            if (rx >= 0 && rx < nx && ry >= 0 && ry < ny) continue;
-            const int mx = clampc(rx, nx) - x0 + 1, my = clampc(ry, ny) - y0 + 1;
-            sTs[s] = fd_ghost<real>(kp, rx, ry, sTs[my * W1 + mx]);
-        }
-        __syncthreads();
-    }
-    // stage 2 on the tile: T^{n+1} = T^n + (h1 + K(Ts)) / 2
-    int flags = 0;
-#pragma unroll
-    for (int q = 0; q < FDR_ROWS; ++q) {
-        const int ly = threadIdx.y + q * FDR_BY;
-        const int gx = x0 + threadIdx.x, gy = y0 + ly;
-        if (gx < nx && gy < ny) {
-            const int c1 = (ly + 1) * W1 + threadIdx.x + 1;
-            const int c2 = (ly + 2) * W2 + threadIdx.x + 2;
-            const real K = fd_K_tile<real>(sTs, W1, c1, sR, W2, c2, sUx[c1], sUy[c1], chi);
-            const real v = sT[c2] + (real)0.5 * (sH1[c1] + K);
-            real* p = T_next + (long long)gy * pitch + gx;
-            *p = v;
-            if (gx < kp.ghost) p[nx] = v;
-            if (gx >= nx - kp.ghost) p[-nx] = v;
-            if (!isfinite(v)) flags = 1 << LB_ERR_NONFINITE;
-        }
     }
     if (flags) atomicOr(kp.err, flags);
 }

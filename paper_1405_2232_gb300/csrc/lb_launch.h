@@ -111,7 +111,9 @@ struct FdLaunch {
     int bmode;
     double chi;           // (tau_g - 1/2) c_s^2
     double a;             // RK2 stage factor: 1 (Heun) or 1/2 (printed form)
-    int strip;            // strip context: the step is k_fd_fused
+    int strip;            // the step is k_fd_fused (strip contexts), else the tile kernels
+    int tile_by;          // rows of their tiles
+    int sms;              // SMs of the device
     int nchunks;          // row chunks per strip (strip contexts)
     cudaStream_t stream;
 };
@@ -180,6 +182,7 @@ inline PopLayout pop_layout(int prec, int nx, int ny, bool strip) {
     cudaError_t launch_scatter_##NAME(void* dst, const KParams& kp, const double* in,  \
                                       cudaStream_t st);                                \
     cudaError_t launch_fd_step_##NAME(const FdLaunch& L);                              \
+    cudaError_t launch_fd_tile_##NAME(const FdLaunch& L);                              \
     cudaError_t launch_fd_moments_##NAME(const FdLaunch& L);                           \
     cudaError_t launch_fd_set_T_##NAME(void* T, const double* T0, const KParams& kp, cudaStream_t st);
 

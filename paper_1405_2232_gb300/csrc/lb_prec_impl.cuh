@@ -178,44 +178,12 @@ cudaError_t fd_fused_launch(const FdLaunch& L) {
     return cudaGetLastError();
 }
 
-template <bool STEP>
-cudaError_t fd_front(const FdLaunch& L) {
-    if constexpr (!kFdSupported) {
-        return cudaErrorNotSupported;
-    } else {
-        using S = Store<LBGB_PREC>;
-        using E = typename S::elem;
-        using R = typename S::real;
-        const dim3 block(FD_BX, FD_BY);
-        const dim3 grid((L.kp.nx + FD_BX - 1) / FD_BX, (L.kp.ny + FD_BY - 1) / FD_BY);
-        const E* src = static_cast<const E*>(L.src);
-        E* dst = static_cast<E*>(L.dst);
-        const R* T = static_cast<const R*>(L.T);
-        R *rho = static_cast<R*>(L.rho), *ux = static_cast<R*>(L.ux), *uy = static_cast<R*>(L.uy);
-        switch (L.bmode) {
-            case BETA_ZERO:
-                k_fd_front<LBGB_PREC, BETA_ZERO, STEP><<<grid, block, 0, L.stream>>>(src, dst, T, rho, ux, uy, L.m_rho,
-                                                                                   L.m_ux, L.m_uy, L.m_T, L.kp);
-                break;
-            case BETA_ONE:
-                k_fd_front<LBGB_PREC, BETA_ONE, STEP><<<grid, block, 0, L.stream>>>(src, dst, T, rho, ux, uy, L.m_rho,
-                                                                                  L.m_ux, L.m_uy, L.m_T, L.kp);
-                break;
-            default:
-                k_fd_front<LBGB_PREC, BETA_MIXED, STEP><<<grid, block, 0, L.stream>>>(src, dst, T, rho, ux, uy,
-                                                                                    L.m_rho, L.m_ux, L.m_uy, L.m_T, L.kp);
-                break;
-        }
-        return cudaGetLastError();
-    }
-}
 }  // namespace
 
 cudaError_t LBGB_CAT(launch_fd_step_, LBGB_NAME)(const FdLaunch& L) {
     if constexpr (!kFdSupported) {
         return cudaErrorNotSupported;
     } else {
-        using R = typename Store<LBGB_PREC>::real;
         if (L.strip) {
             switch (L.bmode) {
                 case BETA_ZERO: return fd_fused_launch<BETA_ZERO>(L);
@@ -223,18 +191,9 @@ cudaError_t LBGB_CAT(launch_fd_step_, LBGB_NAME)(const FdLaunch& L) {
                 default: return fd_fused_launch<BETA_MIXED>(L);
             }
         }
-        cudaError_t e = fd_front<true>(L);
-        if (e != cudaSuccess) return e;
-        const dim3 block(FDR_BX, FDR_BY);
-        const dim3 grid((L.kp.nx + FDR_BX - 1) / FDR_BX, (L.kp.ny + FDR_BY * FDR_ROWS - 1) / (FDR_BY * FDR_ROWS));
-        k_fd_rk2<R><<<grid, block, 0, L.stream>>>(static_cast<const R*>(L.T), static_cast<const R*>(L.rho),
-                                                  static_cast<const R*>(L.ux), static_cast<const R*>(L.uy),
-                                                  static_cast<R*>(L.T_next), L.kp, (R)L.chi, (R)L.a);
-        return cudaGetLastError();
+        return LBGB_CAT(launch_fd_tile_, LBGB_NAME)(L);
     }
 }
-
-cudaError_t LBGB_CAT(launch_fd_moments_, LBGB_NAME)(const FdLaunch& L) { return fd_front<false>(L); }
 
 cudaError_t LBGB_CAT(launch_fd_set_T_, LBGB_NAME)(void* T, const double* T0, const KParams& kp, cudaStream_t st) {
     if constexpr (!kFdSupported) {

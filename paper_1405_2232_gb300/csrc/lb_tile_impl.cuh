@@ -9,6 +9,7 @@
 
 #include <atomic>
 
+#include "lb_fd_tile.cuh"
 #include "lb_launch.h"
 #include "lb_step_tile.cuh"
 
@@ -136,6 +137,69 @@ cudaError_t LBGB_CAT(launch_batch_tile_, LBGB_NAME)(const BatchTileLaunch& L) {
                               L.n_tiles, L.by);
 }
 #endif
+
+// ------------------------------------------------ finite-difference T (Eqs. 26-27)
+namespace {
+constexpr bool kFdTile = LBGB_PREC == LB_PREC_FP64 || LBGB_PREC == LB_PREC_FP32;
+
+// Launch over the lattice's 32-column tiles, programmatic and evenly shared (tile_smem).
+template <class K, class... A>
+cudaError_t fd_launch(std::atomic<unsigned long long>& done, const FdLaunch& L, size_t need, K kern, A... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((L.kp.nx + 31) / 32, (L.kp.ny + L.tile_by - 1) / L.tile_by);
+    cfg.blockDim = dim3(tile_threads(32, L.tile_by));
+    cfg.dynamicSmemBytes = tile_smem(L.sms, (long long)cfg.gridDim.x * cfg.gridDim.y, need);
+    cfg.stream = L.stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    if (cfg.dynamicSmemBytes > 48 * 1024) {
+        cudaError_t e = opt_in_smem(done, kern);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <int BM, bool STEP>
+cudaError_t fd_front(const FdLaunch& L) {
+    using E = typename Store<LBGB_PREC>::elem;
+    using R = typename Store<LBGB_PREC>::real;
+    static std::atomic<unsigned long long> done;
+    return fd_launch(done, L, tile_smem_bytes<LBGB_PREC, BM>(32, L.tile_by), k_fd_front<LBGB_PREC, BM, STEP>,
+                     static_cast<const E*>(L.src), static_cast<E*>(L.dst), static_cast<const R*>(L.T),
+                     static_cast<R*>(L.rho), static_cast<R*>(L.ux), static_cast<R*>(L.uy), L.m_rho, L.m_ux, L.m_uy,
+                     L.m_T, L.kp, L.tile_by);
+}
+template <bool STEP>
+cudaError_t fd_front(const FdLaunch& L) {
+    if (L.bmode == BETA_ZERO) return fd_front<BETA_ZERO, STEP>(L);
+    if (L.bmode == BETA_ONE) return fd_front<BETA_ONE, STEP>(L);
+    return fd_front<BETA_MIXED, STEP>(L);
+}
+}  // namespace
+
+cudaError_t LBGB_CAT(launch_fd_tile_, LBGB_NAME)(const FdLaunch& L) {
+    if constexpr (!kFdTile) {
+        return cudaErrorNotSupported;
+    } else {
+        using R = typename Store<LBGB_PREC>::real;
+        const cudaError_t e = fd_front<true>(L);
+        if (e != cudaSuccess) return e;
+        static std::atomic<unsigned long long> done;
+        return fd_launch(done, L, fd_rk2_smem_bytes<R>(L.tile_by), k_fd_rk2<R>, static_cast<const R*>(L.T),
+                         static_cast<const R*>(L.rho), static_cast<const R*>(L.ux), static_cast<const R*>(L.uy),
+                         static_cast<R*>(L.T_next), L.kp, (R)L.chi, (R)L.a, L.tile_by);
+    }
+}
+
+cudaError_t LBGB_CAT(launch_fd_moments_, LBGB_NAME)(const FdLaunch& L) {
+    if constexpr (!kFdTile)
+        return cudaErrorNotSupported;
+    else
+        return fd_front<false>(L);
+}
 
 namespace {
 template <int BM, bool PART>

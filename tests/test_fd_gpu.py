@@ -128,3 +128,26 @@ def test_fd_strip_front_matches_tile_front(lb, prec, nx, ny, strip):
         assert rel(sr, r) <= 1e-12 and rel(sT, Tn) <= 1e-12
     else:
         assert rel(sr, tr) <= 1e-6 and rel(sT, tT) <= 1e-6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("nx,ny", [(32, 4), (33, 15), (9, 8), (8, 33), (97, 41), (64, 70)])
+def test_fd_fp32_tile_and_strip_kernels_alternate(lb, nx, ny):
+    """Small FP32 lattices step on the tile kernels, and a caller-set wait limit runs the
+    strip kernel: both in turn on one context (f and T keep their ghost columns)
+    against the strip kernel alone.  Both evaluate the same FP32 formulas: one rounding
+    (2^-24, of values below 0.4) per population and step on rho, per stencil on T."""
+    rho, T = I.slab_fields(nx, ny, width=max(2, nx // 2), noise=1e-3)
+    T = T * (1.0 + 0.01 * np.cos(2 * np.pi * np.arange(nx) / nx))
+    kw = dict(nx=nx, ny=ny, precision="fp32", thermal=lb.LB_THERMAL_FD26, psi_uses_local_T=0, T_psi=0.85 * I.CS_TC,
+              beta=1.3)
+    with lb.Lattice(rho, T, **kw) as A, lb.Lattice(rho, T, tile_x=256, tile_y=0, **kw) as B:
+        for k in range(8):
+            lb.lb_set_wait_limit(A.ctx, 0 if k % 2 else 1 << 30)
+            A.step(1)
+        B.step(8)
+        A.synchronize()
+        B.synchronize()
+        a, b = A.moments(), B.moments()
+        assert np.abs(a[0] - b[0]).max() <= 8 * 9 * 2.0 ** -24 * 0.4
+        assert np.abs(a[3] - b[3]).max() <= 8 * 18 * 2.0 ** -24 * 0.1
