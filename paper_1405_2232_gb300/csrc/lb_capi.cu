@@ -16,6 +16,7 @@
 #include "lb.h"
 #include "lb_fd.cuh"
 #include "lb_launch.h"
+#include "lb_step_cluster.cuh"
 #include "tensor_map.h"
 
 using namespace lbgb;
@@ -175,6 +176,7 @@ struct lb_ctx {
     int nchunks = 1;            // strip kernel: row chunks per strip
     int tile_by = 0;            // see StepLaunch (finite-difference strip contexts: > 0
                                 // runs the tile kernels)
+    bool in_cluster = false;    // runs of steps take k_steps_cluster
     int fd_by = 8;              // rows of the finite-difference tile kernels' tiles
     int sms = 152;
     bool have_out_map = false;  // 16-bit strip contexts: out_map[b] describes buf[b]
@@ -257,7 +259,7 @@ KParams make_kparams(const lb_params& p, long long pitch, long long plane, int* 
     return k;
 }
 
-cudaError_t dispatch_step(const lb_ctx* c, const void* src, void* dst) {
+StepLaunch step_launch(const lb_ctx* c, const void* src, void* dst) {
     StepLaunch L;
     L.src = src;
     L.dst = dst;
@@ -275,11 +277,27 @@ cudaError_t dispatch_step(const lb_ctx* c, const void* src, void* dst) {
         L.dst_map = &c->out_map[dst == c->buf[0] ? 0 : 1];
         L.src_maps = &c->in_maps[src == c->buf[0] ? 0 : 1];
     }
+    return L;
+}
+
+cudaError_t dispatch_step(const lb_ctx* c, const void* src, void* dst) {
+    const StepLaunch L = step_launch(c, src, dst);
     switch (c->p.precision) {
         case LB_PREC_FP64: return launch_step_fp64(L);
         case LB_PREC_FP32: return launch_step_fp32(L);
         case LB_PREC_FP16_DEV: return launch_step_fp16(L);
         default: return launch_step_bf16(L);
+    }
+}
+
+// `steps` steps of a tiny lattice in one launch (0: can it be launched?)
+cudaError_t dispatch_cluster(const lb_ctx* c, int steps) {
+    const StepLaunch L = step_launch(c, c->buf[c->cur], c->buf[c->cur ^ (steps & 1)]);
+    switch (c->p.precision) {
+        case LB_PREC_FP32: return launch_cluster_fp32(L, steps);
+        case LB_PREC_FP16_DEV: return launch_cluster_fp16(L, steps);
+        case LB_PREC_BF16_DEV: return launch_cluster_bf16(L, steps);
+        default: return cudaErrorNotSupported;
     }
 }
 
@@ -542,6 +560,12 @@ lb_status create(const lb_params* p, void* stream, lb_ctx** out) {
     sms = c->sms;
     if (c->kp.walls || (strip && !p->tile_x && !p->tile_y && !c->fd))
         c->tile_by = default_tile_rows(p->precision, p->nx, p->ny - 2 * p->halo_rows, sms, c->kp.walls != 0);
+    c->in_cluster = strip && !p->tile_x && !p->tile_y && !c->fd && !p->halo_rows && p->precision != LB_PREC_FP64 &&
+                    cluster_blocks(p->nx, p->ny) > 0;
+    if (c->in_cluster && dispatch_cluster(c, 0) != cudaSuccess) {
+        (void)cudaGetLastError();
+        c->in_cluster = false;
+    }
     if (c->fd) {
         c->fd_by = default_tile_rows(p->precision, p->nx, p->ny, sms, true);
         // two tile launches against one strip pass: 512^2 13.5 us against 16.5, 768^2 26.7
@@ -688,6 +712,16 @@ lb_status lb_step(lb_ctx* c, int64_t n) {
     if (!c) return fail(LB_ERR_ARG, "ctx is NULL");
     if (n < 0) return fail(LB_ERR_ARG, "n must be >= 0");
     CU(cudaSetDevice(c->device), "cudaSetDevice");
+    // a tiny lattice takes a run of steps in one cluster (a caller-set wait limit is about
+    // the strip kernel's waits: it runs then)
+    while (c->in_cluster && n >= CLUSTER_RUN && c->kp.wait_cycles == WAIT_CYCLES_DEFAULT) {
+        const int m = (int)(n < CLUSTER_STEPS ? n : CLUSTER_STEPS);
+        cudaError_t e = dispatch_cluster(c, m);
+        if (e != cudaSuccess) return cuda_fail(e, "cluster kernel launch");
+        c->cur ^= m & 1;
+        c->t += m;
+        n -= m;
+    }
     for (int64_t k = 0; k < n; ++k) {
         cudaError_t e = c->fd ? dispatch_fd_step(c) : dispatch_step(c, c->buf[c->cur], c->buf[c->cur ^ 1]);
         if (e != cudaSuccess) return cuda_fail(e, "step kernel launch");

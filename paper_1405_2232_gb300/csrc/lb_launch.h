@@ -174,6 +174,7 @@ inline PopLayout pop_layout(int prec, int nx, int ny, bool strip) {
 #define LBGB_DECLARE_PREC(NAME)                                                       \
     cudaError_t launch_step_##NAME(const StepLaunch& L);                               \
     cudaError_t launch_tile_##NAME(const StepLaunch& L);                               \
+    cudaError_t launch_cluster_##NAME(const StepLaunch& L, int steps);                 \
     cudaError_t launch_moments_##NAME(const MomentsLaunch& L);                         \
     cudaError_t launch_init_##NAME(void* dst, const KParams& kp, const double* rho0,   \
                                    const double* T0, cudaStream_t st);                 \

@@ -11,6 +11,7 @@
 
 #include "lb_fd_tile.cuh"
 #include "lb_launch.h"
+#include "lb_step_cluster.cuh"
 #include "lb_step_tile.cuh"
 
 namespace lbgb {
@@ -96,6 +97,59 @@ cudaError_t LBGB_CAT(launch_tile_, LBGB_NAME)(const StepLaunch& L) {
     if (L.bx == 32 && (L.by == 8 || L.by == 16)) return step_tile<32, 0>(L, L.by);
     if (L.bx == 64 && L.by == 4) return step_tile<64, 0>(L, L.by);
     return cudaErrorInvalidValue;
+}
+
+// `steps` steps of a tiny lattice in one cluster (see lb_step_cluster.cuh); steps = 0
+// only asks whether the device can hold such a cluster.
+cudaError_t LBGB_CAT(launch_cluster_, LBGB_NAME)(const StepLaunch& L, int steps) {
+    if constexpr (LBGB_PREC == LB_PREC_FP64) {
+        return cudaErrorNotSupported;
+    } else {
+        using E = typename Store<LBGB_PREC>::elem;
+        const int nc = cluster_blocks(L.kp.nx, L.kp.ny);
+        if (!nc || L.kp.walls || L.kp.halo_rows) return cudaErrorInvalidValue;
+        void (*kern)(const E*, E*, const KParams, int);
+        if (L.eq24)
+            kern = L.bmode == BETA_ZERO  ? k_steps_cluster<LBGB_PREC, true, BETA_ZERO>
+                   : L.bmode == BETA_ONE ? k_steps_cluster<LBGB_PREC, true, BETA_ONE>
+                                         : k_steps_cluster<LBGB_PREC, true, BETA_MIXED>;
+        else
+            kern = L.bmode == BETA_ZERO  ? k_steps_cluster<LBGB_PREC, false, BETA_ZERO>
+                   : L.bmode == BETA_ONE ? k_steps_cluster<LBGB_PREC, false, BETA_ONE>
+                                         : k_steps_cluster<LBGB_PREC, false, BETA_MIXED>;
+        // opt in once per kernel and device: 16 blocks and the largest bands
+        static std::atomic<unsigned long long> configured[6];
+        auto& done = configured[(L.eq24 ? 3 : 0) + L.bmode];
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev >= 64 || !(done.load() >> dev & 1ULL)) {
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+            if (e != cudaSuccess) return e;
+            if (dev < 64) done.fetch_or(1ULL << dev);
+        }
+        const int rows = (L.kp.ny + nc - 1) / nc;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)nc;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)nc);
+        cfg.blockDim = dim3((unsigned)((L.kp.nx * (rows + 2) + 31) / 32 * 32));
+        cfg.dynamicSmemBytes = L.bmode == BETA_MIXED ? cluster_smem_bytes<LBGB_PREC, BETA_MIXED>(L.kp.nx, rows)
+                                                     : cluster_smem_bytes<LBGB_PREC, BETA_ONE>(L.kp.nx, rows);
+        cfg.stream = L.stream;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if (steps == 0) {
+            int clusters = 0;
+            e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+            return e == cudaSuccess && clusters == 0 ? cudaErrorNotSupported : e;
+        }
+        return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, steps);
+    }
 }
 
 #ifdef LBGB_BATCH

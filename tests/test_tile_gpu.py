@@ -78,3 +78,32 @@ def test_steps_under_stream_capture(lb):
         s.synchronize()
         for a, b in zip(A.populations(), B.populations()):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,eps", [("fp32", 2.0 ** -24), ("fp16", 2.0 ** -11), ("bf16", 2.0 ** -8)])
+@pytest.mark.parametrize("nx,ny", [(3, 3), (33, 5), (5, 300), (64, 64), (90, 91), (256, 32), (257, 31), (128, 65)])
+def test_runs_of_steps_equal_single_steps(lb, precision, eps, nx, ny):
+    """Tiny lattices take a run of steps in one cluster of blocks, single steps as tiles
+    (the last three sizes: both as tiles): the same state, odd and even runs, ghost columns
+    included (the strip kernel goes on from them)."""
+    ideal = dict(eos=lb.LB_EOS_IDEAL, a=0.0, b=0.0, R=0.5, G=1.0)
+    for thermal, beta, kw in ((lb.LB_THERMAL_EQ24, 1.3, {}), (lb.LB_THERMAL_EQ7, 1.0, {}),
+                              (lb.LB_THERMAL_EQ24, 0.0, ideal)):
+        if kw:
+            rho, T = I.sinusoid_fields(nx, ny, 1.0, 1.0, 0.05, mode=2, axis=0)
+        else:
+            rho, T = I.slab_fields(nx, ny, width=max(2, nx // 2), noise=1e-3)
+            kw = dict(psi_uses_local_T=0, T_psi=0.85 * I.CS_TC)
+        with lb.Lattice(rho, T, nx=nx, ny=ny, precision=precision, beta=beta, thermal=thermal, **kw) as A, \
+                lb.Lattice(rho, T, nx=nx, ny=ny, precision=precision, beta=beta, thermal=thermal, **kw) as B:
+            A.step(17)
+            lb.lb_set_wait_limit(A.ctx, 1 << 30)
+            A.step(1)
+            lb.lb_set_wait_limit(A.ctx, 0)
+            A.step(18)
+            for _ in range(36):
+                B.step(1)
+            A.synchronize()
+            B.synchronize()
+            for a, b in zip(A.populations(), B.populations()):
+                assert np.abs(a - b).max() <= 36 * 9 * eps * 0.2
