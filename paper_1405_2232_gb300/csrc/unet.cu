@@ -16,6 +16,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -915,21 +916,46 @@ lb_status un_warm_fields(int32_t N, int32_t H, int32_t W, const float* d_pred, d
     a.rho = d_rho;
     a.T = d_T;
     a.P = (long long)H * W;
-    // blocks per case: as many as leave each thread at least WARM_KEEP sites
-    int blocks = 1;
-    while (blocks < unk::WARM_MAX_CLUSTER && a.P > (long long)blocks * unk::WARM_THREADS * unk::WARM_KEEP) blocks *= 2;
-    if (blocks > 8)
-        UCU(cudaFuncSetAttribute(unk::k_warm, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "un_warm_fields");
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)blocks;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)N * (unsigned)blocks);
     cfg.blockDim = dim3(unk::WARM_THREADS);
     cfg.stream = static_cast<cudaStream_t>(stream);
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
+    int dev = 0, blocks = 1;
+    UCU(cudaGetDevice(&dev), "un_warm_fields");
+    UCU(cudaFuncSetAttribute(unk::k_warm, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "un_warm_fields");
+    // Blocks per case: the fewest rounds of resident clusters times the time of one,
+    // about 15 + (sites a thread) in units of a kept site (1.4 us), 2.5 for each site past
+    // them.  (7 clusters of 16 fit the chip one block per SM, 8 of 12, 15 of 9, 36 of 4: 8
+    // cases of 256^2 take 46 us in clusters of 12 and 85 in two rounds of 16.  The
+    // device's answers are kept.)
+    static std::atomic<int> resident[64][unk::WARM_MAX_CLUSTER + 1];
+    double best = INFINITY;
+    for (int nc = 1; nc <= unk::WARM_MAX_CLUSTER; ++nc) {
+        int n = dev < 64 ? resident[dev][nc].load() : 0;
+        if (n == 0) {
+            attr.val.clusterDim.x = (unsigned)nc;
+            cfg.gridDim = dim3((unsigned)nc);
+            if (cudaOccupancyMaxActiveClusters(&n, unk::k_warm, &cfg) != cudaSuccess || n < 1) {
+                (void)cudaGetLastError();
+                n = -1;
+            }
+            if (dev < 64) resident[dev][nc].store(n);
+        }
+        if (n < 1) continue;
+        const long long sites = (a.P + (long long)nc * unk::WARM_THREADS - 1) / ((long long)nc * unk::WARM_THREADS);
+        const long long past = sites > unk::WARM_KEEP ? sites - unk::WARM_KEEP : 0;
+        const double cost = (double)((N + n - 1) / n) * (15.0 + (double)sites + 1.5 * (double)past);
+        if (cost < best) {
+            best = cost;
+            blocks = nc;
+        }
+    }
+    attr.val.clusterDim.x = (unsigned)blocks;
+    cfg.gridDim = dim3((unsigned)N * (unsigned)blocks);
     UCU(cudaLaunchKernelEx(&cfg, unk::k_warm, a), "un_warm_fields");
     return LB_OK;
 }

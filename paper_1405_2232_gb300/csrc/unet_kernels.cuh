@@ -23,6 +23,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lb_device.cuh"
+
 namespace unk {
 
 // Programmatic dependent launch (both return at once without it).  grid_wait: what the
@@ -1004,131 +1006,232 @@ struct WarmArgs {
     long long P;  // sites per case
 };
 
-__device__ __forceinline__ double warm_rho_hat(const WarmArgs& a, long long i) {
-    return fmax(a.rho0[i] + a.rho_dev_scale * (double)a.pred[2 * i], a.rho_floor);
+__device__ __forceinline__ double warm_rho_hat(const WarmArgs& a, double rho0, float p) {
+    return fmax(rho0 + a.rho_dev_scale * lbgb::widen(p), a.rho_floor);
 }
-__device__ __forceinline__ double warm_T_hat(const WarmArgs& a, long long i) {
-    return a.T0[i] * (1.0 + a.t_dev_scale * (double)a.pred[2 * i + 1]);
+__device__ __forceinline__ double warm_T_hat(const WarmArgs& a, double T0, float p) {
+    return T0 * (1.0 + a.t_dev_scale * lbgb::widen(p));
 }
 
 constexpr int WARM_THREADS = 512;    // threads of a block
-constexpr int WARM_KEEP = 8;         // sites a thread keeps in registers
+constexpr int WARM_KEEP = 12;        // sites a thread keeps in registers
 constexpr int WARM_MAX_CLUSTER = 16;
 
-// Reduction of NV values over the cluster (sum, or min/max where asked), the same
-// on every thread: lanes, warps and blocks each in a fixed order.  The 16 warps'
-// values and the blocks' are each joined by half a warp per value (every thread
-// joining them cost more FP64 operations than the passes themselves).
-template <int NV>
-__device__ __forceinline__ void cluster_reduce(double (&v)[NV], const int (&op)[NV],
-                                               double (*s_warp)[5], double* s_block, double* s_all) {
+// An integer that orders as the double does (min and max without the FP64 units), and back.
+__device__ __forceinline__ long long order_key(double x) {
+    const long long b = __double_as_longlong(x);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double of_order_key(long long k) {
+    return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+}
+
+struct WarmShared {
+    double sum[WARM_THREADS / 32][4], block_sum[4], out[4];
+    long long lo[WARM_THREADS / 32], hi[WARM_THREADS / 32], block_lo, block_hi;
+};
+
+// Sums v[0..NS) (NS <= 4) and, with MINMAX, the least and greatest key over the
+// cluster: lanes, warps and blocks each in a fixed order.  The first warp of each block
+// then calls fin(sums, lo, hi, out[4]) and every thread returns its out: at one
+// FP64 warp operation in 16 cycles, sixteen warps repeating the last additions and
+// divisions cost more than the passes over the sites.
+template <int NS, bool MINMAX, class Fin>
+__device__ __forceinline__ void cluster_reduce(const double (&vin)[NS], long long lo, long long hi, WarmShared& sh,
+                                               double (&out)[4], Fin fin) {
     namespace cg = cooperative_groups;
-    static_assert(WARM_THREADS == 512 && WARM_MAX_CLUSTER == 16 && NV <= 5, "half a warp per value");
+    static_assert(WARM_THREADS == 512 && WARM_MAX_CLUSTER == 16 && NS <= 4, "half a warp joins them");
+    constexpr unsigned ALL = 0xffffffffu;
     cg::cluster_group cl = cg::this_cluster();
-    const int t = threadIdx.x, k16 = t >> 4, l16 = t & 15;
-    auto join = [](int o, double a, double b) { return o == 0 ? a + b : (o < 0 ? fmin(a, b) : fmax(a, b)); };
-    int my_op = 0;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // the first two exchanges halve the values that a lane carries: six additions for
+    // four sums; lanes 8 k .. 8 k + 7 then hold value k
+    double v[4];
 #pragma unroll
-    for (int k = 0; k < NV; ++k)
-        if (k == k16) my_op = op[k];
-    const double none = my_op == 0 ? 0.0 : (my_op < 0 ? INFINITY : -INFINITY);
-    auto join16 = [&](double x) {
+    for (int k = 0; k < 4; ++k) v[k] = k < NS ? vin[k < NS ? k : 0] : 0.0;
+    const bool up16 = lane & 16, up8 = lane & 8;
+    double x = up16 ? v[2] : v[0];
+    x += __shfl_xor_sync(ALL, up16 ? v[0] : v[2], 16);
+    if (NS > 1) {
+        double y = up16 ? v[3] : v[1];
+        y += __shfl_xor_sync(ALL, up16 ? v[1] : v[3], 16);
+        const double send = up8 ? x : y;
+        x = (up8 ? y : x) + __shfl_xor_sync(ALL, send, 8);
+    } else {
+        x += __shfl_xor_sync(ALL, x, 8);
+    }
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) {
-            const double y = __shfl_xor_sync(0xffffffffu, x, o);
-            x = my_op == 0 ? x + y : (my_op < 0 ? fmin(x, y) : fmax(x, y));
+    for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(ALL, x, o);
+    if ((lane & 7) == 0) sh.sum[warp][lane >> 3] = x;
+    if (MINMAX) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = min(lo, __shfl_xor_sync(ALL, lo, o));
+            hi = max(hi, __shfl_xor_sync(ALL, hi, o));
         }
-        return x;
-    };
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] = join(op[k], v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
-        if ((t & 31) == 0) s_warp[t >> 5][k] = v[k];
+        if (lane == 0) {
+            sh.lo[warp] = lo;
+            sh.hi[warp] = hi;
+        }
     }
     __syncthreads();
-    if (t < 96) {  // (whole warps shuffle; five values are two and a half)
-        const double x = join16(k16 < NV ? s_warp[l16][k16] : none);
-        if (k16 < NV && l16 == 0) s_block[k16] = x;
+    // half a warp joins the sixteen values of one sum (of the warps, then of the blocks)
+    const int k = t >> 4, l = t & 15;
+    auto join = [&](double a) {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(ALL, a, o);
+        return a;
+    };
+    auto join_keys = [&] {
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) {
+            lo = min(lo, __shfl_xor_sync(ALL, lo, o));
+            hi = max(hi, __shfl_xor_sync(ALL, hi, o));
+        }
+    };
+    if (t < 64) {
+        const double a = join(sh.sum[l][k]);
+        if (l == 0) sh.block_sum[k] = a;
+    } else if (MINMAX && t < 96) {
+        lo = sh.lo[l];
+        hi = sh.hi[l];
+        join_keys();
+        if (t == 64) {
+            sh.block_lo = lo;
+            sh.block_hi = hi;
+        }
     }
     cl.sync();
-    if (t < 96) {
-        const double x =
-            join16(k16 < NV && l16 < (int)cl.num_blocks() ? *cl.map_shared_rank(s_block + k16, l16) : none);
-        if (k16 < NV && l16 == 0) s_all[k16] = x;
+    const int blocks = (int)cl.num_blocks();
+    if (t < 32) {
+        // lanes 0 - 15: sums 0 and 2; lanes 16 - 31: sums 1 and 3
+        double s[4];
+#pragma unroll
+        for (int q = 0; q < (NS > 2 ? 2 : 1); ++q) {
+            const double a = join(l < blocks ? *cl.map_shared_rank(&sh.block_sum[2 * q + k], l) : 0.0);
+            s[2 * q] = __shfl_sync(ALL, a, 0);
+            s[2 * q + 1] = __shfl_sync(ALL, a, 16);
+        }
+        if (MINMAX) {
+            const int c = l < blocks ? l : 0;
+            lo = *cl.map_shared_rank(&sh.block_lo, c);
+            hi = *cl.map_shared_rank(&sh.block_hi, c);
+            join_keys();
+        }
+        double o[4] = {0.0, 0.0, 0.0, 0.0};
+        fin(s, of_order_key(lo), of_order_key(hi), o);
+        if (t == 0) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sh.out[q] = o[q];
+        }
     }
     cl.sync();  // (and no block overwrites its values before all have read them)
 #pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = s_all[k];
+    for (int q = 0; q < 4; ++q) out[q] = sh.out[q];
 }
 
 // One cluster of 1 - 16 blocks per case.  Mass is moved inside the interfaces with
 // the weight w = (rho_hat - lo)(hi - rho_hat) (zero in both bulk phases), then a
 // final scaling makes it exact; T is scaled to the initial energy.  Three
 // reductions over the case, each needing the one before, bound by the FP64 units
-// (about 30 operations per site): with one block per case 8 cases of 256^2 kept 8
-// SMs busy for 727 us; a cluster spreads a case over up to 16 SMs, which
-// exchange their sums through distributed shared memory in the same launch, and a
-// thread keeps rho_hat and T_hat of its first WARM_KEEP sites (all, up to 65,536
-// sites per case) between the passes: 86 us.
+// (18 operations per site) and, below some 4,096 sites a block, by the chain of the
+// reductions: with one block per case 8 cases of 256^2 kept 8 SMs busy for 727 us; a
+// cluster spreads a case over up to 16 SMs, which exchange their sums through
+// distributed shared memory in the same launch, and a thread keeps rho_hat, T_hat and w
+// of its first WARM_KEEP sites between the passes.  8 cases of 256^2: 46 us; 86 us with
+// clusters of 16 in two rounds, w formed in each pass and every warp joining the sums.
 __global__ void __launch_bounds__(WARM_THREADS) k_warm(WarmArgs a) {
     namespace cg = cooperative_groups;
-    __shared__ double s_warp[WARM_THREADS / 32][5];
-    __shared__ double s_block[5], s_all[5];
+    __shared__ WarmShared sh;
     cg::cluster_group cl = cg::this_cluster();
     const long long base = (long long)(blockIdx.x / cl.num_blocks()) * a.P;
     const long long first = (long long)cl.block_rank() * WARM_THREADS + threadIdx.x;
     const long long step = (long long)cl.num_blocks() * WARM_THREADS;
-    double rk[WARM_KEEP], tk[WARM_KEEP];
-    // f(i, rho_hat, T_hat) over this thread's sites
-    auto kept = [&](auto f) {
-#pragma unroll
-        for (int k = 0; k < WARM_KEEP; ++k)
-            if (first + k * step < a.P) f(base + first + k * step, rk[k], tk[k]);
-        for (long long i = first + WARM_KEEP * step; i < a.P; i += step)
-            f(base + i, warm_rho_hat(a, base + i), warm_T_hat(a, base + i));
+    // of a kept site: rho_hat (then rho1), T_hat, w
+    double rk[WARM_KEEP], tk[WARM_KEEP], wk[WARM_KEEP];
+    auto weight = [](double r, double lo, double hi) { return (r - lo) * (hi - r); };
+    // pass 1: S0 = sum rho0, S1 = sum rho_hat, E0 = sum rho0 T0, lo, hi
+    double v1[3] = {0.0, 0.0, 0.0}, out[4];
+    long long klo = order_key(INFINITY), khi = order_key(-INFINITY);
+    auto site = [&](long long i, double& r, double& t) {
+        const double r0 = a.rho0[i], t0 = a.T0[i];
+        r = warm_rho_hat(a, r0, a.pred[2 * i]);
+        t = warm_T_hat(a, t0, a.pred[2 * i + 1]);
+        v1[0] += r0;
+        v1[1] += r;
+        v1[2] += r0 * t0;
+        const long long key = order_key(r);
+        klo = min(klo, key);
+        khi = max(khi, key);
     };
+    auto again = [&](long long i, double& r, double& t) {
+        r = warm_rho_hat(a, a.rho0[i], a.pred[2 * i]);
+        t = warm_T_hat(a, a.T0[i], a.pred[2 * i + 1]);
+    };
+    const long long more = first + WARM_KEEP * step;
+    double r, t;
+#pragma unroll
+    for (int k = 0; k < WARM_KEEP; ++k)
+        if (first + k * step < a.P) site(base + first + k * step, rk[k], tk[k]);
+    for (long long i = more; i < a.P; i += step) site(base + i, r, t);
+    double S0 = 0.0, S1 = 0.0, E0 = 0.0;  // (the first warp's)
+    cluster_reduce<3, true>(v1, klo, khi, sh, out, [&](const double* s, double least, double greatest, double* o) {
+        S0 = s[0];
+        S1 = s[1];
+        E0 = s[2];
+        o[0] = least;
+        o[1] = greatest;
+    });
+    const double lo = out[0], hi = out[1];
+    // pass 2: SW = sum w
+    double v2[1] = {0.0};
 #pragma unroll
     for (int k = 0; k < WARM_KEEP; ++k)
         if (first + k * step < a.P) {
-            rk[k] = warm_rho_hat(a, base + first + k * step);
-            tk[k] = warm_T_hat(a, base + first + k * step);
+            wk[k] = weight(rk[k], lo, hi);
+            v2[0] += wk[k];
         }
-    // pass 1: S0 = sum rho0, S1 = sum rho_hat, E0 = sum rho0 T0, lo, hi
-    double v1[5] = {0.0, 0.0, 0.0, INFINITY, -INFINITY};
-    kept([&](long long i, double r, double) {
-        v1[0] += a.rho0[i];
-        v1[1] += r;
-        v1[2] += a.rho0[i] * a.T0[i];
-        v1[3] = fmin(v1[3], r);
-        v1[4] = fmax(v1[4], r);
+    for (long long i = more; i < a.P; i += step) {
+        again(base + i, r, t);
+        v2[0] += weight(r, lo, hi);
+    }
+    cluster_reduce<1, false>(v2, 0, 0, sh, out, [&](const double* s, double, double, double* o) {
+        const double l = s[0] > 0.0 ? (S0 - S1) / s[0] : 0.0;
+        const double cap = hi > lo ? 1.0 / (hi - lo) : 1.0;
+        o[0] = fmin(fmax(l, -cap), cap);
     });
-    const int op1[5] = {0, 0, 0, -1, 1};
-    cluster_reduce<5>(v1, op1, s_warp, s_block, s_all);
-    const double S0 = v1[0], S1 = v1[1], E0 = v1[2], lo = v1[3], hi = v1[4];
-    // pass 2: SW = sum w
-    double v2[1] = {0.0};
-    kept([&](long long, double r, double) { v2[0] += (r - lo) * (hi - r); });
-    const int op2[1] = {0};
-    cluster_reduce<1>(v2, op2, s_warp, s_block, s_all);
-    double lam = v2[0] > 0.0 ? (S0 - S1) / v2[0] : 0.0;
-    const double cap = hi > lo ? 1.0 / (hi - lo) : 1.0;
-    lam = fmin(fmax(lam, -cap), cap);
+    const double lam = out[0];
     // pass 3: S2 = sum rho1, Q = sum rho1 T_hat
     double v3[2] = {0.0, 0.0};
-    kept([&](long long, double r, double t) {
-        const double r1 = r + lam * (r - lo) * (hi - r);
-        v3[0] += r1;
-        v3[1] += r1 * t;
+#pragma unroll
+    for (int k = 0; k < WARM_KEEP; ++k)
+        if (first + k * step < a.P) {
+            rk[k] += lam * wk[k];
+            v3[0] += rk[k];
+            v3[1] += rk[k] * tk[k];
+        }
+    for (long long i = more; i < a.P; i += step) {
+        again(base + i, r, t);
+        r += lam * weight(r, lo, hi);
+        v3[0] += r;
+        v3[1] += r * t;
+    }
+    cluster_reduce<2, false>(v3, 0, 0, sh, out, [&](const double* s, double, double, double* o) {
+        o[0] = S0 / s[0];
+        o[1] = E0 / (o[0] * s[1]);
     });
-    const int op3[2] = {0, 0};
-    cluster_reduce<2>(v3, op3, s_warp, s_block, s_all);
-    const double fr = S0 / v3[0];
-    const double ft = E0 / (fr * v3[1]);
-    kept([&](long long i, double r, double t) {
-        a.rho[i] = (r + lam * (r - lo) * (hi - r)) * fr;
-        a.T[i] = t * ft;
-    });
+    const double fr = out[0], ft = out[1];
+#pragma unroll
+    for (int k = 0; k < WARM_KEEP; ++k)
+        if (first + k * step < a.P) {
+            a.rho[base + first + k * step] = rk[k] * fr;
+            a.T[base + first + k * step] = tk[k] * ft;
+        }
+    for (long long i = more; i < a.P; i += step) {
+        again(base + i, r, t);
+        a.rho[base + i] = (r + lam * weight(r, lo, hi)) * fr;
+        a.T[base + i] = t * ft;
+    }
 }
 
 }  // namespace unk
