@@ -220,12 +220,13 @@ void wgrad_shape(const un_net* n, const Layer& L, long long M, int* MT, int* NT,
 // channel groups, N H rows), box (64, 16, 1, 1): one box is 128 pixels of one
 // channel group of one row, a contiguous 2 KB block moved as 16 rows of 128
 // bytes.  The view's first channel group is applied in the coordinates.
-bool conv_tensor_map(const bf16* x, int xC, int W, int H, int N, CUtensorMap* map, int boxw = unk::TC_M) {
+bool conv_tensor_map(const bf16* x, int xC, int W, int H, int N, CUtensorMap* map, int boxw = unk::TC_M,
+                     int boxg = 1) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return false;
     const cuuint64_t dims[4] = {64, (cuuint64_t)(W / 8), (cuuint64_t)(xC / 8), (cuuint64_t)N * H};
     const cuuint64_t strides[3] = {128, (cuuint64_t)W * 16, (cuuint64_t)xC * W * 2};
-    const cuuint32_t box[4] = {64, (cuuint32_t)boxw / 8, 1, 1};
+    const cuuint32_t box[4] = {64, (cuuint32_t)boxw / 8, (cuuint32_t)boxg, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<bf16*>(x), dims, strides, box, estr,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -326,10 +327,11 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
     const int NBW = xm ? unk::TW_MB : unk::tw_block(L.cin);
     const int W = Wl(n, l), H = Hl(n, l);
     const int segw = unk::tw_segw(W);
+    const int ggroups = (L.cout < unk::TW_MB ? L.cout : unk::TW_MB) / 8, xgroups = (L.cin < NBW ? L.cin : NBW) / 8;
     CUtensorMap gmap, xmap;
     if ((xm || (L.cout % 64 == 0 && L.cout <= 384 && NBW)) && W % 16 == 0 && W % segw == 0 &&
-        M / segw < (1LL << 30) && conv_tensor_map(g, gC, W, H, N, &gmap, segw) &&
-        conv_tensor_map(x, xC, W, H, N, &xmap, segw)) {
+        M / segw < (1LL << 30) && conv_tensor_map(g, gC, W, H, N, &gmap, segw, ggroups) &&
+        conv_tensor_map(x, xC, W, H, N, &xmap, unk::tw_xrow(segw), xgroups)) {
         // fifth-generation tensor cores: (output block, input block, kernel row, pixel split) per CTA
         const int units = (xm ? 1 : (L.cout + unk::TW_MB - 1) / unk::TW_MB) * ((L.cin + NBW - 1) / NBW) * 3;
         const long long items = M / segw;
@@ -355,6 +357,8 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
             a.W = W;
             a.splits = splits;
             a.items_per_split = (int)per;
+            a.ggroups = ggroups;
+            a.xgroups = xgroups;
             a.part = n->wpart + n->wpart_off[k];
             a.bpart = n->bpart + n->bpart_off[k];
             a.err = n->d_err;

@@ -12,9 +12,16 @@
 // y needs exactly one input row, y + dy - 1, so a stage is
 //   g: the row segment of the output gradient, MB / 8 channel groups of segw
 //      pixels (16 bytes each): group j, pixel p -> j * segw * 16 + p * 16;
-//   x: input row y + dy - 1, NBW / 8 channel groups in the halo layout of
-//      k_conv3_tc (slots 8 .. 8 + segw - 1, the wrapped neighbours at slots
-//      7 and 8 + segw): group k, slot q -> GX + k * TC_HROW * 16 + q * 16.
+//   x: input row y + dy - 1, NBW / 8 channel groups of segw + 16 slots (slots
+//      8 .. 8 + segw - 1, the neighbours at 7 and 8 + segw): group k, slot q ->
+//      GX + (k * (segw + 16) + q) * 16.
+// Each arrives as one tensor copy of all its groups; the box of x starts 8 pixels to
+// the left, columns outside the image are filled with zeros, and the edge warp then
+// writes the wrapped neighbours over them.  (A copy per group took about 110 cycles
+// each whatever its kind, more than the MMAs of the stage: with 16 pictures of 256^2 the
+// eleven layers took 768 us so and 587 now, 96 -> 32 at level 0 168 and 118, 384 -> 128 at
+// level 2 97 and 66.  Now the reads of the operands, 24 MMAs in 1,400 - 1,600
+// cycles, and the L2 cache, which gives each row to three kernel rows, bound it.)
 // Both operands are read MN-major (8 channels of one pixel are one 16-byte
 // core-matrix row; 8 pixels of a K step are 128 contiguous bytes): A = g with
 // its channel groups segw * 16 bytes apart, B = x with tap dx's view starting
@@ -28,8 +35,8 @@
 // accumulators are D[ci][co] and the partial sums are written with TMEM lane
 // = input channel.
 //
-// Roles: warp 0 produces (elected lane: barrier byte count and the tensor
-// copies; lanes: the wrapped neighbours, arriving when they land), warp 5
+// Roles: warp 0 produces (elected lane: barrier byte count and the two tensor
+// copies), warp 6 writes the wrapped neighbours and passes the stage on, warp 5
 // issues the MMAs (warp-wide loop, elected lane), warps 1-4 sum g for the bias
 // gradient while the MMAs run (CTAs of input block 0 and dy = 1 only; their
 // arrivals release the stage together with the MMA commit) and write the
@@ -41,8 +48,8 @@
 
 namespace unk {
 
-constexpr int TW_THREADS = 192;
-constexpr int TW_MMA_WARP = 5;
+constexpr int TW_THREADS = 224;
+constexpr int TW_MMA_WARP = 5, TW_EDGE_WARP = 6;
 constexpr int TW_MB = 128;
 
 struct WgradTcArgs {
@@ -52,6 +59,7 @@ struct WgradTcArgs {
     int xC, xoff;
     int Cout, Cin, N, H, W;
     int splits, items_per_split;  // row segments per split
+    int ggroups, xgroups;         // channel groups of a stage's copies (the maps' boxes)
     float* part;                  // [splits][Cout][9][Cin]
     float* bpart;                 // [splits][Cout]
     int* err;
@@ -62,9 +70,10 @@ __host__ __device__ constexpr int tw_segw(int W) { return W < TC_M ? W : TC_M; }
 __host__ __device__ constexpr int tw_gplanes(int NA, bool XM) { return XM ? NA / 8 : TW_MB / 8; }
 __host__ __device__ constexpr int tw_xplanes(int NA, bool XM) { return XM ? TW_MB / 8 : NA / 8; }
 __host__ __device__ constexpr int tw_gbytes(int NA, bool XM, int segw) { return tw_gplanes(NA, XM) * segw * 16; }
-__host__ __device__ constexpr int tw_xbytes(int NA, bool XM) { return tw_xplanes(NA, XM) * TC_HROW * 16; }
+__host__ __device__ constexpr int tw_xrow(int segw) { return segw + 2 * TC_BODY; }  // slots of an x row
+__host__ __device__ constexpr int tw_xbytes(int NA, bool XM, int segw) { return tw_xplanes(NA, XM) * tw_xrow(segw) * 16; }
 __host__ __device__ constexpr int tw_stage_bytes(int NA, bool XM, int segw) {
-    return tw_gbytes(NA, XM, segw) + tw_xbytes(NA, XM);
+    return tw_gbytes(NA, XM, segw) + tw_xbytes(NA, XM, segw);
 }
 __host__ __device__ constexpr int tw_stages(int NA, bool XM, int segw) {
     return (int)((232448 - 1024 - 512) / tw_stage_bytes(NA, XM, segw)) > 6
@@ -94,11 +103,12 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
     const int segw = tw_segw(W);
     const int segs = W / segw;
     const int GB = tw_gbytes(NA, XM, segw);
-    const int SB = GB + tw_xbytes(NA, XM);
+    const int SB = GB + tw_xbytes(NA, XM, segw);
     uint8_t* sS = base;                                                     // [stages][SB]
     uint64_t* full = reinterpret_cast<uint64_t*>(sS + (size_t)stages * SB);  // [stages]
     uint64_t* empty = full + 6;                                             // [stages]
-    uint64_t* mdone = empty + 6;
+    uint64_t* ready = empty + 6;                                            // [stages]
+    uint64_t* mdone = ready + 6;
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(mdone + 1);
     volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
 
@@ -127,7 +137,8 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
 
     if (tid == 0) {
         for (int s = 0; s < stages; ++s) {
-            tc_bar_init(&full[s], 1 + EDGES);
+            tc_bar_init(&full[s], 1);
+            tc_bar_init(&ready[s], 1);
             tc_bar_init(&empty[s], do_bias ? 1 + 4 : 1);
         }
         tc_bar_init(mdone, 1);
@@ -149,8 +160,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
 
     if (warp == 0) {
         // ------------------------------------------------ producer
-        const int ek = lane >> 1, eside = lane & 1;  // edge: input group, side
-        const bool edge = lane < EDGES;
+        const uint32_t bytes = (uint32_t)(a.ggroups * segw + a.xgroups * tw_xrow(segw)) * 16;
         int s = 0;
         uint32_t ph = 0;
         int j = 0;
@@ -171,29 +181,20 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
             const uint32_t st = smem_addr(sS + (size_t)s * SB);
             const uint32_t fb = smem_addr(&full[s]);
             {
-                // arm with every byte of the stage's tensor copies
-                const uint32_t bytes = (uint32_t)((gvalid + xvalid) * segw * 16);
+                // arm with every byte of the stage's two copies (filled columns count)
                 asm volatile(
                     "{\n .reg .pred e;\n .reg .b32 el;\n elect.sync el|e, 0xffffffff;\n"
                     " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(fb),
                     "r"(bytes)
                     : "memory");
             }
-            for (int k = 0; k < gvalid; ++k) ts_tma(&gmap, st + k * segw * 16, fb, x0 / 8, cg0 + k, row);
-            for (int k = 0; k < xvalid; ++k)
-                ts_tma(&xmap, st + GB + (k * TC_HROW + TC_BODY) * 16, fb, x0 / 8, xg0 + k, xrow);
-            if (edge) {
-                const int xx = eside ? wrap(x0 + segw, W) : wrap(x0 - 1, W);
-                cp_async16(sS + (size_t)s * SB + GB + (ek * TC_HROW + (eside ? TC_BODY + segw : TC_BODY - 1)) * 16,
-                           a.x + act_at(xrow, xx, (xg0 + ek) * 8, a.xC, W), true);
-                tc_cp_async_arrive(&full[s]);
-            }
+            ts_tma(&gmap, st, fb, x0 / 8, cg0, row);
+            ts_tma(&xmap, st + GB, fb, x0 / 8 - 1, xg0, xrow);
             if (++s == stages) {
                 s = 0;
                 ph ^= 1u;
             }
         }
-        cp_async_wait<0>();
         if (lane == 0)
             for (int k = (j > stages ? j - stages : 0); k < j; ++k)
                 (void)tc_bar_wait(&full[k % stages], (uint32_t)((k / stages) & 1));
@@ -208,8 +209,8 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
         // stride between MN groups (8 channels)
         // g: channel groups segw * 16 bytes apart
         const uint64_t dg0 = tc_mdesc(smem_addr(sS), 128, (uint32_t)(segw * 16));
-        // x: channel groups one halo row (TC_HROW * 16 bytes) apart
-        const uint64_t dx0 = tc_mdesc(smem_addr(sS) + (uint32_t)(GB + (TC_BODY - 1) * 16), 128, TC_HROW * 16);
+        // x: channel groups one row with its halo apart
+        const uint64_t dx0 = tc_mdesc(smem_addr(sS) + (uint32_t)(GB + (TC_BODY - 1) * 16), 128, (uint32_t)(tw_xrow(segw) * 16));
         const uint64_t da0 = XM ? dx0 : dg0, db0 = XM ? dg0 : dx0;
         const uint32_t ahi = (uint32_t)(da0 >> 32), bhi = (uint32_t)(db0 >> 32);
         const int ksteps = segw / 16;
@@ -219,11 +220,10 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
         for (int i = 0; i < nitems && __shfl_sync(0xffffffffu, *s_abort, 0) == 0; ++i) {
             const uint32_t a_lo = (uint32_t)da0 + (uint32_t)s * (uint32_t)(SB >> 4);
             const uint32_t b_lo = (uint32_t)db0 + (uint32_t)s * (uint32_t)(SB >> 4);
-            if (!__all_sync(0xffffffffu, tc_bar_wait(&full[s], fph))) {
+            if (!__all_sync(0xffffffffu, tc_bar_wait(&ready[s], fph))) {
                 ok = false;
                 break;
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             for (int k = 0; k < ksteps; ++k) {
 #pragma unroll
@@ -243,9 +243,63 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
             if (a.err) atomicOr(a.err, 1 << 6);
         }
         tc_commit_one(mdone);  // arrives once every MMA issued has completed
+    } else if (warp == TW_EDGE_WARP) {
+        // ------------------------------------------------ wrapped neighbours
+        // lane: input group, side.  The values of the next EB items are in registers
+        // while those of this one go into their slots, once the copy has filled these
+        // with zeros.
+        constexpr int EB = 4;
+        const int ek = lane >> 1, eside = lane & 1;
+        auto value = [&](int i) {
+            uint4 v = make_uint4(0, 0, 0, 0);
+            const int item = it0 + i, seg = item % segs, row = item / segs;
+            if (lane < EDGES && i < nitems && seg == (eside ? segs - 1 : 0)) {
+                const int y = row % H, xrow = row - y + wrap(y + dy - 1, H);
+                v = *reinterpret_cast<const uint4*>(
+                    a.x + act_at(xrow, eside ? 0 : W - 1, (xg0 + ek) * 8, a.xC, W));
+            }
+            return v;
+        };
+        uint8_t* slot = sS + GB + (ek * tw_xrow(segw) + (eside ? TC_BODY + segw : TC_BODY - 1)) * 16;
+        uint4 cur[EB], nxt[EB];
+#pragma unroll
+        for (int t = 0; t < EB; ++t) nxt[t] = value(t);
+        int s = 0;
+        uint32_t fph = 0;
+        bool ok = true;
+        for (int i0 = 0; i0 < nitems && ok; i0 += EB) {
+#pragma unroll
+            for (int t = 0; t < EB; ++t) {
+                cur[t] = nxt[t];
+                nxt[t] = value(i0 + EB + t);
+            }
+#pragma unroll
+            for (int t = 0; t < EB; ++t) {
+                const int i = i0 + t;
+                if (i >= nitems || !ok) break;
+                if (!__all_sync(0xffffffffu, tc_bar_wait(&full[s], fph))) {
+                    ok = false;
+                    break;
+                }
+                if (lane < EDGES && (it0 + i) % segs == (eside ? segs - 1 : 0))
+                    *reinterpret_cast<uint4*>(slot + (size_t)s * SB) = cur[t];
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc_bar_arrive(&ready[s]);
+                if (++s == stages) {
+                    s = 0;
+                    fph ^= 1u;
+                }
+            }
+            if (__any_sync(0xffffffffu, *s_abort != 0)) break;
+        }
+        if (!ok && lane == 0) {
+            *s_abort = 1;
+            if (a.err) atomicOr(a.err, 1 << 6);
+        }
     } else {
         // ------------------------------------------------ warps 1-4: bias sums, then the partials
-        const int q = warp & 3;  // TMEM lanes 32 q ..; bias: g groups 4 q .. 4 q + 3
+        const int q = warp & 3;  // TMEM lanes 32 q ..; bias: g groups q, q + 4, ..
         float bs[32];
 #pragma unroll
         for (int k = 0; k < 32; ++k) bs[k] = 0.0f;
@@ -263,14 +317,22 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
                 const uint8_t* gst = sS + (size_t)s * SB;
 #pragma unroll
                 for (int jj = 0; jj < 4; ++jj) {
-                    const int k = 4 * q + jj;
-                    if (k < gvalid)
-                        for (int p = lane; p < segw; p += 32) {
-                            float f[8];
-                            unpack8(*reinterpret_cast<const uint4*>(gst + k * segw * 16 + p * 16), f);
+                    const int k = q + 4 * jj;
+                    if (k < gvalid) {
+                        uint4 u[TC_M / 32];  // (segw <= 128)
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) bs[jj * 8 + e] += f[e];
-                        }
+                        for (int r = 0; r < TC_M / 32; ++r)
+                            if (lane + 32 * r < segw)
+                                u[r] = *reinterpret_cast<const uint4*>(gst + (k * segw + lane + 32 * r) * 16);
+#pragma unroll
+                        for (int r = 0; r < TC_M / 32; ++r)
+                            if (lane + 32 * r < segw) {
+                                float f[8];
+                                unpack8(u[r], f);
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) bs[jj * 8 + e] += f[e];
+                            }
+                    }
                 }
                 __syncwarp();
                 if (lane == 0) tc_bar_arrive(&empty[s]);
@@ -285,11 +347,12 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
             for (int k = 0; k < 32; ++k)
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) bs[k] += __shfl_xor_sync(0xffffffffu, bs[k], o);
-            const int co = cob * TW_MB + 32 * q + lane;
-            if (32 * q + lane < gvalid * 8) {
+            const int k = q + 4 * (lane >> 3);
+            if (k < gvalid) {
+                const int co = cob * TW_MB + 8 * k + (lane & 7);
                 float v = 0.0f;
 #pragma unroll
-                for (int k = 0; k < 32; ++k) v = (k == lane) ? bs[k] : v;
+                for (int i = 0; i < 32; ++i) v = (i == lane) ? bs[i] : v;
                 a.bpart[(long long)split * a.Cout + co] = v;
             }
         }
