@@ -74,10 +74,10 @@ enum {
      * printed with Eq. (27).  Storage FP64 or FP32 only (else
      * LB_ERR_UNSUPPORTED).  Kernels: the whole step in one strip pass
      * (tile (256, 0) in FP32, (128, 0) in FP64; nx >= 8; the FP32 default
-     * where the strip rules hold), or the 32x8 tile front followed by one
-     * launch of both RK2 stages (any other tile_y != 0 request runs 32x8;
-     * the FP64 default); another strip width is LB_ERR_ARG.  Not available
-     * in the batched solver; lb_get/set_populations and the state calls
+     * from 393,217 sites on), or a tile front followed by one launch of both
+     * RK2 stages on tiles 32 wide, their height from the lattice (any
+     * tile_y != 0 request; the FP64 and the small-lattice default); another
+     * strip width is LB_ERR_ARG.  Not available in the batched solver; lb_get/set_populations and the state calls
      * return LB_ERR_UNSUPPORTED (there is no g). */
     LB_THERMAL_FD26 = 2,
     LB_THERMAL_FD26_PRINTED = 3
@@ -110,7 +110,7 @@ enum {
  * rule); psi at a wall node is that of the nearest fluid node; the buoyancy
  * (0, -rho g_grav) is added to the force.  The populations are then stored
  * pre-collision at their site and pushed after the collision.  Cavity
- * contexts: FP64 or FP32, the 32x8 tile kernel (tile_y == 0 is LB_ERR_ARG),
+ * contexts: FP64 or FP32, the tile kernel (tile_y == 0 is LB_ERR_ARG),
  * not in the batched solver; the finite-difference treatment as below. */
 /* CHANNEL (Sec. III A): flow between parallel plates half a spacing below
  * y = 0 and above y = ny - 1 (gap H = ny); f bounces back on the plates; g
@@ -121,7 +121,7 @@ enum {
  * with the symmetric equilibrium at u_in; the outlet (half a spacing right of
  * x = nx - 1) anti-bounces f back at density 1 with the node's velocity, and
  * copies g from column nx - 2 (zero gradient); psi outside = psi of the
- * nearest node; no gravity.  FP64 or FP32, the 32x8 tile kernel, not in the
+ * nearest node; no gravity.  FP64 or FP32, the tile kernel, not in the
  * batched solver.  With the finite-difference treatment (cavity and channel)
  * K of Eq. (26) reads ghosts outside: the temperature reflected about the
  * boundary value (2 T_b - T of the mirror node) across an isothermal
@@ -285,7 +285,9 @@ lb_status lb_halo_unpack(lb_ctx* ctx, int32_t face, const void* d_buf);
  * reports LB_ERR_TIMEOUT; the state of the step that timed out is undefined
  * (restore it with lb_load_state or lb_set_populations), the context and the
  * device stay usable.  A tiny limit makes the wait give up on purpose (tests
- * of the error path).  Applies to steps launched after the call; the tile
+ * of the error path).  Small periodic lattices created without a tile shape step
+ * on tiles or in one cluster of blocks, which do not wait on copies; while
+ * a limit other than the default is set they run the strip kernel.  Applies to steps launched after the call; the tile
  * kernels and the batched solver do not wait and ignore it.  LB_ERR_ARG for
  * cycles < 0. */
 lb_status lb_set_wait_limit(lb_ctx* ctx, int64_t cycles);
