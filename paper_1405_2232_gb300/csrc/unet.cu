@@ -333,7 +333,8 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
     const long long nw = (long long)L.cout * 9 * L.cin;
     // the swapped orientation (M = input channels) for 32 output channels
     // and at least 64 input channels; otherwise M = output channels
-    const bool xm = L.cout == 32 && L.cin >= 64 && L.cin % 32 == 0;
+    const bool rows3 = L.cout == 32 && L.cin == 32;  // three kernel rows as M
+    const bool xm = rows3 || (L.cout == 32 && L.cin >= 64 && L.cin % 32 == 0);
     const int NBW = xm ? unk::TW_MB : unk::tw_block(L.cin);
     const int W = Wl(n, l), H = Hl(n, l);
     const int segw = unk::tw_segw(W);
@@ -343,7 +344,8 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
         M / segw < (1LL << 30) && conv_tensor_map(g, gC, W, H, N, &gmap, segw, ggroups) &&
         conv_tensor_map(x, xC, W, H, N, &xmap, unk::tw_xrow(segw), xgroups)) {
         // fifth-generation tensor cores: (output block, input block, kernel row, pixel split) per CTA
-        const int units = (xm ? 1 : (L.cout + unk::TW_MB - 1) / unk::TW_MB) * ((L.cin + NBW - 1) / NBW) * 3;
+        const int units =
+            rows3 ? 1 : (xm ? 1 : (L.cout + unk::TW_MB - 1) / unk::TW_MB) * ((L.cin + NBW - 1) / NBW) * 3;
         const long long items = M / segw;
         long long S = n->sms / units;
         if (S < 1) S = 1;
@@ -376,7 +378,9 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
             const int stages = unk::tw_stages(na, xm, segw);
             const size_t smem = unk::tw_smem_bytes(na, xm, segw);
             const unsigned grid = (unsigned)(units * splits);
-            if (xm)
+            if (rows3)
+                launch(unk::k_wgrad_tc<32, true, true>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
+            else if (xm)
                 launch(unk::k_wgrad_tc<32, true>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
             else if (NBW == 128)
                 launch(unk::k_wgrad_tc<128, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
@@ -782,6 +786,8 @@ lb_status un_create(const un_config* cfg, void* stream, un_net** out) {
         e = cudaFuncSetAttribute(unk::k_wgrad_tc<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(unk::k_wgrad_tc<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(unk::k_wgrad_tc<32, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(unk::k_conv3_halo, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)unk::halo_smem_bytes());

@@ -1,6 +1,6 @@
 // unet_tcw.cuh -- weight (and bias) gradient of the 3x3 circular convolution
 // on the tcgen05 tensor cores, for layers with at least 64 output channels
-// (levels 1 .. 3 of the network):
+// (levels 1 .. 3 of the network) or 32 (level 0, XM and ROWS3 below):
 //   dW[co][tap][ci] = sum_p g[p][co] x[p + shift_tap][ci],   db[co] = sum_p g[p][co]
 // as one GEMM per tap with M = 128 output channels (a block; rows past Cout
 // are computed and dropped), N = NBW input channels (a block) and K = pixels.
@@ -34,6 +34,12 @@
 // output channels three quarters of every MMA would be empty); the
 // accumulators are D[ci][co] and the partial sums are written with TMEM lane
 // = input channel.
+//
+// With ROWS3 (32 input and 32 output channels, the full-resolution layers) the input
+// rows y - 1, y, y + 1 of a stage lie one after the other, so that A's 128 rows are
+// three kernel rows of 32 input channels (96 used) and one pass over the pixels
+// takes all nine taps: the three layers of 16 x 256^2 took 86 us each on the mma.sync kernel,
+// the training step 2,464 us with them and 2,319 so.
 //
 // Roles: warp 0 produces (elected lane: barrier byte count and the two tensor
 // copies), warp 6 writes the wrapped neighbours and passes the stage on, warp 5
@@ -88,7 +94,7 @@ __host__ __device__ constexpr int tw_block(int Cin) {
     return Cin % 128 == 0 ? 128 : (Cin % 64 == 0 ? 64 : (Cin % 32 == 0 ? 32 : 0));
 }
 
-template <int NA, bool XM>
+template <int NA, bool XM, bool ROWS3 = false>
 __global__ void __launch_bounds__(TW_THREADS, 1)
     k_wgrad_tc(WgradTcArgs a, const __grid_constant__ CUtensorMap gmap, const __grid_constant__ CUtensorMap xmap,
                int stages) {
@@ -96,7 +102,8 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
     constexpr int NBW = XM ? TW_MB : NA;            // input channels of a block
     constexpr int XG = tw_xplanes(NA, XM);          // input channel groups staged
     constexpr uint32_t COLS = 3 * NA <= 128 ? 128u : (3 * NA <= 256 ? 256u : 512u);
-    static_assert(2 * XG <= 32, "one edge copy per producer lane");
+    static_assert(2 * XG <= 32, "one edge value per lane");
+    static_assert(!ROWS3 || XM, "the rows stack along the 128 rows of A");
     extern __shared__ __align__(1024) uint8_t tw_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tw_raw) + 1023) & ~uintptr_t(1023));
     const int H = a.H, W = a.W;
@@ -116,23 +123,24 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
     // unit: output block, input block, dy, split (split outermost: the CTAs
     // working on the same pixels run together)
     const int ncob = XM ? 1 : (a.Cout + TW_MB - 1) / TW_MB;
-    const int ncib = (a.Cin + NBW - 1) / NBW;
+    const int ncib = ROWS3 ? 1 : (a.Cin + NBW - 1) / NBW;
     int u = blockIdx.x;
     const int cob = u % ncob;
     u /= ncob;
     const int cib = u % ncib;
     u /= ncib;
-    const int dy = u % 3;
-    const int split = u / 3;
+    const int dy = ROWS3 ? 0 : u % 3;
+    const int split = ROWS3 ? u : u / 3;
     const int items = a.N * H * segs;
     const int it0 = split * a.items_per_split;
     const int it1 = min(it0 + a.items_per_split, items);
     const int nitems = it1 > it0 ? it1 - it0 : 0;
-    const bool do_bias = cib == 0 && dy == 1;
+    const bool do_bias = ROWS3 || (cib == 0 && dy == 1);
     const int cg0 = (a.goff + cob * TW_MB) / 8;         // first g channel group of the block
     const int gvalid = XM ? a.Cout / 8 : min(TW_MB, a.Cout - cob * TW_MB) / 8;  // g groups that exist
     const int xg0 = (a.xoff + cib * NBW) / 8;
-    const int xvalid = min(NBW, a.Cin - cib * NBW) / 8;  // x groups that exist
+    // x groups that exist (ROWS3: those of the three rows, one after the other)
+    const int xvalid = ROWS3 ? 3 * a.xgroups : min(NBW, a.Cin - cib * NBW) / 8;
     const int EDGES = 2 * xvalid;                        // wrapped neighbours per stage
 
     if (tid == 0) {
@@ -160,7 +168,7 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
 
     if (warp == 0) {
         // ------------------------------------------------ producer
-        const uint32_t bytes = (uint32_t)(a.ggroups * segw + a.xgroups * tw_xrow(segw)) * 16;
+        const uint32_t bytes = (uint32_t)(a.ggroups * segw + (ROWS3 ? 3 : 1) * a.xgroups * tw_xrow(segw)) * 16;
         int s = 0;
         uint32_t ph = 0;
         int j = 0;
@@ -169,7 +177,6 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
             const int seg = item % segs;
             const int row = item / segs;  // n H + y
             const int y = row % H, n = row / H;
-            const int xrow = n * H + wrap(y + dy - 1, H);
             const int x0 = seg * segw;
             if (j >= stages && !__all_sync(0xffffffffu, tc_bar_wait(&empty[s], ph ^ 1u))) {
                 if (lane == 0) {
@@ -189,7 +196,10 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
                     : "memory");
             }
             ts_tma(&gmap, st, fb, x0 / 8, cg0, row);
-            ts_tma(&xmap, st + GB, fb, x0 / 8 - 1, xg0, xrow);
+#pragma unroll
+            for (int r = 0; r < (ROWS3 ? 3 : 1); ++r)
+                ts_tma(&xmap, st + GB + r * a.xgroups * tw_xrow(segw) * 16, fb, x0 / 8 - 1, xg0,
+                       n * H + wrap(y + dy + r - 1, H));
             if (++s == stages) {
                 s = 0;
                 ph ^= 1u;
@@ -254,9 +264,10 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
             uint4 v = make_uint4(0, 0, 0, 0);
             const int item = it0 + i, seg = item % segs, row = item / segs;
             if (lane < EDGES && i < nitems && seg == (eside ? segs - 1 : 0)) {
-                const int y = row % H, xrow = row - y + wrap(y + dy - 1, H);
+                const int r = ROWS3 ? ek / a.xgroups : 0;
+                const int y = row % H, xrow = row - y + wrap(y + dy + r - 1, H);
                 v = *reinterpret_cast<const uint4*>(
-                    a.x + act_at(xrow, eside ? 0 : W - 1, (xg0 + ek) * 8, a.xC, W));
+                    a.x + act_at(xrow, eside ? 0 : W - 1, (xg0 + ek - r * a.xgroups) * 8, a.xC, W));
             }
             return v;
         };
@@ -364,11 +375,12 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
         const int col = 32 * q + lane;
         const int co = cob * TW_MB + col;
         const bool valid = col < (XM ? xvalid : gvalid) * 8 && nitems > 0 && done;
-        float* out = XM ? a.part + (long long)split * a.Cout * 9 * a.Cin + cib * NBW + col
+        const int r = ROWS3 ? col / a.Cin : 0;  // kernel row of this lane
+        float* out = XM ? a.part + (long long)split * a.Cout * 9 * a.Cin + cib * NBW + (col - r * a.Cin)
                         : a.part + ((long long)split * a.Cout + co) * 9 * a.Cin;
 #pragma unroll 1
         for (int dx = 0; dx < 3; ++dx) {
-            const int tap = dy * 3 + dx;
+            const int tap = (dy + r) * 3 + dx;
 #pragma unroll 1
             for (int cc = 0; cc < NA; cc += 32) {
                 uint32_t v[32];
