@@ -77,8 +77,9 @@ enum {
      * from 393,217 sites on), or a tile front followed by one launch of both
      * RK2 stages on tiles 32 wide, their height from the lattice (any
      * tile_y != 0 request; the FP64 and the small-lattice default); another
-     * strip width is LB_ERR_ARG.  Not available in the batched solver; lb_get/set_populations and the state calls
-     * return LB_ERR_UNSUPPORTED (there is no g). */
+     * strip width is LB_ERR_ARG.  Not available in the batched solver;
+     * lb_get/set_populations and the state calls return LB_ERR_UNSUPPORTED
+     * (there is no g). */
     LB_THERMAL_FD26 = 2,
     LB_THERMAL_FD26_PRINTED = 3
 };
