@@ -3,7 +3,8 @@
 //
 // Both kernels have the structure of lb_step_tile.cuh: tiles of 32 columns and a height
 // that balances them over the SMs, one site per thread, the ring around the tile in
-// threads of its own, launched before the kernel ahead of them ends.
+// threads of its own, launched before the kernel ahead of them ends (whose outputs they
+// read, so these are not __restrict__: see k_step_tile).
 //  k_fd_front: rho (pulled f), T and psi of the tile and a ring of one site; force,
 //   u and the f collision of the tile.  STEP stores f and writes rho^n, u^n; else the
 //   moments outputs.
@@ -46,8 +47,8 @@ __device__ __forceinline__ real fd_ghost(const KParams& kp, int rx, int ry, real
 
 template <int PREC, int BMODE, bool STEP>
 __global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
-    k_fd_front(const typename Store<PREC>::elem* __restrict__ src, typename Store<PREC>::elem* __restrict__ dst,
-               const typename Store<PREC>::real* __restrict__ Tf, typename Store<PREC>::real* __restrict__ rho_n,
+    k_fd_front(const typename Store<PREC>::elem* src, typename Store<PREC>::elem* __restrict__ dst,
+               const typename Store<PREC>::real* Tf, typename Store<PREC>::real* __restrict__ rho_n,
                typename Store<PREC>::real* __restrict__ ux_n, typename Store<PREC>::real* __restrict__ uy_n,
                double* __restrict__ m_rho, double* __restrict__ m_ux, double* __restrict__ m_uy,
                double* __restrict__ m_T, const KParams kp, int by) {
@@ -154,8 +155,8 @@ __host__ __device__ constexpr size_t fd_rk2_smem_bytes(int by) {
 // reads the ghost of fd_ghost; rho and u the mirror node's.
 template <typename real>
 __global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
-    k_fd_rk2(const real* __restrict__ T, const real* __restrict__ rho, const real* __restrict__ ux,
-             const real* __restrict__ uy, real* __restrict__ T_next, const KParams kp, real chi, real a, int by) {
+    k_fd_rk2(const real* T, const real* rho, const real* ux, const real* uy,
+             real* __restrict__ T_next, const KParams kp, real chi, real a, int by) {
     constexpr int BX = 32, W2 = BX + 4, W1 = BX + 2;
     extern __shared__ __align__(16) unsigned char tile_smem[];
     real* sT = reinterpret_cast<real*>(tile_smem);  // [by + 4][W2]

@@ -246,10 +246,11 @@ __device__ __forceinline__ void tile_step(const typename Store<PREC>::elem* src,
 // One step per launch; grid (tiles in x, tiles in y), tile_threads(BX, by)
 // threads.  Launched so that its blocks may become resident while the step before
 // it still runs (programmatic dependent launch); they wait for its end before
-// they read anything.
+// they read anything.  So src is not __restrict__: that would say that nobody writes it
+// while the kernel runs, and let a load move above the wait.
 template <int PREC, int BX, int WALLS, bool EQ24, int BMODE>
 __global__ void __launch_bounds__(tile_threads(BX, tile_max_by(BX)))
-    k_step_tile(const typename Store<PREC>::elem* __restrict__ src, typename Store<PREC>::elem* __restrict__ dst,
+    k_step_tile(const typename Store<PREC>::elem* src, typename Store<PREC>::elem* __restrict__ dst,
                 const KParams kp, int by) {
     using real = typename Store<PREC>::real;
     extern __shared__ __align__(16) unsigned char tile_smem[];
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(tile_threads(BX, tile_max_by(BX)))
 // lb_batch_device.cuh re-reads less and takes over for large batches.)
 template <int PREC, bool EQ24, int BMODE>
 __global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
-    k_batch_tile(const typename Store<PREC>::elem* __restrict__ src, typename Store<PREC>::elem* __restrict__ dst,
+    k_batch_tile(const typename Store<PREC>::elem* src, typename Store<PREC>::elem* __restrict__ dst,
                  const BatchDomain* __restrict__ doms, const BatchStepTile* __restrict__ tiles,
                  const int* __restrict__ n_tiles, int by) {
     using real = typename Store<PREC>::real;

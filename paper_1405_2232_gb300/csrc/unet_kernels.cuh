@@ -32,6 +32,9 @@ namespace unk {
 // grid_launch: the next kernel's blocks may become resident; in a kernel that
 // allocates TMEM only once it holds it, since a waiting block of the next kernel
 // could otherwise hold the columns that this one needs to finish.
+// Inputs are not const __restrict__ and not read with __ldg: both say that nobody writes
+// them while the kernel runs, which the kernel ahead may do, and let a load move above
+// the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_begin() {
@@ -715,7 +718,7 @@ __global__ void __launch_bounds__(256) k_sum_splits(const __grid_constant__ SumJ
 // ------------------------------------------------------ element-wise parts
 // network input: 3 float32 planes [P][3] (pixel-major) -> BF16, 32 channels
 // (zero padded); one thread per (row, channel group, x), x fastest
-__global__ void k_input(const float* __restrict__ in, long long rows, int W, bf16* __restrict__ x0) {
+__global__ void k_input(const float* in, long long rows, int W, bf16* __restrict__ x0) {
     grid_begin();
     const long long total = rows * 4 * W;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
@@ -733,7 +736,7 @@ __global__ void k_input(const float* __restrict__ in, long long rows, int W, bf1
 
 // 2x2 average pool of a view (H, W: input size) into a dense tensor of
 // N x H/2 x W/2 pixels and C channels; one thread per output (row, group, x)
-__global__ void k_pool(const bf16* __restrict__ s, int sC, int soff, int C, int N, int H, int W,
+__global__ void k_pool(const bf16* s, int sC, int soff, int C, int N, int H, int W,
                        bf16* __restrict__ out) {
     grid_begin();
     const int C8 = C / 8, H2 = H / 2, W2 = W / 2;
@@ -761,7 +764,7 @@ __global__ void k_pool(const bf16* __restrict__ s, int sC, int soff, int C, int 
 
 // gradient through nearest upsampling: out (coarse, dense, C channels) at
 // (y, x) = (sum of the 2x2 fine block of g) * (mask at fine (2y, 2x) > 0)
-__global__ void k_up_bwd(const bf16* __restrict__ g, int gC, int goff, const bf16* __restrict__ mask, int mC,
+__global__ void k_up_bwd(const bf16* g, int gC, int goff, const bf16* mask, int mC,
                          int moff, int C, int N, int H, int W, bf16* __restrict__ out) {
     grid_begin();
     const int C8 = C / 8, H2 = H / 2, W2 = W / 2;
@@ -791,8 +794,8 @@ __global__ void k_up_bwd(const bf16* __restrict__ g, int gC, int goff, const bf1
 
 // skip gradient: out (fine, dense, C channels) at p =
 // (gp[parent(p)] / 4 + gcat[p]) * (s[p] > 0), gp coarse dense with C channels
-__global__ void k_skip_bwd(const bf16* __restrict__ gp, const bf16* __restrict__ gcat, int gC, int goff,
-                           const bf16* __restrict__ s, int sC, int soff, int C, int N, int H, int W,
+__global__ void k_skip_bwd(const bf16* gp, const bf16* gcat, int gC, int goff,
+                           const bf16* s, int sC, int soff, int C, int N, int H, int W,
                            bf16* __restrict__ out) {
     grid_begin();
     const int C8 = C / 8;
@@ -815,8 +818,8 @@ __global__ void k_skip_bwd(const bf16* __restrict__ gp, const bf16* __restrict__
 // ------------------------------------------------------------------ head
 // y[p][j] = sum_c Wh[j][c] h[p][c] + bh[j], j = 0, 1 (FP32 weights)
 template <int C>
-__global__ void k_head_fwd(const bf16* __restrict__ h, const float* __restrict__ Wh, const float* __restrict__ bh,
-                           long long P, int W, float* __restrict__ y) {
+__global__ void k_head_fwd(const bf16* h, const float* Wh, const float* bh, long long P, int W,
+                           float* __restrict__ y) {
     grid_begin();
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P; p += (long long)gridDim.x * blockDim.x) {
         float y0 = bh[0], y1 = bh[1];
@@ -841,8 +844,7 @@ __global__ void k_head_fwd(const bf16* __restrict__ h, const float* __restrict__
 // block.  gh[p][c] = (sum_j gy_j Wh[j][c]) * (h > 0), gy = 2 (y - t) / count.
 // Per-block partials: pw[block][2C + 2] (dWh then dbh), pl[block] (sum of squares).
 template <int C>
-__global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, const float* __restrict__ Wh,
-                                                   const float* __restrict__ bh, const float* __restrict__ tgt,
+__global__ void __launch_bounds__(256) k_head_bwd(const bf16* h, const float* Wh, const float* bh, const float* tgt,
                                                    long long P, int W, int rows_per_block, float inv_count2,
                                                    bf16* __restrict__ gh, float* __restrict__ pw,
                                                    double* __restrict__ pl) {
@@ -918,7 +920,7 @@ __global__ void __launch_bounds__(256) k_head_bwd(const bf16* __restrict__ h, co
 }
 
 // *out = sum of n doubles: strided per-thread sums, fixed-order tree (one block of 256)
-__global__ void __launch_bounds__(256) k_sum_doubles(const double* __restrict__ part, int n, double* __restrict__ out) {
+__global__ void __launch_bounds__(256) k_sum_doubles(const double* part, int n, double* __restrict__ out) {
     grid_begin();
     __shared__ double red[256];
     double s = 0.0;

@@ -431,7 +431,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (a.mask)
 #pragma unroll
                 for (int kk = 0; kk < N / 8; ++kk)
-                    mraw[kk] = __ldg(reinterpret_cast<const uint4*>(a.mask + act_at(row, x, a.moff + 8 * kk, a.mC, W)));
+                    mraw[kk] = *reinterpret_cast<const uint4*>(a.mask + act_at(row, x, a.moff + 8 * kk, a.mC, W));
             // one decision per warp (the TMEM loads below are warp-wide)
             if (!__all_sync(0xffffffffu, tc_bar_wait(&accf[b], rnd))) {
                 *s_abort = 1;

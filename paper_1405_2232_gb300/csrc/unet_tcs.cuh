@@ -98,7 +98,7 @@ __device__ __forceinline__ void ts_tma(const CUtensorMap* map, uint32_t dst, uin
 
 template <int NB>
 __global__ void __launch_bounds__(TS_THREADS, 1)
-    k_conv3_tcs(ConvArgs a, const __grid_constant__ CUtensorMap xmap, const bf16* __restrict__ wimg) {
+    k_conv3_tcs(ConvArgs a, const __grid_constant__ CUtensorMap xmap, const bf16* wimg) {
     constexpr int R = ts_rows(NB);
     constexpr int GSTR = ts_gstr(R);
     constexpr int ABYTES = ts_abytes(R);
@@ -309,8 +309,8 @@ __global__ void __launch_bounds__(TS_THREADS, 1)
                         if (a.mask && live)
 #pragma unroll
                             for (int k = 0; k < 4; ++k)
-                                mraw[k] = __ldg(reinterpret_cast<const uint4*>(
-                                    a.mask + act_at(row, x, a.moff + co0 + cc + 8 * k, a.mC, W)));
+                                mraw[k] = *reinterpret_cast<const uint4*>(
+                                    a.mask + act_at(row, x, a.moff + co0 + cc + 8 * k, a.mC, W));
                         uint32_t v[32];
                         const uint32_t taddr =
                             tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(grp * R * NB + r * NB + cc);
