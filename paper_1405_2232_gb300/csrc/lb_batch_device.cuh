@@ -346,9 +346,7 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
 //
 // Bound by the FP64 units (a warp instruction per 16 cycles of an SM, conversions
 // from FP32 included).  So in FP32 the nine populations of a site are summed as a
-// float and its accumulated rounding errors (the two-sum of Knuth: the float is
-// the step's rho, and both together are the exact sum that nine FP64 additions
-// gave), floats are widened on the integer units, and a thread sums its eight sites
+// float and its rounding errors (sum9: the float is the step's rho), floats are widened on the integer units, and a thread sums its eight sites
 // before the block reduction: about 12 FP64 operations per site instead of 75.  28
 // domains of 3.3 million sites: 104 us, 475 us before.
 struct BatchTile {
@@ -379,25 +377,11 @@ __global__ void __launch_bounds__(256)
         const int y = s / kp.nx, x = s - y * kp.nx;
         real f[9], g[9];
         pull18<S>(src_base + D.off, kp, x, y, f, g);
-        real rho = f[0], e = g[0], rho_err = (real)0, e_err = (real)0;
-#pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            if constexpr (sizeof(real) == 4) {
-                add_exact(rho, f[i], rho_err);
-                add_exact(e, g[i], e_err);
-            } else {
-                rho += f[i];
-                e += g[i];
-            }
-        }
+        real rho, e;
+        v[0] += sum9(f, rho);
+        v[1] += sum9(g, e);
         const double r = widen(rho), T = widen(e / (rho * cv));
         const long long fo = D.fld_off + s;
-        v[0] += r;
-        v[1] += widen(e);
-        if constexpr (sizeof(real) == 4) {
-            v[0] += widen(rho_err);
-            v[1] += widen(e_err);
-        }
         if (have_ref) {
             const double a = r - ref_rho[fo], c = T - ref_T[fo];
             v[2] = fma(a, a, v[2]);

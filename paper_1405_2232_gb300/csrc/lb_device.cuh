@@ -341,11 +341,33 @@ __device__ __forceinline__ double widen(float x) {
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 
-// s += x, the rounding error of the addition added to err
-__device__ __forceinline__ void add_exact(float& s, float x, float& err) {
-    const float t = s + x, d = t - s;
-    err += (s - (t - d)) + (x - d);
-    s = t;
+// a += x; returns the rounding error of the addition, exactly (the two-sum of Knuth)
+__device__ __forceinline__ float two_sum(float& a, float x) {
+    const float t = a + x, d = t - a, err = (a - (t - d)) + (x - d);
+    a = t;
+    return err;
+}
+
+// s: the sum of nine populations in index order, the step's float.  Returns the same
+// sum in FP64: s and its rounding errors, which one float holds exactly for the
+// populations of a smooth state; where it does not (populations of very different
+// magnitude, infinities, NaN), the nine FP64 additions.
+__device__ __forceinline__ double sum9(const float v[9], float& s) {
+    float err = 0.0f, lost = 0.0f;
+    s = v[0];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) lost += fabsf(two_sum(err, two_sum(s, v[i])));
+    if (lost == 0.0f) return widen(s) + widen(err);
+    double m = (double)v[0];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) m += (double)v[i];
+    return m;
+}
+__device__ __forceinline__ double sum9(const double v[9], double& s) {
+    s = v[0];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) s += v[i];
+    return s;
 }
 
 template <typename real>

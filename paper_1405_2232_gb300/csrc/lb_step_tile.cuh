@@ -358,20 +358,9 @@ __global__ void __launch_bounds__(tile_threads(32, 8))
             my = (f[2] - f[4]) + ((f[5] - f[7]) + (f[6] - f[8]));
         }
         if constexpr (PART) {
-            if constexpr (sizeof(real) == 8) {
-                m = rho;
-                en = e;
-            } else {
-                // rho and e with their rounding errors: the exact sums
-                float r = f[0], q = g[0], r_err = 0.0f, q_err = 0.0f;
-#pragma unroll
-                for (int i = 1; i < 9; ++i) {
-                    add_exact(r, f[i], r_err);
-                    add_exact(q, g[i], q_err);
-                }
-                m = widen(r) + widen(r_err);
-                en = widen(q) + widen(q_err);
-            }
+            real s;
+            m = sum9(f, s);
+            en = sum9(g, s);
         }
     }
     if (flags) atomicOr(kp.err, flags);
