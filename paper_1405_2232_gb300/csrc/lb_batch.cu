@@ -92,7 +92,7 @@ struct lb_batch {
     int tile_by = 0;
     bool strip_asked = false;     // the caller set a chunk height: the strip kernel
     int n_step_tiles = 0;
-    int cap_step_tiles = 0;
+    int max_step_tiles = 0;
     BatchStepTile* d_step_tiles = nullptr;
     int* d_next = nullptr;        // takes from the work counter in the current step (the step resets it)
     int max_items = 0;
@@ -171,15 +171,18 @@ cudaError_t launch_batch_check(lb_batch* b) {
     return cudaGetLastError();
 }
 
-// Height of the tiles the active domains step in (0: the strip kernel): up to 1.5 x
-// 2^20 sites in FP32 (12 domains of 174,000 sites 84 -> 7.6 us per step, a lone 64^2 68
-// -> 2.8 us; 2.1 million sites in 128 domains 84 us on strips against 90), 2^20 in FP64.
+// Most active sites that step on tiles: 1.5 x 2^20 in FP32 (12 domains of 174,000 sites
+// 84 -> 7.6 us per step, a lone 64^2 68 -> 2.8 us; 2.1 million sites in 128 domains 84 us
+// on strips against 90), 2^20 in FP64.
+long long tile_sites(int prec) { return prec == LB_PREC_FP32 ? 3LL << 19 : (1LL << 20) - 1; }
+
+// Height of the tiles the active domains step in (0: the strip kernel).
 int batch_tile_rows(const lb_batch* b) {
     if (b->strip_asked) return 0;
     long long sites = 0;
     for (int d = 0; d < b->n; ++d)
         if (b->frozen[d] < 0) sites += (long long)b->params[d].nx * b->params[d].ny;
-    if (sites > (b->prec == LB_PREC_FP32 ? 3LL << 19 : (1LL << 20) - 1)) return 0;
+    if (sites > tile_sites(b->prec)) return 0;
     return balanced_tile_rows(b->prec, b->sms, 1, [&](int by) {
         long long t = 0;
         for (int d = 0; d < b->n; ++d)
@@ -232,7 +235,27 @@ int chunk_rows_used(const lb_batch* b) {
     return best;
 }
 
-// Rebuild the step work list and the check tile list from the active set.
+// Most tiles that active domains with at most tile_sites sites can have, tiles of one
+// row included: the domains with the most tiles per site first, until their sites pass it.
+long long most_step_tiles(int prec, const std::vector<lb_params>& params) {
+    auto per_row = [](const lb_params& p) { return (long long)((p.nx + 31) / 32); };
+    std::vector<const lb_params*> order;
+    for (const lb_params& p : params)
+        if ((long long)p.nx * p.ny <= tile_sites(prec)) order.push_back(&p);
+    std::sort(order.begin(), order.end(),
+              [&](const lb_params* p, const lb_params* q) { return per_row(*p) * q->nx > per_row(*q) * p->nx; });
+    long long sites = 0, tiles = 0;
+    for (const lb_params* p : order) {
+        if (sites > tile_sites(prec)) break;
+        sites += (long long)p->nx * p->ny;
+        tiles += per_row(*p) * p->ny;
+    }
+    return tiles;
+}
+
+// Rebuild the step work list and the check tile list from the active set.  (Into the
+// lists allocated at the start: a failed allocation here would leave the batch with
+// a list that is not there.)
 lb_status rebuild_lists(lb_batch* b) {
     std::vector<BatchStepTile> step_tiles;
     b->tile_by = batch_tile_rows(b);
@@ -241,18 +264,11 @@ lb_status rebuild_lists(lb_batch* b) {
         for (int y = 0; y < b->params[d].ny; y += b->tile_by)
             for (int x = 0; x < b->params[d].nx; x += 32) step_tiles.push_back(BatchStepTile{d, x, y, 0});
     }
-    b->n_step_tiles = (int)step_tiles.size();
-    if (b->n_step_tiles > b->cap_step_tiles) {
-        if (b->graph) {  // it holds the list's address
-            cudaGraphExecDestroy(b->graph);
-            b->graph = nullptr;
-        }
-        cudaFree(b->d_step_tiles);
-        b->d_step_tiles = nullptr;
-        b->cap_step_tiles = 0;
-        BCU(cudaMalloc(&b->d_step_tiles, sizeof(BatchStepTile) * step_tiles.size()), "step tile list");
-        b->cap_step_tiles = b->n_step_tiles;
+    if ((long long)step_tiles.size() > b->max_step_tiles) {  // (never: most_step_tiles)
+        step_tiles.clear();
+        b->tile_by = 0;
     }
+    b->n_step_tiles = (int)step_tiles.size();
     if (b->graph && (b->graph_by != b->tile_by || b->n_step_tiles > b->graph_grid ||
                      (b->tile_by && 4 * b->n_step_tiles < b->graph_grid))) {
         cudaGraphExecDestroy(b->graph);  // another kernel, or a grid too small or mostly idle
@@ -467,6 +483,7 @@ lb_status lb_batch_init(const lb_params* params, int32_t n, const double* const*
     b->buf_bytes = (size_t)off * es;
     b->max_items = max_items;
     b->max_tiles = max_tiles;
+    b->max_step_tiles = (int)most_step_tiles(prec, b->params);
     if (e == cudaSuccess) e = cudaMalloc(&b->buf[0], b->buf_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&b->buf[1], b->buf_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_err, sizeof(int) * n);
@@ -476,6 +493,7 @@ lb_status lb_batch_init(const lb_params* params, int32_t n, const double* const*
     if (e == cudaSuccess) e = cudaMalloc(&b->d_next, sizeof(int) * 2);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_next, 0, sizeof(int) * 2, b->stream);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tiles, sizeof(BatchTile) * (max_tiles > 0 ? max_tiles : 1));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_step_tiles, sizeof(BatchStepTile) * (b->max_step_tiles > 0 ? b->max_step_tiles : 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tile_begin, sizeof(int) * (n + 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_part, sizeof(double) * 6 * (max_tiles > 0 ? max_tiles : 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_out6, sizeof(double) * 6 * n);
