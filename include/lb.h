@@ -390,16 +390,25 @@ lb_status lb_batch_free(lb_batch* b);
  * the height in 16 .. 64 that balances the active domains on the others.
  * lb_batch_set_chunk_rows runs the strip kernel at that height (rebuilds the lists,
  * synchronises); LB_ERR_ARG for rows < 16.  lb_batch_chunk_rows returns the height
- * set or tuned (64 before; -1 for NULL).
+ * set or tuned (64 before; -1 for NULL), lb_batch_tile_rows the height of the tiles of
+ * the next step (0: the strip kernel; -1 for NULL).
  * lb_batch_autotune times `steps` batched steps (after 2 warm-up steps) for
  * each of the LB_BATCH_TUNE_N heights 16, 32, 64, 128, keeps the fastest (or the
  * tile kernel, where the library would run it and it is faster still) and
  * writes it to *chunk_rows (may be NULL); ms_per_step[k] (may be NULL) gets
  * each height's time per step.  The batch state, its time and its error
  * words are restored afterwards, bit for bit (one temporary device copy of
- * the state is allocated and freed).  Synchronises. */
+ * the state is allocated and freed).  A tuning that chose the strip kernel holds while at
+ * least half of the sites that were active then still are; after that the library
+ * chooses for the active domains, as without a tuning.  Synchronises.
+ * lb_batch_apply_tuning gives the batch the outcome of such a tuning of the active
+ * domains without timing anything: the height and, from lb_batch_tile_rows after the
+ * tuning, whether the tile kernel was the faster (tiles 1) or not (0).  Synchronises.
+ * LB_ERR_ARG for rows < 16 or another value of tiles. */
 lb_status lb_batch_set_chunk_rows(lb_batch* b, int32_t rows);
 int32_t lb_batch_chunk_rows(const lb_batch* b);
+int32_t lb_batch_tile_rows(const lb_batch* b);
+lb_status lb_batch_apply_tuning(lb_batch* b, int32_t rows, int32_t tiles);
 lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
                             double ms_per_step[LB_BATCH_TUNE_N]);
 

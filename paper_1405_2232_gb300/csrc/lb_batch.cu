@@ -38,6 +38,7 @@ constexpr int BATCH_BX_FP64 = 128;
 // row-chunk heights the autotuner tries; the work list is sized for the smallest
 constexpr int kChunkCand[LB_BATCH_TUNE_N] = {16, 32, 64, 128};
 constexpr int MIN_CHUNK_ROWS = 16;
+constexpr int DEFAULT_CHUNK_ROWS = 64;
 
 lb_status err(lb_status st, const char* fmt, ...) __attribute__((format(printf, 2, 3)));
 lb_status err(lb_status st, const char* fmt, ...) {
@@ -70,7 +71,7 @@ struct lb_batch {
     int eq24 = 1;
     int bmode = BETA_ONE;
     int bx = BATCH_BX_FP32;
-    int chunk_rows = 64;
+    int chunk_rows = DEFAULT_CHUNK_ROWS;  // the height set or tuned
     int device = 0;
     int sms = 152;
     cudaStream_t stream = nullptr;
@@ -91,6 +92,8 @@ struct lb_batch {
     // tile step (tile_by > 0): its tiles instead of the strip kernel's items
     int tile_by = 0;
     bool strip_asked = false;     // the caller set a chunk height: the strip kernel
+    bool strip_tuned = false;     // a tuning found the strip kernel at chunk_rows the fastest ...
+    long long tuned_sites = 0;    // ... with this many active sites
     int n_step_tiles = 0;
     int max_step_tiles = 0;
     BatchStepTile* d_step_tiles = nullptr;
@@ -176,13 +179,24 @@ cudaError_t launch_batch_check(lb_batch* b) {
 // on strips against 90), 2^20 in FP64.
 long long tile_sites(int prec) { return prec == LB_PREC_FP32 ? 3LL << 19 : (1LL << 20) - 1; }
 
-// Height of the tiles the active domains step in (0: the strip kernel).
-int batch_tile_rows(const lb_batch* b) {
-    if (b->strip_asked) return 0;
+long long active_sites(const lb_batch* b) {
     long long sites = 0;
     for (int d = 0; d < b->n; ++d)
         if (b->frozen[d] < 0) sites += (long long)b->params[d].nx * b->params[d].ny;
-    if (sites > tile_sites(b->prec)) return 0;
+    return sites;
+}
+
+// The strip kernel at chunk_rows, whatever the active set: the caller set the height, or a
+// tuning chose it and at least half of the sites that it was measured on are still
+// active (what is fastest depends on them: the last domains of a sweep take 84 us per step
+// on strips and 7.6 on tiles).
+bool strip_fixed(const lb_batch* b) {
+    return b->strip_asked || (b->strip_tuned && 2 * active_sites(b) >= b->tuned_sites);
+}
+
+// Height of the tiles the active domains step in (0: the strip kernel).
+int batch_tile_rows(const lb_batch* b) {
+    if (strip_fixed(b) || active_sites(b) > tile_sites(b->prec)) return 0;
     return balanced_tile_rows(b->prec, b->sms, 1, [&](int by) {
         long long t = 0;
         for (int d = 0; d < b->n; ++d)
@@ -201,17 +215,17 @@ long long item_cost(const lb_batch* b, int nx, int strip, int y0, int y1, int ha
     return (long long)(y1 - y0 + 2) * (w + 64);
 }
 
-// Height of the strip kernel's row chunks: the caller's, or with none asked the one
-// in 16 .. chunk_rows whose items finish first by their cost, where the tallest gives
+// Height of the strip kernel's row chunks: the caller's or the tuned one, else the one
+// in 16 .. 64 whose items finish first by their cost, where the tallest gives
 // the persistent CTAs fewer than four items each (n items of mean m and longest c on G
 // CTAs: the lesser of ceil(n/G) c and sum/G + m/2).  28 domains of 3.3 million sites:
 // 64 rows 123 us per step, 16 rows 110; 128 domains of 128^2: 84 and 90.
 int chunk_rows_used(const lb_batch* b) {
-    if (b->strip_asked) return b->chunk_rows;
+    if (strip_fixed(b)) return b->chunk_rows;
     const double G = 2.0 * b->sms;
-    int best = b->chunk_rows;
+    int best = DEFAULT_CHUNK_ROWS;
     double best_cost = 0.0;
-    for (int rows = b->chunk_rows; rows >= MIN_CHUNK_ROWS; rows -= MIN_CHUNK_ROWS / 2) {
+    for (int rows = DEFAULT_CHUNK_ROWS; rows >= MIN_CHUNK_ROWS; rows -= MIN_CHUNK_ROWS / 2) {
         double sum = 0.0, longest = 0.0, n = 0.0;
         for (int d = 0; d < b->n; ++d) {
             if (b->frozen[d] >= 0) continue;
@@ -225,9 +239,9 @@ int chunk_rows_used(const lb_batch* b) {
                 longest = std::max(longest, c);
             }
         }
-        if (rows == b->chunk_rows && n >= 4.0 * G) return rows;
+        if (rows == DEFAULT_CHUNK_ROWS && n >= 4.0 * G) return rows;
         const double cost = std::max(sum / G, std::min(std::ceil(n / G) * longest, sum / G + 0.5 * sum / std::max(n, 1.0)));
-        if (rows == b->chunk_rows || cost < 0.98 * best_cost) {
+        if (rows == DEFAULT_CHUNK_ROWS || cost < 0.98 * best_cost) {
             best = rows;
             best_cost = cost;
         }
@@ -735,6 +749,19 @@ lb_status lb_batch_set_chunk_rows(lb_batch* b, int32_t rows) {
 
 int32_t lb_batch_chunk_rows(const lb_batch* b) { return b ? b->chunk_rows : -1; }
 
+int32_t lb_batch_tile_rows(const lb_batch* b) { return b ? b->tile_by : -1; }
+
+lb_status lb_batch_apply_tuning(lb_batch* b, int32_t rows, int32_t tiles) {
+    if (!b || rows < MIN_CHUNK_ROWS || rows > 1 << 20 || tiles < 0 || tiles > 1)
+        return err(LB_ERR_ARG, "lb_batch_apply_tuning: rows must be >= %d, tiles 0 or 1", MIN_CHUNK_ROWS);
+    BCU(cudaSetDevice(b->device), "cudaSetDevice");
+    b->chunk_rows = rows;
+    b->strip_asked = false;
+    b->strip_tuned = !tiles;
+    b->tuned_sites = active_sites(b);
+    return rebuild_lists(b);
+}
+
 lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
                             double ms_per_step[LB_BATCH_TUNE_N]) {
     if (!b || steps < 1) return err(LB_ERR_ARG, "lb_batch_autotune: NULL batch or steps < 1");
@@ -756,7 +783,8 @@ lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
     int best_rows = rows0;
     // the strip kernel at every height, then the tile step where the library would
     // run it (the tuned batch keeps the faster kernel)
-    const bool asked0 = b->strip_asked;
+    const bool asked0 = b->strip_asked, tuned0 = b->strip_tuned;
+    b->strip_tuned = false;
     bool strip_best = true;
     for (int k = 0; k <= LB_BATCH_TUNE_N && e == cudaSuccess && st == LB_OK; ++k) {
         const bool strip = k < LB_BATCH_TUNE_N;
@@ -790,7 +818,6 @@ lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
     }
     // restore the snapshot, whatever happened
     b->cur = cur0;
-    b->strip_asked = e == cudaSuccess && st == LB_OK ? strip_best : asked0;
     cudaError_t e2 = cudaMemcpyAsync(b->buf[cur0], snap, b->buf_bytes, cudaMemcpyDeviceToDevice, b->stream);
     if (e2 == cudaSuccess)
         e2 = cudaMemcpyAsync(b->d_err, errw.data(), sizeof(int) * b->n, cudaMemcpyHostToDevice, b->stream);
@@ -798,11 +825,16 @@ lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
     if (ev[0]) cudaEventDestroy(ev[0]);
     if (ev[1]) cudaEventDestroy(ev[1]);
     cudaFree(snap);
-    if (e != cudaSuccess) return cuerr(e, "batch autotune");
-    if (e2 != cudaSuccess) return cuerr(e2, "batch autotune restore");
-    if (st != LB_OK) return st;
-    b->chunk_rows = st == LB_OK && std::isfinite(best) ? best_rows : rows0;
-    st = rebuild_lists(b);
+    if (e != cudaSuccess || e2 != cudaSuccess || st != LB_OK) {
+        b->chunk_rows = rows0;
+        b->strip_asked = asked0;
+        b->strip_tuned = tuned0;
+        const lb_status back = rebuild_lists(b);  // the lists of the choice before
+        if (e != cudaSuccess) return cuerr(e, "batch autotune");
+        if (e2 != cudaSuccess) return cuerr(e2, "batch autotune restore");
+        return st != LB_OK ? st : back;
+    }
+    st = lb_batch_apply_tuning(b, std::isfinite(best) ? best_rows : rows0, !strip_best);
     if (st == LB_OK && chunk_rows) *chunk_rows = b->chunk_rows;
     return st;
 }

@@ -76,6 +76,7 @@ EXPORTED = [
     "lb_batch_init", "lb_batch_step", "lb_batch_check", "lb_batch_run", "lb_batch_fields",
     "lb_batch_time", "lb_batch_free", "lb_tune_candidate", "lb_autotune",
     "lb_batch_set_chunk_rows", "lb_batch_chunk_rows", "lb_batch_autotune", "lb_batch_restart",
+    "lb_batch_tile_rows", "lb_batch_apply_tuning",
 ]
 
 
@@ -136,6 +137,8 @@ def load(path: str | None = None):
         "lb_autotune": (st, [P, ctypes.c_int32, vp, P, dp]),
         "lb_batch_set_chunk_rows": (st, [vp, ctypes.c_int32]),
         "lb_batch_chunk_rows": (ctypes.c_int32, [vp]),
+        "lb_batch_tile_rows": (ctypes.c_int32, [vp]),
+        "lb_batch_apply_tuning": (st, [vp, ctypes.c_int32, ctypes.c_int32]),
         "lb_batch_autotune": (st, [vp, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32), dp]),
         "lb_batch_restart": (st, [vp, ctypes.c_int32, vp, vp, ctypes.c_int32]),
     }
@@ -443,6 +446,15 @@ def lb_batch_chunk_rows(b) -> int:
     return int(load().lb_batch_chunk_rows(b))
 
 
+def lb_batch_tile_rows(b) -> int:
+    return int(load().lb_batch_tile_rows(b))
+
+
+def lb_batch_apply_tuning(b, rows: int, tiles: bool):
+    """The outcome of an earlier tuning (height, and whether the tile kernel was faster)."""
+    _check(load().lb_batch_apply_tuning(b, int(rows), int(tiles)))
+
+
 def lb_batch_autotune(b, steps: int):
     """Time the row-chunk heights; returns (chosen height, ms per step per height)."""
     rows = ctypes.c_int32()
@@ -495,8 +507,16 @@ class Batch:
     def chunk_rows(self, rows):
         lb_batch_set_chunk_rows(self.b, rows)
 
+    @property
+    def tile_rows(self):
+        """Rows of the tiles of the next step; 0: it runs the strip kernel."""
+        return lb_batch_tile_rows(self.b)
+
     def autotune(self, steps=20):
         return lb_batch_autotune(self.b, steps)
+
+    def apply_tuning(self, rows, tiles):
+        lb_batch_apply_tuning(self.b, rows, tiles)
 
     def close(self):
         if self.b is not None:

@@ -80,3 +80,33 @@ def test_batch_autotune_restores_state(lb):
         B_.step(2)
         for d in range(len(specs)):
             assert np.array_equal(A_.fields(d)[0], B_.fields(d)[0]), d
+
+
+def uniform_batch(lb, sizes):
+    params = [lb.lb_params_default(nx=nx, ny=ny, precision="fp32", psi_uses_local_T=0, T_psi=0.075) for nx, ny in sizes]
+    return params, [np.full((ny, nx), 0.1) for nx, ny in sizes], [np.full((ny, nx), 0.075) for nx, ny in sizes]
+
+
+@pytest.mark.gpu
+def test_tuned_strips_hold_for_half_of_the_sites(lb):
+    """A tuning that chose strips applies while half of its sites are active; then the
+    library's rule: tiles for the domains that are left, narrow ones among them (the
+    longest tile list).  A height set by the caller stays."""
+    # 2.6 million sites, too many for tiles; all but two domains are at rest and converge
+    sizes = [(1024, 1024), (1024, 1024), (3, 100000), (5, 50000)]
+    params, rhos, Ts = uniform_batch(lb, sizes)
+    for d in (2, 3):
+        nx, ny = sizes[d]
+        rhos[d] = 0.1 + 1e-3 * np.sin(2 * np.pi * np.arange(ny) / 100)[:, None] * np.ones((1, nx))
+    with lb.Batch(params, rhos, Ts) as B, lb.Batch(params, rhos, Ts) as C:
+        B.apply_tuning(32, False)
+        C.chunk_rows = 32
+        assert (B.tile_rows, C.tile_rows) == (0, 0) and B.chunk_rows == 32
+        rb, rc = B.run(1e-7, K=20, max_steps=40), C.run(1e-7, K=20, max_steps=40)
+        assert rb[2][:2].tolist() == [0, 0] and rb[2][2] == lb.LB_ERR_NOT_CONVERGED
+        assert B.tile_rows > 0 and C.tile_rows == 0 and B.chunk_rows == 32
+        assert np.array_equal(rb[0], rc[0])
+        for d in range(len(sizes)):
+            assert np.array_equal(B.fields(d)[0], C.fields(d)[0]), d
+        with pytest.raises(lb.LbError):
+            B.apply_tuning(8, False)
