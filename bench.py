@@ -406,13 +406,14 @@ def run_sweep(lb, torch, dist, world, rank, args):
     sites = sum(q.nx * q.ny for q in params)
     with lb.Batch(params, [d.rho for d in doms], [d.T for d in doms]) as B:
         rows, _ = B.autotune(20)
+        tiles = B.tile_rows > 0
         torch.cuda.synchronize()
         t0 = time.perf_counter()
         B.step(200)
         B.check()  # synchronises
         t_step = (time.perf_counter() - t0) / 200
     with lb.Batch(params, [d.rho for d in doms], [d.T for d in doms]) as B:
-        B.chunk_rows = rows
+        B.apply_tuning(rows, tiles)
         if dist:
             dist.barrier()
         t0 = time.perf_counter()

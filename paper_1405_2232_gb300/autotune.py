@@ -9,7 +9,9 @@ temperature treatment (Eq. 7 or Eq. 24), force form (beta = 0, 1 or mixed,
 Eq. 2 / Eq. 4), the lattice's size class (nx and ny rounded up to powers of
 two) and whether nx meets the strip kernel's 16-byte row rule.  A batch
 tuning is keyed by the device, precision, treatment, force form, the number
-of domains and the total site count (both rounded up to powers of two).
+of domains and the total site count (both rounded up to powers of two), and the
+kernel that the library would run the batch on.  Its entry holds that the tile kernel
+was the fastest, or the fastest height of the strip kernel.
 
 The cache is a flat JSON object ``{key: entry}``; it is written atomically
 (temporary file + rename).  Its default path is ``$LBGB_TUNE_CACHE`` or
@@ -120,17 +122,22 @@ def tuned_params(p, cache: TuneCache | None = None, steps: int | None = None,
 
 def tuned_batch(batch, cache: TuneCache | None = None, steps: int = 20,
                 device_name: str | None = None, timer=None) -> int:
-    """Set the batch's row-chunk height to the fastest (cached per key); returns it.
+    """Run the batch on its fastest kernel and row-chunk height (cached per key);
+    returns the height.
 
-    ``timer(batch, steps) -> (rows, ms_per_height)`` defaults to Batch.autotune."""
+    ``timer(batch, steps) -> (rows, ms_per_height)`` defaults to Batch.autotune, which
+    leaves the batch on the faster kernel (``tile_rows``)."""
     cache = cache or TuneCache()
     key = batch_key(batch.params, device_name or _device_name())
+    key += "|tiles" if getattr(batch, "tile_rows", 0) else "|strips"
     hit = cache.get(key)
     if hit is None:
         rows, ms = (timer or (lambda b, s: b.autotune(s)))(batch, steps)
-        hit = {"chunk_rows": int(rows),
+        hit = {"chunk_rows": int(rows), "tiles": bool(getattr(batch, "tile_rows", 0)),
                "ms_per_step": [None if math.isnan(v) else float(v) for v in ms]}
         cache.put(key, hit)
+    elif hasattr(batch, "apply_tuning"):
+        batch.apply_tuning(hit["chunk_rows"], hit["tiles"])
     else:
         batch.chunk_rows = hit["chunk_rows"]
     return hit["chunk_rows"]

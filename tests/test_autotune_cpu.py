@@ -103,3 +103,31 @@ def test_default_steps():
     assert A.default_steps(64 * 64) == 200
     assert A.default_steps(10 ** 10) == 4
     assert all(A.default_steps(s) % 2 == 0 for s in (3, 1000, 123457, 10 ** 8))
+
+
+def test_batch_cache_keeps_the_kernel(tmp_path):
+    """A cold and a warm cache leave the batch on the same kernel; a batch that the
+    library would run on another one is tuned on its own."""
+    class FakeBatch:
+        def __init__(self, tile_rows):
+            self.params = [lb.lb_params_default(nx=64, ny=64)]
+            self.tile_rows, self.applied = tile_rows, None
+
+        def apply_tuning(self, rows, tiles):
+            self.applied = (rows, tiles)
+
+    path = str(tmp_path / "tune.json")
+    n = []
+
+    def timer(b, steps):
+        n.append(b)
+        return 16, np.array([1.0, 2.0, 3.0, 4.0])
+
+    assert A.tuned_batch(FakeBatch(7), A.TuneCache(path), device_name="dev", timer=timer) == 16
+    warm = FakeBatch(7)
+    assert A.tuned_batch(warm, A.TuneCache(path), device_name="dev", timer=timer) == 16
+    assert warm.applied == (16, True) and len(n) == 1
+    A.tuned_batch(FakeBatch(0), A.TuneCache(path), device_name="dev", timer=timer)
+    strips = FakeBatch(0)
+    A.tuned_batch(strips, A.TuneCache(path), device_name="dev", timer=timer)
+    assert strips.applied == (16, False) and len(n) == 2

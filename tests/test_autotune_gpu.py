@@ -88,6 +88,20 @@ def uniform_batch(lb, sizes):
 
 
 @pytest.mark.gpu
+def test_batch_steps_on_the_same_kernel_with_a_cold_and_a_warm_cache(lb, tmp_path):
+    cache = str(tmp_path / "t.json")
+    args = uniform_batch(lb, [(64, 64), (90, 70)])
+    kernels = []
+    for _ in range(2):
+        with lb.Batch(*args) as B:
+            untuned = B.tile_rows
+            rows = A.tuned_batch(B, A.TuneCache(cache), steps=4)
+            assert B.chunk_rows == rows
+            kernels.append(B.tile_rows)
+    assert untuned > 0 and kernels[0] == kernels[1]
+
+
+@pytest.mark.gpu
 def test_tuned_strips_hold_for_half_of_the_sites(lb):
     """A tuning that chose strips applies while half of its sites are active; then the
     library's rule: tiles for the domains that are left, narrow ones among them (the
