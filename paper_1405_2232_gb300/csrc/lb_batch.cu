@@ -818,6 +818,7 @@ lb_status lb_batch_autotune(lb_batch* b, int32_t steps, int32_t* chunk_rows,
     }
     // restore the snapshot, whatever happened
     b->cur = cur0;
+    b->checked_t = -1;  // (fields() reads the restored state, not the check before)
     cudaError_t e2 = cudaMemcpyAsync(b->buf[cur0], snap, b->buf_bytes, cudaMemcpyDeviceToDevice, b->stream);
     if (e2 == cudaSuccess)
         e2 = cudaMemcpyAsync(b->d_err, errw.data(), sizeof(int) * b->n, cudaMemcpyHostToDevice, b->stream);

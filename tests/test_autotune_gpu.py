@@ -124,3 +124,22 @@ def test_tuned_strips_hold_for_half_of_the_sites(lb):
             assert np.array_equal(B.fields(d)[0], C.fields(d)[0]), d
         with pytest.raises(lb.LbError):
             B.apply_tuning(8, False)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_batch_state_around_a_tuning_read_anew(lb, prec):
+    """Mass, energy and fields after a tuning, each from the state (a check), equal those
+    before; a step in between changes them."""
+    rho, T = I.slab_fields(70, 45, noise=1e-3)
+    p = [lb.lb_params_default(nx=70, ny=45, precision=prec, psi_uses_local_T=0, T_psi=0.08)] * 2
+    with lb.Batch(p, [rho, rho], [T, T]) as B:
+        B.step(7)
+        before = B.check()[1:3], B.fields(1)
+        B.autotune(3)
+        after = B.fields(1), B.check()[1:3]
+        B.step(1)
+        moved = B.fields(1)
+    assert np.array_equal(before[0], after[1])
+    for k in range(2):
+        assert np.array_equal(before[1][k], after[0][k]) and not np.array_equal(before[1][k], moved[k])
