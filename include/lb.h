@@ -315,10 +315,19 @@ lb_status lb_free(lb_ctx* ctx);
  * the fastest tile_x, tile_y; ms_per_step[k] (may be NULL) = each shape's
  * time per step in ms, NaN for shapes not valid here.  Allocates and frees
  * one trial context at a time (two population buffers of the lattice);
- * synchronises.  LB_ERR_ARG for NULL params/best or steps < 1. */
+ * synchronises.  LB_ERR_ARG for NULL params/best or steps < 1.
+ * Without a shape (tile_x = tile_y = 0) the library chooses: beside the strip kernel,
+ * tiles whose height balances the lattice over the SMs, and runs of 16 and more steps of a
+ * tiny lattice in one launch.  None of the shapes above is these, so on small lattices the
+ * library's choice is usually faster than the fastest shape.
+ * lb_time_step: *ms_per_step = the time per step of *p as it is (its own tile fields, so
+ * also the library's choice) over one lb_step of `steps`, after one such call, otherwise
+ * as lb_autotune times a shape.  LB_ERR_ARG for NULL pointers or steps < 1, else what
+ * lb_init returns for *p. */
 lb_status lb_tune_candidate(int32_t k, int32_t* tile_x, int32_t* tile_y);
 lb_status lb_autotune(const lb_params* p, int32_t steps, void* stream, lb_params* best,
                       double ms_per_step[LB_TUNE_N]);
+lb_status lb_time_step(const lb_params* p, int32_t steps, void* stream, double* ms_per_step);
 
 /* ------------------------------------------------------------------ batch
  * Many independent periodic domains (a parameter sweep) advanced together by

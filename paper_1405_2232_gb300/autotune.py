@@ -1,8 +1,8 @@
 """Autotuned step shapes and batch work-list granularity, with a JSON cache.
 
-The timing itself is native (``lb_autotune`` and ``lb_batch_autotune`` in the
-library, CUDA events on the device); this module only keys, stores and
-reuses the winners.
+The timing itself is native (``lb_autotune``, ``lb_time_step`` and
+``lb_batch_autotune`` in the library, CUDA events on the device); this module
+only keys, stores and reuses the winners.
 
 A single-lattice tuning is keyed by the device name, storage precision,
 temperature treatment (Eq. 7 or Eq. 24), force form (beta = 0, 1 or mixed,
@@ -99,18 +99,31 @@ class TuneCache:
         os.replace(tmp, self.path)
 
 
+def fastest_shape(p, steps: int):
+    """lb_autotune's result, with the library's own choice (tile_x = tile_y = 0) as the
+    best where it is faster than every shape."""
+    best, ms = lb.lb_autotune(p, steps)
+    own = ctypes_copy(lb.lb_params(), p)
+    own.tile_x = own.tile_y = 0
+    if lb.lb_time_step(own, steps) <= min((v for v in ms if not math.isnan(v)), default=math.inf):
+        best = own
+    return best, ms
+
+
 def tuned_params(p, cache: TuneCache | None = None, steps: int | None = None,
                  device_name: str | None = None, timer=None):
-    """p with tile_x/tile_y set to the fastest step shape (cached per key).
+    """p with tile_x/tile_y set to the fastest step shape, 0 if that is the library's own
+    choice (cached per key).
 
-    ``timer(p, steps) -> (best_params, ms_per_shape)`` defaults to lb.lb_autotune."""
+    ``timer(p, steps) -> (best_params, ms_per_shape)`` defaults to fastest_shape."""
     cache = cache or TuneCache()
-    key = tune_key(p, device_name or _device_name())
+    # (an entry whose key does not say so was found without the library's choice)
+    key = tune_key(p, device_name or _device_name()) + "|own"
     hit = cache.get(key)
     out = lb.lb_params()
     ctypes_copy(out, p)
     if hit is None:
-        timer = timer or lb.lb_autotune
+        timer = timer or fastest_shape
         best, ms = timer(p, steps or default_steps(p.nx * p.ny))
         hit = {"tile_x": int(best.tile_x), "tile_y": int(best.tile_y),
                "ms_per_step": [None if math.isnan(v) else float(v) for v in ms],

@@ -76,7 +76,7 @@ EXPORTED = [
     "lb_batch_init", "lb_batch_step", "lb_batch_check", "lb_batch_run", "lb_batch_fields",
     "lb_batch_time", "lb_batch_free", "lb_tune_candidate", "lb_autotune",
     "lb_batch_set_chunk_rows", "lb_batch_chunk_rows", "lb_batch_autotune", "lb_batch_restart",
-    "lb_batch_tile_rows", "lb_batch_apply_tuning",
+    "lb_batch_tile_rows", "lb_batch_apply_tuning", "lb_time_step",
 ]
 
 
@@ -135,6 +135,7 @@ def load(path: str | None = None):
         "lb_tune_candidate": (st, [ctypes.c_int32, ctypes.POINTER(ctypes.c_int32),
                                    ctypes.POINTER(ctypes.c_int32)]),
         "lb_autotune": (st, [P, ctypes.c_int32, vp, P, dp]),
+        "lb_time_step": (st, [P, ctypes.c_int32, vp, dp]),
         "lb_batch_set_chunk_rows": (st, [vp, ctypes.c_int32]),
         "lb_batch_chunk_rows": (ctypes.c_int32, [vp]),
         "lb_batch_tile_rows": (ctypes.c_int32, [vp]),
@@ -436,6 +437,13 @@ def lb_autotune(p: lb_params, steps: int, stream=None):
     _check(load().lb_autotune(ctypes.byref(p), int(steps), _stream(stream), ctypes.byref(best),
                               _dptr(ms)))
     return best, ms
+
+
+def lb_time_step(p: lb_params, steps: int, stream=None) -> float:
+    """ms per step of p as it is (tile_x = tile_y = 0: the library's choice)."""
+    ms = ctypes.c_double()
+    _check(load().lb_time_step(ctypes.byref(p), int(steps), _stream(stream), ctypes.byref(ms)))
+    return ms.value
 
 
 def lb_batch_set_chunk_rows(b, rows: int):

@@ -131,3 +131,32 @@ def test_batch_cache_keeps_the_kernel(tmp_path):
     strips = FakeBatch(0)
     A.tuned_batch(strips, A.TuneCache(path), device_name="dev", timer=timer)
     assert strips.applied == (16, False) and len(n) == 2
+
+
+def test_an_entry_without_the_librarys_choice_is_tuned_again(tmp_path, monkeypatch):
+    """tuned_params keeps tile_x = tile_y = 0 where that is faster than every shape; an
+    entry found among the shapes alone does not count."""
+    p = lb.lb_params_default(nx=64, ny=64, precision="fp32", tau_f=0.7)
+    path = str(tmp_path / "tune.json")
+    A.TuneCache(path).put(A.tune_key(p, "dev"), {"tile_x": 32, "tile_y": 8, "ms_per_step": [], "shapes": []})
+
+    def shapes(q, steps):
+        best = A.ctypes_copy(lb.lb_params(), q)
+        best.tile_x, best.tile_y = 32, 8
+        return best, np.array([14.0, 15.0, 2.2, 2.5, np.nan])
+
+    for own, tile in ((1.2, (0, 0)), (2.6, (32, 8))):
+        monkeypatch.setattr(lb, "lb_autotune", shapes)
+        monkeypatch.setattr(lb, "lb_time_step", lambda q, steps: own if (q.tile_x, q.tile_y) == (0, 0) else None)
+        q = A.tuned_params(p, A.TuneCache(path), device_name=f"dev{own}")
+        assert (q.tile_x, q.tile_y, q.tau_f) == (*tile, 0.7)
+    monkeypatch.setattr(lb, "lb_time_step", lambda q, steps: 1.2)
+    q = A.tuned_params(p, A.TuneCache(path), device_name="dev")
+    assert (q.tile_x, q.tile_y) == (0, 0)
+
+
+def test_time_step_argument_checks(lib):
+    p, ms = lb.lb_params_default(nx=64, ny=64), ctypes.c_double()
+    assert lib.lb_time_step(None, 4, None, ctypes.byref(ms)) == lb.LB_ERR_ARG
+    assert lib.lb_time_step(ctypes.byref(p), 4, None, None) == lb.LB_ERR_ARG
+    assert lib.lb_time_step(ctypes.byref(p), 0, None, ctypes.byref(ms)) == lb.LB_ERR_ARG
