@@ -293,7 +293,10 @@ lb_status lb_halo_unpack(lb_ctx* ctx, int32_t face, const void* d_buf);
  * cycles < 0. */
 lb_status lb_set_wait_limit(lb_ctx* ctx, int64_t cycles);
 
-/* Parameters the context runs with (tile sizes resolved). */
+/* Parameters the context runs with: a context created from them runs the same kernels.
+ * Tile sizes are resolved where a shape is (tile_y == 0: the strip kernel, tile_x columns
+ * wide); tile_x = tile_y = 0 where the library steps a small lattice created without
+ * a shape on tiles of its own height or in one cluster of blocks. */
 lb_status lb_get_params(const lb_ctx* ctx, lb_params* out);
 
 /* Release the context and its device memory.  NULL is accepted. */

@@ -930,6 +930,8 @@ lb_status lb_set_wait_limit(lb_ctx* c, int64_t cycles) {
 lb_status lb_get_params(const lb_ctx* c, lb_params* out) {
     if (!c || !out) return fail(LB_ERR_ARG, "NULL argument");
     *out = c->p;
+    // tiles or cluster runs of the library's choice: no shape that could be asked for is these
+    if (c->p.tile_y == 0 && (c->tile_by || c->in_cluster)) out->tile_x = 0;
     return LB_OK;
 }
 

@@ -106,3 +106,24 @@ def test_batch_kernels_give_the_same_bits(lb, prec):
                         L.step(25)
                         m = L.moments()
                     assert np.array_equal(a[0], m[0]) and np.array_equal(a[1], m[3]), (k, sizes[d])
+
+
+@pytest.mark.parametrize("prec,thermal,nx,ny,shape", [
+    ("fp32", None, 64, 64, (0, 0)), ("fp64", None, 90, 70, (0, 0)), ("bf16", None, 300, 200, (0, 0)),
+    ("fp32", "fd", 128, 96, (0, 0)), ("fp32", None, 2048, 1100, (256, 0)), ("fp64", None, 1100, 1000, (128, 0))])
+def test_a_context_from_the_reported_parameters_runs_the_same_kernels(lb, prec, thermal, nx, ny, shape):
+    """lb_get_params of a context without a shape: the strip kernel's width where it runs, else
+    no shape; a context created from the parameters reports them again.  An explicit
+    shape is reported as it is."""
+    rho, T = np.full((ny, nx), 0.1), np.full((ny, nx), 0.075)
+    kw = dict(nx=nx, ny=ny, precision=prec, thermal=lb.LB_THERMAL_FD26 if thermal else lb.LB_THERMAL_EQ24)
+    with lb.Lattice(rho, T, **kw) as L:
+        p = lb.lb_get_params(L.ctx)
+    assert (p.tile_x, p.tile_y) == shape
+    with lb.Lattice(rho, T, **{n: getattr(p, n) for n, _ in p._fields_}) as L:
+        q = lb.lb_get_params(L.ctx)
+    assert (q.tile_x, q.tile_y) == shape
+    width = 128 if prec == "fp64" else 256
+    with lb.Lattice(rho, T, tile_x=width, tile_y=0, **kw) as L:
+        q = lb.lb_get_params(L.ctx)
+    assert (q.tile_x, q.tile_y) == (width, 0)
