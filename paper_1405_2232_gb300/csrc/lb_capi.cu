@@ -399,12 +399,14 @@ cudaError_t dispatch_fd_set_T(lb_ctx* c, const double* d_T0) {
 // SMs best with the kernel's registers (seven rows: four blocks of ten warps in FP32;
 // six rows: four of nine in the 16-bit modes).  The strip kernel reads less and takes
 // over where the state outgrows the L2 cache: at 2^21 sites in FP32 (1448^2: 61.6 us
-// against 59.4, 2048^2: 109 against 114), at 1.5 x 2^20 in the 16-bit modes (1024^2:
-// 28.7 against 26.7, 1448^2: 51 against 52).
+// against 59.4, 2048^2: 109 against 114), at 7 x 2^17 in the 16-bit modes, whose strips
+// load a row in seven copies (1016 x 765: 20.5 - 21.1 us against 18.6 - 19.0, 1024 x 896:
+// 22.6 against 22.3 - 22.9, 1024^2: 24.8 - 26.1 against 26.2 - 26.6, 1536 x 1024: 36.9
+// against 38.5 - 39.0; FP16 and BF16, Eq. (7) and (24)).
 int default_tile_rows(int prec, int nx, int rows, int sms, bool walls) {
     const bool fp64 = prec == LB_PREC_FP64, fp32 = prec == LB_PREC_FP32;
     const long long sites = (long long)nx * rows;
-    if (!walls && sites > (fp64 ? (1LL << 20) - 1 : (fp32 ? 1LL << 21 : 3LL << 19))) return 0;
+    if (!walls && sites > (fp64 ? (1LL << 20) - 1 : (fp32 ? 1LL << 21 : 7LL << 17))) return 0;
     const long long cols = (nx + 31) / 32;
     const int low = (rows + 65534) / 65535;  // (at most 65,535 blocks down a grid)
     if (!walls && low > (fp64 ? 1 : TILE_FILL_DEV)) return 0;

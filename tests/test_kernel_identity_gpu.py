@@ -127,3 +127,12 @@ def test_a_context_from_the_reported_parameters_runs_the_same_kernels(lb, prec, 
     with lb.Lattice(rho, T, tile_x=width, tile_y=0, **kw) as L:
         q = lb.lb_get_params(L.ctx)
     assert (q.tile_x, q.tile_y) == (width, 0)
+
+
+@pytest.mark.parametrize("prec", ["fp16", "bf16"])
+@pytest.mark.parametrize("nx,ny,tiles", [(1016, 765, True), (1024, 896, True), (1032, 896, False), (1024, 1024, False)])
+def test_16bit_lattices_leave_the_tiles_where_strips_are_faster(lb, prec, nx, ny, tiles):
+    """1024^2: 24.8 - 26.1 us per step on strips, 26.2 - 26.6 on tiles; 1016 x 765: 20.5 and
+    18.6 at least."""
+    with lb.Lattice(np.full((ny, nx), 0.1), np.full((ny, nx), 0.075), nx=nx, ny=ny, precision=prec) as L:
+        assert lb.lb_get_params(L.ctx).tile_x == (0 if tiles else 256)
