@@ -102,6 +102,7 @@ struct lb_batch {
     BatchTile* d_tiles = nullptr;
     int* d_tile_begin = nullptr;  // [n + 1]
     int max_tiles = 0;
+    int check_sites = 256;        // sites of a check tile
     double* d_part = nullptr;     // [max_tiles][6]
     double* d_out6 = nullptr;     // [n][6]
     double* d_ref_rho = nullptr;  // dense reference fields (all domains)
@@ -249,6 +250,15 @@ int chunk_rows_used(const lb_batch* b) {
     return best;
 }
 
+// Sites of a check tile: eight per thread keep the block reductions cheap where the tiles
+// still fill the SMs twice; fewer on smaller batches, whose check is the latency of one
+// tile (a lone 64^2, the call: FP32 34.6 us at one site per thread, 44 at eight; FP64 35.7
+// and 49.5).  From the whole batch, so that a domain's sums do not depend on which others are active.
+int check_tile_sites(long long sites, int sms) {
+    const long long k = (sites + 512LL * sms - 1) / (512LL * sms);
+    return 256 * (int)std::min(std::max(k, 1LL), 8LL);
+}
+
 // Most tiles that active domains with at most tile_sites sites can have, tiles of one
 // row included: the domains with the most tiles per site first, until their sites pass it.
 long long most_step_tiles(int prec, const std::vector<lb_params>& params) {
@@ -315,7 +325,9 @@ lb_status rebuild_lists(lb_batch* b) {
                 items.push_back(it);
             }
         }
-        for (int first = 0; first < nx * ny; first += CHECK_SITES) tiles.push_back(BatchTile{d, first});
+        const long long n = (long long)nx * ny;
+        for (long long first = 0; first < n; first += b->check_sites)
+            tiles.push_back(BatchTile{d, (int)first, (int)std::min(first + b->check_sites, n)});
     }
     begin[b->n] = (int)tiles.size();
     if ((int)items.size() > b->max_items || (int)tiles.size() > b->max_tiles)
@@ -491,9 +503,11 @@ lb_status lb_batch_init(const lb_params* params, int32_t n, const double* const*
         off += 18 * plane;
         fld += (long long)p.nx * p.ny;
         max_items += ((p.nx + b->bx - 1) / b->bx) * ((p.ny + MIN_CHUNK_ROWS - 1) / MIN_CHUNK_ROWS);
-        max_tiles += (p.nx * p.ny + CHECK_SITES - 1) / CHECK_SITES;
     }
     b->n_sites = fld;
+    b->check_sites = check_tile_sites(fld, b->sms);
+    for (int d = 0; d < n; ++d)
+        max_tiles += (int)(((long long)params[d].nx * params[d].ny + b->check_sites - 1) / b->check_sites);
     b->buf_bytes = (size_t)off * es;
     b->max_items = max_items;
     b->max_tiles = max_tiles;

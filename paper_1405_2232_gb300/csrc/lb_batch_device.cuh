@@ -339,10 +339,10 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     if (aborted && t == 0) atomicOr(doms[0].kp.err, 1 << LB_ERR_TIMEOUT);
 }
 
-// Per-domain partial sums over tiles of CHECK_SITES sites: rho, rho c_v T (sum g),
+// Per-domain partial sums over tiles of 256 to 2,048 sites: rho, rho c_v T (sum g),
 // |d rho|^2, rho^2, |dT|^2, T^2 against the reference fields, and the new
-// reference fields are written.  One CTA per (domain, tile) item, eight sites per
-// thread.
+// reference fields are written.  One CTA per (domain, tile) item, one to eight sites
+// per thread (check_tile_sites in lb_batch.cu).
 //
 // Bound by the FP64 units (a warp instruction per 16 cycles of an SM, conversions
 // from FP32 included).  So in FP32 the nine populations of a site are summed as a
@@ -351,9 +351,8 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
 // domains of 3.3 million sites: 104 us, 475 us before.
 struct BatchTile {
     int domain;
-    int first;   // first site (row-major) of the tile in the domain
+    int first, end;   // sites (row-major) of the tile in the domain
 };
-constexpr int CHECK_SITES = 2048;
 
 template <int PREC>
 __global__ void __launch_bounds__(256)
@@ -369,11 +368,10 @@ __global__ void __launch_bounds__(256)
     const BatchTile tile = tiles[b];
     const BatchDomain& D = doms[tile.domain];
     const KParams& kp = D.kp;
-    const int n = kp.nx * kp.ny;
     const real cv = kpick<real>(kp.cv, kp.f.cv);
     double v[6] = {0, 0, 0, 0, 0, 0};
     bool bad = false;
-    for (int s = tile.first + (int)threadIdx.x; s < n && s < tile.first + CHECK_SITES; s += 256) {
+    for (int s = tile.first + (int)threadIdx.x; s < tile.end; s += 256) {
         const int y = s / kp.nx, x = s - y * kp.nx;
         real f[9], g[9];
         pull18<S>(src_base + D.off, kp, x, y, f, g);

@@ -327,3 +327,30 @@ def test_tile_and_strip_steps_agree(lb, prec, eps):
             assert len(set(ra[0].tolist())) > 1  # some left the list before others
             for d in range(len(sizes)):
                 assert np.array_equal(A.fields(d)[0], B.fields(d)[0]), d
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("side", [3, 250, 520, 1100])
+def test_check_sums_at_every_tile_size(lb, prec, side):
+    """The check's tiles have 256 to 2,048 sites, by the sites of the whole batch (the last
+    domain sets them): mass and energy are the FP64 sums of the stored populations, and a
+    domain's fields do not depend on the others.  At most 1.21 million terms of equal
+    sign, 2^-53 a rounding of partial sums: 1e-13."""
+    sizes = [(3, 3), (45, 45), (64, 33), (90, 61), (side, side)]
+    params, rhos, Ts = [], [], []
+    for k, (nx, ny) in enumerate(sizes):
+        rho, T = I.slab_fields(nx, ny, width=max(2, nx // 2), noise=1e-3, seed=k + 1)
+        params.append(lb.lb_params_default(nx=nx, ny=ny, precision=prec, psi_uses_local_T=0, T_psi=0.85 * I.CS_TC))
+        rhos.append(rho)
+        Ts.append(T)
+    with lb.Batch(params, rhos, Ts) as B:
+        _, mass, energy, status = B.check()
+        fields = [B.fields(d) for d in range(len(sizes))]
+    assert not status.any()
+    for d, p in enumerate(params):
+        with lb.Lattice(rhos[d], Ts[d], nx=p.nx, ny=p.ny, precision=prec) as L:
+            f, g = L.populations()
+            m = L.moments()
+        assert abs(mass[d] - f.sum()) <= 1e-13 * f.sum() and abs(energy[d] - g.sum()) <= 1e-13 * g.sum()
+        assert np.array_equal(fields[d][0], m[0]) and np.array_equal(fields[d][1], m[3])
