@@ -253,7 +253,8 @@ int chunk_rows_used(const lb_batch* b) {
 // Sites of a check tile: eight per thread keep the block reductions cheap where the tiles
 // still fill the SMs twice; fewer on smaller batches, whose check is the latency of one
 // tile (a lone 64^2, the call: FP32 34.6 us at one site per thread, 44 at eight; FP64 35.7
-// and 49.5).  From the whole batch, so that a domain's sums do not depend on which others are active.
+// and 49.5).  From the whole batch, so that a domain's sums do not depend on which others are
+// active.
 int check_tile_sites(long long sites, int sms) {
     const long long k = (sites + 512LL * sms - 1) / (512LL * sms);
     return 256 * (int)std::min(std::max(k, 1LL), 8LL);
