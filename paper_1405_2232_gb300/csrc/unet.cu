@@ -936,6 +936,11 @@ lb_status un_warm_fields(int32_t N, int32_t H, int32_t W, const float* d_pred, d
     a.rho = d_rho;
     a.T = d_T;
     a.P = (long long)H * W;
+    if (a.P <= unk::WARM_BLOCK_SITES) {
+        unk::k_warm_block<<<N, 256, 0, static_cast<cudaStream_t>(stream)>>>(a);
+        UCU(cudaGetLastError(), "un_warm_fields");
+        return LB_OK;
+    }
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.y = attr.val.clusterDim.z = 1;

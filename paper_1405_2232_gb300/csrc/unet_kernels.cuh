@@ -1132,6 +1132,80 @@ __device__ __forceinline__ void cluster_reduce(const double (&vin)[NS], long lon
     for (int q = 0; q < 4; ++q) out[q] = sh.out[q];
 }
 
+// Cases of at most WARM_BLOCK_SITES sites: one block of 256 threads per case, each pass
+// from the inputs.  Little shared memory and few registers, so eight blocks share an SM;
+// the cluster kernel below has one block of 512 threads on an SM, whose three reductions
+// alone take 25 us.  A case of 16^2 11.4 us (cluster kernel 24.6), 500 of 32^2 58 (105),
+// 1000 of 32^2 98 (184); at 48^2 one case 34 (26), 1000 cases 208 (211): the line
+// lies between 32^2 and 48^2.
+constexpr int WARM_BLOCK_SITES = 1536;
+
+// fixed-order reduction over a block of 256 threads (op 0: sum, -1: least, 1: greatest)
+template <int NV>
+__device__ __forceinline__ void warm_block_reduce(double (&v)[NV], double (*red)[256], const int (&op)[NV]) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) red[k][threadIdx.x] = v[k];
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+        if (threadIdx.x < w)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const double a = red[k][threadIdx.x], b = red[k][threadIdx.x + w];
+                red[k][threadIdx.x] = op[k] == 0 ? a + b : (op[k] < 0 ? fmin(a, b) : fmax(a, b));
+            }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = red[k][0];
+    __syncthreads();
+}
+
+// The handoff of k_warm (see there).
+__global__ void __launch_bounds__(256) k_warm_block(WarmArgs a) {
+    __shared__ double red[5][256];
+    const long long base = (long long)blockIdx.x * a.P;
+    auto rho_hat = [&](long long i) { return warm_rho_hat(a, a.rho0[base + i], a.pred[2 * (base + i)]); };
+    auto T_hat = [&](long long i) { return warm_T_hat(a, a.T0[base + i], a.pred[2 * (base + i) + 1]); };
+    double v1[5] = {0.0, 0.0, 0.0, INFINITY, -INFINITY};
+    for (long long i = threadIdx.x; i < a.P; i += 256) {
+        const double r = rho_hat(i);
+        v1[0] += a.rho0[base + i];
+        v1[1] += r;
+        v1[2] += a.rho0[base + i] * a.T0[base + i];
+        v1[3] = fmin(v1[3], r);
+        v1[4] = fmax(v1[4], r);
+    }
+    const int op1[5] = {0, 0, 0, -1, 1};
+    warm_block_reduce<5>(v1, red, op1);
+    const double S0 = v1[0], S1 = v1[1], E0 = v1[2], lo = v1[3], hi = v1[4];
+    double v2[1] = {0.0};
+    for (long long i = threadIdx.x; i < a.P; i += 256) {
+        const double r = rho_hat(i);
+        v2[0] += (r - lo) * (hi - r);
+    }
+    const int op2[1] = {0};
+    warm_block_reduce<1>(v2, red, op2);
+    double lam = v2[0] > 0.0 ? (S0 - S1) / v2[0] : 0.0;
+    const double cap = hi > lo ? 1.0 / (hi - lo) : 1.0;
+    lam = fmin(fmax(lam, -cap), cap);
+    double v3[2] = {0.0, 0.0};
+    for (long long i = threadIdx.x; i < a.P; i += 256) {
+        const double r = rho_hat(i);
+        const double r1 = r + lam * (r - lo) * (hi - r);
+        v3[0] += r1;
+        v3[1] += r1 * T_hat(i);
+    }
+    const int op3[2] = {0, 0};
+    warm_block_reduce<2>(v3, red, op3);
+    const double fr = S0 / v3[0], ft = E0 / (fr * v3[1]);
+    for (long long i = threadIdx.x; i < a.P; i += 256) {
+        const double r = rho_hat(i);
+        const double t = T_hat(i);  // (read before the fields, which may be the inputs, are written)
+        a.rho[base + i] = (r + lam * (r - lo) * (hi - r)) * fr;
+        a.T[base + i] = t * ft;
+    }
+}
+
 // One cluster of 1 - 16 blocks per case.  Mass is moved inside the interfaces with
 // the weight w = (rho_hat - lo)(hi - rho_hat) (zero in both bulk phases), then a
 // final scaling makes it exact; T is scaled to the initial energy.  Three

@@ -296,3 +296,22 @@ def test_warmstart_training_learns_without_per_step_sync(torch, N):
     zero = float((Y ** 2).mean().sqrt())
     net.close()
     assert fit < zero / 3, (fit, zero, losses[::8])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,h,w", [(1, 1, 1), (3, 1, 2), (7, 5, 3), (5, 16, 16), (200, 16, 17), (3, 32, 48), (3, 29, 53)])
+def test_warm_handoff_small_cases(torch, N, n, h, w):
+    """Cases that one small block takes, up to the line (32 x 48) and past it, in place."""
+    r = np.random.default_rng(31)
+    pred = r.standard_normal((n, h, w, 2)).astype(np.float32)
+    rho0 = 0.05 + 0.3 * r.random((n, h, w))
+    T0 = 0.08 + 0.01 * r.random((n, h, w))
+    d = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    d_rho, d_T = d(rho0), d(T0)
+    N.warm_fields(n, h, w, d(pred), I.UNET_NORM, d_rho, d_T, d_rho, d_T)
+    torch.cuda.synchronize()
+    nm = I.UNET_NORM
+    rh, th = U.denormalise(pred.astype(np.float64), nm["rho_dev_scale"], nm["t_dev_scale"], rho0, T0)
+    rr, tr = U.warm_project(rh, th, rho0, T0)
+    assert np.allclose(d_rho.cpu().numpy(), rr, rtol=1e-12, atol=0)
+    assert np.allclose(d_T.cpu().numpy(), tr, rtol=1e-12, atol=0)
