@@ -174,6 +174,13 @@ cudaError_t alloc(un_net* n, T** p, long long count) {
     return e;
 }
 
+// the error of a launch ends the pass
+#define UTRY(call)                          \
+    do {                                    \
+        const cudaError_t e_ = (call);      \
+        if (e_ != cudaSuccess) return e_;   \
+    } while (0)
+
 int grid_for(long long work, int per_block = 256) {
     long long b = (work + per_block - 1) / per_block;
     return (int)(b < 1 ? 1 : (b > 1 << 20 ? 1 << 20 : b));
@@ -185,7 +192,8 @@ int grid_for(long long work, int per_block = 256) {
 // block start-up then overlap the kernel ahead.  256^2 x 16 training step 2.68 -> 2.63 ms, eight cases through the network and
 // the handoff 524 -> 483 us.
 template <class... P, class... A>
-cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
+[[nodiscard]] cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                 A&&... args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -204,9 +212,14 @@ cudaError_t launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cud
 // and their own time is that of the fullest SM: training steps that run on them
 // took 4,030 us so at 240 x 232 x 5 and 3,510 us launched after it.
 template <class... P, class... A>
-cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A&&... args) {
-    kernel<<<grid, block, smem, stream>>>(static_cast<P>(args)...);
-    return cudaGetLastError();
+[[nodiscard]] cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                       A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 // splits of the weight-gradient kernel for a layer at M pixels
@@ -250,8 +263,9 @@ const bf16* blocked_of(const un_net* n, const bf16* w) {
     return nullptr;
 }
 
-cudaError_t conv(un_net* n, const bf16* x, int xC, int xoff, int Cin, const bf16* w, const float* bias, int Cout,
-                 bf16* y, int yC, int yoff, const bf16* mask, int mC, int moff, int N, int l, int relu, int up) {
+[[nodiscard]] cudaError_t conv(un_net* n, const bf16* x, int xC, int xoff, int Cin, const bf16* w, const float* bias,
+                               int Cout, bf16* y, int yC, int yoff, const bf16* mask, int mC, int moff, int N, int l,
+                               int relu, int up) {
     unk::ConvArgs a;
     a.x = x;
     a.xC = xC;
@@ -282,11 +296,10 @@ cudaError_t conv(un_net* n, const bf16* x, int xC, int xoff, int Cin, const bf16
         const size_t smem = unk::tc_smem_bytes(Cout, Cin);
         const int stages = unk::tc_stages(Cout, Cin);
         switch (Cout) {
-            case 32: launch(unk::k_conv3_tc<32>, grid, unk::TC_THREADS, smem, n->stream, a, xmap, stages); break;
-            case 64: launch(unk::k_conv3_tc<64>, grid, unk::TC_THREADS, smem, n->stream, a, xmap, stages); break;
-            default: launch(unk::k_conv3_tc<96>, grid, unk::TC_THREADS, smem, n->stream, a, xmap, stages); break;
+            case 32: return launch(unk::k_conv3_tc<32>, grid, unk::TC_THREADS, smem, n->stream, a, xmap, stages);
+            case 64: return launch(unk::k_conv3_tc<64>, grid, unk::TC_THREADS, smem, n->stream, a, xmap, stages);
+            default: return launch(unk::k_conv3_tc<96>, grid, unk::TC_THREADS, smem, n->stream, a, xmap, stages);
         }
-        return cudaGetLastError();
     }
     const int NB = unk::ts_block(Cout);
     const int segw = a.W < unk::TC_M ? a.W : unk::TC_M;
@@ -298,36 +311,33 @@ cudaError_t conv(un_net* n, const bf16* x, int xC, int xoff, int Cin, const bf16
         const long long tiles = (M / segw) / unk::ts_rows(NB) * (Cout / NB);
         const int grid = (int)(tiles < n->sms ? tiles : n->sms);
         if (NB == 128)
-            launch(unk::k_conv3_tcs<128>, grid, unk::TS_THREADS, unk::ts_smem_bytes(128), n->stream, a, xmap, wimg);
-        else
-            launch(unk::k_conv3_tcs<64>, grid, unk::TS_THREADS, unk::ts_smem_bytes(64), n->stream, a, xmap, wimg);
-        return cudaGetLastError();
+            return launch(unk::k_conv3_tcs<128>, grid, unk::TS_THREADS, unk::ts_smem_bytes(128), n->stream, a, xmap,
+                          wimg);
+        return launch(unk::k_conv3_tcs<64>, grid, unk::TS_THREADS, unk::ts_smem_bytes(64), n->stream, a, xmap, wimg);
     }
     if (a.W % unk::HT_W == 0 && a.H % unk::HT_H == 0 && Cout % unk::HT_NT == 0) {
         // halo-tile form: one staged input halo serves all nine taps
         const unsigned tiles = (unsigned)((long long)N * (a.H / unk::HT_H) * (a.W / unk::HT_W));
-        launch_after(unk::k_conv3_halo, dim3(tiles, Cout / unk::HT_NT), 256, unk::halo_smem_bytes(), n->stream, a);
-        return cudaGetLastError();
+        return launch_after(unk::k_conv3_halo, dim3(tiles, Cout / unk::HT_NT), 256, unk::halo_smem_bytes(), n->stream,
+                            a);
     }
     const unsigned gx = (unsigned)((M + unk::CV_MT - 1) / unk::CV_MT);
-    if (Cout % 64 == 0)
-        launch_after(unk::k_conv3<64>, dim3(gx, Cout / 64), 256, 0, n->stream, a);
-    else
-        launch_after(unk::k_conv3<32>, dim3(gx, Cout / 32), 256, 0, n->stream, a);
-    return cudaGetLastError();
+    if (Cout % 64 == 0) return launch_after(unk::k_conv3<64>, dim3(gx, Cout / 64), 256, 0, n->stream, a);
+    return launch_after(unk::k_conv3<32>, dim3(gx, Cout / 32), 256, 0, n->stream, a);
 }
 
 // the sums over layer k's splits, for the launch at the end of the pass
-cudaError_t queue_sums(un_net* n, int k, int splits) {
+[[nodiscard]] cudaError_t queue_sums(un_net* n, int k, int splits) {
     const Layer& L = n->L[k];
     const bool ok =
         n->sums.add(n->wpart + n->wpart_off[k], splits, (long long)L.cout * 9 * L.cin, false, n->grad + L.woff) &&
         n->sums.add(n->bpart + n->bpart_off[k], splits, L.cout, true, n->grad + L.boff);
-    return ok ? cudaGetLastError() : cudaErrorInvalidValue;
+    return ok ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // weight and bias gradient of layer k: g (gradient at its output) and x (its input)
-cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16* x, int xC, int xoff, int N, int l) {
+[[nodiscard]] cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16* x, int xC, int xoff,
+                                int N, int l) {
     const Layer& L = n->L[k];
     const long long M = Pl(n, l, N);
     const long long nw = (long long)L.cout * 9 * L.cin;
@@ -378,17 +388,18 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
             const int stages = unk::tw_stages(na, xm, segw);
             const size_t smem = unk::tw_smem_bytes(na, xm, segw);
             const unsigned grid = (unsigned)(units * splits);
+            cudaError_t e;
             if (rows3)
-                launch(unk::k_wgrad_tc<32, true, true>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
+                e = launch(unk::k_wgrad_tc<32, true, true>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
             else if (xm)
-                launch(unk::k_wgrad_tc<32, true>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
+                e = launch(unk::k_wgrad_tc<32, true>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
             else if (NBW == 128)
-                launch(unk::k_wgrad_tc<128, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
+                e = launch(unk::k_wgrad_tc<128, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
             else if (NBW == 64)
-                launch(unk::k_wgrad_tc<64, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
+                e = launch(unk::k_wgrad_tc<64, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
             else
-                launch(unk::k_wgrad_tc<32, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
-            return queue_sums(n, k, splits);
+                e = launch(unk::k_wgrad_tc<32, false>, grid, unk::TW_THREADS, smem, n->stream, a, gmap, xmap, stages);
+            return e == cudaSuccess ? queue_sums(n, k, splits) : e;
         }
     }
     if (W % unk::HT_W == 0 && H % unk::HT_H == 0) {
@@ -415,8 +426,9 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
         a.tiles_per_split = (int)tps;
         a.part = n->wpart + n->wpart_off[k];
         a.bpart = n->bpart + n->bpart_off[k];
-        launch_after(unk::k_wgrad_halo, dim3(blocks, splits), 256, unk::wgrad_halo_smem_bytes(), n->stream, a);
-        return queue_sums(n, k, splits);
+        const cudaError_t e =
+            launch_after(unk::k_wgrad_halo, dim3(blocks, splits), 256, unk::wgrad_halo_smem_bytes(), n->stream, a);
+        return e == cudaSuccess ? queue_sums(n, k, splits) : e;
     }
     int MT, NT, tiles, splits, cps;
     wgrad_shape(n, L, M, &MT, &NT, &tiles, &splits, &cps);
@@ -436,12 +448,13 @@ cudaError_t wgrad(un_net* n, int k, const bf16* g, int gC, int goff, const bf16*
     a.part = n->wpart + n->wpart_off[k];
     a.bpart = n->bpart + n->bpart_off[k];
     const dim3 grid(tiles, splits);
-    if (MT == 32 && NT == 32) launch_after(unk::k_wgrad<32, 32>, grid, 256, 0, n->stream, a);
-    else if (MT == 32) launch_after(unk::k_wgrad<32, 64>, grid, 256, 0, n->stream, a);
-    else if (NT == 32) launch_after(unk::k_wgrad<64, 32>, grid, 256, 0, n->stream, a);
-    else launch_after(unk::k_wgrad<64, 64>, grid, 256, 0, n->stream, a);
+    cudaError_t e;
+    if (MT == 32 && NT == 32) e = launch_after(unk::k_wgrad<32, 32>, grid, 256, 0, n->stream, a);
+    else if (MT == 32) e = launch_after(unk::k_wgrad<32, 64>, grid, 256, 0, n->stream, a);
+    else if (NT == 32) e = launch_after(unk::k_wgrad<64, 32>, grid, 256, 0, n->stream, a);
+    else e = launch_after(unk::k_wgrad<64, 64>, grid, 256, 0, n->stream, a);
     // (bias: partials of the centre-tap CTAs, summed over the splits in order)
-    return queue_sums(n, k, splits);
+    return e == cudaSuccess ? queue_sums(n, k, splits) : e;
 }
 
 const bf16* Wb(const un_net* n, int k) { return n->wb + n->L[k].qoff; }
@@ -481,65 +494,64 @@ cudaError_t adam_refresh(un_net* n, int adam, float lr, float b1, float b2, floa
         a.nbt[a.nl] = L.cout % 16 == 0 ? unk::ts_block(L.cin) : 0;
         ++a.nl;
     }
-    launch(unk::k_adam_refresh, grid_for(n->nparam), 256, 0, n->stream, a);
-    return cudaGetLastError();
+    return launch(unk::k_adam_refresh, grid_for(n->nparam), 256, 0, n->stream, a);
 }
 
 cudaError_t refresh_weights(un_net* n) { return adam_refresh(n, 0, 0.0f, 0.0f, 0.0f, 1.0f, 1.0f, 1.0f); }
 
-cudaError_t forward(un_net* n, int N, const float* d_in) {
+[[nodiscard]] cudaError_t forward(un_net* n, int N, const float* d_in) {
     const int LV = UN_LEVELS;
-    launch(unk::k_input, grid_for(Pl(n, 0, N) * 4), 256, 0, n->stream, d_in, (long long)N * Hl(n, 0), Wl(n, 0), n->x0);
+    UTRY(launch(unk::k_input, grid_for(Pl(n, 0, N) * 4), 256, 0, n->stream, d_in, (long long)N * Hl(n, 0), Wl(n, 0),
+                n->x0));
     for (int l = 0; l < LV; ++l) {
         const bf16* src = l == 0 ? n->x0 : n->pl[l - 1];
         const int sC = l == 0 ? UN_IN_PAD : Cl(n, l - 1);
-        conv(n, src, sC, 0, sC, Wb(n, LE(l, 0)), Bias(n, LE(l, 0)), Cl(n, l), n->a[l], Cl(n, l), 0, nullptr, 0, 0, N,
-             l, 1, 0);
+        UTRY(conv(n, src, sC, 0, sC, Wb(n, LE(l, 0)), Bias(n, LE(l, 0)), Cl(n, l), n->a[l], Cl(n, l), 0, nullptr, 0, 0, N,
+                  l, 1, 0));
         if (l < LV - 1) {
             const int catC = Cl(n, l + 1) + Cl(n, l);
-            conv(n, n->a[l], Cl(n, l), 0, Cl(n, l), Wb(n, LE(l, 1)), Bias(n, LE(l, 1)), Cl(n, l), n->cat[l], catC,
-                 Cl(n, l + 1), nullptr, 0, 0, N, l, 1, 0);
-            launch(unk::k_pool, grid_for(Pl(n, l + 1, N) * Cl(n, l) / 8), 256, 0, n->stream, 
-                n->cat[l], catC, Cl(n, l + 1), Cl(n, l), N, Hl(n, l), Wl(n, l), n->pl[l]);
+            UTRY(conv(n, n->a[l], Cl(n, l), 0, Cl(n, l), Wb(n, LE(l, 1)), Bias(n, LE(l, 1)), Cl(n, l), n->cat[l], catC,
+                      Cl(n, l + 1), nullptr, 0, 0, N, l, 1, 0));
+            UTRY(launch(unk::k_pool, grid_for(Pl(n, l + 1, N) * Cl(n, l) / 8), 256, 0, n->stream,
+                        n->cat[l], catC, Cl(n, l + 1), Cl(n, l), N, Hl(n, l), Wl(n, l), n->pl[l]));
         } else {
             // bottleneck output, upsampled into cat[LV - 2]
             const int catC = Cl(n, l) + Cl(n, l - 1);
-            conv(n, n->a[l], Cl(n, l), 0, Cl(n, l), Wb(n, LE(l, 1)), Bias(n, LE(l, 1)), Cl(n, l), n->cat[l - 1], catC,
-                 0, nullptr, 0, 0, N, l, 1, 1);
+            UTRY(conv(n, n->a[l], Cl(n, l), 0, Cl(n, l), Wb(n, LE(l, 1)), Bias(n, LE(l, 1)), Cl(n, l), n->cat[l - 1], catC,
+                      0, nullptr, 0, 0, N, l, 1, 1));
         }
     }
     for (int l = LV - 2; l >= 0; --l) {
         const int catC = Cl(n, l + 1) + Cl(n, l);
-        conv(n, n->cat[l], catC, 0, catC, Wb(n, LD(l, 0)), Bias(n, LD(l, 0)), Cl(n, l), n->c[l], Cl(n, l), 0, nullptr,
-             0, 0, N, l, 1, 0);
+        UTRY(conv(n, n->cat[l], catC, 0, catC, Wb(n, LD(l, 0)), Bias(n, LD(l, 0)), Cl(n, l), n->c[l], Cl(n, l), 0, nullptr,
+                  0, 0, N, l, 1, 0));
         if (l > 0)
-            conv(n, n->c[l], Cl(n, l), 0, Cl(n, l), Wb(n, LD(l, 1)), Bias(n, LD(l, 1)), Cl(n, l), n->cat[l - 1],
-                 Cl(n, l) + Cl(n, l - 1), 0, nullptr, 0, 0, N, l, 1, 1);
+            UTRY(conv(n, n->c[l], Cl(n, l), 0, Cl(n, l), Wb(n, LD(l, 1)), Bias(n, LD(l, 1)), Cl(n, l), n->cat[l - 1],
+                      Cl(n, l) + Cl(n, l - 1), 0, nullptr, 0, 0, N, l, 1, 1));
         else
-            conv(n, n->c[0], Cl(n, 0), 0, Cl(n, 0), Wb(n, LD(0, 1)), Bias(n, LD(0, 1)), Cl(n, 0), n->d0, Cl(n, 0), 0,
-                 nullptr, 0, 0, N, 0, 1, 0);
+            UTRY(conv(n, n->c[0], Cl(n, 0), 0, Cl(n, 0), Wb(n, LD(0, 1)), Bias(n, LD(0, 1)), Cl(n, 0), n->d0, Cl(n, 0), 0,
+                      nullptr, 0, 0, N, 0, 1, 0));
     }
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
-cudaError_t head_fwd(un_net* n, int N, float* out) {
+[[nodiscard]] cudaError_t head_fwd(un_net* n, int N, float* out) {
     const Layer& H = n->L[LHEAD];
     const long long P = Pl(n, 0, N);
     const int C = n->cfg.base;
     const int g = grid_for(P);
     switch (C) {
         case 32:
-            launch(unk::k_head_fwd<32>, g, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, P, Wl(n, 0), out);
-            break;
+            return launch(unk::k_head_fwd<32>, g, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, P, Wl(n, 0),
+                          out);
         case 64:
-            launch(unk::k_head_fwd<64>, g, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, P, Wl(n, 0), out);
-            break;
+            return launch(unk::k_head_fwd<64>, g, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, P, Wl(n, 0),
+                          out);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
-cudaError_t backward(un_net* n, int N, const float* d_target) {
+[[nodiscard]] cudaError_t backward(un_net* n, int N, const float* d_target) {
     const int LV = UN_LEVELS;
     const Layer& H = n->L[LHEAD];
     const long long P = Pl(n, 0, N);
@@ -549,49 +561,48 @@ cudaError_t backward(un_net* n, int N, const float* d_target) {
     const float inv2 = (float)(2.0 / ((double)P * UN_OUT));
     switch (C) {
         case 32:
-            launch(unk::k_head_bwd<32>, hb, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, d_target, P, Wl(n, 0),
-                                                           rows, inv2, n->gd0, n->hpart, n->lpart);
+            UTRY(launch(unk::k_head_bwd<32>, hb, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, d_target, P,
+                        Wl(n, 0), rows, inv2, n->gd0, n->hpart, n->lpart));
             break;
         case 64:
-            launch(unk::k_head_bwd<64>, hb, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, d_target, P, Wl(n, 0),
-                                                           rows, inv2, n->gd0, n->hpart, n->lpart);
+            UTRY(launch(unk::k_head_bwd<64>, hb, 256, 0, n->stream, n->d0, n->p + H.woff, n->p + H.boff, d_target, P,
+                        Wl(n, 0), rows, inv2, n->gd0, n->hpart, n->lpart));
             break;
         default: return cudaErrorInvalidValue;
     }
     n->sums.count = 0;
-    n->sums.add(n->hpart, hb, 2LL * C + 2, true, n->grad + H.woff);
-    launch(unk::k_sum_doubles, 1, 256, 0, n->stream, n->lpart, hb, n->d_loss);
+    if (!n->sums.add(n->hpart, hb, 2LL * C + 2, true, n->grad + H.woff)) return cudaErrorInvalidValue;
+    UTRY(launch(unk::k_sum_doubles, 1, 256, 0, n->stream, n->lpart, hb, n->d_loss));
     // decoder, finest level first
     for (int l = 0; l < LV - 1; ++l) {
         const bf16* gin = l == 0 ? n->gd0 : n->gup[l];
         const int c = Cl(n, l), catC = Cl(n, l + 1) + Cl(n, l);
-        wgrad(n, LD(l, 1), gin, c, 0, n->c[l], c, 0, N, l);
-        conv(n, gin, c, 0, c, Wt(n, LD(l, 1)), nullptr, c, n->gc[l], c, 0, n->c[l], c, 0, N, l, 0, 0);
-        wgrad(n, LD(l, 0), n->gc[l], c, 0, n->cat[l], catC, 0, N, l);
-        conv(n, n->gc[l], c, 0, c, Wt(n, LD(l, 0)), nullptr, catC, n->gcat[l], catC, 0, nullptr, 0, 0, N, l, 0, 0);
+        UTRY(wgrad(n, LD(l, 1), gin, c, 0, n->c[l], c, 0, N, l));
+        UTRY(conv(n, gin, c, 0, c, Wt(n, LD(l, 1)), nullptr, c, n->gc[l], c, 0, n->c[l], c, 0, N, l, 0, 0));
+        UTRY(wgrad(n, LD(l, 0), n->gc[l], c, 0, n->cat[l], catC, 0, N, l));
+        UTRY(conv(n, n->gc[l], c, 0, c, Wt(n, LD(l, 0)), nullptr, catC, n->gcat[l], catC, 0, nullptr, 0, 0, N, l, 0, 0));
         const int cu = Cl(n, l + 1);
-        launch(unk::k_up_bwd, grid_for(Pl(n, l + 1, N) * cu / 8), 256, 0, n->stream, 
-            n->gcat[l], catC, 0, n->cat[l], catC, 0, cu, N, Hl(n, l), Wl(n, l), n->gup[l + 1]);
+        UTRY(launch(unk::k_up_bwd, grid_for(Pl(n, l + 1, N) * cu / 8), 256, 0, n->stream,
+                    n->gcat[l], catC, 0, n->cat[l], catC, 0, cu, N, Hl(n, l), Wl(n, l), n->gup[l + 1]));
     }
     // encoder, coarsest level first
     for (int l = LV - 1; l >= 0; --l) {
         const bf16* gin = l == LV - 1 ? n->gup[LV - 1] : n->gs[l];
         const int c = Cl(n, l);
-        wgrad(n, LE(l, 1), gin, c, 0, n->a[l], c, 0, N, l);
-        conv(n, gin, c, 0, c, Wt(n, LE(l, 1)), nullptr, c, n->ga[l], c, 0, n->a[l], c, 0, N, l, 0, 0);
+        UTRY(wgrad(n, LE(l, 1), gin, c, 0, n->a[l], c, 0, N, l));
+        UTRY(conv(n, gin, c, 0, c, Wt(n, LE(l, 1)), nullptr, c, n->ga[l], c, 0, n->a[l], c, 0, N, l, 0, 0));
         const bf16* src = l == 0 ? n->x0 : n->pl[l - 1];
         const int sC = l == 0 ? UN_IN_PAD : Cl(n, l - 1);
-        wgrad(n, LE(l, 0), n->ga[l], c, 0, src, sC, 0, N, l);
+        UTRY(wgrad(n, LE(l, 0), n->ga[l], c, 0, src, sC, 0, N, l));
         if (l > 0) {
             const int cp = Cl(n, l - 1), catC = c + cp;
-            conv(n, n->ga[l], c, 0, c, Wt(n, LE(l, 0)), nullptr, cp, n->gp[l - 1], cp, 0, nullptr, 0, 0, N, l, 0, 0);
-            launch(unk::k_skip_bwd, grid_for(Pl(n, l - 1, N) * cp / 8), 256, 0, n->stream, 
-                n->gp[l - 1], n->gcat[l - 1], catC, c, n->cat[l - 1], catC, c, cp, N, Hl(n, l - 1), Wl(n, l - 1),
-                n->gs[l - 1]);
+            UTRY(conv(n, n->ga[l], c, 0, c, Wt(n, LE(l, 0)), nullptr, cp, n->gp[l - 1], cp, 0, nullptr, 0, 0, N, l, 0, 0));
+            UTRY(launch(unk::k_skip_bwd, grid_for(Pl(n, l - 1, N) * cp / 8), 256, 0, n->stream,
+                        n->gp[l - 1], n->gcat[l - 1], catC, c, n->cat[l - 1], catC, c, cp, N, Hl(n, l - 1), Wl(n, l - 1),
+                        n->gs[l - 1]));
         }
     }
-    launch(unk::k_sum_splits, n->sums.first[n->sums.count], 256, 0, n->stream, n->sums);
-    return cudaGetLastError();
+    return launch(unk::k_sum_splits, n->sums.first[n->sums.count], 256, 0, n->stream, n->sums);
 }
 
 // tensor table for un_get_tensor: pointer, element count at N, channels and

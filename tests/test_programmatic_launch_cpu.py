@@ -52,3 +52,15 @@ def test_no_read_only_promise_on_what_the_kernel_ahead_writes(name, params, body
         params = params.replace(table, "")
     assert not re.search(r"const [^,*]*\*\s*(const\s*)?__restrict__", params), params
     assert "__ldg" not in body and ".nc" not in body
+
+
+def test_no_launch_of_the_network_drops_its_error():
+    """Every launch, convolution and weight gradient of a pass is used in an expression (a
+    return, an assignment or UTRY), not called as a statement."""
+    s = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, "unet.cu")).read())
+    names = r"(?:launch|launch_after|conv|wgrad|queue_sums)\("
+    statements = [t.strip() for t in re.split(r"[;{}]", s)]
+    assert sum(bool(re.search(r"\b" + names, t)) for t in statements) > 30
+    dropped = [t for t in statements
+               if re.match(r"(?:(?:if|for) \(.*\)\s*|else\s+|case \w+:\s*|default:\s*)*" + names, t, flags=re.S)]
+    assert not dropped, dropped
