@@ -9,6 +9,15 @@
 
 namespace lbgb {
 
+// cudaLaunchKernelEx that does not leave its error behind as the runtime's last one: the next
+// launch with <<<>>>, of any context, would read it there and fail.
+template <class... P, class... A>
+inline cudaError_t launch_kernel(const cudaLaunchConfig_t& cfg, void (*kernel)(P...), A&&... args) {
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+
 // Most rows of a tile, and the threads of a block for a tile of bx x by
 // (tile and ring, each in whole warps).
 __host__ __device__ constexpr int tile_max_by(int bx) { return bx == 32 ? 16 : 4; }

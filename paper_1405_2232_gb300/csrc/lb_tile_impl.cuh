@@ -80,7 +80,7 @@ cudaError_t step_tile(const StepLaunch& L, int by) {
         cudaError_t e = opt_in_smem(configured[(L.eq24 ? 3 : 0) + L.bmode], kern);
         if (e != cudaSuccess) return e;
     }
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, by);
+    return launch_kernel(cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, by);
 }
 
 }  // namespace
@@ -148,7 +148,7 @@ cudaError_t LBGB_CAT(launch_cluster_, LBGB_NAME)(const StepLaunch& L, int steps)
             e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
             return e == cudaSuccess && clusters == 0 ? cudaErrorNotSupported : e;
         }
-        return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, steps);
+        return launch_kernel(cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.kp, steps);
     }
 }
 
@@ -187,8 +187,8 @@ cudaError_t LBGB_CAT(launch_batch_tile_, LBGB_NAME)(const BatchTileLaunch& L) {
     cfg.stream = L.stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.doms, L.tiles,
-                              L.n_tiles, L.by);
+    return launch_kernel(cfg, kern, static_cast<const E*>(L.src), static_cast<E*>(L.dst), L.doms, L.tiles,
+                         L.n_tiles, L.by);
 }
 #endif
 
@@ -213,7 +213,7 @@ cudaError_t fd_launch(std::atomic<unsigned long long>& done, const FdLaunch& L, 
         cudaError_t e = opt_in_smem(done, kern);
         if (e != cudaSuccess) return e;
     }
-    return cudaLaunchKernelEx(&cfg, kern, args...);
+    return launch_kernel(cfg, kern, args...);
 }
 
 template <int BM, bool STEP>

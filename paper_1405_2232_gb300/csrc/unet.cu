@@ -24,6 +24,7 @@
 #include <new>
 #include <vector>
 
+#include "lb_launch.h"
 #include "tensor_map.h"
 #include "lb.h"
 #include "unet.h"
@@ -204,7 +205,7 @@ template <class... P, class... A>
     cfg.stream = stream;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    return lbgb::launch_kernel(cfg, kernel, args...);
 }
 
 // The same after the kernel ahead has ended: for the mma.sync kernels, which have several
@@ -219,7 +220,7 @@ template <class... P, class... A>
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    return lbgb::launch_kernel(cfg, kernel, args...);
 }
 
 // splits of the weight-gradient kernel for a layer at M pixels
@@ -992,7 +993,7 @@ lb_status un_warm_fields(int32_t N, int32_t H, int32_t W, const float* d_pred, d
     }
     attr.val.clusterDim.x = (unsigned)blocks;
     cfg.gridDim = dim3((unsigned)N * (unsigned)blocks);
-    UCU(cudaLaunchKernelEx(&cfg, unk::k_warm, a), "un_warm_fields");
+    UCU(lbgb::launch_kernel(cfg, unk::k_warm, a), "un_warm_fields");
     return LB_OK;
 }
 

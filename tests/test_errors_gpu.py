@@ -88,3 +88,19 @@ def test_bounded_wait_times_out_and_context_recovers(lb, precision, thermal):
             assert np.all(np.isfinite(L.moments()[0]))
     with pytest.raises(lb.LbError):
         lb.lb_set_wait_limit(None, 1)
+
+
+def test_a_refused_launch_fails_its_own_call_only(lb):
+    """600,000 rows of 32 x 8 tiles are more blocks down a grid than CUDA takes: the runtime
+    refuses the launch and lb_step returns its error.  Another context goes on."""
+    rho, T = np.full((600000, 3), 0.1), np.full((600000, 3), 0.075)
+    with lb.Lattice(rho, T, nx=3, ny=600000, precision="fp32", tile_x=32, tile_y=8) as A, \
+            lattice(lb, 64, 48, "fp32") as B:
+        before = B.moments()
+        with pytest.raises(lb.LbError) as ei:
+            A.step(1)
+        assert ei.value.status == lb.LB_ERR_CUDA
+        for a, b in zip(before, B.moments()):
+            assert np.array_equal(a, b)
+        B.step(3)
+        B.synchronize()
