@@ -136,3 +136,24 @@ def test_16bit_lattices_leave_the_tiles_where_strips_are_faster(lb, prec, nx, ny
     18.6 at least."""
     with lb.Lattice(np.full((ny, nx), 0.1), np.full((ny, nx), 0.075), nx=nx, ny=ny, precision=prec) as L:
         assert lb.lb_get_params(L.ctx).tile_x == (0 if tiles else 256)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_cluster_runs_under_stream_capture(lb, prec):
+    """A captured run of an even number of steps replays in place."""
+    import torch
+    s = torch.cuda.Stream()
+    rho, T = I.slab_fields(64, 48, noise=1e-3)
+    kw = dict(nx=64, ny=48, precision=prec, psi_uses_local_T=0, T_psi=0.85 * I.CS_TC)
+    with lb.Lattice(rho, T, stream=s, **kw) as A, lb.Lattice(rho, T, stream=s, **kw) as B:
+        g = torch.cuda.CUDAGraph()
+        s.synchronize()
+        with torch.cuda.graph(g, stream=s):
+            A.step(32)
+        with torch.cuda.stream(s):
+            for _ in range(3):
+                g.replay()
+        for _ in range(96):
+            B.step(1)
+        a, b = state(A), state(B)
+        assert all(np.array_equal(x, y) for x, y in zip(a, b))
