@@ -198,13 +198,13 @@ struct KParams {
     long long wait_cycles;       // limit of the strip kernels' pipeline waits (<= 0: default)
     int halo_rows;               // 0: periodic in y; H > 0: rows [0, H) and [ny - H, ny) are ghost
                                  // rows of a y-decomposed lattice, the step updates [H, ny - H)
-    // 16-bit modes, collision in deviation variables (collide_dev):
     // FP64 step: products and scalings of the parameters above that are formed
     // once on the host (kp_fill_derived); each is the double the printed
     // formula forms per site
     double b4;                   // b / 4 (exact)
     double gw[3], cwc[3];        // guo_pre w and corr_pre w c_v (rest, axis, diagonal)
     int g_pow2;                  // |G| is a power of two: 2 x / G = x (2 / G), both exact scalings
+    // 16-bit modes, collision in deviation variables (collide_dev):
     float sum_bf, sum_bg;        // sum_i base_f[i], sum_i base_g[i]
     float dsum_f, dsum_g;        // sum_i base_f[i] - rho0, sum_i base_g[i] - rho0 c_v T0
     float cw_f[3], cw_g[3];      // w rho0 - base_f, w rho0 c_v T0 - base_g (rest, axis, diagonal)
@@ -292,6 +292,21 @@ __device__ __forceinline__ real kpick(double d, float f) {
 // Default limit of a bounded device wait, in clock cycles (about one second
 // at GB300 clocks).
 constexpr long long WAIT_CYCLES_DEFAULT = 2000000000LL;
+
+// Programmatic dependent launch (both return at once without it).  grid_wait: what the
+// kernel before this one wrote is complete; before any access to global memory.
+// grid_launch: the next kernel's blocks may become resident; in a kernel that
+// allocates TMEM only once it holds it, since a waiting block of the next kernel
+// could otherwise hold the columns that this one needs to finish.
+// Inputs of such a kernel are not const __restrict__ and not read with __ldg: both say that
+// nobody writes them while the kernel runs, which the kernel ahead may do, and let a load
+// move above the wait.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_begin() {
+    grid_launch();
+    grid_wait();
+}
 
 enum BetaMode { BETA_ZERO = 0, BETA_ONE = 1, BETA_MIXED = 2 };
 

@@ -174,144 +174,145 @@ __global__ void __launch_bounds__(strip_threads<BX>(), 2)
     real *rho_cur = r_rho, *rho_prv = r_rho + 4 * RA, *T_cur = r_T, *T_prv = r_T + 4 * RA;
     for (int jb = 0; jb < njobs + 2 && !aborted; jb += 4) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = jb + u;
-        if (j >= njobs + 2) break;
-        auto row8 = [&](real* cur, real* prv, int r) { return ((r >= 0 || r < -4) ? cur : prv) + (r & 3) * RA; };
-        // A(j)
-        if (j < njobs) {
-            const int s = u;
-            if (!mbar_wait_bounded(&full[s], ph, kp.wait_cycles)) s_abort[u & 1] = 1;
-            if (colA != -99) {
-                const elem* st = stage + (size_t)s * NP * SEGW;
-                const int c = colA + HALO;
-                real f[9], psi, psi2;
+        for (int u = 0; u < 4; ++u) {
+            const int j = jb + u;
+            if (j >= njobs + 2) break;
+            auto row8 = [&](real* cur, real* prv, int r) { return ((r >= 0 || r < -4) ? cur : prv) + (r & 3) * RA; };
+            // A(j)
+            if (j < njobs) {
+                const int s = u;
+                if (!mbar_wait_bounded(&full[s], ph, kp.wait_cycles)) s_abort[u & 1] = 1;
+                if (colA != -99) {
+                    const elem* st = stage + (size_t)s * NP * SEGW;
+                    const int c = colA + HALO;
+                    real f[9], psi, psi2;
 #pragma unroll
-                for (int i = 0; i < 9; ++i) f[i] = S::load(st + i * SEGW + c - ex(i), (real)kp.base_f[i]);
-                real rho = f[0];
+                    for (int i = 0; i < 9; ++i) f[i] = S::load(st + i * SEGW + c - ex(i), (real)kp.base_f[i]);
+                    real rho = f[0];
 #pragma unroll
-                for (int i = 1; i < 9; ++i) rho += f[i];
-                const real T = (real)st[9 * SEGW + c];
-                site_psi_T<real, BMODE>(kp, rho, T, psi, psi2, flags);
-                const int ia = colA + 2;
-                if (BMODE != BETA_ZERO) r_psi[u * RA + ia] = psi;
-                if (BMODE != BETA_ONE) r_psi2[u * RA + ia] = psi2;
-                row8(rho_cur, rho_prv, u)[ia] = rho;
-                row8(T_cur, T_prv, u)[ia] = T;
+                    for (int i = 1; i < 9; ++i) rho += f[i];
+                    const real T = (real)st[9 * SEGW + c];
+                    site_psi_T<real, BMODE>(kp, rho, T, psi, psi2, flags);
+                    const int ia = colA + 2;
+                    if (BMODE != BETA_ZERO) r_psi[u * RA + ia] = psi;
+                    if (BMODE != BETA_ONE) r_psi2[u * RA + ia] = psi2;
+                    row8(rho_cur, rho_prv, u)[ia] = rho;
+                    row8(T_cur, T_prv, u)[ia] = T;
+                }
             }
-        }
-        consumer_sync<BX + 32>();
-        // (a thread that times out at job j + 1 writes the other slot than the
-        // one read here, so every consumer leaves at the same job)
-        if (s_abort[u & 1]) {
-            aborted = true;
-            break;
-        }
-        // B(k), k = j - 1: force, u; own rows: f collision and store
-        {
-            const int k = j - 1;
-            if (k >= 1 && k <= njobs - 2 && colB != -99) {
-                const elem* st = stage + (size_t)((u + 3) & 3) * NP * SEGW;
-                const int c = colB + HALO;
-                real f[9], g[9];
+            consumer_sync<BX + 32>();
+            // (a thread that times out at job j + 1 writes the other slot than the
+            // one read here, so every consumer leaves at the same job)
+            if (s_abort[u & 1]) {
+                aborted = true;
+                break;
+            }
+            // B(k), k = j - 1: force, u; own rows: f collision and store
+            {
+                const int k = j - 1;
+                if (k >= 1 && k <= njobs - 2 && colB != -99) {
+                    const elem* st = stage + (size_t)((u + 3) & 3) * NP * SEGW;
+                    const int c = colB + HALO;
+                    real f[9], g[9];
 #pragma unroll
-                for (int i = 0; i < 9; ++i) {
-                    f[i] = S::load(st + i * SEGW + c - ex(i), (real)kp.base_f[i]);
-                    g[i] = (real)0;
-                }
-                const int ia = colB + 2;
-                const real rho = row8(rho_cur, rho_prv, u - 1)[ia];
-                real Fx, Fy, ux, uy, Tg;
-                force_from_rows<real, BMODE>(
-                    kp, r_psi + ((u + 2) & 3) * RA + ia, r_psi + ((u + 3) & 3) * RA + ia, r_psi + ((u + 0) & 3) * RA + ia,
-                    r_psi2 + ((u + 2) & 3) * RA + ia, r_psi2 + ((u + 3) & 3) * RA + ia,
-                    r_psi2 + ((u + 0) & 3) * RA + ia, Fx, Fy);
-                // the f half of the collision; g (zero here) is not used
-                // (FP32: the fused multiply-add form, faster in this kernel)
-                collide<real, false, true>(kp, f, g, rho, Fx, Fy, ux, uy, Tg);
-                if constexpr (sizeof(real) == 4) {
-                    // FP32: the rings keep a = chi grad(rho) / rho - u, which
-                    // both stages' K share (fd_K_rows_a)
-                    real ax, ay;
-                    fd_a_rows(row8(rho_cur, rho_prv, u - 2) + ia, row8(rho_cur, rho_prv, u - 1) + ia,
-                              row8(rho_cur, rho_prv, u) + ia, ux, uy, chi, ax, ay);
-                    r_ux[((u + 3) & 3) * RB + colB + 1] = ax;
-                    r_uy[((u + 3) & 3) * RB + colB + 1] = ay;
-                } else {
-                    r_ux[((u + 3) & 3) * RB + colB + 1] = ux;
-                    r_uy[((u + 3) & 3) * RB + colB + 1] = uy;
-                }
-                if (own_col && k >= 2 && k <= njobs - 3) {
-                    int y = y_start - 2 + k;
-                    y = y >= ny ? y - ny : y;
-                    const int xg = x0 + t;
-                    const uint32_t off = (uint32_t)y * pitch + (uint32_t)xg;
-                    const bool ghost_lo = xg < ghost, ghost_hi = xg >= nx - ghost;
+                    for (int i = 0; i < 9; ++i) {
+                        f[i] = S::load(st + i * SEGW + c - ex(i), (real)kp.base_f[i]);
+                        g[i] = (real)0;
+                    }
+                    const int ia = colB + 2;
+                    const real rho = row8(rho_cur, rho_prv, u - 1)[ia];
+                    real Fx, Fy, ux, uy, Tg;
+                    force_from_rows<real, BMODE>(
+                        kp, r_psi + ((u + 2) & 3) * RA + ia, r_psi + ((u + 3) & 3) * RA + ia, r_psi + u * RA + ia,
+                        r_psi2 + ((u + 2) & 3) * RA + ia, r_psi2 + ((u + 3) & 3) * RA + ia,
+                        r_psi2 + u * RA + ia, Fx, Fy);
+                    // the f half of the collision; g (zero here) is not used
+                    // (FP32: the fused multiply-add form, faster in this kernel)
+                    collide<real, false, true>(kp, f, g, rho, Fx, Fy, ux, uy, Tg);
+                    if constexpr (sizeof(real) == 4) {
+                        // FP32: the rings keep a = chi grad(rho) / rho - u, which
+                        // both stages' K share (fd_K_rows_a)
+                        real ax, ay;
+                        fd_a_rows(row8(rho_cur, rho_prv, u - 2) + ia, row8(rho_cur, rho_prv, u - 1) + ia,
+                                  row8(rho_cur, rho_prv, u) + ia, ux, uy, chi, ax, ay);
+                        r_ux[((u + 3) & 3) * RB + colB + 1] = ax;
+                        r_uy[((u + 3) & 3) * RB + colB + 1] = ay;
+                    } else {
+                        r_ux[((u + 3) & 3) * RB + colB + 1] = ux;
+                        r_uy[((u + 3) & 3) * RB + colB + 1] = uy;
+                    }
+                    if (own_col && k >= 2 && k <= njobs - 3) {
+                        int y = y_start - 2 + k;
+                        y = y >= ny ? y - ny : y;
+                        const int xg = x0 + t;
+                        const uint32_t off = (uint32_t)y * pitch + (uint32_t)xg;
+                        const bool ghost_lo = xg < ghost, ghost_hi = xg >= nx - ghost;
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) S::put(dst + ((uint32_t)i * plane + off), f[i], (real)kp.base_f[i]);
-                    // the periodic ghost copies: one branch per site, not per plane
-                    if (ghost_lo || ghost_hi) {
+                        for (int i = 0; i < 9; ++i) S::put(dst + ((uint32_t)i * plane + off), f[i], (real)kp.base_f[i]);
+                        // the periodic ghost copies: one branch per site, not per plane
+                        if (ghost_lo || ghost_hi) {
 #pragma unroll
-                        for (int i = 0; i < 9; ++i) {
-                            elem* pf = dst + ((uint32_t)i * plane + off);
-                            if (ghost_lo) S::put(pf + nx, f[i], (real)kp.base_f[i]);
-                            if (ghost_hi) S::put(pf - nx, f[i], (real)kp.base_f[i]);
+                            for (int i = 0; i < 9; ++i) {
+                                elem* pf = dst + ((uint32_t)i * plane + off);
+                                if (ghost_lo) S::put(pf + nx, f[i], (real)kp.base_f[i]);
+                                if (ghost_hi) S::put(pf - nx, f[i], (real)kp.base_f[i]);
+                            }
                         }
                     }
                 }
             }
-        }
-        // C(k), k = j - 2: stage 1
-        {
-            const int k = j - 2;
-            if (k >= 1 && k <= njobs - 2 && colB != -99) {
-                const int ia = colB + 2, ib = colB + 1;
-                const real* Ts_ = row8(T_cur, T_prv, u - 3) + ia;
-                const real* Tc_ = row8(T_cur, T_prv, u - 2) + ia;
-                const real* Tn_ = row8(T_cur, T_prv, u - 1) + ia;
-                real K;
-                if constexpr (sizeof(real) == 4)
-                    K = fd_K_rows_a(Ts_, Tc_, Tn_, r_ux[((u + 2) & 3) * RB + ib], r_uy[((u + 2) & 3) * RB + ib], chi);
-                else
-                    K = fd_K_rows(Ts_, Tc_, Tn_, row8(rho_cur, rho_prv, u - 3) + ia, row8(rho_cur, rho_prv, u - 2) + ia,
-                                        row8(rho_cur, rho_prv, u - 1) + ia, r_ux[((u + 2) & 3) * RB + ib],
-                                        r_uy[((u + 2) & 3) * RB + ib], chi);
-                r_h1[((u + 2) & 3) * RB + ib] = K;
-                r_Ts[((u + 2) & 3) * RB + ib] = Tc_[0] + a * K;
+            // C(k), k = j - 2: stage 1
+            {
+                const int k = j - 2;
+                if (k >= 1 && k <= njobs - 2 && colB != -99) {
+                    const int ia = colB + 2, ib = colB + 1;
+                    const real* Ts_ = row8(T_cur, T_prv, u - 3) + ia;
+                    const real* Tc_ = row8(T_cur, T_prv, u - 2) + ia;
+                    const real* Tn_ = row8(T_cur, T_prv, u - 1) + ia;
+                    real K;
+                    if constexpr (sizeof(real) == 4)
+                        K = fd_K_rows_a(Ts_, Tc_, Tn_, r_ux[((u + 2) & 3) * RB + ib], r_uy[((u + 2) & 3) * RB + ib],
+                                        chi);
+                    else
+                        K = fd_K_rows(Ts_, Tc_, Tn_, row8(rho_cur, rho_prv, u - 3) + ia,
+                                      row8(rho_cur, rho_prv, u - 2) + ia, row8(rho_cur, rho_prv, u - 1) + ia,
+                                      r_ux[((u + 2) & 3) * RB + ib], r_uy[((u + 2) & 3) * RB + ib], chi);
+                    r_h1[((u + 2) & 3) * RB + ib] = K;
+                    r_Ts[((u + 2) & 3) * RB + ib] = Tc_[0] + a * K;
+                }
+            }
+            // D(k), k = j - 4: stage 2 on own rows and columns
+            {
+                const int k = j - 4;
+                if (k >= 2 && k <= njobs - 3 && own_col) {
+                    const int ia = t + 2, ib = t + 1;
+                    real K;
+                    if constexpr (sizeof(real) == 4)
+                        K = fd_K_rows_a(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + u * RB + ib,
+                                        r_Ts + ((u + 1) & 3) * RB + ib, r_ux[u * RB + ib], r_uy[u * RB + ib],
+                                        chi);
+                    else
+                        K = fd_K_rows(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + u * RB + ib,
+                                      r_Ts + ((u + 1) & 3) * RB + ib, row8(rho_cur, rho_prv, u - 5) + ia,
+                                      row8(rho_cur, rho_prv, u - 4) + ia, row8(rho_cur, rho_prv, u - 3) + ia,
+                                      r_ux[u * RB + ib], r_uy[u * RB + ib], chi);
+                    const real v = row8(T_cur, T_prv, u - 4)[ia] + (real)0.5 * (r_h1[u * RB + ib] + K);
+                    int y = y_start - 2 + k;
+                    y = y >= ny ? y - ny : y;
+                    const int xg = x0 + t;
+                    real* p = Tnext + (long long)y * pitch + xg;
+                    *p = v;
+                    if (xg < ghost) p[nx] = v;
+                    if (xg >= nx - ghost) p[-nx] = v;
+                    if (!isfinite(v)) flags |= 1 << LB_ERR_NONFINITE;
+                }
+            }
+            // the stage of job j-1 has had its last reader (A at j-1, B at j)
+            if (j >= 1 && j <= njobs - 1 && !halo) {
+                __syncwarp();
+                if ((t & 31) == 0) mbar_arrive(&empty[(u + 3) & 3]);
             }
         }
-        // D(k), k = j - 4: stage 2 on own rows and columns
-        {
-            const int k = j - 4;
-            if (k >= 2 && k <= njobs - 3 && own_col) {
-                const int ia = t + 2, ib = t + 1;
-                real K;
-                if constexpr (sizeof(real) == 4)
-                    K = fd_K_rows_a(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + ((u + 0) & 3) * RB + ib,
-                                    r_Ts + ((u + 1) & 3) * RB + ib, r_ux[((u + 0) & 3) * RB + ib], r_uy[((u + 0) & 3) * RB + ib],
-                                    chi);
-                else
-                    K = fd_K_rows(r_Ts + ((u + 3) & 3) * RB + ib, r_Ts + ((u + 0) & 3) * RB + ib,
-                                        r_Ts + ((u + 1) & 3) * RB + ib, row8(rho_cur, rho_prv, u - 5) + ia,
-                                        row8(rho_cur, rho_prv, u - 4) + ia, row8(rho_cur, rho_prv, u - 3) + ia,
-                                        r_ux[((u + 0) & 3) * RB + ib], r_uy[((u + 0) & 3) * RB + ib], chi);
-                const real v = row8(T_cur, T_prv, u - 4)[ia] + (real)0.5 * (r_h1[((u + 0) & 3) * RB + ib] + K);
-                int y = y_start - 2 + k;
-                y = y >= ny ? y - ny : y;
-                const int xg = x0 + t;
-                real* p = Tnext + (long long)y * pitch + xg;
-                *p = v;
-                if (xg < ghost) p[nx] = v;
-                if (xg >= nx - ghost) p[-nx] = v;
-                if (!isfinite(v)) flags |= 1 << LB_ERR_NONFINITE;
-            }
-        }
-        // the stage of job j-1 has had its last reader (A at j-1, B at j)
-        if (j >= 1 && j <= njobs - 1 && !halo) {
-            __syncwarp();
-            if ((t & 31) == 0) mbar_arrive(&empty[(u + 3) & 3]);
-        }
-      }
         ph ^= 1u;
         real* x = rho_cur;
         rho_cur = rho_prv;

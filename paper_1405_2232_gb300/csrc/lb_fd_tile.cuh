@@ -4,7 +4,7 @@
 // Both kernels have the structure of lb_step_tile.cuh: tiles of 32 columns and a height
 // that balances them over the SMs, one site per thread, the ring around the tile in
 // threads of its own, launched before the kernel ahead of them ends (whose outputs they
-// read, so these are not __restrict__: see k_step_tile).
+// read: grid_wait).
 //  k_fd_front: rho (pulled f), T and psi of the tile and a ring of one site; force,
 //   u and the f collision of the tile.  STEP stores f and writes rho^n, u^n; else the
 //   moments outputs.
@@ -71,8 +71,7 @@ __global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
     const long long off = (long long)gy * kp.pitch + gx;
     real f[9], g[9], rho = 0, T = 0;
     const int at = (ly + 1) * WX + lx + 1;
-    grid_dependency_launch();
-    grid_dependency_wait();
+    grid_begin();
     if (need) {
         const PullAt<false> pull(kp, gx, gy);
 #pragma unroll
@@ -171,8 +170,7 @@ __global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
     tile_site<BX>(tid, by, lx, ly);
     const bool need = tid - BX * by < tile_ring(BX, by) && lx <= W && ly <= Hh;
     const int rx = x0 + lx, ry = y0 + ly;
-    grid_dependency_launch();
-    grid_dependency_wait();
+    grid_begin();
     for (int s = tid; s < W2 * (Hh + 4); s += (int)blockDim.x) {
         const int j = s / W2, i = s - j * W2;
         if (i >= W + 4) continue;

@@ -19,8 +19,8 @@
 // kernel is chosen for.  The strip kernels, which re-read and recompute less, take
 // the larger lattices (default_tile_rows in lb_capi.cu has the rule).  Per step, before
 // (strip kernel; cavity and channel: a tile kernel that pulled its sites twice) and now:
-// FP32 64^2 14.4 -> 2.2 us, 512^2 16.4 -> 7.2 us, FP16 1016 x 765 22.6 -> 18.5 us, FP64
-// 384 x 320 129 -> 90 us, 150 x 150 cavity 26 -> 19 us, 500 x 60 channel 32 -> 28 us.
+// FP32 64^2 14.4 -> 2.2 us, 512^2 16.4 -> 7.2 us, FP16 1016 x 765 22.6 -> 18.6 us, FP64
+// 384 x 320 130 -> 91 us, 150 x 150 cavity 31 -> 19 us, 500 x 60 channel 41 -> 29 us.
 //
 // Walls: nx-by-ny fluid nodes inside walls half a lattice spacing outside the
 // outermost nodes.  The populations are stored pre-collision at their own site and
@@ -58,9 +58,6 @@ __host__ __device__ constexpr size_t tile_smem_bytes(int bx, int by) {
 }
 
 constexpr size_t TILE_SM_SMEM = 228 * 1024;  // shared memory of an SM
-
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Post-collision populations of fluid node (gx, gy) to the nodes they reach
 // (cavity and channel).
@@ -246,8 +243,7 @@ __device__ __forceinline__ void tile_step(const typename Store<PREC>::elem* src,
 // One step per launch; grid (tiles in x, tiles in y), tile_threads(BX, by)
 // threads.  Launched so that its blocks may become resident while the step before
 // it still runs (programmatic dependent launch); they wait for its end before
-// they read anything.  So src is not __restrict__: that would say that nobody writes it
-// while the kernel runs, and let a load move above the wait.
+// they read anything (grid_wait: src is not __restrict__).
 template <int PREC, int BX, int WALLS, bool EQ24, int BMODE>
 __global__ void __launch_bounds__(tile_threads(BX, tile_max_by(BX)))
     k_step_tile(const typename Store<PREC>::elem* src, typename Store<PREC>::elem* __restrict__ dst,
@@ -257,8 +253,7 @@ __global__ void __launch_bounds__(tile_threads(BX, tile_max_by(BX)))
     real* s_psi = reinterpret_cast<real*>(tile_smem);
     real* s_psi2 = BMODE == BETA_MIXED ? s_psi + (BX + 2) * (by + 2) : s_psi;
     int flags = 0;
-    grid_dependency_launch();
-    grid_dependency_wait();
+    grid_begin();
     tile_step<PREC, BX, WALLS, EQ24, BMODE>(src, dst, kp, blockIdx.x * BX, kp.halo_rows + blockIdx.y * by, by, s_psi,
                                             s_psi2, flags);
     if (flags) atomicOr(kp.err, flags);
@@ -279,16 +274,16 @@ __global__ void __launch_bounds__(tile_threads(32, tile_max_by(32)))
     extern __shared__ __align__(16) unsigned char tile_smem[];
     real* s_psi = reinterpret_cast<real*>(tile_smem);
     real* s_psi2 = BMODE == BETA_MIXED ? s_psi + 34 * (by + 2) : s_psi;
-    grid_dependency_launch();
+    grid_launch();
     if ((int)blockIdx.x >= *n_tiles) {  // the grid covers the longest list
-        grid_dependency_wait();         // (no block ends before the step ahead of it)
+        grid_wait();         // (no block ends before the step ahead of it)
         return;
     }
     const BatchStepTile t = tiles[blockIdx.x];
     const BatchDomain& D = doms[t.domain];
     const long long off = D.off;
     int flags = 0;
-    grid_dependency_wait();
+    grid_wait();
     tile_step<PREC, 32, 0, EQ24, BMODE>(src + off, dst + off, D.kp, t.x0, t.y0, by, s_psi, s_psi2, flags);
     if (flags) atomicOr(D.kp.err, flags);
 }

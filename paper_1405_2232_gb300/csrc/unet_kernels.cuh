@@ -27,20 +27,9 @@
 
 namespace unk {
 
-// Programmatic dependent launch (both return at once without it).  grid_wait: what the
-// kernel before this one wrote is complete; before any access to global memory.
-// grid_launch: the next kernel's blocks may become resident; in a kernel that
-// allocates TMEM only once it holds it, since a waiting block of the next kernel
-// could otherwise hold the columns that this one needs to finish.
-// Inputs are not const __restrict__ and not read with __ldg: both say that nobody writes
-// them while the kernel runs, which the kernel ahead may do, and let a load move above
-// the wait.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_begin() {
-    grid_launch();
-    grid_wait();
-}
+using lbgb::grid_begin;
+using lbgb::grid_launch;
+using lbgb::grid_wait;
 
 typedef __nv_bfloat16 bf16;
 
