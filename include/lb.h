@@ -288,9 +288,9 @@ lb_status lb_halo_unpack(lb_ctx* ctx, int32_t face, const void* d_buf);
  * device stay usable.  A tiny limit makes the wait give up on purpose (tests
  * of the error path).  Small periodic lattices created without a tile shape step
  * on tiles or in one cluster of blocks, which do not wait on copies; while
- * a limit other than the default is set they run the strip kernel.  Applies to steps launched after the call; the tile
- * kernels and the batched solver do not wait and ignore it.  LB_ERR_ARG for
- * cycles < 0. */
+ * a limit other than the default is set they run the strip kernel.  Applies to
+ * steps launched after the call; the tile kernels and the batched solver do not
+ * wait and ignore it.  LB_ERR_ARG for cycles < 0. */
 lb_status lb_set_wait_limit(lb_ctx* ctx, int64_t cycles);
 
 /* Parameters the context runs with: a context created from them runs the same kernels.
@@ -372,7 +372,8 @@ lb_status lb_batch_run(lb_batch* b, double tol, int64_t K, int64_t max_steps, in
                        double* residual_out, int32_t* status_out);
 
 /* Host float64 rho and T [ny][nx] of domain d (either may be NULL).  For an
- * active domain this runs a check (the new residual reference).  Synchronises. */
+ * active domain this runs a check (the new residual reference), unless one has run
+ * at this time.  Synchronises. */
 lb_status lb_batch_fields(lb_batch* b, int32_t d, double* rho, double* T);
 
 /* Restart domain d from the float64 fields rho0, T0 [ny][nx] (host or device,
